@@ -40,9 +40,30 @@ struct Problem {
 //   a32     fp32 [BH][p][d]        key-side summary, feature-major
 //   aT16    fp16 [BH][d][p]        the same, transposed, as the tensor-core B operand
 //   part    fp32 partial results of a key-split stage 2 (tensor-core path only)
+//   efpad   E, F with padded rows (tensor-core path, N no multiple of 8); last, the only part that depends on N
 struct Layout {
-  size_t status, status_bytes, kpvp, kpvp_end, weight, a32, aT16, part, total;
+  size_t status, status_bytes, kpvp, kpvp_end, weight, a32, aT16, part, efpad, total;
 };
+
+// Ragged lengths (N no multiple of 8) pay a copy of E, F into rows on 16-byte boundaries (pad_rows.cuh).  Against the
+// CUDA-core kernels that is a gain at every length tried from 257 on; shorter ones keep the three-launch path.
+constexpr int kRaggedMin = 256;
+
+bool tensor_path_ok(const Problem& pr) {
+  if (pr.fp32) return false;
+  if (pr.d != 64 && pr.d != 128) return false;
+  if (pr.N % 8 && pr.N < kRaggedMin) return false;
+  if (pr.k % 64 || pr.k > 512) return false;
+  if (pr.kernel == FLURKA_PERFORMER && (pr.m % 64 || pr.m > 256)) return false;
+  return true;
+}
+
+// Elements between the rows of E, F as the tensor-core kernels read them: N, or whole 128-byte lines above it
+// where N is ragged and the rows are copied.
+int ef_pitch(const Problem& pr) { return pr.N % 8 ? (pr.N + 63) & ~63 : pr.N; }
+size_t efpad_bytes(const Problem& pr) {
+  return pr.N % 8 && tensor_path_ok(pr) ? (size_t)2 * pr.k * (pr.ef_per_head ? pr.H : 1) * ef_pitch(pr) * 2 : 0;
+}
 
 size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }
 
@@ -61,6 +82,7 @@ Layout make_layout(const Problem& pr, bool with_split_scratch = true) {
                                  ? k2_part_floats(pr.kernel == FLURKA_PERFORMER, pr.BH(), pr.d, pr.k, pr.p())
                                  : 0;
   L.part = off;   off = align256(off + part_floats * 4);
+  L.efpad = off;  off = align256(off + (with_split_scratch ? efpad_bytes(pr) : 0));
   L.total = off;
   return L;
 }
@@ -136,15 +158,6 @@ bool overlaps(const void* a, size_t na, const void* b, size_t nb) {
   return x < y + nb && y < x + na;
 }
 
-bool tensor_path_ok(const Problem& pr) {
-  if (pr.fp32) return false;
-  if (pr.d != 64 && pr.d != 128) return false;
-  if (pr.N % 8) return false;       // row pitch of E, F (N elements) must be a multiple of 16 bytes for TMA
-  if (pr.k % 64 || pr.k > 512) return false;
-  if (pr.kernel == FLURKA_PERFORMER && (pr.m % 64 || pr.m > 256)) return false;
-  return true;
-}
-
 // The library-owned workspace grows in stream order: the old block is released and the new one
 // obtained on the call's stream, so nothing waits on the host and earlier work queued on that
 // stream still finds its block.
@@ -180,6 +193,20 @@ int check_device() {
     return FLURKA_ERR_DEVICE;
   }
   return major == 10 ? FLURKA_OK : FLURKA_ERR_DEVICE;
+}
+
+// Copies E, F into `pad` with padded rows where the tensor-core kernels need that, and points *E, *F there.
+int pad_projections(const Problem& pr, char* pad, const void** E, const void** F, cudaStream_t st, int* launches) {
+  if (pr.N % 8 == 0) return FLURKA_OK;
+  const int rows = pr.k * (pr.ef_per_head ? pr.H : 1);
+  char* Fp = pad + efpad_bytes(pr) / 2;
+  int cuda_err = 0;
+  const int rc = launch_pad_rows(*E, *F, pad, Fp, rows, pr.N, ef_pitch(pr), st, &cuda_err);
+  if (rc) { g_last_cuda_error = cuda_err; return rc; }
+  *E = pad;
+  *F = Fp;
+  ++*launches;
+  return FLURKA_OK;
 }
 
 template <typename T>
@@ -311,8 +338,11 @@ int run_pipeline(const Problem& pr, const Layout& L, char* ws, const void* Q, co
   auto stage1 = [&](float* kpvp, int* status, int* n) -> int {
     if (tc1) {
       int cuda_err = 0;
-      int rc = launch_k1(*tc, K, V, E, F, kpvp, pr.BH(), pr.seq_major_heads(), pr.N, pr.d, pr.k, status, st, &cuda_err,
-                         pr.ef_heads());
+      const void *Ep = E, *Fp = F;
+      int rc = pad_projections(pr, ws + L.efpad, &Ep, &Fp, st, n);
+      if (rc) return rc;
+      rc = launch_k1(*tc, K, V, Ep, Fp, kpvp, pr.BH(), pr.seq_major_heads(), pr.N, pr.d, pr.k, status, st, &cuda_err,
+                     pr.ef_heads(), ef_pitch(pr));
       if (rc) { g_last_cuda_error = cuda_err; return rc; }
       ++*n;
       return FLURKA_OK;
@@ -715,7 +745,11 @@ int fused_pipeline(const Problem& pr, int dm, const FusedLayout& FL, char* ws, c
       // dm/64 pseudo-heads of width 64, then W^K, W^V on the k contracted rows
       rc = launch_k0_query_map(*tc, Xq, Wq, qp, pr.B, pr.N, pr.H, dm, pr.d, status, st, &cuda_err);
       if (rc) { g_last_cuda_error = cuda_err; return rc; }
-      rc = launch_k1(*tc, Xk, Xv, E, F, kt, pr.B * (dm / 64), dm / 64, pr.N, 64, pr.k, status, st, &cuda_err);
+      const void *Ep = E, *Fp = F;
+      rc = pad_projections(pr, ws + FL.L.efpad, &Ep, &Fp, st, n);
+      if (rc) return rc;
+      rc = launch_k1(*tc, Xk, Xv, Ep, Fp, kt, pr.B * (dm / 64), dm / 64, pr.N, 64, pr.k, status, st, &cuda_err, 0,
+                     ef_pitch(pr));
       if (rc) { g_last_cuda_error = cuda_err; return rc; }
       rc = launch_k0_key_value_maps(*tc, kt, (__nv_bfloat16*)(ws + FL.a3), Wk, Wv, kpvp, pr.B, pr.H, dm, pr.d, pr.k,
                                     status, st, &cuda_err);
@@ -810,7 +844,7 @@ namespace {
 // memset), then dK', dV' [2][BH][k][d]; all fp32.
 struct BackwardLayout {
   Layout L;
-  size_t da, dab_bytes, db, dkpvp, abf, split, rowstat, total;
+  size_t da, dab_bytes, db, dkpvp, abf, split, rowstat, efpad, total;
 };
 
 // the query side of the backward has a tensor-core kernel for d = 64 (PERFORMER: any feature count the
@@ -837,6 +871,8 @@ BackwardLayout make_backward_layout(const Problem& pr) {
     off = align256(off + (size_t)pr.BH() * ((pr.N + 127) / 128) * 128 * 8);
   b.split = off;
   if (tensor_path_ok(pr)) off = align256(off + (size_t)2 * pr.k * 2 * pr.BH() * pr.d * 2);      // dK', dV' as two bf16 terms
+  b.efpad = off;
+  off = align256(off + efpad_bytes(pr));
   b.total = off;
   return b;
 }
@@ -861,8 +897,12 @@ int backward_pipeline(const Problem& pr, const BackwardLayout& BL, char* ws, con
   // the forward's stages 1 and 2 again: K', V', a_i, b_i (or z_i)
   int rc = FLURKA_OK;
   int cuda_err = 0;
+  const void *Ep = E, *Fp = F;           // what the tensor-core kernels read: E, F, or copies with padded rows
   if (tc) {
-    rc = launch_k1(*tc, K, V, E, F, kpvp, pr.BH(), smh, pr.N, pr.d, pr.k, (int*)(ws + L.status), st, &cuda_err, efh);
+    rc = pad_projections(pr, ws + BL.efpad, &Ep, &Fp, st, launches);
+    if (rc) return rc;
+    rc = launch_k1(*tc, K, V, Ep, Fp, kpvp, pr.BH(), smh, pr.N, pr.d, pr.k, (int*)(ws + L.status), st, &cuda_err, efh,
+                   ef_pitch(pr));
     if (rc) { g_last_cuda_error = cuda_err; return rc; }
     ++*launches;
   } else {
@@ -908,10 +948,17 @@ int backward_pipeline(const Problem& pr, const BackwardLayout& BL, char* ws, con
     ++*launches;
   }
   if (tc && efh == 0) {
-    rc = launch_k5(*tc, E, F, K, V, dkpvp, (__nv_bfloat16*)(ws + BL.split), dK, dV, dE, dF, pr.BH(), smh, pr.N, pr.d, pr.k,
-                   (int*)(ws + L.status), st, &cuda_err);
+    const bool padded = Ep != E;
+    void *dEp = padded ? (void*)Ep : dE, *dFp = padded ? (void*)Fp : dF;   // the copies are not read again after this
+    rc = launch_k5(*tc, Ep, Fp, K, V, dkpvp, (__nv_bfloat16*)(ws + BL.split), dK, dV, dEp, dFp, pr.BH(), smh, pr.N, pr.d,
+                   pr.k, ef_pitch(pr), (int*)(ws + L.status), st, &cuda_err);
     if (rc) { g_last_cuda_error = cuda_err; return rc; }
     *launches += 3;
+    if (padded) {
+      rc = launch_unpad_rows(dEp, dFp, dE, dF, pr.k, pr.N, ef_pitch(pr), st, &cuda_err);
+      if (rc) { g_last_cuda_error = cuda_err; return rc; }
+      ++*launches;
+    }
   } else {
     dim3 grid((pr.N + 31) / 32, pr.BH(), 2);
     simt_bwd_inputs<T><<<grid, 256, 0, st>>>((const T*)E, (const T*)F, dkpvp, (T*)dK, (T*)dV, pr.BH(), pr.N, pr.d,

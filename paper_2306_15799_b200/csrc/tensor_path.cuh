@@ -14,6 +14,7 @@
 #include "k4_bwd_query_side.cuh"
 #include "k5_bwd_projections.cuh"
 #include "k6_bwd_key_side.cuh"
+#include "pad_rows.cuh"
 
 namespace flurka {
 
@@ -64,20 +65,22 @@ inline EncodeTiledFn encode_tiled_fn() {
 struct CachedMap {
   CUtensorMap map;
   const void* ptr = nullptr;
-  unsigned long long key[8] = {0, 0, 0, 0, 0, 0, 0, 0};
+  unsigned long long key[9] = {0, 0, 0, 0, 0, 0, 0, 0, 0};
   bool valid = false;
 };
 
 // rank <= 3; dims/box in elements (innermost first); 128-byte swizzle; out-of-range reads give zero.
+// pitch: elements between rows where they are further apart than dims[0] (0: dense)
 inline bool encode_map(CachedMap* cm, CUtensorMapDataType dt, int esize, int rank, const void* ptr,
-                       const unsigned long long* dims, const unsigned* box) {
-  unsigned long long key[8] = {(unsigned long long)dt, (unsigned long long)rank, dims[0], dims[1],
-                               rank > 2 ? dims[2] : 1ull, box[0], box[1], rank > 2 ? box[2] : 1u};
+                       const unsigned long long* dims, const unsigned* box, unsigned long long pitch = 0) {
+  if (!pitch) pitch = dims[0];
+  unsigned long long key[9] = {(unsigned long long)dt, (unsigned long long)rank, dims[0], dims[1],
+                               rank > 2 ? dims[2] : 1ull, box[0], box[1], rank > 2 ? box[2] : 1u, pitch};
   if (cm->valid && cm->ptr == ptr && memcmp(key, cm->key, sizeof(key)) == 0) return true;
   EncodeTiledFn fn = encode_tiled_fn();
   if (!fn) return false;
   cuuint64_t gdim[3] = {dims[0], dims[1], rank > 2 ? dims[2] : 1};
-  cuuint64_t gstride[2] = {dims[0] * (cuuint64_t)esize, dims[0] * dims[1] * (cuuint64_t)esize};
+  cuuint64_t gstride[2] = {pitch * (cuuint64_t)esize, pitch * dims[1] * (cuuint64_t)esize};
   cuuint32_t bdim[3] = {box[0], box[1], rank > 2 ? box[2] : 1};
   cuuint32_t estr[3] = {1, 1, 1};
   CUresult r = fn(&cm->map, dt, (cuuint32_t)rank, const_cast<void*>(ptr), gdim, gstride, bdim, estr,
@@ -138,6 +141,25 @@ inline int TensorContext::sm_count() {
   return (lim > 0 && lim < n) ? lim : n;
 }
 
+// ---- E, F with rows on 16-byte boundaries (N no multiple of 8), and dE, dF back ------------------------------
+inline int launch_pad_rows(const void* E, const void* F, void* Ep, void* Fp, int rows, int N, int pitch, cudaStream_t st,
+                           int* cuda_err) {
+  dim3 grid((N + 2047) / 2048, rows < 65535 ? rows : 65535, 2);
+  pad_rows<<<grid, 256, 0, st>>>((const uint16_t*)E, (const uint16_t*)F, (uint16_t*)Ep, (uint16_t*)Fp, rows, N, pitch);
+  cudaError_t e = cudaGetLastError();
+  if (e != cudaSuccess) { *cuda_err = (int)e; return -6; }
+  return 0;
+}
+inline int launch_unpad_rows(const void* dEp, const void* dFp, void* dE, void* dF, int rows, int N, int pitch,
+                             cudaStream_t st, int* cuda_err) {
+  const long long blocks = ((long long)rows * N + 2047) / 2048;
+  dim3 grid((unsigned)(blocks < 65535 ? blocks : 65535), 1, 2);
+  unpad_rows<<<grid, 256, 0, st>>>((const uint16_t*)dEp, (const uint16_t*)dFp, (uint16_t*)dE, (uint16_t*)dF, rows, N, pitch);
+  cudaError_t e = cudaGetLastError();
+  if (e != cudaSuccess) { *cuda_err = (int)e; return -6; }
+  return 0;
+}
+
 // Sequence splits of stage 1: as few as fill the machine once.  Every split adds a full copy of
 // the output to the fp32 reduction (measured: the reduce-add traffic of all CTAs drains at about
 // 2.5 TB/s after the last MMA, so more, shorter CTAs lose more in that tail than they gain).
@@ -151,9 +173,10 @@ inline int k1_choose_nsplit(int sms, int units, int chunks) {
 // ---- stage 1: K' = E K, V' = F V into kpvp (already zeroed) ----------------------------------
 // H > 0: K, V are [B,N,H,d] (H heads merged into the row); H == 0: [B,H,N,d]
 // ef_heads > 0: E, F are [ef_heads][k][N] (one pair per head; head index = bh % ef_heads)
+// ef_pitch: elements between the rows of E, F (N, or a multiple of 8 above it)
 inline int launch_k1(TensorContext& tc, const void* K, const void* V, const void* E, const void* F, float* kpvp,
                      int BH, int H, int N, int d, int k, int* status, cudaStream_t st, int* cuda_err,
-                     int ef_heads = 0) {
+                     int ef_heads, int ef_pitch) {
   TensorMaps& tm = tc.maps;
   const unsigned long long dE[3] = {(unsigned long long)N, (unsigned long long)k,
                                     (unsigned long long)(ef_heads > 0 ? ef_heads : 1)};
@@ -164,8 +187,8 @@ inline int launch_k1(TensorContext& tc, const void* K, const void* V, const void
   const unsigned bX[3] = {64, 64, 1};
   const unsigned long long dO[3] = {(unsigned long long)d, (unsigned long long)k, (unsigned long long)2 * BH};
   const unsigned bO[3] = {32, 32, 1};
-  if (!encode_map(&tm.E, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, 3, E, dE, bE) ||
-      !encode_map(&tm.F, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, 3, F, dE, bE) ||
+  if (!encode_map(&tm.E, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, 3, E, dE, bE, ef_pitch) ||
+      !encode_map(&tm.F, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, 3, F, dE, bE, ef_pitch) ||
       !encode_map(&tm.K, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, 3, K, dX, bX) ||
       !encode_map(&tm.V, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, 3, V, dX, bX) ||
       !encode_map(&tm.kpvp, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, 3, kpvp, dO, bO)) {
@@ -490,9 +513,11 @@ inline int launch_k4(TensorContext& tc, bool performer, const void* Q, const voi
 
 // ---- backward of the down-projection: dK, dV, dE, dF from the fp32 dK', dV' (shared E, F) -------------
 // split: scratch for the two bf16 terms of dK', dV', [2][k][2][BH][d]
+// ef_pitch: elements between the rows of E, F, dE, dF.  When it is not N, E, F are padded copies that the last
+// product overwrites with dE, dF (dE == E, dF == F), and the caller copies those to their dense form.
 inline int launch_k5(TensorContext& tc, const void* E, const void* F, const void* K, const void* V, const float* dkpvp,
                      __nv_bfloat16* split, void* dK, void* dV, void* dE, void* dF, int BH, int H, int N, int d, int k,
-                     int* status, cudaStream_t st, int* cuda_err) {
+                     int ef_pitch, int* status, cudaStream_t st, int* cuda_err) {
   TensorMaps& tm = tc.maps;
   const unsigned long long hd = (unsigned long long)BH * d;
   const unsigned long long dEF[2] = {(unsigned long long)N, (unsigned long long)k};
@@ -503,11 +528,11 @@ inline int launch_k5(TensorContext& tc, const void* E, const void* F, const void
   const unsigned long long dS[3] = {2 * hd, (unsigned long long)k, 2};
   const unsigned bS64[3] = {64, 64, 1}, bS128[3] = {64, 128, 1};
   const CUtensorMapDataType bf = CU_TENSOR_MAP_DATA_TYPE_BFLOAT16;
-  if (!encode_map(&tm.bE, bf, 2, 2, E, dEF, bEF) || !encode_map(&tm.bF, bf, 2, 2, F, dEF, bEF) ||
+  if (!encode_map(&tm.bE, bf, 2, 2, E, dEF, bEF, ef_pitch) || !encode_map(&tm.bF, bf, 2, 2, F, dEF, bEF, ef_pitch) ||
       !encode_map(&tm.bK, bf, 2, 3, K, dKV, bKV) || !encode_map(&tm.bV, bf, 2, 3, V, dKV, bKV) ||
       !encode_map(&tm.split64, bf, 2, 3, split, dS, bS64) || !encode_map(&tm.split128, bf, 2, 3, split, dS, bS128) ||
       !encode_map(&tm.gK, bf, 2, 3, dK, dKV, bGK) || !encode_map(&tm.gV, bf, 2, 3, dV, dKV, bGK) ||
-      !encode_map(&tm.gE, bf, 2, 2, dE, dEF, bGE) || !encode_map(&tm.gF, bf, 2, 2, dF, dEF, bGE)) {
+      !encode_map(&tm.gE, bf, 2, 2, dE, dEF, bGE, ef_pitch) || !encode_map(&tm.gF, bf, 2, 2, dF, dEF, bGE, ef_pitch)) {
     *cuda_err = (int)cudaErrorInvalidValue;
     return -6;
   }

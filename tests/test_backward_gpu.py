@@ -227,3 +227,16 @@ def test_backward_argument_errors():
     assert lib.flurka_backward(*base, *dims, None, *outs[1:], None) == -1
     assert lib.flurka_backward(*base, *dims, *outs, None) == 0
     assert binding.flurka_backward_workspace_bytes(RNN, torch.float32, 1, 1, 32, 8, 4, 0) > 0
+
+
+@pytest.mark.parametrize("w,layout,per_head", [
+    (Workload("bwd_odd_n257", PERFORMER, "bf16", 1, 2, 257, 64, 64, 64, 351), "bhnd", False),
+    (Workload("bwd_odd_k256", PERFORMER, "bf16", 2, 2, 643, 64, 256, 256, 352), "bnhd", False),
+    (Workload("bwd_odd_d128", PERFORMER, "bf16", 1, 2, 390, 128, 128, 128, 353), "bhnd", False),
+    (Workload("bwd_odd_rnn", RNN, "bf16", 1, 3, 1001, 64, 192, 0, 354), "bhnd", False),
+    (Workload("bwd_odd_per_head", PERFORMER, "bf16", 2, 2, 301, 64, 64, 128, 355), "bhnd", True),
+], ids=lambda v: v.name if hasattr(v, "name") else str(v))
+def test_backward_of_ragged_lengths_on_the_tensor_path(w, layout, per_head):
+    """N no multiple of 8: E, F are read from padded copies, dE, dF leave through them."""
+    _check(w, layout=layout, per_head=per_head)
+    assert binding.flurka_last_path() == binding.PATH_TENSOR

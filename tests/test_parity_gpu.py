@@ -460,3 +460,30 @@ def test_stage1_pairs_and_single_ctas_match_oracle(shape):
                     assert np.abs(got - want).max() <= 3e-5 * max(1.0, np.abs(want).max())
         got = out.cpu().double().numpy()
         pu.assert_close(got[B - 1, H - 1], pu.oracle_head(x, w, B - 1, H - 1), "bf16", "stage 1 %s" % ("pairs" if on else "single"))
+
+
+@pytest.mark.parametrize("w,layout,per_head", [
+    # one position past a multiple of 8, 64, 128; an even remainder; the shortest ragged length of the tensor path
+    (_wl("odd_perf_n257", PERFORMER, "bf16", 1, 2, 257, 64, 64, 64, 141), "bhnd", False),
+    (_wl("odd_perf_pairs", PERFORMER, "bf16", 2, 4, 1281, 64, 256, 256, 142), "bnhd", False),
+    (_wl("odd_perf_d128", PERFORMER, "bf16", 1, 3, 1003, 128, 128, 128, 143), "bhnd", False),
+    (_wl("odd_rnn_n262", RNN, "bf16", 2, 2, 262, 64, 128, 0, 144), "bnhd", False),
+    (_wl("odd_perf_per_head", PERFORMER, "bf16", 2, 2, 519, 64, 64, 128, 145), "bhnd", True),
+], ids=lambda v: v.name if hasattr(v, "name") else str(v))
+def test_ragged_lengths_on_the_tensor_path(w, layout, per_head):
+    """N no multiple of 8: E, F are read from copies whose rows start on 16-byte boundaries."""
+    x = synth.make_inputs(w)
+    if per_head:
+        gen = torch.Generator().manual_seed(w.seed)
+        for name in ("E", "F"):
+            x[name] = (torch.randn(w.H, w.k, w.N, generator=gen, dtype=torch.float64) * float(w.k) ** -0.5).bfloat16()
+    dev = pu.to_device(x)
+    t = (lambda a: a.transpose(1, 2).contiguous()) if layout == "bnhd" else (lambda a: a)
+    out = binding.flurka_forward(t(dev["Q"]), t(dev["K"]), t(dev["V"]), dev["E"], dev["F"], dev["W"], w.variant, layout=layout)
+    torch.cuda.synchronize()
+    assert binding.flurka_last_status() == 0 and binding.flurka_last_path() == binding.PATH_TENSOR
+    got = t(out).cpu().double().numpy()
+    for b in range(w.B):
+        for h in range(w.H):
+            one = dict(x, E=x["E"][h], F=x["F"][h]) if per_head else x
+            pu.assert_close(got[b, h], pu.oracle_head(one, w, b, h), "bf16", "%s head (%d,%d)" % (w.name, b, h))
