@@ -209,56 +209,76 @@ int pad_projections(const Problem& pr, char* pad, const void** E, const void** F
   return FLURKA_OK;
 }
 
+template <typename T, int R, int NB>
+void launch_simt_down_project_as(const Problem& pr, const void* K, const void* V, const void* E, const void* Fin,
+                                 float* kpvp, cudaStream_t st) {
+  // enough sequence splits for about four blocks per SM; a split is a multiple of one step
+  const int jt = (pr.k + 16 * R - 1) / (16 * R);
+  int nsplit = 4 * 148 / (jt * pr.BH() * 2);
+  const int max_split = (pr.N + kSimtTN - 1) / kSimtTN;
+  nsplit = std::max(1, std::min(nsplit, std::min(max_split, 16384)));
+  int chunk = (pr.N + nsplit - 1) / nsplit;
+  chunk = (chunk + kSimtTN - 1) / kSimtTN * kSimtTN;
+  nsplit = (pr.N + chunk - 1) / chunk;
+  dim3 grid(jt, pr.BH(), 2 * nsplit);
+  simt_down_project<T, R, NB><<<grid, kSimtThreads, 0, st>>>((const T*)K, (const T*)V, (const T*)E, (const T*)Fin, kpvp,
+                                                           pr.BH(), pr.N, pr.d, pr.k, nsplit, chunk,
+                                                           pr.seq_major_heads(), pr.ef_heads());
+}
+
 template <typename T>
 int launch_simt_down_project(const Problem& pr, const void* K, const void* V, const void* E,
                              const void* F, float* kpvp, cudaStream_t st, int* launches) {
-  // enough sequence splits to fill the machine; each split is a multiple of the 32-wide tile
-  const int jt = (pr.k + 31) / 32;
-  int nsplit = (4 * 148 + jt * pr.BH() * 2 - 1) / (jt * pr.BH() * 2);
-  const int max_split = (pr.N + 255) / 256;
-  if (nsplit > max_split) nsplit = max_split;
-  if (nsplit < 1) nsplit = 1;
-  if (nsplit > 16384) nsplit = 16384;
-  int chunk = (pr.N + nsplit - 1) / nsplit;
-  chunk = (chunk + 31) / 32 * 32;
-  nsplit = (pr.N + chunk - 1) / chunk;
-  dim3 grid(jt, pr.BH(), 2 * nsplit);
-  simt_down_project<T><<<grid, 256, 0, st>>>((const T*)K, (const T*)V, (const T*)E, (const T*)F, kpvp,
-                                            pr.BH(), pr.N, pr.d, pr.k, nsplit, chunk, pr.seq_major_heads(),
-                                            pr.ef_heads());
+  // rows per block: the largest tile that k fills (the larger the tile, the fewer shared memory reads per FMA)
+  const bool wide = pr.d > 64;
+  if (pr.k > 64) wide ? launch_simt_down_project_as<T, 8, 2>(pr, K, V, E, F, kpvp, st)
+                      : launch_simt_down_project_as<T, 8, 1>(pr, K, V, E, F, kpvp, st);
+  else if (pr.k > 32) wide ? launch_simt_down_project_as<T, 4, 2>(pr, K, V, E, F, kpvp, st)
+                           : launch_simt_down_project_as<T, 4, 1>(pr, K, V, E, F, kpvp, st);
+  else wide ? launch_simt_down_project_as<T, 2, 2>(pr, K, V, E, F, kpvp, st)
+            : launch_simt_down_project_as<T, 2, 1>(pr, K, V, E, F, kpvp, st);
   ++*launches;
   return FLURKA_OK;
+}
+
+template <typename T, bool P, bool kKeySide, int R, int NB>
+int launch_simt_attend_as(const Problem& pr, const void* Q, const void* W, const float* kpvp, float* weight, float* a32,
+                          __half* aT16, void* out, cudaStream_t st) {
+  const size_t smem = simt_attend_smem(R, NB, pr.d);
+  auto fn = simt_attend<T, P, kKeySide, R, NB>;
+  if (smem > 48 * 1024) {
+    cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return cuda_fail(e);
+  }
+  dim3 grid(((kKeySide ? pr.p() : pr.N) + 16 * R - 1) / (16 * R), pr.BH());
+  fn<<<grid, kSimtThreads, smem, st>>>((const T*)Q, (const T*)W, kpvp, weight, a32, aT16, (T*)out, pr.BH(), pr.N, pr.d,
+                                  pr.k, pr.p(), pr.seq_major_heads());
+  return FLURKA_OK;
+}
+
+template <typename T, bool P, bool kKeySide>
+int launch_simt_attend(const Problem& pr, const void* Q, const void* W, const float* kpvp, float* weight, float* a32,
+                       __half* aT16, void* out, cudaStream_t st, int* launches) {
+  // 128 rows per block as soon as that gives every SM a block; 32 below, where the length of one block is the time
+  const bool big = (long long)(((kKeySide ? pr.p() : pr.N) + 127) / 128) * pr.BH() >= 148;
+  ++*launches;
+  if (pr.d > 64)
+    return big ? launch_simt_attend_as<T, P, kKeySide, 8, 2>(pr, Q, W, kpvp, weight, a32, aT16, out, st)
+               : launch_simt_attend_as<T, P, kKeySide, 2, 2>(pr, Q, W, kpvp, weight, a32, aT16, out, st);
+  return big ? launch_simt_attend_as<T, P, kKeySide, 8, 1>(pr, Q, W, kpvp, weight, a32, aT16, out, st)
+             : launch_simt_attend_as<T, P, kKeySide, 2, 1>(pr, Q, W, kpvp, weight, a32, aT16, out, st);
 }
 
 template <typename T, bool P>
 int launch_simt_key_side(const Problem& pr, const float* kpvp, const void* W, float* weight, float* a32,
                          __half* aT16, cudaStream_t st, int* launches) {
-  const size_t smem = ((size_t)8 * pr.k + 32 * (pr.d + 1)) * 4;
-  auto fn = simt_key_side<T, P>;
-  if (smem > 24 * 1024) {
-    cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return cuda_fail(e);
-  }
-  dim3 grid((pr.p() + 7) / 8, pr.BH());
-  fn<<<grid, 256, smem, st>>>(kpvp, (const T*)W, weight, a32, aT16, pr.BH(), pr.d, pr.k, pr.p());
-  ++*launches;
-  return FLURKA_OK;
+  return launch_simt_attend<T, P, true>(pr, nullptr, W, kpvp, weight, a32, aT16, nullptr, st, launches);
 }
 
 template <typename T, bool P>
-int launch_simt_query_side(const Problem& pr, const void* Q, const void* W, const float* weight,
-                           const float* a32, void* out, cudaStream_t st, int* launches) {
-  const size_t smem = ((size_t)32 * (pr.d + 1) + 32 * pr.d) * 4;
-  dim3 grid((pr.N + 31) / 32, pr.BH());
-  if (smem > 24 * 1024) {   // static (16.6 KB) + dynamic may pass the 48 KB default limit
-    cudaError_t e = cudaFuncSetAttribute(simt_query_side<T, P>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)smem);
-    if (e != cudaSuccess) return cuda_fail(e);
-  }
-  simt_query_side<T, P><<<grid, 256, smem, st>>>((const T*)Q, (const T*)W, weight, a32, (T*)out, pr.N,
-                                                 pr.d, pr.p(), pr.seq_major_heads());
-  ++*launches;
-  return FLURKA_OK;
+int launch_simt_query_side(const Problem& pr, const void* Q, const void* W, float* weight, float* a32, void* out,
+                           cudaStream_t st, int* launches) {
+  return launch_simt_attend<T, P, false>(pr, Q, W, nullptr, weight, a32, nullptr, out, st, launches);
 }
 
 template <typename T>

@@ -44,263 +44,319 @@ __device__ __forceinline__ void store_out(float* p, float v) { *p = v; }
 __device__ __forceinline__ void store_out(__nv_bfloat16* p, float v) { *p = __float2bfloat16_rn(v); }
 
 // ---------------------------------------------------------------------------------------------
-// Stage 1.  grid = (ceil(k/32), B*H, 2*nsplit); block = 256.
+// Building blocks.  A block is 256 threads, ty = tid / 16, tx = tid % 16; a thread owns the R rows ty + 16 r and, in
+// each of NB 64-wide column blocks, the columns 4 tx .. 4 tx + 3.  Both kinds of product below read shared memory as
+// 16-byte pieces only: with R = 8, 12 loads per 128 FFMA of a warp.  B = 2, H = 8, N = 4096, d = 64, k = m = 256, fp32:
+// stage 1 443 -> 117 us, stage 3 617 -> 150 us against scalar reads and four rows per thread.  Tried and slower:
+// 8 x 8 outputs per thread (half the warps: 120 and 164 us), two-wide FMA on pairs of contraction steps (147 and
+// 215 us: it has no higher rate than FFMA and twice the accumulator registers).  Smaller R keeps more blocks busy
+// where there are few rows.
+// ---------------------------------------------------------------------------------------------
+constexpr int kSimtThreads = 256;
+
+__device__ __forceinline__ float4 simt_load4(const float* p) { return *reinterpret_cast<const float4*>(p); }
+__device__ __forceinline__ float4 simt_load4(const __nv_bfloat16* p) {
+  const uint2 v = *reinterpret_cast<const uint2*>(p);       // a bf16 is the upper half of an fp32
+  return make_float4(__uint_as_float(v.x << 16), __uint_as_float(v.x & 0xffff0000u), __uint_as_float(v.y << 16),
+                     __uint_as_float(v.y & 0xffff0000u));
+}
+// the first `live` (<= 0: none) of four consecutive elements, zeros after them; `vec`: p is aligned for one load
+template <typename T>
+__device__ __forceinline__ float4 simt_load_row4(const T* p, int live, bool vec) {
+  if (vec && live >= 4) return simt_load4(p);
+  float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+  if (live > 0) v.x = to_f32(p[0]);
+  if (live > 1) v.y = to_f32(p[1]);
+  if (live > 2) v.z = to_f32(p[2]);
+  if (live > 3) v.w = to_f32(p[3]);
+  return v;
+}
+// floats between the rows of a tile that is read row-wise in 16-byte pieces: an odd number of pieces, so that eight
+// consecutive rows fall into different banks
+__host__ __device__ __forceinline__ int simt_ld(int cols) { return (((cols + 3) >> 2) | 1) << 2; }
+
+// acc[r][..] += A[row][0 .. kk) B[0 .. kk)[cols]; A rows `lda` floats apart, B rows 64 NB; kk a multiple of 4
+template <int R, int NB>
+__device__ __forceinline__ void simt_product(float (&acc)[R][NB * 4], const float* A, int lda, const float* Bt, int kk) {
+  const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
+  for (int t = 0; t < kk; t += 4) {
+    float4 b[4][NB];
+#pragma unroll
+    for (int u = 0; u < 4; ++u)
+#pragma unroll
+      for (int q = 0; q < NB; ++q) b[u][q] = *reinterpret_cast<const float4*>(Bt + (t + u) * (64 * NB) + q * 64 + tx * 4);
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+      const float4 a = *reinterpret_cast<const float4*>(A + (ty + 16 * r) * lda + t);
+      const float av[4] = {a.x, a.y, a.z, a.w};
+#pragma unroll
+      for (int u = 0; u < 4; ++u)
+#pragma unroll
+        for (int q = 0; q < NB; ++q) {
+          acc[r][q * 4 + 0] = fmaf(av[u], b[u][q].x, acc[r][q * 4 + 0]);
+          acc[r][q * 4 + 1] = fmaf(av[u], b[u][q].y, acc[r][q * 4 + 1]);
+          acc[r][q * 4 + 2] = fmaf(av[u], b[u][q].z, acc[r][q * 4 + 2]);
+          acc[r][q * 4 + 3] = fmaf(av[u], b[u][q].w, acc[r][q * 4 + 3]);
+        }
+    }
+  }
+}
+
+// s[r][f] += X[row] . Y[tx + 16 f] over `cols` (a multiple of 4) columns; rows of both `ld` floats apart
+template <int R>
+__device__ __forceinline__ void simt_dots(float (&s)[R][4], const float* X, const float* Y, int ld, int cols) {
+  const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
+  for (int c = 0; c < cols; c += 4) {
+    float4 y[4];
+#pragma unroll
+    for (int f = 0; f < 4; ++f) y[f] = *reinterpret_cast<const float4*>(Y + (tx + 16 * f) * ld + c);
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+      const float4 x = *reinterpret_cast<const float4*>(X + (ty + 16 * r) * ld + c);
+#pragma unroll
+      for (int f = 0; f < 4; ++f) {
+        s[r][f] = fmaf(x.x, y[f].x, s[r][f]);
+        s[r][f] = fmaf(x.y, y[f].y, s[r][f]);
+        s[r][f] = fmaf(x.z, y[f].z, s[r][f]);
+        s[r][f] = fmaf(x.w, y[f].w, s[r][f]);
+      }
+    }
+  }
+}
+
+// ---------------------------------------------------------------------------------------------
+// Stage 1.  grid = (ceil(k / 16R), B*H, 2*nsplit).
 // blockIdx.z = t*nsplit + s: t = 0 projects K with E, t = 1 projects V with F; split s covers the
 // sequence range [s*chunk, min(N,(s+1)*chunk)).  Partial sums are added into KpVp (zeroed before).
 // KpVp layout: [2][B*H][k][d] fp32.  E, F: [k][N] shared by all heads, or [H][k][N] (ef_heads = H).
+// The next 32 positions travel in registers while the current ones are multiplied.
 // ---------------------------------------------------------------------------------------------
-template <typename T>
-__global__ void __launch_bounds__(256)
+constexpr int kSimtTN = 32;            // sequence positions per step
+template <typename T, int R, int NB>
+__global__ void __launch_bounds__(kSimtThreads, R == 8 && NB == 2 ? 1 : 2)
 simt_down_project(const T* __restrict__ Kin, const T* __restrict__ Vin, const T* __restrict__ E,
-                  const T* __restrict__ F, float* __restrict__ KpVp, int BH, int N, int d, int k,
+                  const T* __restrict__ Fin, float* __restrict__ KpVp, int BH, int N, int d, int k,
                   int nsplit, int chunk, int seq_major_heads, int ef_heads) {
-  constexpr int TJ = 32, TN = 32;
-  __shared__ float Ps[TJ][TN + 1];
-  __shared__ float Xs[TN][128];
-
-  const int t = blockIdx.z / nsplit;
-  const int s = blockIdx.z % nsplit;
-  const int bh = blockIdx.y;
-  const int j0 = blockIdx.x * TJ;
+  constexpr int kRows = 16 * R, kLd = kSimtTN + 4;
+  __shared__ __align__(16) float Ps[kRows * kLd];      // [j][n]
+  __shared__ __align__(16) float Xs[kSimtTN * 64 * NB];  // [n][c]
+  const int t = blockIdx.z / nsplit, s = blockIdx.z % nsplit;
+  const int bh = blockIdx.y, j0 = blockIdx.x * kRows;
   // ef_heads > 0: E and F are [ef_heads][k][N], one pair per head (head = bh % ef_heads)
-  const T* __restrict__ P = (t ? F : E) + (ef_heads > 0 ? (size_t)(bh % ef_heads) * k * N : 0);
+  const T* __restrict__ P = (t ? Fin : E) + (ef_heads > 0 ? (size_t)(bh % ef_heads) * k * N : 0);
   const HeadView hv = head_view(bh, seq_major_heads, N, d);
   const T* __restrict__ X = (t ? Vin : Kin) + hv.base;
   float* __restrict__ out = KpVp + ((size_t)t * BH + bh) * (size_t)k * d;
+  const int n_begin = s * chunk, n_end = min(N, n_begin + chunk);
+  const bool vec_p = (N & 3) == 0, vec_x = (d & 3) == 0;
 
-  const int n_begin = s * chunk;
-  const int n_end = min(N, n_begin + chunk);
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-
-  float acc[4][4];
+  constexpr int kPV = R / 2, kXV = 2 * NB;             // 16-byte pieces of each tile per thread
+  float4 rp[kPV], rx[kXV];
+  auto fetch = [&](int n0) {
 #pragma unroll
-  for (int a = 0; a < 4; ++a)
+    for (int i = 0; i < kPV; ++i) {
+      const int idx = threadIdx.x + i * kSimtThreads, jj = idx >> 3, nn = (idx & 7) * 4;
+      rp[i] = simt_load_row4(P + (size_t)(j0 + jj) * N + n0 + nn, j0 + jj < k ? n_end - (n0 + nn) : 0, vec_p);
+    }
 #pragma unroll
-    for (int b = 0; b < 4; ++b) acc[a][b] = 0.f;
-
-  for (int n0 = n_begin; n0 < n_end; n0 += TN) {
-    // stage the projection tile [32 j][32 n] and the input tile [32 n][d]
-    for (int idx = threadIdx.x; idx < TJ * TN; idx += 256) {
-      const int jj = idx / TN, nn = idx % TN;
-      const int j = j0 + jj, n = n0 + nn;
-      Ps[jj][nn] = (j < k && n < n_end) ? to_f32(P[(size_t)j * N + n]) : 0.f;
+    for (int i = 0; i < kXV; ++i) {
+      const int idx = threadIdx.x + i * kSimtThreads, nn = idx / (16 * NB), c = (idx % (16 * NB)) * 4;
+      rx[i] = simt_load_row4(X + (size_t)(n0 + nn) * hv.row_stride + c, n0 + nn < n_end ? d - c : 0, vec_x);
     }
-    for (int idx = threadIdx.x; idx < TN * 128; idx += 256) {
-      const int nn = idx >> 7, c = idx & 127;
-      const int n = n0 + nn;
-      Xs[nn][c] = (n < n_end && c < d) ? to_f32(X[(size_t)n * hv.row_stride + c]) : 0.f;
+  };
+  float acc[R][NB * 4];
+#pragma unroll
+  for (int r = 0; r < R; ++r)
+#pragma unroll
+    for (int c = 0; c < NB * 4; ++c) acc[r][c] = 0.f;
+  fetch(n_begin);
+  for (int n0 = n_begin; n0 < n_end; n0 += kSimtTN) {
+#pragma unroll
+    for (int i = 0; i < kPV; ++i) {
+      const int idx = threadIdx.x + i * kSimtThreads;
+      *reinterpret_cast<float4*>(Ps + (idx >> 3) * kLd + (idx & 7) * 4) = rp[i];
     }
+#pragma unroll
+    for (int i = 0; i < kXV; ++i) *reinterpret_cast<float4*>(Xs + (threadIdx.x + i * kSimtThreads) * 4) = rx[i];
     __syncthreads();
-#pragma unroll 4
-    for (int nn = 0; nn < TN; ++nn) {
-      float p[4], x[4];
-#pragma unroll
-      for (int a = 0; a < 4; ++a) p[a] = Ps[warp * 4 + a][nn];
-#pragma unroll
-      for (int b = 0; b < 4; ++b) x[b] = Xs[nn][lane + 32 * b];
-#pragma unroll
-      for (int a = 0; a < 4; ++a)
-#pragma unroll
-        for (int b = 0; b < 4; ++b) acc[a][b] = fmaf(p[a], x[b], acc[a][b]);
-    }
+    if (n0 + kSimtTN < n_end) fetch(n0 + kSimtTN);
+    simt_product<R, NB>(acc, Ps, kLd, Xs, kSimtTN);
     __syncthreads();
   }
+  const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
 #pragma unroll
-  for (int a = 0; a < 4; ++a) {
-    const int j = j0 + warp * 4 + a;
+  for (int r = 0; r < R; ++r) {
+    const int j = j0 + ty + 16 * r;
     if (j >= k) continue;
 #pragma unroll
-    for (int b = 0; b < 4; ++b) {
-      const int c = lane + 32 * b;
-      if (c < d) atomicAdd(out + (size_t)j * d + c, acc[a][b]);
+    for (int q = 0; q < NB; ++q) {
+      const int c = q * 64 + tx * 4;
+      float* o = out + (size_t)j * d + c;
+      if (vec_x && c < d) {
+        atomicAdd(reinterpret_cast<float4*>(o), make_float4(acc[r][q * 4], acc[r][q * 4 + 1], acc[r][q * 4 + 2], acc[r][q * 4 + 3]));
+      } else {
+#pragma unroll
+        for (int e = 0; e < 4; ++e)
+          if (c + e < d) atomicAdd(o + e, acc[r][q * 4 + e]);
+      }
     }
   }
 }
 
 // ---------------------------------------------------------------------------------------------
-// Stage 2.  grid = (ceil(p/8), B*H); block = 256 (8 warps, one feature each); p = m or d.
-// Dynamic shared memory: 8*k floats (the exponents / feature values of this block's features)
-// followed by 32*(d+1) floats (one chunk of K' rows).
-// Outputs: weight[bh][i] (b_i or z_i), a32[bh][i][c] fp32, aT16[bh][c][i] fp16 (either may be NULL).
+// Stages 2 and 3 share one form: every row (a feature i on the key side, a query n on the query side) weighs a list
+// of items (projected keys j, or features i), normalises the weights, and takes the weighted mean of the items'
+// vectors (v'_j, or a_i), items in steps of 64 with a running maximum.
+//   key side    rows W_i, items K'_j with bias -|k'_j|^2/2 and vectors V'_j   (PERFORMER)
+//               weight elu(k'_ji) + 1                                          (RNN)
+//               out: weight[bh][i] (b_i or z_i), a32[bh][i][c] fp32, aT16[bh][c][i] fp16 (either may be NULL)
+//   query side  rows Q_n, items W_i with bias b_i and vectors a_i               (PERFORMER)
+//               weight (elu(q_ni) + 1) z_i                                      (RNN)
+// grid = (ceil(rows / 16R), B*H).  Dynamic shared memory: simt_attend_smem().
 // ---------------------------------------------------------------------------------------------
-template <typename T, bool kPerformer>
-__global__ void __launch_bounds__(256)
-simt_key_side(const float* __restrict__ KpVp, const T* __restrict__ W, float* __restrict__ weight,
-              float* __restrict__ a32, __half* __restrict__ aT16, int BH, int d, int k, int p) {
-  extern __shared__ float smem[];
-  float* Ls = smem;                 // [8][k]
-  float* Ks = smem + 8 * k;         // [32][d+1]
-  __shared__ float nrm[32];
-  __shared__ float wrow[8][128];
-
-  const int bh = blockIdx.y;
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int i = blockIdx.x * 8 + warp;          // this warp's feature
-  const bool live = i < p;
-  const float* __restrict__ Kp = KpVp + (size_t)bh * k * d;
-  const float* __restrict__ Vp = KpVp + ((size_t)BH + bh) * (size_t)k * d;
-
-  if (kPerformer) {
-    for (int c = lane; c < d; c += 32) wrow[warp][c] = live ? to_f32(W[(size_t)i * d + c]) : 0.f;
-  }
-  // pass 1: exponents L_ji (PERFORMER) or feature values elu(k'_ji)+1 (RNN), all keys j
-  for (int j0 = 0; j0 < k; j0 += 32) {
-    __syncthreads();
-    for (int idx = threadIdx.x; idx < 32 * d; idx += 256) {
-      const int jj = idx / d, c = idx % d;
-      Ks[jj * (d + 1) + c] = (j0 + jj < k) ? Kp[(size_t)(j0 + jj) * d + c] : 0.f;
-    }
-    __syncthreads();
-    if (kPerformer) {
-      if (warp == 0) {
-        float s = 0.f;
-        for (int c = 0; c < d; ++c) { const float v = Ks[lane * (d + 1) + c]; s = fmaf(v, v, s); }
-        nrm[lane] = 0.5f * s;
-      }
-      __syncthreads();
-      float dot = 0.f;
-      for (int c = 0; c < d; ++c) dot = fmaf(wrow[warp][c], Ks[lane * (d + 1) + c], dot);
-      if (j0 + lane < k) Ls[warp * k + j0 + lane] = dot - nrm[lane];
-    } else {
-      if (j0 + lane < k) {
-        const float x = live ? Ks[lane * (d + 1) + i] : 0.f;
-        Ls[warp * k + j0 + lane] = x > 0.f ? x + 1.f : expf(x);
-      }
-    }
-  }
-  __syncwarp();
-  // per-feature maximum (PERFORMER); RNN needs none
-  float cmax = 0.f;
-  if (kPerformer) {
-    cmax = -INFINITY;
-    for (int j = lane; j < k; j += 32) cmax = fmaxf(cmax, Ls[warp * k + j]);
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) cmax = fmaxf(cmax, __shfl_xor_sync(0xffffffffu, cmax, o));
-    for (int j = lane; j < k; j += 32) Ls[warp * k + j] = expf(Ls[warp * k + j] - cmax);
-    __syncwarp();
-  }
-  // pass 2: z_i and the weighted sum of V' rows; lane owns columns lane, lane+32, ...
-  float z = 0.f, acc[4] = {0.f, 0.f, 0.f, 0.f};
-  for (int j = 0; j < k; ++j) {
-    const float e = Ls[warp * k + j];
-    z += e;
-#pragma unroll
-    for (int b = 0; b < 4; ++b) {
-      const int c = lane + 32 * b;
-      if (c < d) acc[b] = fmaf(e, Vp[(size_t)j * d + c], acc[b]);
-    }
-  }
-  if (!live) return;
-  const float inv = 1.f / z;
-  if (lane == 0) weight[(size_t)bh * p + i] = kPerformer ? cmax + logf(z) : z;
-#pragma unroll
-  for (int b = 0; b < 4; ++b) {
-    const int c = lane + 32 * b;
-    if (c < d) {
-      const float a = acc[b] * inv;
-      if (a32) a32[((size_t)bh * p + i) * d + c] = a;
-      if (aT16) aT16[((size_t)bh * d + c) * p + i] = __float2half_rn(a);
-    }
-  }
+inline size_t simt_attend_smem(int R, int NB, int d) {
+  return ((size_t)(16 * R + 64) * simt_ld(d) + (size_t)64 * 64 * NB + (size_t)16 * R * 68 + 64) * 4;
 }
 
-// ---------------------------------------------------------------------------------------------
-// Stage 3.  grid = (ceil(N/32), B*H); block = 256: warp w owns rows 4w..4w+3 of the 32-row tile,
-// lane owns feature (i0 + lane) while scoring and columns lane + 32t while accumulating.
-// Features are streamed in chunks of 32 with an online (running-maximum) normalisation.
-// Dynamic shared memory: 32*(d+1) floats (W chunk) + 32*d floats (a chunk).
-// ---------------------------------------------------------------------------------------------
-template <typename T, bool kPerformer>
-__global__ void __launch_bounds__(256)
-simt_query_side(const T* __restrict__ Q, const T* __restrict__ W, const float* __restrict__ weight,
-                const float* __restrict__ a32, T* __restrict__ out, int N, int d, int p, int seq_major_heads) {
-  extern __shared__ float smem[];
-  float* Ws = smem;                  // [32][d+1]
-  float* As = smem + 32 * (d + 1);   // [32][d]
-  __shared__ float qs[32][128];
-  __shared__ float ws[32];
-
-  const int bh = blockIdx.y;
-  const int n0 = blockIdx.x * 32;
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+template <typename T, bool kPerformer, bool kKeySide, int R, int NB>
+__global__ void __launch_bounds__(kSimtThreads, R == 8 && NB == 2 ? 1 : 2)
+simt_attend(const T* __restrict__ Q, const T* __restrict__ W, const float* __restrict__ KpVp, float* __restrict__ weight,
+            float* __restrict__ a32, __half* __restrict__ aT16, T* __restrict__ out, int BH, int N, int d, int k, int p,
+            int seq_major_heads) {
+  extern __shared__ __align__(16) float smem[];
+  constexpr int kRows = 16 * R, kLd = 68;
+  const int ld = simt_ld(d), cols = (d + 3) & ~3;
+  float* Xs = smem;                        // [16R][ld]    rows
+  float* Ys = Xs + kRows * ld;             // [64][ld]     items
+  float* Vs = Ys + 64 * ld;                // [64][64 NB]  the items' vectors
+  float* Ps = Vs + 64 * 64 * NB;           // [16R][68]    weights
+  float* bias = Ps + kRows * kLd;          // [64]
+  const int bh = blockIdx.y, row0 = blockIdx.x * kRows;
+  const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
+  const bool vec = (d & 3) == 0;
+  const int rows = kKeySide ? p : N, items = kKeySide ? k : p;
   const HeadView hv = head_view(bh, seq_major_heads, N, d);
-  const T* __restrict__ Qh = Q + hv.base;
-  const float* __restrict__ ah = a32 + (size_t)bh * p * d;
-  const float* __restrict__ wh = weight + (size_t)bh * p;
+  const float* __restrict__ Vh = kKeySide ? KpVp + ((size_t)BH + bh) * (size_t)k * d : a32 + (size_t)bh * p * d;
 
-  for (int idx = threadIdx.x; idx < 32 * d; idx += 256) {
-    const int r = idx / d, c = idx % d;
-    qs[r][c] = (n0 + r < N) ? to_f32(Qh[(size_t)(n0 + r) * hv.row_stride + c]) : 0.f;
+  if (kPerformer || !kKeySide) {
+    for (int idx = threadIdx.x; idx < kRows * (cols >> 2); idx += kSimtThreads) {
+      const int r = idx / (cols >> 2), c = (idx % (cols >> 2)) * 4;
+      const T* src = kKeySide ? W + (size_t)(row0 + r) * d : Q + hv.base + (size_t)(row0 + r) * hv.row_stride;
+      *reinterpret_cast<float4*>(Xs + r * ld + c) = simt_load_row4(src + c, row0 + r < rows ? d - c : 0, vec);
+    }
   }
-  float run_max[4], run_sum[4], acc[4][4];
+  float run_max[R], run_sum[R], acc[R][NB * 4];
 #pragma unroll
-  for (int r = 0; r < 4; ++r) {
+  for (int r = 0; r < R; ++r) {
     run_max[r] = -INFINITY;
     run_sum[r] = 0.f;
 #pragma unroll
-    for (int b = 0; b < 4; ++b) acc[r][b] = 0.f;
+    for (int c = 0; c < NB * 4; ++c) acc[r][c] = 0.f;
   }
-
-  for (int i0 = 0; i0 < p; i0 += 32) {
+  for (int i0 = 0; i0 < items; i0 += 64) {
     __syncthreads();
-    if (kPerformer) {
-      for (int idx = threadIdx.x; idx < 32 * d; idx += 256) {
-        const int ii = idx / d, c = idx % d;
-        Ws[ii * (d + 1) + c] = (i0 + ii < p) ? to_f32(W[(size_t)(i0 + ii) * d + c]) : 0.f;
+    if (kPerformer || kKeySide) {
+      for (int idx = threadIdx.x; idx < 64 * (cols >> 2); idx += kSimtThreads) {
+        const int r = idx / (cols >> 2), c = (idx % (cols >> 2)) * 4;
+        const int live = i0 + r < items ? d - c : 0;
+        float4 y;
+        if (kKeySide) y = simt_load_row4(KpVp + ((size_t)bh * k + i0 + r) * d + c, live, vec);
+        else y = simt_load_row4(W + (size_t)(i0 + r) * d + c, live, vec);
+        *reinterpret_cast<float4*>(Ys + r * ld + c) = y;
       }
     }
-    for (int idx = threadIdx.x; idx < 32 * d; idx += 256) {
-      const int ii = idx / d, c = idx % d;
-      As[ii * d + c] = (i0 + ii < p) ? ah[(size_t)(i0 + ii) * d + c] : 0.f;
+    for (int idx = threadIdx.x; idx < 64 * 16 * NB; idx += kSimtThreads) {
+      const int r = idx / (16 * NB), c = (idx % (16 * NB)) * 4;
+      *reinterpret_cast<float4*>(Vs + idx * 4) = simt_load_row4(Vh + (size_t)(i0 + r) * d + c, i0 + r < items ? d - c : 0, vec);
     }
-    if (threadIdx.x < 32) ws[threadIdx.x] = (i0 + threadIdx.x < p) ? wh[i0 + threadIdx.x] : 0.f;
+    if (!kKeySide && threadIdx.x < 64) bias[threadIdx.x] = i0 + threadIdx.x < items ? weight[(size_t)bh * p + i0 + threadIdx.x] : 0.f;
     __syncthreads();
-    const bool feat_live = (i0 + lane) < p;
+    if (kKeySide && kPerformer) {
+      // -|k'_j|^2 / 2: a few threads per key
+      constexpr int kPer = kSimtThreads / 64;
+      const int r = threadIdx.x / kPer;
+      float sq = 0.f;
+      for (int c = (threadIdx.x % kPer) * 4; c < cols; c += 4 * kPer) {
+        const float4 v = *reinterpret_cast<const float4*>(Ys + r * ld + c);
+        sq = fmaf(v.x, v.x, fmaf(v.y, v.y, fmaf(v.z, v.z, fmaf(v.w, v.w, sq))));
+      }
 #pragma unroll
-    for (int r = 0; r < 4; ++r) {
-      const int row = warp * 4 + r;
-      float pv;
+      for (int o = 1; o < kPer; o <<= 1) sq += __shfl_xor_sync(0xffffffffu, sq, o);
+      if (threadIdx.x % kPer == 0) bias[r] = -0.5f * sq;
+      __syncthreads();
+    }
+    float s[R][4];
+#pragma unroll
+    for (int r = 0; r < R; ++r)
+#pragma unroll
+      for (int f = 0; f < 4; ++f) s[r][f] = 0.f;
+    if (kPerformer) simt_dots<R>(s, Xs, Ys, ld, cols);
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+      const int row = ty + 16 * r;
       if (kPerformer) {
-        float s = 0.f;
-        for (int c = 0; c < d; ++c) s = fmaf(qs[row][c], Ws[lane * (d + 1) + c], s);
-        s = feat_live ? s + ws[lane] : -INFINITY;
-        float cm = s;
+        float cm = -INFINITY;
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) cm = fmaxf(cm, __shfl_xor_sync(0xffffffffu, cm, o));
+        for (int f = 0; f < 4; ++f) {
+          s[r][f] = i0 + tx + 16 * f < items ? s[r][f] + bias[tx + 16 * f] : -INFINITY;
+          cm = fmaxf(cm, s[r][f]);
+        }
+#pragma unroll
+        for (int o = 8; o > 0; o >>= 1) cm = fmaxf(cm, __shfl_xor_sync(0xffffffffu, cm, o));
         const float new_max = fmaxf(run_max[r], cm);
-        const float rescale = expf(run_max[r] - new_max);   // exp(-inf) = 0 on the first chunk
+        const float rescale = expf(run_max[r] - new_max);       // exp(-inf) = 0 on the first step
         run_max[r] = new_max;
         run_sum[r] *= rescale;
 #pragma unroll
-        for (int b = 0; b < 4; ++b) acc[r][b] *= rescale;
-        pv = feat_live ? expf(s - new_max) : 0.f;
+        for (int c = 0; c < NB * 4; ++c) acc[r][c] *= rescale;
+#pragma unroll
+        for (int f = 0; f < 4; ++f) s[r][f] = expf(s[r][f] - new_max);
       } else {
-        const float x = feat_live ? qs[row][i0 + lane] : 0.f;
-        pv = feat_live ? (x > 0.f ? x + 1.f : expf(x)) * ws[lane] : 0.f;
-      }
-      float psum = pv;
 #pragma unroll
-      for (int o = 16; o > 0; o >>= 1) psum += __shfl_xor_sync(0xffffffffu, psum, o);
-      run_sum[r] += psum;
-      for (int ii = 0; ii < 32; ++ii) {
-        const float pi = __shfl_sync(0xffffffffu, pv, ii);
-#pragma unroll
-        for (int b = 0; b < 4; ++b) {
-          const int c = lane + 32 * b;
-          if (c < d) acc[r][b] = fmaf(pi, As[ii * d + c], acc[r][b]);
+        for (int f = 0; f < 4; ++f) {
+          const int i = tx + 16 * f;
+          float v = 0.f;
+          if (i0 + i < items) {
+            const float x = kKeySide ? (row0 + row < rows ? Ys[i * ld + row0 + row] : 0.f) : Xs[row * ld + i0 + i];
+            v = (x > 0.f ? x + 1.f : expf(x)) * (kKeySide ? 1.f : bias[i]);
+          }
+          s[r][f] = v;
         }
       }
+      float part = 0.f;                                           // this thread's share of the row
+#pragma unroll
+      for (int f = 0; f < 4; ++f) {
+        part += s[r][f];
+        Ps[row * kLd + tx + 16 * f] = s[r][f];
+      }
+      run_sum[r] += part;
     }
+    __syncthreads();
+    simt_product<R, NB>(acc, Ps, kLd, Vs, min(64, (items - i0 + 3) & ~3));
   }
 #pragma unroll
-  for (int r = 0; r < 4; ++r) {
-    const int n = n0 + warp * 4 + r;
-    if (n >= N) continue;
-    const float inv = 1.f / fmaxf(run_sum[r], 1.17549435e-38f);
+  for (int r = 0; r < R; ++r) {
+    float sum = run_sum[r];
 #pragma unroll
-    for (int b = 0; b < 4; ++b) {
-      const int c = lane + 32 * b;
-      if (c < d) store_out(out + hv.base + (size_t)n * hv.row_stride + c, acc[r][b] * inv);
+    for (int o = 8; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+    const int row = row0 + ty + 16 * r;
+    if (row >= rows) continue;
+    const float inv = 1.f / fmaxf(sum, 1.17549435e-38f);
+    if (kKeySide && tx == 0) weight[(size_t)bh * p + row] = kPerformer ? run_max[r] + logf(sum) : sum;
+#pragma unroll
+    for (int q = 0; q < NB; ++q) {
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        const int c = q * 64 + tx * 4 + e;
+        if (c >= d) continue;
+        const float v = acc[r][q * 4 + e] * inv;
+        if (kKeySide) {
+          if (a32) a32[((size_t)bh * p + row) * d + c] = v;
+          if (aT16) aT16[((size_t)bh * d + c) * p + row] = __float2half_rn(v);
+        } else {
+          store_out(out + hv.base + (size_t)row * hv.row_stride + c, v);
+        }
+      }
     }
   }
 }

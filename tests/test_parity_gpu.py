@@ -487,3 +487,17 @@ def test_ragged_lengths_on_the_tensor_path(w, layout, per_head):
         for h in range(w.H):
             one = dict(x, E=x["E"][h], F=x["F"][h]) if per_head else x
             pu.assert_close(got[b, h], pu.oracle_head(one, w, b, h), "bf16", "%s head (%d,%d)" % (w.name, b, h))
+
+
+@pytest.mark.parametrize("w", [
+    # tiles of 32, 64 and 128 projection rows and their remainders; head dimensions around one and two 64-column blocks
+    _wl("simt_edge_k33_d66", PERFORMER, "fp32", 1, 2, 97, 66, 33, 65, 151),
+    _wl("simt_edge_k65_d100", PERFORMER, "bf16", 1, 2, 130, 100, 65, 63, 152),
+    _wl("simt_edge_k129_d63", RNN, "fp32", 1, 2, 161, 63, 129, 0, 153),
+    # enough heads for 128-row tiles on the query side (and, with m = 129, on the key side)
+    _wl("simt_edge_many_heads", PERFORMER, "fp32", 2, 40, 129, 31, 40, 129, 154),
+    _wl("simt_edge_many_heads_d128", PERFORMER, "fp32", 2, 38, 255, 128, 64, 130, 155),
+    _wl("simt_edge_many_heads_rnn", RNN, "fp32", 4, 38, 127, 70, 96, 0, 156),
+], ids=lambda w: w.name)
+def test_simt_path_at_the_edges_of_its_tiles(w):
+    pu.check_all_heads(w, path=binding.PATH_SIMT)
