@@ -213,7 +213,7 @@ int flurka_set_stage1_pairs(int on);
 /* The path the most recent successful flurka_forward (or flurka_backward) took (never FLURKA_PATH_AUTO). */
 int flurka_last_path(void);
 
-/* Number of kernels the most recent successful flurka_forward launched. */
+/* Number of kernels the most recent successful flurka_forward launched (the clearing of its accumulators not counted). */
 int flurka_last_launches(void);
 
 /*

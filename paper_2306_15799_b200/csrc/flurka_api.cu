@@ -35,7 +35,7 @@ struct Problem {
 //   status  int32[4] at offset 0 whatever the problem, then one arrival counter per
 //           (head, 128-feature tile) of stage 2
 //   kpvp    fp32 [2][BH][k][d]     K' then V'
-//           (status and kpvp are adjacent: one memset per forward clears both)
+//           (status and kpvp are adjacent: one range to clear per forward)
 //   weight  fp32 [BH][p]           b_i (PERFORMER) or z_i (RNN)
 //   a32     fp32 [BH][p][d]        key-side summary, feature-major
 //   aT16    fp16 [BH][d][p]        the same, transposed, as the tensor-core B operand
@@ -210,7 +210,7 @@ int pad_projections(const Problem& pr, char* pad, const void** E, const void** F
 }
 
 template <typename T, int R, int NB>
-void launch_simt_down_project_as(const Problem& pr, const void* K, const void* V, const void* E, const void* Fin,
+cudaError_t launch_simt_down_project_as(const Problem& pr, const void* K, const void* V, const void* E, const void* Fin,
                                  float* kpvp, cudaStream_t st) {
   // enough sequence splits for about four blocks per SM; a split is a multiple of one step
   const int jt = (pr.k + 16 * R - 1) / (16 * R);
@@ -221,9 +221,9 @@ void launch_simt_down_project_as(const Problem& pr, const void* K, const void* V
   chunk = (chunk + kSimtTN - 1) / kSimtTN * kSimtTN;
   nsplit = (pr.N + chunk - 1) / chunk;
   dim3 grid(jt, pr.BH(), 2 * nsplit);
-  simt_down_project<T, R, NB><<<grid, kSimtThreads, 0, st>>>((const T*)K, (const T*)V, (const T*)E, (const T*)Fin, kpvp,
-                                                           pr.BH(), pr.N, pr.d, pr.k, nsplit, chunk,
-                                                           pr.seq_major_heads(), pr.ef_heads());
+  return launch_after_predecessor(simt_down_project<T, R, NB>, grid, kSimtThreads, 0, st, (const T*)K, (const T*)V,
+                                  (const T*)E, (const T*)Fin, kpvp, pr.BH(), pr.N, pr.d, pr.k, nsplit, chunk,
+                                  pr.seq_major_heads(), pr.ef_heads());
 }
 
 template <typename T>
@@ -231,12 +231,14 @@ int launch_simt_down_project(const Problem& pr, const void* K, const void* V, co
                              const void* F, float* kpvp, cudaStream_t st, int* launches) {
   // rows per block: the largest tile that k fills (the larger the tile, the fewer shared memory reads per FMA)
   const bool wide = pr.d > 64;
-  if (pr.k > 64) wide ? launch_simt_down_project_as<T, 8, 2>(pr, K, V, E, F, kpvp, st)
-                      : launch_simt_down_project_as<T, 8, 1>(pr, K, V, E, F, kpvp, st);
-  else if (pr.k > 32) wide ? launch_simt_down_project_as<T, 4, 2>(pr, K, V, E, F, kpvp, st)
-                           : launch_simt_down_project_as<T, 4, 1>(pr, K, V, E, F, kpvp, st);
-  else wide ? launch_simt_down_project_as<T, 2, 2>(pr, K, V, E, F, kpvp, st)
-            : launch_simt_down_project_as<T, 2, 1>(pr, K, V, E, F, kpvp, st);
+  cudaError_t e;
+  if (pr.k > 64) e = wide ? launch_simt_down_project_as<T, 8, 2>(pr, K, V, E, F, kpvp, st)
+                          : launch_simt_down_project_as<T, 8, 1>(pr, K, V, E, F, kpvp, st);
+  else if (pr.k > 32) e = wide ? launch_simt_down_project_as<T, 4, 2>(pr, K, V, E, F, kpvp, st)
+                               : launch_simt_down_project_as<T, 4, 1>(pr, K, V, E, F, kpvp, st);
+  else e = wide ? launch_simt_down_project_as<T, 2, 2>(pr, K, V, E, F, kpvp, st)
+                : launch_simt_down_project_as<T, 2, 1>(pr, K, V, E, F, kpvp, st);
+  if (e != cudaSuccess) return cuda_fail(e);
   ++*launches;
   return FLURKA_OK;
 }
@@ -251,8 +253,9 @@ int launch_simt_attend_as(const Problem& pr, const void* Q, const void* W, const
     if (e != cudaSuccess) return cuda_fail(e);
   }
   dim3 grid(((kKeySide ? pr.p() : pr.N) + 16 * R - 1) / (16 * R), pr.BH());
-  fn<<<grid, kSimtThreads, smem, st>>>((const T*)Q, (const T*)W, kpvp, weight, a32, aT16, (T*)out, pr.BH(), pr.N, pr.d,
-                                  pr.k, pr.p(), pr.seq_major_heads());
+  cudaError_t e = launch_after_predecessor(fn, grid, kSimtThreads, smem, st, (const T*)Q, (const T*)W, kpvp, weight, a32,
+                                           aT16, (T*)out, pr.BH(), pr.N, pr.d, pr.k, pr.p(), pr.seq_major_heads());
+  if (e != cudaSuccess) return cuda_fail(e);
   return FLURKA_OK;
 }
 
@@ -298,7 +301,8 @@ int key_side_dispatch(const Problem& pr, const float* kpvp, const void* W, float
 template <typename T, typename Stage1>
 int run_pipeline_with(const Problem& pr, const Layout& L, char* ws, const void* Q, const void* W, void* out,
                       cudaStream_t st, bool tc2, bool tc3, TensorContext* tc, StageTimer* timer, bool keep_status,
-                      int* launches, Stage1&& stage1, int phases = 3) {
+                      int* launches, Stage1&& stage1, int phases = 3, void* more = nullptr, size_t more_bytes = 0) {
+  // more: one further range of the workspace that has to start at zero
   // phases: bit 0 = clear the accumulators and run stage 1, bit 1 = run stages 2 and 3 (a sequence-sharded
   // forward does the two halves in separate calls, with the sum over the shards in between)
   float* kpvp = (float*)(ws + L.kpvp);
@@ -308,12 +312,12 @@ int run_pipeline_with(const Problem& pr, const Layout& L, char* ws, const void* 
   int* status = (int*)(ws + L.status);
   const bool performer = pr.kernel == FLURKA_PERFORMER;
   int cuda_err = 0;
-  // one memset: the status words, the arrival counters and the K', V' accumulators the kernels add into
+  // one range: the status words, the arrival counters and the K', V' accumulators the kernels add into
   const size_t clear_from = L.status + (keep_status ? 16 : 0);
   cudaError_t e = cudaSuccess;
   int rc = FLURKA_OK;
   if (phases & 1) {
-    e = cudaMemsetAsync(ws + clear_from, 0, L.kpvp_end - clear_from, st);
+    e = launch_clear(ws + clear_from, L.kpvp_end - clear_from, more, more_bytes, st);
     if (e != cudaSuccess) return cuda_fail(e);
     if (timer) timer->mark(0, st);
     rc = stage1(kpvp, status, launches);
@@ -758,8 +762,6 @@ int fused_pipeline(const Problem& pr, int dm, const FusedLayout& FL, char* ws, c
   void* qp = ws + FL.qp;
   auto stage1 = [&](float* kpvp, int* status, int* n) -> int {
     int cuda_err = 0, rc;
-    cudaError_t e = cudaMemsetAsync(kt, 0, FL.kt_bytes, st);
-    if (e != cudaSuccess) return cuda_fail(e);
     if (tensor) {
       // Q = Xq W^Q first (the long one), then the contraction of the un-projected keys and values as
       // dm/64 pseudo-heads of width 64, then W^K, W^V on the k contracted rows
@@ -787,7 +789,7 @@ int fused_pipeline(const Problem& pr, int dm, const FusedLayout& FL, char* ws, c
     return simt_map<T>(Xq, Wq, qp, false, sizeof(T) == 4, pr.B * pr.N, dm, pr.H * pr.d, 1, 0, 0, 0, 0, st, n);
   };
   return run_pipeline_with<T>(pr, FL.L, ws, qp, W, out, st, tensor, tensor, tc, timer, /*keep_status=*/false, launches,
-                              stage1);
+                              stage1, 3, tensor ? kt : nullptr, tensor ? FL.kt_bytes : 0);
 }
 
 }  // namespace
@@ -861,7 +863,7 @@ int flurka_forward_fused(const void* Xq, const void* Xk, const void* Xv, const v
 namespace {
 
 // Scratch of the backward pass, after the forward layout: da [BH][p][d], db [BH][p] (adjacent: one
-// memset), then dK', dV' [2][BH][k][d]; all fp32.
+// range to clear), then dK', dV' [2][BH][k][d]; all fp32.
 struct BackwardLayout {
   Layout L;
   size_t da, dab_bytes, db, dkpvp, abf, split, rowstat, efpad, total;
@@ -911,9 +913,8 @@ int backward_pipeline(const Problem& pr, const BackwardLayout& BL, char* ws, con
   float* db = (float*)(ws + BL.db);
   float* dkpvp = (float*)(ws + BL.dkpvp);
   const int smh = pr.seq_major_heads(), efh = pr.ef_heads();
-  cudaError_t e = cudaMemsetAsync(ws + L.status, 0, L.kpvp_end - L.status, st);
+  cudaError_t e = launch_clear(ws + L.status, L.kpvp_end - L.status, da, BL.dab_bytes, st);
   if (e != cudaSuccess) return cuda_fail(e);
-  if ((e = cudaMemsetAsync(da, 0, BL.dab_bytes, st)) != cudaSuccess) return cuda_fail(e);
   // the forward's stages 1 and 2 again: K', V', a_i, b_i (or z_i)
   int rc = FLURKA_OK;
   int cuda_err = 0;

@@ -23,6 +23,7 @@ struct K1Params {
   int nsplit;      // CTAs along the sequence
   int col_groups;  // ceil(BH * d / group_cols)
   int k_halves;    // ceil(k / 256)
+  int wait_inputs; // E, F are the previous kernel's results (padded copies)
   int* status;
 };
 
@@ -96,6 +97,7 @@ k1_down_project(const __grid_constant__ CUtensorMap tmE, const __grid_constant__
       const CUtensorMap* tmX = t ? &tmV : &tmK;
       prefetch_tmap(tmP);
       prefetch_tmap(tmX);
+      if (p.wait_inputs) grid_dependency_wait_async();
       const uint32_t tx_bytes = (uint32_t)(mt * 16384 + nb * 8192);
       const int dblocks = p.d >> 6;                         // 64-column slabs per head
       int issued = 0;
@@ -151,6 +153,7 @@ k1_down_project(const __grid_constant__ CUtensorMap tmE, const __grid_constant__
       const int q = warp & 3;                                // TMEM lane quadrant of this warp
       bool ok = mbar_wait(bar_accum, 0, p.status, &abort_flag);
       if (warp == 2 && lane == 0) grid_launch_dependents();   // only the epilogue is left
+      grid_dependency_wait_async();                           // K', V' have been zeroed
       if (ok) {
         tcgen05_fence_after();
         const uint32_t stage_buf = smem_base + (warp - 2) * 32768;   // 8 x 4 KB, pipeline is drained

@@ -28,6 +28,7 @@ struct K1PairParams {
   int nsplit;      // CTA pairs along the sequence
   int col_groups;  // ceil(BH * d / 512)
   int k_halves;    // k / 256
+  int wait_inputs; // E, F are the previous kernel's results (padded copies)
   int* status;
 };
 
@@ -164,6 +165,7 @@ k1_down_project_pair(const __grid_constant__ CUtensorMap tmE, const __grid_const
         const CUtensorMap* tmX = t ? &tmV : &tmK;
         prefetch_tmap(tmP);
         prefetch_tmap(tmX);
+        if (p.wait_inputs) grid_dependency_wait_async();
         const uint32_t tx_bytes = (uint32_t)(16384 + nj * 16384);
         const int dblocks = p.d >> 6;                         // 64-column slabs per head
         int issued = 0;
@@ -229,6 +231,7 @@ k1_down_project_pair(const __grid_constant__ CUtensorMap tmE, const __grid_const
       const int q = warp & 3;                                // TMEM lane quadrant of this warp
       bool ok = mbar_wait(bar_accum, 0, p.status, &abort_flag);
       if (warp == 2 && lane == 0) grid_launch_dependents();   // only the epilogue is left
+      grid_dependency_wait_async();                           // K', V' have been zeroed
       if (ok) {
         tcgen05_fence_after();
         const uint32_t stage_buf = smem_base + (warp - 2) * 32768;   // 8 x 4 KB per warp, the pipeline is drained

@@ -11,6 +11,8 @@
 #include <cuda_bf16.h>
 #include <stdint.h>
 
+#include "tc_common.cuh"
+
 namespace flurka {
 
 // Eight bf16 from src[at .. at + 7], `at` not aligned: the two 16-byte pieces they lie in, shifted into place.
@@ -45,6 +47,8 @@ __device__ __forceinline__ uint4 load8_unaligned(const uint16_t* __restrict__ sr
 __global__ void __launch_bounds__(256)
 pad_rows(const uint16_t* __restrict__ src0, const uint16_t* __restrict__ src1, uint16_t* __restrict__ dst0,
          uint16_t* __restrict__ dst1, int rows, int N, int pitch) {
+  tc::grid_launch_dependents();
+  tc::grid_dependency_wait();       // (so that its own completion says that everything before it is complete)
   const uint16_t* __restrict__ src = blockIdx.z ? src1 : src0;
   uint16_t* __restrict__ dst = blockIdx.z ? dst1 : dst0;
   const int c = (blockIdx.x * 256 + threadIdx.x) * 8;

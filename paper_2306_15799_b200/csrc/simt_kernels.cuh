@@ -19,6 +19,8 @@
 #include <cuda_runtime.h>
 #include <math.h>
 
+#include "tc_common.cuh"
+
 namespace flurka {
 
 // Where head bh of a [B,H,N,d] tensor (H == 0) or of a [B,N,H,d] tensor (H = number of heads) starts,
@@ -140,6 +142,7 @@ simt_down_project(const T* __restrict__ Kin, const T* __restrict__ Vin, const T*
   constexpr int kRows = 16 * R, kLd = kSimtTN + 4;
   __shared__ __align__(16) float Ps[kRows * kLd];      // [j][n]
   __shared__ __align__(16) float Xs[kSimtTN * 64 * NB];  // [n][c]
+  tc::grid_launch_dependents();
   const int t = blockIdx.z / nsplit, s = blockIdx.z % nsplit;
   const int bh = blockIdx.y, j0 = blockIdx.x * kRows;
   // ef_heads > 0: E and F are [ef_heads][k][N], one pair per head (head = bh % ef_heads)
@@ -183,6 +186,7 @@ simt_down_project(const T* __restrict__ Kin, const T* __restrict__ Vin, const T*
     simt_product<R, NB>(acc, Ps, kLd, Xs, kSimtTN);
     __syncthreads();
   }
+  tc::grid_dependency_wait();          // KpVp has been zeroed
   const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
 #pragma unroll
   for (int r = 0; r < R; ++r) {
@@ -231,6 +235,7 @@ simt_attend(const T* __restrict__ Q, const T* __restrict__ W, const float* __res
   float* Vs = Ys + 64 * ld;                // [64][64 NB]  the items' vectors
   float* Ps = Vs + 64 * 64 * NB;           // [16R][68]    weights
   float* bias = Ps + kRows * kLd;          // [64]
+  tc::grid_launch_dependents();
   const int bh = blockIdx.y, row0 = blockIdx.x * kRows;
   const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
   const bool vec = (d & 3) == 0;
@@ -245,6 +250,7 @@ simt_attend(const T* __restrict__ Q, const T* __restrict__ W, const float* __res
       *reinterpret_cast<float4*>(Xs + r * ld + c) = simt_load_row4(src + c, row0 + r < rows ? d - c : 0, vec);
     }
   }
+  tc::grid_dependency_wait();          // rows are inputs of the call; everything else comes from the kernels before
   float run_max[R], run_sum[R], acc[R][NB * 4];
 #pragma unroll
   for (int r = 0; r < R; ++r) {

@@ -40,6 +40,11 @@ __device__ __forceinline__ bool elect_one() {
 // returns once the predecessor has completed and its writes are visible).  Without the launch
 // attribute the wait returns at once.
 __device__ __forceinline__ void grid_dependency_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+// The same before this thread's asynchronous copies (TMA, bulk) touch global memory that kernel wrote.
+__device__ __forceinline__ void grid_dependency_wait_async() {
+  grid_dependency_wait();
+  asm volatile("fence.proxy.async.global;" ::: "memory");
+}
 // Lets the next kernel in the stream be scheduled once every CTA of this grid has said so or has
 // exited.  Called late in a CTA's life: when the last CTA calls it, every CTA of this grid already
 // holds its SM, so the successor's CTAs can never keep one of ours from starting.

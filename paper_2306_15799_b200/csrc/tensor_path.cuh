@@ -6,6 +6,9 @@
 #include <cuda_runtime.h>
 #include <string.h>
 
+#include <algorithm>
+
+#include "clear.cuh"
 #include "k0_linear_maps.cuh"
 #include "k1_down_project.cuh"
 #include "k1_down_project_pair.cuh"
@@ -17,6 +20,39 @@
 #include "pad_rows.cuh"
 
 namespace flurka {
+
+// Launch with programmatic stream serialisation: the kernel may be scheduled while the previous
+// kernel in the stream is finishing (its CTAs call griddepcontrol.launch_dependents) and waits in
+// griddepcontrol.wait before it touches that kernel's results.  Every kernel of a chain waits somewhere before it
+// ends, so that the completion of one says that all before it are complete.
+template <typename... KArgs, typename... Args>
+inline cudaError_t launch_after_predecessor(void (*fn)(KArgs...), dim3 grid, int block, size_t smem, cudaStream_t st,
+                                            Args... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = dim3((unsigned)block, 1, 1);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, fn, KArgs(args)...);
+}
+
+// Zeroes [p0, p0 + n0) and [p1, p1 + n1) (16-byte aligned; lengths are rounded up to 16 bytes).
+inline cudaError_t launch_clear(void* p0, size_t n0, void* p1, size_t n1, cudaStream_t st) {
+  ClearRanges r;
+  r.ptr[0] = reinterpret_cast<uint4*>(p0);
+  r.ptr[1] = reinterpret_cast<uint4*>(p1);
+  r.count[0] = (n0 + 15) >> 4;
+  r.count[1] = (n1 + 15) >> 4;
+  // four 16-byte words per thread, at most eight blocks per SM
+  size_t blocks = (std::max(r.count[0], r.count[1]) + 1023) / 1024;
+  blocks = std::max<size_t>(1, std::min<size_t>(blocks, 148 * 8));
+  return launch_after_predecessor(clear_ranges, dim3((unsigned)blocks), 256, 0, st, r);
+}
 
 // Optional per-stage timing: events recorded on the launch stream around the three stages.
 struct StageTimer {
@@ -145,8 +181,8 @@ inline int TensorContext::sm_count() {
 inline int launch_pad_rows(const void* E, const void* F, void* Ep, void* Fp, int rows, int N, int pitch, cudaStream_t st,
                            int* cuda_err) {
   dim3 grid((N + 2047) / 2048, rows < 65535 ? rows : 65535, 2);
-  pad_rows<<<grid, 256, 0, st>>>((const uint16_t*)E, (const uint16_t*)F, (uint16_t*)Ep, (uint16_t*)Fp, rows, N, pitch);
-  cudaError_t e = cudaGetLastError();
+  cudaError_t e = launch_after_predecessor(pad_rows, grid, 256, 0, st, (const uint16_t*)E, (const uint16_t*)F,
+                                           (uint16_t*)Ep, (uint16_t*)Fp, rows, N, pitch);
   if (e != cudaSuccess) { *cuda_err = (int)e; return -6; }
   return 0;
 }
@@ -202,6 +238,7 @@ inline int launch_k1(TensorContext& tc, const void* K, const void* V, const void
     pp.col_groups = (BH * d + 511) / 512;
     pp.k_halves = k / 256;
     pp.nsplit = k1_choose_nsplit(tc.sm_count() / 2, 2 * pp.col_groups * pp.k_halves, (N + 63) / 64);
+    pp.wait_inputs = ef_pitch != N;
     pp.status = status;
     if (!tc.k1p_attr) {
       cudaError_t e = cudaFuncSetAttribute(k1_down_project_pair, cudaFuncAttributeMaxDynamicSharedMemorySize, kK1PSmemBytes);
@@ -209,9 +246,8 @@ inline int launch_k1(TensorContext& tc, const void* K, const void* V, const void
       tc.k1p_attr = true;
     }
     const int pairs = 2 * pp.k_halves * pp.col_groups * pp.nsplit;
-    k1_down_project_pair<<<2 * pairs, kK1PThreads, kK1PSmemBytes, st>>>(tm.E.map, tm.F.map, tm.K.map, tm.V.map,
-                                                                        tm.kpvp.map, pp);
-    cudaError_t e = cudaGetLastError();
+    cudaError_t e = launch_after_predecessor(k1_down_project_pair, 2 * pairs, kK1PThreads, kK1PSmemBytes, st, tm.E.map,
+                                             tm.F.map, tm.K.map, tm.V.map, tm.kpvp.map, pp);
     if (e != cudaSuccess) { *cuda_err = (int)e; return -6; }
     return 0;
   }
@@ -222,6 +258,7 @@ inline int launch_k1(TensorContext& tc, const void* K, const void* V, const void
   p.col_groups = (BH * d + p.group_cols - 1) / p.group_cols;
   p.k_halves = (k + 255) / 256;
   p.nsplit = k1_choose_nsplit(tc.sm_count(), 2 * p.col_groups * p.k_halves, (N + 63) / 64);
+  p.wait_inputs = ef_pitch != N;
   p.status = status;
   if (!tc.k1_attr) {
     cudaError_t e = cudaFuncSetAttribute(k1_down_project, cudaFuncAttributeMaxDynamicSharedMemorySize, kK1SmemBytes);
@@ -229,16 +266,11 @@ inline int launch_k1(TensorContext& tc, const void* K, const void* V, const void
     tc.k1_attr = true;
   }
   const int grid = 2 * p.k_halves * p.col_groups * p.nsplit;
-  k1_down_project<<<grid, kK1Threads, kK1SmemBytes, st>>>(tm.E.map, tm.F.map, tm.K.map, tm.V.map, tm.kpvp.map, p);
-  cudaError_t e = cudaGetLastError();
+  cudaError_t e = launch_after_predecessor(k1_down_project, grid, kK1Threads, kK1SmemBytes, st, tm.E.map, tm.F.map,
+                                           tm.K.map, tm.V.map, tm.kpvp.map, p);
   if (e != cudaSuccess) { *cuda_err = (int)e; return -6; }
   return 0;
 }
-
-// Forward declaration (defined below).
-template <typename... KArgs, typename... Args>
-inline cudaError_t launch_after_predecessor(void (*fn)(KArgs...), int grid, int block, size_t smem, cudaStream_t st,
-                                            Args... args);
 
 inline int k0_set_attr(TensorContext& tc, int* cuda_err) {
   if (!tc.k0_attr) {
@@ -321,45 +353,26 @@ inline int launch_k0_query_map(TensorContext& tc, const void* Xq, const void* Wq
       if (e != cudaSuccess) { *cuda_err = (int)e; (void)cudaGetLastError(); return -6; }
       tc.k0p_attr = true;
     }
-    k0_query_map_pair<<<2 * p.row_blocks * p.col_groups, kK0Threads, kK0PSmemBytes, st>>>(tm.Xq.map, tm.Wq.map, tm.Qp.map, p);
-    cudaError_t e = cudaGetLastError();
+    cudaError_t e = launch_after_predecessor(k0_query_map_pair, 2 * p.row_blocks * p.col_groups, kK0Threads, kK0PSmemBytes,
+                                             st, tm.Xq.map, tm.Wq.map, tm.Qp.map, p);
     if (e != cudaSuccess) { *cuda_err = (int)e; return -6; }
     return 0;
   }
   int rc = k0_set_attr(tc, cuda_err);
   if (rc) return rc;
-  k0_linear_map<<<p.row_blocks * p.col_groups, kK0Threads, kK0SmemBytes, st>>>(tm.Xq.map, tm.Wq.map, tm.Wq.map,
-                                                                               tm.Qp.map, p);
-  cudaError_t e = cudaGetLastError();
+  cudaError_t e = launch_after_predecessor(k0_linear_map, p.row_blocks * p.col_groups, kK0Threads, kK0SmemBytes, st,
+                                           tm.Xq.map, tm.Wq.map, tm.Wq.map, tm.Qp.map, p);
   if (e != cudaSuccess) { *cuda_err = (int)e; return -6; }
   return 0;
 }
 
-// Launch with programmatic stream serialisation: the kernel may be scheduled while the previous
-// kernel in the stream is finishing (its CTAs call griddepcontrol.launch_dependents late in their
-// life) and waits in griddepcontrol.wait before it touches that kernel's results.
-template <typename... KArgs, typename... Args>
-inline cudaError_t launch_after_predecessor(void (*fn)(KArgs...), int grid, int block, size_t smem, cudaStream_t st,
-                                            Args... args) {
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((unsigned)grid, 1, 1);
-  cfg.blockDim = dim3((unsigned)block, 1, 1);
-  cfg.dynamicSmemBytes = smem;
-  cfg.stream = st;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, fn, KArgs(args)...);
-}
-
-// Key splits of stage 2: with few (head, feature tile) pairs the keys are divided over up to four
-// CTAs per pair, as long as all of them fit on the machine at once.
-inline int k2_nsplit(int sms, bool performer, int BH, int k, int p) {
+// Key splits of stage 2: with few (head, feature tile) pairs the key blocks are divided over up to four
+// CTAs per pair, as long as all of them fit on the machine at once.  (A block is not divided: the merge costs
+// about what half a block does.)
+inline int k2_nsplit(int sms, bool performer, int BH, int d, int k, int p) {
   if (!performer) return 1;
   const int units = BH * ((p + 127) / 128);
-  const int chunks = (k + kK2Chunk - 1) / kK2Chunk;
+  const int chunks = (k * d + kK2BlockElems - 1) / kK2BlockElems;
   int ns = sms / units;
   if (ns > chunks) ns = chunks;
   if (ns > 4) ns = 4;
@@ -370,7 +383,7 @@ inline int k2_nsplit(int sms, bool performer, int BH, int k, int p) {
 // problem could get on any device (so the workspace size does not depend on the device)
 inline size_t k2_part_floats(bool performer, int BH, int d, int k, int p) {
   if (!performer) return 0;
-  int chunks = (k + kK2Chunk - 1) / kK2Chunk;
+  int chunks = (k * d + kK2BlockElems - 1) / kK2BlockElems;
   if (chunks > 4) chunks = 4;
   if (chunks < 2) return 0;
   return (size_t)BH * ((p + 127) / 128) * chunks * (size_t)(d + 2) * 128;
@@ -397,10 +410,11 @@ inline int launch_k2(TensorContext& tc, bool performer, const float* kpvp, const
   prm.aT16 = aT16;
   prm.a32 = a32;
   prm.status = status;
-  prm.nsplit = (part && counters) ? k2_nsplit(tc.sm_total(), performer, BH, k, p) : 1;
+  prm.nsplit = (part && counters) ? k2_nsplit(tc.sm_total(), performer, BH, d, k, p) : 1;
   prm.part = part;
   prm.counters = counters;
-  auto fn = performer ? k2_key_side<true> : k2_key_side<false>;
+  auto fn = d == 64 ? (performer ? k2_key_side<true, 64> : k2_key_side<false, 64>)
+                    : (performer ? k2_key_side<true, 128> : k2_key_side<false, 128>);
   cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, kK2SmemBytes);
   if (e != cudaSuccess) { *cuda_err = (int)e; (void)cudaGetLastError(); return -6; }
   // the RNN kernel ignores tmW; pass any valid map
