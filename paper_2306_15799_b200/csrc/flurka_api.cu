@@ -932,8 +932,8 @@ int backward_pipeline(const Problem& pr, const BackwardLayout& BL, char* ws, con
   }
   if (tc) {
     // the key side on its tensor-core kernel, one CTA per (head, feature tile), with a in fp32 as well
-    rc = launch_k2(*tc, P, kpvp, W, weight, (__half*)(ws + L.aT16), nullptr, nullptr, pr.BH(), pr.d, pr.k, pr.p(),
-                   (int*)(ws + L.status), st, &cuda_err, a32);
+    rc = launch_k2(*tc, P, kpvp, W, weight, nullptr, nullptr, nullptr, pr.BH(), pr.d, pr.k, pr.p(),
+                   (int*)(ws + L.status), st, &cuda_err, a32, tcq ? (__nv_bfloat16*)(ws + BL.abf) : nullptr);
     if (rc) { g_last_cuda_error = cuda_err; return rc; }
     ++*launches;
   } else {
@@ -941,10 +941,15 @@ int backward_pipeline(const Problem& pr, const BackwardLayout& BL, char* ws, con
     if (rc) return rc;
   }
   if (tc && tcq) {
-    rc = launch_k4(*tc, P, Q, dO, W, a32, weight, (__nv_bfloat16*)(ws + BL.abf), dQ, da, db, pr.BH(), smh, pr.N, pr.d, pr.p(),
-                   (int*)(ws + L.status), st, &cuda_err, ws + BL.rowstat);
+    const __nv_bfloat16* abf = (const __nv_bfloat16*)(ws + BL.abf);
+    if (pr.d == 64)
+      rc = launch_k7(*tc, P, Q, dO, W, a32, weight, abf, dQ, da, db, pr.BH(), smh, pr.N, pr.p(), (int*)(ws + L.status), st,
+                     &cuda_err);
+    else
+      rc = launch_k4(*tc, P, Q, dO, W, a32, weight, abf, dQ, da, db, pr.BH(), smh, pr.N, pr.d, pr.p(),
+                     (int*)(ws + L.status), st, &cuda_err, ws + BL.rowstat);
     if (rc) { g_last_cuda_error = cuda_err; return rc; }
-    *launches += 2;
+    ++*launches;
   } else {
     auto fn = simt_bwd_query_side<T, P>;
     const size_t smem = ((size_t)2 * 32 * (pr.d + 1) + 32 * 33 + 32 * pr.d) * 4;

@@ -38,8 +38,9 @@ struct K2Params {
   int ftiles;               // ceil(p / 128)
   const float* kpvp;        // [2][BH][k][d] fp32
   float* weight;            // [BH][p]      b_i (PERFORMER) or z_i (RNN)
-  __half* aT16;             // [BH][d][p]   a^T
+  __half* aT16;             // [BH][d][p]   a^T, or NULL
   float* a32;               // [BH][p][d]   a in fp32 as well (the backward pass wants it), or NULL
+  __nv_bfloat16* abf;       // [BH][2][p][d]  a as two bf16 terms (the backward pass), or NULL
   int* status;
   int nsplit;               // CTAs per (head, feature tile) along the keys (1..4; PERFORMER only)
   float* part;              // nsplit > 1: [BH * ftiles][nsplit][d + 2][128]  max, sum, accumulator columns
@@ -68,6 +69,22 @@ __device__ __forceinline__ float k2_ex2(float x) {
 }
 __device__ __forceinline__ void st_shared_v2(uint32_t addr, uint32_t a, uint32_t b) {
   asm volatile("st.shared.v2.b32 [%0], {%1, %2};" ::"r"(addr), "r"(a), "r"(b) : "memory");
+}
+// kCols consecutive values of a feature's a, as two bf16 terms `term` elements apart
+template <int kCols>
+__device__ __forceinline__ void k2_store_split(__nv_bfloat16* dst, size_t term, const float (&v)[kCols]) {
+#pragma unroll
+  for (int c = 0; c < kCols; c += 8) {
+    uint32_t hi[4], lo[4];
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+      const float x = v[c + 2 * e], y = v[c + 2 * e + 1];
+      hi[e] = pack_bf16x2(x, y);
+      lo[e] = pack_bf16x2(x - __uint_as_float(hi[e] << 16), y - __uint_as_float(hi[e] & 0xffff0000u));
+    }
+    *reinterpret_cast<uint4*>(dst + c) = make_uint4(hi[0], hi[1], hi[2], hi[3]);
+    *reinterpret_cast<uint4*>(dst + term + c) = make_uint4(lo[0], lo[1], lo[2], lo[3]);
+  }
 }
 __device__ __forceinline__ uint32_t half2_bits(__half2 h) { return *reinterpret_cast<const uint32_t*>(&h); }
 
@@ -392,9 +409,11 @@ k2_key_side(const __grid_constant__ CUtensorMap tmW, const K2Params prm) {
 #pragma unroll
         for (int c = 0; c < kColsPer; c += 4) arow[c >> 2] = make_float4(acc[c], acc[c + 1], acc[c + 2], acc[c + 3]);
       }
+      if (prm.abf && feat < p)
+        k2_store_split(prm.abf + ((size_t)head * 2 * p + feat) * kD + qd * kColsPer, (size_t)p * kD, acc);
     }
     __syncthreads();
-    if (ok) {
+    if (ok && prm.aT16) {
       const int cpr = min(128, p - i0) >> 3;                // 16-byte pieces per row
       __half* dst = prm.aT16 + (size_t)head * kD * p + i0;
       const uint4* tile = reinterpret_cast<const uint4*>(base_ptr + kK2K3);
@@ -448,9 +467,11 @@ k2_key_side(const __grid_constant__ CUtensorMap tmW, const K2Params prm) {
       if (feat < p) {
 #pragma unroll
         for (int c = 0; c < kColsPer; ++c) {
-          dst[(size_t)c * p] = __float2half_rn(acc[c] * inv);
-          if (prm.a32) prm.a32[((size_t)head * p + feat) * kD + qd * kColsPer + c] = acc[c] * inv;
+          acc[c] *= inv;
+          if (prm.aT16) dst[(size_t)c * p] = __float2half_rn(acc[c]);
+          if (prm.a32) prm.a32[((size_t)head * p + feat) * kD + qd * kColsPer + c] = acc[c];
         }
+        if (prm.abf) k2_store_split(prm.abf + ((size_t)head * 2 * p + feat) * kD + qd * kColsPer, (size_t)p * kD, acc);
       }
       if (tid == 0) prm.counters[unit] = 0;
     }

@@ -17,6 +17,7 @@
 #include "k4_bwd_query_side.cuh"
 #include "k5_bwd_projections.cuh"
 #include "k6_bwd_key_side.cuh"
+#include "k7_bwd_query_side.cuh"
 #include "pad_rows.cuh"
 
 namespace flurka {
@@ -26,19 +27,29 @@ namespace flurka {
 // griddepcontrol.wait before it touches that kernel's results.  Every kernel of a chain waits somewhere before it
 // ends, so that the completion of one says that all before it are complete.
 template <typename... KArgs, typename... Args>
-inline cudaError_t launch_after_predecessor(void (*fn)(KArgs...), dim3 grid, int block, size_t smem, cudaStream_t st,
-                                            Args... args) {
+inline cudaError_t launch_cluster_after_predecessor(int cluster, void (*fn)(KArgs...), dim3 grid, int block, size_t smem,
+                                                    cudaStream_t st, Args... args) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = grid;
   cfg.blockDim = dim3((unsigned)block, 1, 1);
   cfg.dynamicSmemBytes = smem;
   cfg.stream = st;
-  cudaLaunchAttribute attr[1];
+  cudaLaunchAttribute attr[2];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[0].val.programmaticStreamSerializationAllowed = 1;
+  attr[1].id = cudaLaunchAttributeClusterDimension;
+  attr[1].val.clusterDim.x = (unsigned)cluster;
+  attr[1].val.clusterDim.y = 1;
+  attr[1].val.clusterDim.z = 1;
   cfg.attrs = attr;
-  cfg.numAttrs = 1;
+  cfg.numAttrs = cluster > 1 ? 2 : 1;
   return cudaLaunchKernelEx(&cfg, fn, KArgs(args)...);
+}
+// (kernels with __cluster_dims__ bring their own cluster size)
+template <typename... KArgs, typename... Args>
+inline cudaError_t launch_after_predecessor(void (*fn)(KArgs...), dim3 grid, int block, size_t smem, cudaStream_t st,
+                                            Args... args) {
+  return launch_cluster_after_predecessor(1, fn, grid, block, smem, st, args...);
 }
 
 // Zeroes [p0, p0 + n0) and [p1, p1 + n1) (16-byte aligned; lengths are rounded up to 16 bytes).
@@ -392,7 +403,7 @@ inline size_t k2_part_floats(bool performer, int BH, int d, int k, int p) {
 // ---- stage 2: per-feature summaries a (fp16, transposed) and weights b / z from K', V' --------
 inline int launch_k2(TensorContext& tc, bool performer, const float* kpvp, const void* W, float* weight,
                      __half* aT16, float* part, int* counters, int BH, int d, int k, int p, int* status,
-                     cudaStream_t st, int* cuda_err, float* a32 = nullptr) {
+                     cudaStream_t st, int* cuda_err, float* a32 = nullptr, __nv_bfloat16* abf = nullptr) {
   TensorMaps& tm = tc.maps;
   if (performer) {
     const unsigned long long dW[2] = {(unsigned long long)d, (unsigned long long)p};
@@ -409,6 +420,7 @@ inline int launch_k2(TensorContext& tc, bool performer, const float* kpvp, const
   prm.weight = weight;
   prm.aT16 = aT16;
   prm.a32 = a32;
+  prm.abf = abf;
   prm.status = status;
   prm.nsplit = (part && counters) ? k2_nsplit(tc.sm_total(), performer, BH, d, k, p) : 1;
   prm.part = part;
@@ -476,10 +488,47 @@ inline int launch_k3(TensorContext& tc, bool performer, const void* Q, const voi
   return 0;
 }
 
+// ---- backward of the query side, d = 64: dQ, and da, db added to ---------------------------------------
+// abf: the two bf16 terms of a, [BH][2][p][64]
+inline int launch_k7(TensorContext& tc, bool performer, const void* Q, const void* dO, const void* W, const float* a32,
+                     const float* weight, const __nv_bfloat16* abf, void* dQ, float* da, float* db, int BH, int H, int N,
+                     int p, int* status, cudaStream_t st, int* cuda_err) {
+  TensorMaps& tm = tc.maps;
+  const unsigned long long dQd[3] = {(unsigned long long)(H > 0 ? H * 64 : 64), (unsigned long long)N,
+                                     (unsigned long long)(H > 0 ? BH / H : BH)};
+  const unsigned bQ[3] = {64, 128, 1};
+  const unsigned long long dW[2] = {64ull, (unsigned long long)p};
+  const unsigned bW[2] = {64, 128};                       // 128 features of a CTA; rows past p read as zero
+  const unsigned long long dA[3] = {64ull, (unsigned long long)p, (unsigned long long)BH * 2};
+  const CUtensorMapDataType bf = CU_TENSOR_MAP_DATA_TYPE_BFLOAT16;
+  if (!encode_map(&tm.Q, bf, 2, 3, Q, dQd, bQ) || !encode_map(&tm.dO, bf, 2, 3, dO, dQd, bQ) ||
+      (performer && !encode_map(&tm.W2, bf, 2, 2, W, dW, bW)) || !encode_map(&tm.abf, bf, 2, 3, abf, dA, bQ)) {
+    *cuda_err = (int)cudaErrorInvalidValue;
+    return -6;
+  }
+  K7Params prm;
+  prm.N = N; prm.p = p; prm.BH = BH; prm.H = H;
+  prm.tiles_per_head = (N + 127) / 128;
+  prm.total_tiles = prm.tiles_per_head * BH;
+  prm.weight = weight; prm.a32 = a32;
+  prm.dQ = reinterpret_cast<__nv_bfloat16*>(dQ);
+  prm.da = da; prm.db = db; prm.status = status;
+  const int parts = (p + 127) / 128;                      // 1 or 2 CTAs share a tile
+  auto fn = !performer ? k7_bwd_query_side<false, 1> : (parts == 2 ? k7_bwd_query_side<true, 2> : k7_bwd_query_side<true, 1>);
+  cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, kK7SmemBytes);
+  if (e != cudaSuccess) { *cuda_err = (int)e; (void)cudaGetLastError(); return -6; }
+  const int groups = std::max(1, std::min(tc.sm_count() / parts, prm.total_tiles));
+  // the RNN kernel ignores tmW; pass any valid map
+  e = launch_cluster_after_predecessor(parts, fn, groups * parts, kK7Threads, kK7SmemBytes, st, tm.Q.map, tm.dO.map,
+                                       performer ? tm.W2.map : tm.Q.map, tm.abf.map, prm);
+  if (e != cudaSuccess) { *cuda_err = (int)e; (void)cudaGetLastError(); return -6; }
+  return 0;
+}
+
 // ---- backward of the query side (PERFORMER, d = 64, p = 64, 128, 192 or 256): dQ, and da, db added to --
 // abf: scratch for the two bf16 terms of a, [BH][2][p][64]
 inline int launch_k4(TensorContext& tc, bool performer, const void* Q, const void* dO, const void* W, const float* a32,
-                     const float* weight, __nv_bfloat16* abf, void* dQ, float* da, float* db, int BH, int H, int N,
+                     const float* weight, const __nv_bfloat16* abf, void* dQ, float* da, float* db, int BH, int H, int N,
                      int d, int p, int* status, cudaStream_t st, int* cuda_err, void* rowstat = nullptr) {
   // rowstat: d = 128 only, 8 bytes per query row of every 128-row tile (BH * ceil(N / 128) * 128 rows)
   TensorMaps& tm = tc.maps;
@@ -498,12 +547,6 @@ inline int launch_k4(TensorContext& tc, bool performer, const void* Q, const voi
       !encode_map(&tm.abf, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, 3, abf, dA, bA)) {
     *cuda_err = (int)cudaErrorInvalidValue;
     return -6;
-  }
-  {
-    const long long total = (long long)BH * p * d;
-    int grid = (int)((total + 255) / 256);
-    if (grid > 148 * 8) grid = 148 * 8;
-    k4_split_a<<<grid, 256, 0, st>>>(a32, abf, BH, p, d);
   }
   K4Params prm;
   prm.N = N; prm.p = p; prm.BH = BH; prm.H = H; prm.d = d;
