@@ -515,11 +515,12 @@ inline int launch_k7(TensorContext& tc, bool performer, const void* Q, const voi
   prm.da = da; prm.db = db; prm.status = status;
   const int parts = (p + 127) / 128;                      // 1 or 2 CTAs share a tile
   auto fn = !performer ? k7_bwd_query_side<false, 1> : (parts == 2 ? k7_bwd_query_side<true, 2> : k7_bwd_query_side<true, 1>);
-  cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, kK7SmemBytes);
+  const int smem = performer ? K7Smem<true>::bytes : K7Smem<false>::bytes;
+  cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
   if (e != cudaSuccess) { *cuda_err = (int)e; (void)cudaGetLastError(); return -6; }
   const int groups = std::max(1, std::min(tc.sm_count() / parts, prm.total_tiles));
   // the RNN kernel ignores tmW; pass any valid map
-  e = launch_cluster_after_predecessor(parts, fn, groups * parts, kK7Threads, kK7SmemBytes, st, tm.Q.map, tm.dO.map,
+  e = launch_cluster_after_predecessor(parts, fn, groups * parts, kK7Threads, smem, st, tm.Q.map, tm.dO.map,
                                        performer ? tm.W2.map : tm.Q.map, tm.abf.map, prm);
   if (e != cudaSuccess) { *cuda_err = (int)e; (void)cudaGetLastError(); return -6; }
   return 0;
