@@ -899,6 +899,30 @@ BackwardLayout make_backward_layout(const Problem& pr) {
   return b;
 }
 
+template <typename T, bool P, int R, int NB>
+int launch_simt_bwd_key_side_as(const Problem& pr, const float* kpvp, const void* W, const float* weight, const float* a32,
+                                const float* da, const float* db, float* dkpvp, __nv_bfloat16* split, cudaStream_t st) {
+  const size_t smem = simt_bwd_key_side_smem(R, pr.d);
+  auto fn = simt_bwd_key_side<T, P, R, NB>;
+  cudaError_t e = cudaSuccess;
+  if (smem > 48 * 1024) e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (e == cudaSuccess)
+    e = launch_after_predecessor(fn, dim3((pr.k + 16 * R - 1) / (16 * R), pr.BH()), kSimtThreads, smem, st, kpvp,
+                                 (const T*)W, weight, a32, da, db, dkpvp, split, pr.BH(), pr.d, pr.k, pr.p());
+  return e == cudaSuccess ? FLURKA_OK : cuda_fail(e);
+}
+
+template <typename T, bool P>
+int launch_simt_bwd_key_side(const Problem& pr, const float* kpvp, const void* W, const float* weight, const float* a32,
+                             const float* da, const float* db, float* dkpvp, __nv_bfloat16* split, cudaStream_t st) {
+  // 64 keys per block where that still gives every SM a block, else 32
+  const bool big = (long long)((pr.k + 63) / 64) * pr.BH() >= 148;
+  if (pr.d > 64) return big ? launch_simt_bwd_key_side_as<T, P, 4, 2>(pr, kpvp, W, weight, a32, da, db, dkpvp, split, st)
+                            : launch_simt_bwd_key_side_as<T, P, 2, 2>(pr, kpvp, W, weight, a32, da, db, dkpvp, split, st);
+  return big ? launch_simt_bwd_key_side_as<T, P, 4, 1>(pr, kpvp, W, weight, a32, da, db, dkpvp, split, st)
+             : launch_simt_bwd_key_side_as<T, P, 2, 1>(pr, kpvp, W, weight, a32, da, db, dkpvp, split, st);
+}
+
 template <typename T, bool P>
 int backward_pipeline(const Problem& pr, const BackwardLayout& BL, char* ws, const void* Q, const void* K,
                       const void* V, const void* E, const void* F, const void* W, const void* dO, void* dQ, void* dK,
@@ -960,28 +984,25 @@ int backward_pipeline(const Problem& pr, const BackwardLayout& BL, char* ws, con
                                 pr.p(), smh);
     ++*launches;
   }
+  __nv_bfloat16* split = tc ? (__nv_bfloat16*)(ws + BL.split) : nullptr;
   if (tc && P && pr.d == 64) {
-    rc = launch_k6(*tc, W, kpvp, weight, a32, da, db, dkpvp, pr.BH(), pr.k, pr.p(), (int*)(ws + L.status), st, &cuda_err);
+    rc = launch_k6(*tc, W, kpvp, weight, a32, da, db, split, pr.BH(), pr.k, pr.p(), (int*)(ws + L.status), st, &cuda_err);
     if (rc) { g_last_cuda_error = cuda_err; return rc; }
     ++*launches;
   } else {
-    auto fn = simt_bwd_key_side<T, P>;
-    const size_t smem = ((size_t)3 * 32 * (pr.d + 1) + (size_t)2 * 8 * kBwdKeysPerWarp * pr.d) * 4;
-    if ((e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess)
-      return cuda_fail(e);
-    dim3 grid((pr.k + 8 * kBwdKeysPerWarp - 1) / (8 * kBwdKeysPerWarp), pr.BH());
-    fn<<<grid, 256, smem, st>>>(kpvp, (const T*)W, weight, a32, da, db, dkpvp, pr.BH(), pr.d, pr.k, pr.p());
+    rc = launch_simt_bwd_key_side<T, P>(pr, kpvp, W, weight, a32, da, db, dkpvp, split, st);
+    if (rc) return rc;
     ++*launches;
   }
-  if (tc && efh == 0) {
+  if (tc) {
     const bool padded = Ep != E;
     void *dEp = padded ? (void*)Ep : dE, *dFp = padded ? (void*)Fp : dF;   // the copies are not read again after this
-    rc = launch_k5(*tc, Ep, Fp, K, V, dkpvp, (__nv_bfloat16*)(ws + BL.split), dK, dV, dEp, dFp, pr.BH(), smh, pr.N, pr.d,
-                   pr.k, ef_pitch(pr), (int*)(ws + L.status), st, &cuda_err);
+    rc = launch_k5(*tc, Ep, Fp, K, V, split, dK, dV, dEp, dFp, pr.BH(), smh, pr.N, pr.d, pr.k, efh, ef_pitch(pr),
+                   (int*)(ws + L.status), st, &cuda_err);
     if (rc) { g_last_cuda_error = cuda_err; return rc; }
-    *launches += 3;
+    *launches += 2;
     if (padded) {
-      rc = launch_unpad_rows(dEp, dFp, dE, dF, pr.k, pr.N, ef_pitch(pr), st, &cuda_err);
+      rc = launch_unpad_rows(dEp, dFp, dE, dF, pr.k * (efh > 0 ? efh : 1), pr.N, ef_pitch(pr), st, &cuda_err);
       if (rc) { g_last_cuda_error = cuda_err; return rc; }
       ++*launches;
     }

@@ -12,11 +12,12 @@
 //     dV' += A^T da,   dK' += dL^T W,   s += dL^T 1      (A, dL as bf16 tiles the feature owners write into
 //     shared memory in the canonical 128-byte-swizzled layout, read as MN-major A operands),
 // and the key owners finish with dk'_j = (dL^T W)_j - k'_j s_j.  Nothing is shared between CTAs: dK', dV' rows
-// are written once, with plain stores.
+// are written once, with plain stores, as the two bf16 terms the products with E, F, K, V read.
 #pragma once
 
 #include <cuda_bf16.h>
 
+#include "k2_key_side.cuh"
 #include "tc_common.cuh"
 
 namespace flurka {
@@ -28,7 +29,7 @@ struct K6Params {
   const float* a32;             // [BH][p][64]
   const float* da;              // [BH][p][64]
   const float* db;              // [BH][p]
-  float* dkpvp;                 // [2][BH][k][64]  dK', dV'
+  __nv_bfloat16* split;         // [2][2 terms][k][BH][64]  dK', dV' as two bf16 terms
   int* status;
 };
 
@@ -116,6 +117,7 @@ k6_bwd_key_side(const __grid_constant__ CUtensorMap tmW, const K6Params prm) {
       o16[e] = __float2bfloat16_rn(c == 0 && n < 128 ? 1.f : 0.f);
     }
   }
+  grid_dependency_wait();
   // ---- K' and V' of the chunk, once: fp32 rows from the workspace -> bf16 terms; n_j = -|k'_j|^2 / 2
   {
     const int ccol = (lane & 15) * 4;                   // 16 lanes per row of 64 floats
@@ -288,6 +290,7 @@ k6_bwd_key_side(const __grid_constant__ CUtensorMap tmW, const K6Params prm) {
     }
   }
 
+  if (tid == 0) grid_launch_dependents();
   // ---- key owners: dv'_j and dk'_j = (dL^T W)_j - k'_j s_j, one row of 64 floats each
   if (ok && warp < 4) {
     tcgen05_fence_after();
@@ -297,8 +300,9 @@ k6_bwd_key_side(const __grid_constant__ CUtensorMap tmW, const K6Params prm) {
     tmem_wait_ld(rs);
     const float sj = __uint_as_float(rs[0]);
     const bool live = j < keys;
-    float* dk = prm.dkpvp + ((size_t)head * k + j0 + (live ? j : 0)) * 64;
-    float* dv = prm.dkpvp + (((size_t)prm.BH + head) * k + j0 + (live ? j : 0)) * 64;
+    const size_t hd = (size_t)prm.BH * 64, term = (size_t)k * hd;
+    __nv_bfloat16* dk = prm.split + (size_t)(j0 + (live ? j : 0)) * hd + (size_t)head * 64;
+    __nv_bfloat16* dv = dk + 2 * term;
     const float* kr = Kp + (size_t)(live ? j : 0) * 64;
 #pragma unroll 1
     for (int c = 0; c < 64; c += 32) {
@@ -308,15 +312,19 @@ k6_bwd_key_side(const __grid_constant__ CUtensorMap tmW, const K6Params prm) {
       tmem_wait_ld(r1);
       tmem_wait_ld(r2);
       if (live) {
+        float x[32];
 #pragma unroll
         for (int e = 0; e < 32; e += 4) {
           const float4 kv = *reinterpret_cast<const float4*>(kr + c + e);
-          *reinterpret_cast<float4*>(dk + c + e) =
-              make_float4(fmaf(-kv.x, sj, __uint_as_float(r1[e])), fmaf(-kv.y, sj, __uint_as_float(r1[e + 1])),
-                          fmaf(-kv.z, sj, __uint_as_float(r1[e + 2])), fmaf(-kv.w, sj, __uint_as_float(r1[e + 3])));
-          *reinterpret_cast<float4*>(dv + c + e) = make_float4(__uint_as_float(r2[e]), __uint_as_float(r2[e + 1]),
-                                                               __uint_as_float(r2[e + 2]), __uint_as_float(r2[e + 3]));
+          x[e] = fmaf(-kv.x, sj, __uint_as_float(r1[e]));
+          x[e + 1] = fmaf(-kv.y, sj, __uint_as_float(r1[e + 1]));
+          x[e + 2] = fmaf(-kv.z, sj, __uint_as_float(r1[e + 2]));
+          x[e + 3] = fmaf(-kv.w, sj, __uint_as_float(r1[e + 3]));
         }
+        k2_store_split(dk + c, term, x);
+#pragma unroll
+        for (int e = 0; e < 32; ++e) x[e] = __uint_as_float(r2[e]);
+        k2_store_split(dv + c, term, x);
       }
     }
   }

@@ -213,139 +213,151 @@ simt_bwd_query_side(const T* __restrict__ Q, const T* __restrict__ W, const T* _
 }
 
 // ---------------------------------------------------------------------------------------------
-// Key side.  grid = (ceil(k/32), B*H); block = 256: a warp owns four projected keys, so that every
-// chunk of W, a, da a block brings into shared memory (32 features at a time) serves 32 keys and every
-// value read from it in the inner loops serves four.  Lane = feature for the scalar parts (A_ij, g_ij),
-// lane = column for the sums over features; A and dL of a chunk go through shared memory so that the
-// column loop reads the four keys' values of a feature with one 16-byte broadcast load each.
-// Inputs: K', V' (KpVp), W, a, b (weight), da, db.  Outputs: dKpVp [2][B*H][k][d] fp32 (dK' then dV').
-// Dynamic shared memory: 3 * 32 * (d+1) floats (W, a, da chunks) + 2 * 32 * d floats (the block's keys, values).
+// Key side.  grid = (ceil(k / 16R), B*H); block = 256 (the building blocks of simt_kernels.cuh): a block owns 16 R
+// projected keys and walks the features 64 at a time: the exponents k'_j . w_i and the products v'_j . da_i are dot
+// products of rows, the weights A and dL go through shared memory, and dv'_j = sum_i A_ij da_i,
+// dk'_j = sum_i dL_ij w_i - k'_j sum_i dL_ij are register-tile products that read da and W where the dot products left
+// them.  Inputs: K', V' (KpVp), W, a, b (weight), da, db.  Outputs: dKpVp [2][B*H][k][d] fp32 (dK' then dV').
+// Bound by shared memory reads (R = 2: six 16-byte reads per 32 FMA).  RNN, B H = 96, k = 256, d = 64: BKR_FIG;
+// PERFORMER, B H = 8, k = 512, m = 256, d = 128: BKP_FIG (a warp with four keys, scalar reads, before).
 // ---------------------------------------------------------------------------------------------
-constexpr int kBwdKeysPerWarp = 4;
-template <typename T, bool kPerformer>
-__global__ void __launch_bounds__(256, 4)
+inline size_t simt_bwd_key_side_smem(int R, int d) {
+  return ((size_t)(2 * 64 + 2 * 16 * R) * simt_ld(d) + (size_t)2 * 16 * R * 68 + 128 + 128) * 4;
+}
+template <typename T, bool kPerformer, int R, int NB>
+__global__ void __launch_bounds__(kSimtThreads, NB == 1 ? 2 : 1)
 simt_bwd_key_side(const float* __restrict__ KpVp, const T* __restrict__ W, const float* __restrict__ weight,
                   const float* __restrict__ a32, const float* __restrict__ da, const float* __restrict__ db,
-                  float* __restrict__ dKpVp, int BH, int d, int k, int p) {
-  constexpr int KW = kBwdKeysPerWarp;
-  extern __shared__ float smem[];
-  float* Ws = smem;                          // [32][d+1]
-  float* As = Ws + 32 * (d + 1);             // [32][d+1]
-  float* Ds = As + 32 * (d + 1);             // [32][d+1]  da chunk
-  // the block's 8 * KW keys and values, rows of d floats (dynamic: d = 64 leaves room for a fourth block per SM)
-  float* ks = Ds + 32 * (d + 1);             // [8 * KW][d]
-  float* vs = ks + 8 * KW * d;               // [8 * KW][d]
-  __shared__ __align__(16) float sA[8][32][KW], sdL[8][32][KW];
-  __shared__ float bs[32], dbs[32];
-
-  const int bh = blockIdx.y;
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int j0 = (blockIdx.x * 8 + warp) * KW;                 // this warp's keys j0 .. j0 + KW - 1
+                  float* __restrict__ dKpVp, __nv_bfloat16* __restrict__ split, int BH, int d, int k, int p) {
+  // split != NULL: the results leave as two bf16 terms, [2][2 terms][k][BH][d] (what k5_bwd_projections reads), else
+  // as fp32 into dKpVp
+  extern __shared__ __align__(16) float smem[];
+  constexpr int kRows = 16 * R, kLd = 68;
+  const int ld = simt_ld(d), cols = (d + 3) & ~3;
+  float* Ks = smem;                        // [16R][ld]
+  float* Vs = Ks + kRows * ld;             // [16R][ld]
+  float* Ws = Vs + kRows * ld;             // [64][ld]
+  float* Ds = Ws + 64 * ld;                // [64][ld]  da (the products below may read past its end: columns nobody keeps)
+  float* As = Ds + 64 * ld;                // [16R][68] A
+  float* Ls = As + kRows * kLd;            // [16R][68] dL
+  float* bs = Ls + kRows * kLd;            // [64] b_i (RNN: 1 / z_i)
+  float* es = bs + 64;                     // [64] db_i - da_i . a_i
+  float* nrm = es + 64;                    // [16R <= 128] |k'_j|^2 / 2
+  const int bh = blockIdx.y, j0 = blockIdx.x * kRows;
+  const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
+  const bool vec = (d & 3) == 0;
   const float* __restrict__ Kp = KpVp + (size_t)bh * k * d;
   const float* __restrict__ Vp = KpVp + ((size_t)BH + bh) * (size_t)k * d;
-  float half_sq[KW];
-#pragma unroll
-  for (int q = 0; q < KW; ++q) {
-    const bool key_live = j0 + q < k;
-    float hs = 0.f;
-    for (int c = lane; c < d; c += 32) {
-      const float x = key_live ? Kp[(size_t)(j0 + q) * d + c] : 0.f;
-      ks[(warp * KW + q) * d + c] = x;
-      vs[(warp * KW + q) * d + c] = key_live ? Vp[(size_t)(j0 + q) * d + c] : 0.f;
-      hs = fmaf(x, x, hs);
+  tc::grid_launch_dependents();
+  tc::grid_dependency_wait();
+
+  const size_t hd = (size_t)BH * d, term = (size_t)k * hd;
+  auto put = [&](int z, int j, int c, float v) {       // element (j, c) of dK' (z = 0) or dV'
+    if (split) {
+      __nv_bfloat16* o = split + (size_t)z * 2 * term + (size_t)j * hd + (size_t)bh * d + c;
+      const __nv_bfloat16 hi = __float2bfloat16_rn(v);
+      o[0] = hi;
+      o[term] = __float2bfloat16_rn(v - __bfloat162float(hi));
+    } else {
+      dKpVp[(((size_t)z * BH + bh) * k + j) * d + c] = v;
     }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) hs += __shfl_xor_sync(0xffffffffu, hs, o);
-    half_sq[q] = 0.5f * hs;
+  };
+  for (int idx = threadIdx.x; idx < kRows * (cols >> 2); idx += kSimtThreads) {
+    const int r = idx / (cols >> 2), c = (idx % (cols >> 2)) * 4;
+    const int live = j0 + r < k ? d - c : 0;
+    *reinterpret_cast<float4*>(Ks + r * ld + c) = simt_load_row4(Kp + (size_t)(j0 + r) * d + c, live, vec);
+    *reinterpret_cast<float4*>(Vs + r * ld + c) = simt_load_row4(Vp + (size_t)(j0 + r) * d + c, live, vec);
   }
-  float dk[KW][4], dv[KW][4], dl_sum[KW];
+  float dk[R][NB * 4], dv[R][NB * 4], dl_sum[R];
 #pragma unroll
-  for (int q = 0; q < KW; ++q) {
-    dl_sum[q] = 0.f;
+  for (int r = 0; r < R; ++r) {
+    dl_sum[r] = 0.f;
 #pragma unroll
-    for (int b = 0; b < 4; ++b) dk[q][b] = dv[q][b] = 0.f;
+    for (int c = 0; c < NB * 4; ++c) dk[r][c] = dv[r][c] = 0.f;
   }
-  for (int i0 = 0; i0 < p; i0 += 32) {
+  __syncthreads();
+  if (kPerformer && threadIdx.x < kRows) {
+    float s = 0.f;
+    for (int c = 0; c < cols; ++c) s = fmaf(Ks[threadIdx.x * ld + c], Ks[threadIdx.x * ld + c], s);
+    nrm[threadIdx.x] = 0.5f * s;
+  }
+  for (int i0 = 0; i0 < p; i0 += 64) {
     __syncthreads();
-    for (int idx = threadIdx.x; idx < 32 * d; idx += 256) {
-      const int ii = idx / d, c = idx % d;
-      const bool in = i0 + ii < p;
-      const size_t g = ((size_t)bh * p + i0 + ii) * d + c;
-      if (kPerformer) Ws[ii * (d + 1) + c] = in ? to_f32(W[(size_t)(i0 + ii) * d + c]) : 0.f;
-      As[ii * (d + 1) + c] = in ? a32[g] : 0.f;
-      Ds[ii * (d + 1) + c] = in ? da[g] : 0.f;
-    }
-    if (threadIdx.x < 32) {
-      const bool in = i0 + threadIdx.x < p;
-      bs[threadIdx.x] = in ? weight[(size_t)bh * p + i0 + threadIdx.x] : 0.f;
-      dbs[threadIdx.x] = in ? db[(size_t)bh * p + i0 + threadIdx.x] : 0.f;
+    for (int idx = threadIdx.x; idx < 64 * (cols >> 2); idx += kSimtThreads) {
+      const int r = idx / (cols >> 2), c = (idx % (cols >> 2)) * 4;
+      const int live = i0 + r < p ? d - c : 0;
+      if (kPerformer) *reinterpret_cast<float4*>(Ws + r * ld + c) = simt_load_row4(W + (size_t)(i0 + r) * d + c, live, vec);
+      *reinterpret_cast<float4*>(Ds + r * ld + c) = simt_load_row4(da + ((size_t)bh * p + i0 + r) * d + c, live, vec);
     }
     __syncthreads();
-    const bool feat_live = (i0 + lane) < p;
-    // A_ij and g_ij for feature i = i0 + lane and the warp's four keys
-    float e1[KW], wk[KW];
-#pragma unroll
-    for (int q = 0; q < KW; ++q) e1[q] = wk[q] = 0.f;
-    for (int c = 0; c < d; ++c) {
-      const float dsv = Ds[lane * (d + 1) + c], asv = As[lane * (d + 1) + c];
-      const float wsv = kPerformer ? Ws[lane * (d + 1) + c] : 0.f;
-#pragma unroll
-      for (int q = 0; q < KW; ++q) {
-        e1[q] = fmaf(dsv, vs[(warp * KW + q) * d + c] - asv, e1[q]);
-        if (kPerformer) wk[q] = fmaf(wsv, ks[(warp * KW + q) * d + c], wk[q]);
+    {
+      // e_i, four threads per feature
+      const int r = threadIdx.x >> 2;
+      const bool in = i0 + r < p;
+      float s = 0.f;
+      for (int c = (threadIdx.x & 3) * 4; c < cols; c += 16) {
+        const float4 x = *reinterpret_cast<const float4*>(Ds + r * ld + c);
+        const float4 y = simt_load_row4(a32 + ((size_t)bh * p + i0 + r) * d + c, in ? d - c : 0, vec);
+        s = fmaf(x.x, y.x, fmaf(x.y, y.y, fmaf(x.z, y.z, fmaf(x.w, y.w, s))));
+      }
+      s += __shfl_xor_sync(0xffffffffu, s, 1);
+      s += __shfl_xor_sync(0xffffffffu, s, 2);
+      if ((threadIdx.x & 3) == 0) {
+        es[r] = in ? db[(size_t)bh * p + i0 + r] - s : 0.f;
+        const float w = in ? weight[(size_t)bh * p + i0 + r] : 0.f;
+        bs[r] = kPerformer ? w : (in ? 1.f / w : 0.f);
       }
     }
+    __syncthreads();
+    float s[R][4], t[R][4];
 #pragma unroll
-    for (int q = 0; q < KW; ++q) {
-      const bool live = feat_live && (j0 + q < k);
-      float A = 0.f, g = 0.f;
-      if (live) {
-        g = e1[q] + dbs[lane];
-        if (kPerformer) A = expf(wk[q] - half_sq[q] - bs[lane]);     // b_i = log sum_j exp(L_ji): A <= 1
-        else A = elu1(ks[(warp * KW + q) * d + i0 + lane]) / bs[lane];      // weight holds z_i for RNN
-      }
-      const float dL = A * g;
-      dl_sum[q] += dL;
-      if (!kPerformer && live) {
-        const float x = ks[(warp * KW + q) * d + i0 + lane];
-        dKpVp[((size_t)bh * k + j0 + q) * d + i0 + lane] = dL * elu1_slope(x) / elu1(x);
-      }
-      sA[warp][lane][q] = A;
-      sdL[warp][lane][q] = dL;
-    }
-    __syncwarp();
-    for (int ii = 0; ii < 32; ++ii) {
-      const float4 A4 = *reinterpret_cast<const float4*>(&sA[warp][ii][0]);
-      const float4 L4 = *reinterpret_cast<const float4*>(&sdL[warp][ii][0]);
-      const float Aq[KW] = {A4.x, A4.y, A4.z, A4.w}, Lq[KW] = {L4.x, L4.y, L4.z, L4.w};
+    for (int r = 0; r < R; ++r)
 #pragma unroll
-      for (int b = 0; b < 4; ++b) {
-        const int c = lane + 32 * b;
-        if (c < d) {
-          const float dsv = Ds[ii * (d + 1) + c];
-          const float wsv = kPerformer ? Ws[ii * (d + 1) + c] : 0.f;
+      for (int f = 0; f < 4; ++f) s[r][f] = t[r][f] = 0.f;
+    if (kPerformer) simt_dots<R>(s, Ks, Ws, ld, cols);
+    simt_dots<R>(t, Vs, Ds, ld, cols);
 #pragma unroll
-          for (int q = 0; q < KW; ++q) {
-            dv[q][b] = fmaf(Aq[q], dsv, dv[q][b]);
-            if (kPerformer) dk[q][b] = fmaf(Lq[q], wsv, dk[q][b]);
+    for (int r = 0; r < R; ++r) {
+      const int row = ty + 16 * r;
+#pragma unroll
+      for (int f = 0; f < 4; ++f) {
+        const int i = tx + 16 * f;
+        float A = 0.f, x = 0.f;
+        if (i0 + i < p && j0 + row < k) {
+          if (kPerformer) {
+            A = expf(s[r][f] - nrm[row] - bs[i]);       // b_i = log sum_j exp(L_ji): A <= 1
+          } else {
+            x = Ks[row * ld + i0 + i];
+            A = elu1(x) * bs[i];
           }
         }
+        const float dL = A * (t[r][f] + es[i]);
+        dl_sum[r] += dL;
+        As[row * kLd + i] = A;
+        Ls[row * kLd + i] = dL;
+        if (!kPerformer && i0 + i < p && j0 + row < k) put(0, j0 + row, i0 + i, dL * elu1_slope(x) / elu1(x));
       }
     }
-    __syncwarp();
+    __syncthreads();
+    const int kk = min(64, (p - i0 + 3) & ~3);
+    simt_product<R, NB>(dv, As, kLd, Ds, ld, kk);
+    if (kPerformer) simt_product<R, NB>(dk, Ls, kLd, Ws, ld, kk);
   }
 #pragma unroll
-  for (int q = 0; q < KW; ++q) {
-    if (j0 + q >= k) continue;
-    float ds = dl_sum[q];
+  for (int r = 0; r < R; ++r) {
+    float ds = dl_sum[r];
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) ds += __shfl_xor_sync(0xffffffffu, ds, o);
+    for (int o = 8; o > 0; o >>= 1) ds += __shfl_xor_sync(0xffffffffu, ds, o);
+    const int row = ty + 16 * r;
+    if (j0 + row >= k) continue;
 #pragma unroll
-    for (int b = 0; b < 4; ++b) {
-      const int c = lane + 32 * b;
-      if (c < d) {
-        if (kPerformer) dKpVp[((size_t)bh * k + j0 + q) * d + c] = dk[q][b] - ks[(warp * KW + q) * d + c] * ds;
-        dKpVp[(((size_t)BH + bh) * k + j0 + q) * d + c] = dv[q][b];
+    for (int q = 0; q < NB; ++q) {
+      const int c0 = q * 64 + tx * 4;
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        if (c0 + e >= d) continue;
+        if (kPerformer) put(0, j0 + row, c0 + e, dk[r][q * 4 + e] - Ks[row * ld + c0 + e] * ds);
+        put(1, j0 + row, c0 + e, dv[r][q * 4 + e]);
       }
     }
   }

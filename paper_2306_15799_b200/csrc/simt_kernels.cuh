@@ -77,16 +77,16 @@ __device__ __forceinline__ float4 simt_load_row4(const T* p, int live, bool vec)
 // consecutive rows fall into different banks
 __host__ __device__ __forceinline__ int simt_ld(int cols) { return (((cols + 3) >> 2) | 1) << 2; }
 
-// acc[r][..] += A[row][0 .. kk) B[0 .. kk)[cols]; A rows `lda` floats apart, B rows 64 NB; kk a multiple of 4
+// acc[r][..] += A[row][0 .. kk) B[0 .. kk)[cols]; A rows `lda`, B rows `ldb` floats apart; kk a multiple of 4
 template <int R, int NB>
-__device__ __forceinline__ void simt_product(float (&acc)[R][NB * 4], const float* A, int lda, const float* Bt, int kk) {
+__device__ __forceinline__ void simt_product(float (&acc)[R][NB * 4], const float* A, int lda, const float* Bt, int ldb, int kk) {
   const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
   for (int t = 0; t < kk; t += 4) {
     float4 b[4][NB];
 #pragma unroll
     for (int u = 0; u < 4; ++u)
 #pragma unroll
-      for (int q = 0; q < NB; ++q) b[u][q] = *reinterpret_cast<const float4*>(Bt + (t + u) * (64 * NB) + q * 64 + tx * 4);
+      for (int q = 0; q < NB; ++q) b[u][q] = *reinterpret_cast<const float4*>(Bt + (t + u) * ldb + q * 64 + tx * 4);
 #pragma unroll
     for (int r = 0; r < R; ++r) {
       const float4 a = *reinterpret_cast<const float4*>(A + (ty + 16 * r) * lda + t);
@@ -183,7 +183,7 @@ simt_down_project(const T* __restrict__ Kin, const T* __restrict__ Vin, const T*
     for (int i = 0; i < kXV; ++i) *reinterpret_cast<float4*>(Xs + (threadIdx.x + i * kSimtThreads) * 4) = rx[i];
     __syncthreads();
     if (n0 + kSimtTN < n_end) fetch(n0 + kSimtTN);
-    simt_product<R, NB>(acc, Ps, kLd, Xs, kSimtTN);
+    simt_product<R, NB>(acc, Ps, kLd, Xs, 64 * NB, kSimtTN);
     __syncthreads();
   }
   tc::grid_dependency_wait();          // KpVp has been zeroed
@@ -338,7 +338,7 @@ simt_attend(const T* __restrict__ Q, const T* __restrict__ W, const float* __res
       run_sum[r] += part;
     }
     __syncthreads();
-    simt_product<R, NB>(acc, Ps, kLd, Vs, min(64, (items - i0 + 3) & ~3));
+    simt_product<R, NB>(acc, Ps, kLd, Vs, 64 * NB, min(64, (items - i0 + 3) & ~3));
   }
 #pragma unroll
   for (int r = 0; r < R; ++r) {

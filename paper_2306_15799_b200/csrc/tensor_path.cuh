@@ -156,7 +156,6 @@ struct TensorContext {
   bool k1p_attr = false;
   bool k0_attr = false;
   bool k0p_attr = false;
-  bool k5_attr = false;
   int sm_total() {
     if (!sms) {
       int dev = 0;
@@ -569,73 +568,68 @@ inline int launch_k4(TensorContext& tc, bool performer, const void* Q, const voi
   return 0;
 }
 
-// ---- backward of the down-projection: dK, dV, dE, dF from the fp32 dK', dV' (shared E, F) -------------
-// split: scratch for the two bf16 terms of dK', dV', [2][k][2][BH][d]
+// ---- backward of the down-projection: dK, dV, dE, dF from dK', dV' as two bf16 terms ----------------------------
+// split: [2][2 terms][k][BH][d] bf16; ef_heads > 0: E, F, dE, dF are [ef_heads][k][N]
 // ef_pitch: elements between the rows of E, F, dE, dF.  When it is not N, E, F are padded copies that the last
 // product overwrites with dE, dF (dE == E, dF == F), and the caller copies those to their dense form.
-inline int launch_k5(TensorContext& tc, const void* E, const void* F, const void* K, const void* V, const float* dkpvp,
-                     __nv_bfloat16* split, void* dK, void* dV, void* dE, void* dF, int BH, int H, int N, int d, int k,
-                     int ef_pitch, int* status, cudaStream_t st, int* cuda_err) {
+template <int kMode, int kN>
+inline cudaError_t launch_k5_as(TensorContext& tc, const CachedMap& p0, const CachedMap& p1, const CachedMap& s,
+                                const CachedMap& o0, const CachedMap& o1, K5Params p, cudaStream_t st) {
+  using Sh = K5Shape<kMode, kN>;
+  const int rows = kMode == 0 ? p.N : p.k, cols = kMode == 0 ? p.slabs * 64 : p.N;
+  p.row_tiles = (rows + 255) / 256;
+  p.col_tiles = (cols + kN - 1) / kN;
+  p.tiles = 2 * p.groups * p.row_tiles * p.col_tiles;
+  auto fn = k5_bwd_projections<kMode, kN>;
+  cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, Sh::kSmemBytes);
+  if (e != cudaSuccess) return e;
+  const int pairs = std::max(1, std::min(tc.sm_count() / 2, p.tiles));
+  return launch_after_predecessor(fn, 2 * pairs, kK5Threads, Sh::kSmemBytes, st, p0.map, p1.map, s.map, o0.map, o1.map, p);
+}
+inline int launch_k5(TensorContext& tc, const void* E, const void* F, const void* K, const void* V,
+                     const __nv_bfloat16* split, void* dK, void* dV, void* dE, void* dF, int BH, int H, int N, int d, int k,
+                     int ef_heads, int ef_pitch, int* status, cudaStream_t st, int* cuda_err) {
   TensorMaps& tm = tc.maps;
+  const int groups = ef_heads > 0 ? ef_heads : 1;
+  K5Params p;
+  p.N = N; p.k = k; p.d = d; p.BH = BH; p.H = H; p.status = status;
+  p.groups = groups;
+  p.slabs = BH / groups * (d >> 6);
+  // 256 x 128 tiles where 256 x 256 ones would leave more than a third of the pairs of SMs without one: such a
+  // launch is bound by the length of one tile
+  const int few = tc.sm_count() / 3;
+  const bool narrow0 = 2 * groups * ((N + 255) / 256) * ((p.slabs + 3) / 4) < few;
+  const bool narrow1 = 2 * groups * ((k + 255) / 256) * ((N + 255) / 256) < few;
   const unsigned long long hd = (unsigned long long)BH * d;
-  const unsigned long long dEF[2] = {(unsigned long long)N, (unsigned long long)k};
-  const unsigned bEF[2] = {64, 64}, bGE[2] = {64, 32};
+  const unsigned long long dEF[3] = {(unsigned long long)N, (unsigned long long)k, (unsigned long long)groups};
+  const unsigned bEF[3] = {64, 64, 1}, bGE[3] = {64, 32, 1};
   const unsigned long long dKV[3] = {(unsigned long long)(H > 0 ? H * d : d), (unsigned long long)N,
                                      (unsigned long long)(H > 0 ? BH / H : BH)};
-  const unsigned bKV[3] = {64, 256, 1}, bGK[3] = {64, 32, 1};
-  const unsigned long long dS[3] = {2 * hd, (unsigned long long)k, 2};
+  const unsigned bKV[3] = {64, narrow1 ? 64u : 128u, 1}, bGK[3] = {64, 32, 1};
+  const unsigned long long dS[3] = {hd, (unsigned long long)k, 4};
   const unsigned bS64[3] = {64, 64, 1}, bS128[3] = {64, 128, 1};
   const CUtensorMapDataType bf = CU_TENSOR_MAP_DATA_TYPE_BFLOAT16;
-  if (!encode_map(&tm.bE, bf, 2, 2, E, dEF, bEF, ef_pitch) || !encode_map(&tm.bF, bf, 2, 2, F, dEF, bEF, ef_pitch) ||
+  if (!encode_map(&tm.bE, bf, 2, 3, E, dEF, bEF, ef_pitch) || !encode_map(&tm.bF, bf, 2, 3, F, dEF, bEF, ef_pitch) ||
       !encode_map(&tm.bK, bf, 2, 3, K, dKV, bKV) || !encode_map(&tm.bV, bf, 2, 3, V, dKV, bKV) ||
       !encode_map(&tm.split64, bf, 2, 3, split, dS, bS64) || !encode_map(&tm.split128, bf, 2, 3, split, dS, bS128) ||
       !encode_map(&tm.gK, bf, 2, 3, dK, dKV, bGK) || !encode_map(&tm.gV, bf, 2, 3, dV, dKV, bGK) ||
-      !encode_map(&tm.gE, bf, 2, 2, dE, dEF, bGE, ef_pitch) || !encode_map(&tm.gF, bf, 2, 2, dF, dEF, bGE, ef_pitch)) {
+      !encode_map(&tm.gE, bf, 2, 3, dE, dEF, bGE, ef_pitch) || !encode_map(&tm.gF, bf, 2, 3, dF, dEF, bGE, ef_pitch)) {
     *cuda_err = (int)cudaErrorInvalidValue;
     return -6;
   }
-  if (!tc.k5_attr) {
-    cudaError_t e = cudaFuncSetAttribute(k5_bwd_projections<0>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         K5Shape<0>::kSmemBytes);
-    if (e == cudaSuccess)
-      e = cudaFuncSetAttribute(k5_bwd_projections<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, K5Shape<1>::kSmemBytes);
-    if (e == cudaSuccess)
-      e = cudaFuncSetAttribute(k5_bwd_projections<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, K5Shape<2>::kSmemBytes);
-    if (e != cudaSuccess) { *cuda_err = (int)e; (void)cudaGetLastError(); return -6; }
-    tc.k5_attr = true;
-  }
-  {
-    const long long total = (long long)2 * BH * k * (d / 4);
-    int grid = (int)((total + 255) / 256);
-    if (grid > 148 * 8) grid = 148 * 8;
-    k5_split_rows<<<grid, 256, 0, st>>>(dkpvp, split, BH, k, d);
-  }
-  K5Params p;
-  p.N = N; p.k = k; p.d = d; p.BH = BH; p.H = H; p.status = status;
-  p.row_blocks = (N + K5Shape<0>::kRows - 1) / K5Shape<0>::kRows;
-  p.col_groups = (int)((hd + 255) / 256);
-  k5_bwd_projections<0><<<2 * p.row_blocks * p.col_groups, kK5Threads, K5Shape<0>::kSmemBytes, st>>>(
-      tm.bE.map, tm.bF.map, tm.split64.map, tm.gK.map, tm.gV.map, p);
-  p.row_blocks = (k + 255) / 256;
-  p.col_groups = (N + 255) / 256;
-  if (2 * p.row_blocks * p.col_groups >= 100) {
-    k5_bwd_projections<1><<<2 * p.row_blocks * p.col_groups, kK5Threads, K5Shape<1>::kSmemBytes, st>>>(
-        tm.bK.map, tm.bV.map, tm.split128.map, tm.gE.map, tm.gF.map, p);
-  } else {
-    // few tiles: 128-row tiles put twice as many CTAs to work, each with four smaller stages in flight
-    p.row_blocks = (k + 127) / 128;
-    k5_bwd_projections<2><<<2 * p.row_blocks * p.col_groups, kK5Threads, K5Shape<2>::kSmemBytes, st>>>(
-        tm.bK.map, tm.bV.map, tm.split128.map, tm.gE.map, tm.gF.map, p);
-  }
-  cudaError_t e = cudaGetLastError();
-  if (e != cudaSuccess) { *cuda_err = (int)e; return -6; }
+  cudaError_t e = narrow0 ? launch_k5_as<0, 128>(tc, tm.bE, tm.bF, tm.split64, tm.gK, tm.gV, p, st)
+                          : launch_k5_as<0, 256>(tc, tm.bE, tm.bF, tm.split64, tm.gK, tm.gV, p, st);
+  if (e == cudaSuccess)
+    e = narrow1 ? launch_k5_as<1, 128>(tc, tm.bK, tm.bV, tm.split128, tm.gE, tm.gF, p, st)
+                : launch_k5_as<1, 256>(tc, tm.bK, tm.bV, tm.split128, tm.gE, tm.gF, p, st);
+  if (e != cudaSuccess) { *cuda_err = (int)e; (void)cudaGetLastError(); return -6; }
   return 0;
 }
 
 // ---- backward of the key side (PERFORMER, d = 64): dK', dV' from da, db ---------------------------------
 inline int launch_k6(TensorContext& tc, const void* W, const float* kpvp, const float* weight, const float* a32,
-                     const float* da, const float* db, float* dkpvp, int BH, int k, int p, int* status, cudaStream_t st,
-                     int* cuda_err) {
+                     const float* da, const float* db, __nv_bfloat16* split, int BH, int k, int p, int* status,
+                     cudaStream_t st, int* cuda_err) {
   TensorMaps& tm = tc.maps;
   const unsigned long long dW[2] = {64ull, (unsigned long long)p};
   const unsigned bW[2] = {64, 128};
@@ -645,12 +639,11 @@ inline int launch_k6(TensorContext& tc, const void* W, const float* kpvp, const 
   }
   K6Params prm;
   prm.k = k; prm.p = p; prm.BH = BH;
-  prm.kpvp = kpvp; prm.weight = weight; prm.a32 = a32; prm.da = da; prm.db = db; prm.dkpvp = dkpvp; prm.status = status;
+  prm.kpvp = kpvp; prm.weight = weight; prm.a32 = a32; prm.da = da; prm.db = db; prm.split = split; prm.status = status;
   cudaError_t e = cudaFuncSetAttribute(k6_bwd_key_side, cudaFuncAttributeMaxDynamicSharedMemorySize, kK6SmemBytes);
   if (e != cudaSuccess) { *cuda_err = (int)e; (void)cudaGetLastError(); return -6; }
-  k6_bwd_key_side<<<BH * ((k + 127) / 128), kK6Threads, kK6SmemBytes, st>>>(tm.W2.map, prm);
-  e = cudaGetLastError();
-  if (e != cudaSuccess) { *cuda_err = (int)e; return -6; }
+  e = launch_after_predecessor(k6_bwd_key_side, BH * ((k + 127) / 128), kK6Threads, kK6SmemBytes, st, tm.W2.map, prm);
+  if (e != cudaSuccess) { *cuda_err = (int)e; (void)cudaGetLastError(); return -6; }
   return 0;
 }
 
