@@ -862,11 +862,11 @@ int flurka_forward_fused(const void* Xq, const void* Xk, const void* Xv, const v
 
 namespace {
 
-// Scratch of the backward pass, after the forward layout: da [BH][p][d], db [BH][p] (adjacent: one
+// Scratch of the backward pass, after the forward layout: da [BH][p][d], e [BH][p] (adjacent: one
 // range to clear), then dK', dV' [2][BH][k][d]; all fp32.
 struct BackwardLayout {
   Layout L;
-  size_t da, dab_bytes, db, dkpvp, abf, split, rowstat, efpad, total;
+  size_t da, dae_bytes, ei, dkpvp, abf, split, rowstat, efpad, total;
 };
 
 // the query side of the backward has a tensor-core kernel for d = 64 (PERFORMER: any feature count the
@@ -882,9 +882,9 @@ BackwardLayout make_backward_layout(const Problem& pr) {
   size_t off = b.L.total;
   const size_t da_bytes = (size_t)pr.BH() * pr.p() * pr.d * 4;
   b.da = off;
-  b.db = off + da_bytes;
-  b.dab_bytes = da_bytes + (size_t)pr.BH() * pr.p() * 4;
-  off = align256(off + b.dab_bytes);
+  b.ei = off + da_bytes;
+  b.dae_bytes = da_bytes + (size_t)pr.BH() * pr.p() * 4;
+  off = align256(off + b.dae_bytes);
   b.dkpvp = off; off = align256(off + (size_t)2 * pr.BH() * pr.k * pr.d * 4);
   b.abf = off;
   if (backward_tensor_ok(pr)) off = align256(off + (size_t)2 * pr.BH() * pr.p() * pr.d * 2);   // a as two bf16 terms
@@ -899,28 +899,35 @@ BackwardLayout make_backward_layout(const Problem& pr) {
   return b;
 }
 
-template <typename T, bool P, int R, int NB>
-int launch_simt_bwd_key_side_as(const Problem& pr, const float* kpvp, const void* W, const float* weight, const float* a32,
-                                const float* da, const float* db, float* dkpvp, __nv_bfloat16* split, cudaStream_t st) {
+template <typename T, bool P, int R, int NB, int kD>
+int launch_simt_bwd_key_side_at(const Problem& pr, const float* kpvp, const void* W, const float* weight, const float* da,
+                                const float* ei, float* dkpvp, __nv_bfloat16* split, cudaStream_t st) {
   const size_t smem = simt_bwd_key_side_smem(R, pr.d);
-  auto fn = simt_bwd_key_side<T, P, R, NB>;
+  auto fn = simt_bwd_key_side<T, P, R, NB, kD>;
   cudaError_t e = cudaSuccess;
   if (smem > 48 * 1024) e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e == cudaSuccess)
     e = launch_after_predecessor(fn, dim3((pr.k + 16 * R - 1) / (16 * R), pr.BH()), kSimtThreads, smem, st, kpvp,
-                                 (const T*)W, weight, a32, da, db, dkpvp, split, pr.BH(), pr.d, pr.k, pr.p());
+                                 (const T*)W, weight, da, ei, dkpvp, split, pr.BH(), pr.d, pr.k, pr.p());
   return e == cudaSuccess ? FLURKA_OK : cuda_fail(e);
 }
 
+template <typename T, bool P, int R, int NB>
+int launch_simt_bwd_key_side_as(const Problem& pr, const float* kpvp, const void* W, const float* weight, const float* da,
+                                const float* ei, float* dkpvp, __nv_bfloat16* split, cudaStream_t st) {
+  return pr.d == 64 * NB ? launch_simt_bwd_key_side_at<T, P, R, NB, 64 * NB>(pr, kpvp, W, weight, da, ei, dkpvp, split, st)
+                         : launch_simt_bwd_key_side_at<T, P, R, NB, 0>(pr, kpvp, W, weight, da, ei, dkpvp, split, st);
+}
+
 template <typename T, bool P>
-int launch_simt_bwd_key_side(const Problem& pr, const float* kpvp, const void* W, const float* weight, const float* a32,
-                             const float* da, const float* db, float* dkpvp, __nv_bfloat16* split, cudaStream_t st) {
+int launch_simt_bwd_key_side(const Problem& pr, const float* kpvp, const void* W, const float* weight, const float* da,
+                             const float* ei, float* dkpvp, __nv_bfloat16* split, cudaStream_t st) {
   // 64 keys per block where that still gives every SM a block, else 32
   const bool big = (long long)((pr.k + 63) / 64) * pr.BH() >= 148;
-  if (pr.d > 64) return big ? launch_simt_bwd_key_side_as<T, P, 4, 2>(pr, kpvp, W, weight, a32, da, db, dkpvp, split, st)
-                            : launch_simt_bwd_key_side_as<T, P, 2, 2>(pr, kpvp, W, weight, a32, da, db, dkpvp, split, st);
-  return big ? launch_simt_bwd_key_side_as<T, P, 4, 1>(pr, kpvp, W, weight, a32, da, db, dkpvp, split, st)
-             : launch_simt_bwd_key_side_as<T, P, 2, 1>(pr, kpvp, W, weight, a32, da, db, dkpvp, split, st);
+  if (pr.d > 64) return big ? launch_simt_bwd_key_side_as<T, P, 4, 2>(pr, kpvp, W, weight, da, ei, dkpvp, split, st)
+                            : launch_simt_bwd_key_side_as<T, P, 2, 2>(pr, kpvp, W, weight, da, ei, dkpvp, split, st);
+  return big ? launch_simt_bwd_key_side_as<T, P, 4, 1>(pr, kpvp, W, weight, da, ei, dkpvp, split, st)
+             : launch_simt_bwd_key_side_as<T, P, 2, 1>(pr, kpvp, W, weight, da, ei, dkpvp, split, st);
 }
 
 template <typename T, bool P>
@@ -934,10 +941,10 @@ int backward_pipeline(const Problem& pr, const BackwardLayout& BL, char* ws, con
   float* weight = (float*)(ws + L.weight);
   float* a32 = (float*)(ws + L.a32);
   float* da = (float*)(ws + BL.da);
-  float* db = (float*)(ws + BL.db);
+  float* ei = (float*)(ws + BL.ei);
   float* dkpvp = (float*)(ws + BL.dkpvp);
   const int smh = pr.seq_major_heads(), efh = pr.ef_heads();
-  cudaError_t e = launch_clear(ws + L.status, L.kpvp_end - L.status, da, BL.dab_bytes, st);
+  cudaError_t e = launch_clear(ws + L.status, L.kpvp_end - L.status, da, BL.dae_bytes, st);
   if (e != cudaSuccess) return cuda_fail(e);
   // the forward's stages 1 and 2 again: K', V', a_i, b_i (or z_i)
   int rc = FLURKA_OK;
@@ -957,7 +964,7 @@ int backward_pipeline(const Problem& pr, const BackwardLayout& BL, char* ws, con
   if (tc) {
     // the key side on its tensor-core kernel, one CTA per (head, feature tile), with a in fp32 as well
     rc = launch_k2(*tc, P, kpvp, W, weight, nullptr, nullptr, nullptr, pr.BH(), pr.d, pr.k, pr.p(),
-                   (int*)(ws + L.status), st, &cuda_err, a32, tcq ? (__nv_bfloat16*)(ws + BL.abf) : nullptr);
+                   (int*)(ws + L.status), st, &cuda_err, tcq ? nullptr : a32, tcq ? (__nv_bfloat16*)(ws + BL.abf) : nullptr);
     if (rc) { g_last_cuda_error = cuda_err; return rc; }
     ++*launches;
   } else {
@@ -967,10 +974,10 @@ int backward_pipeline(const Problem& pr, const BackwardLayout& BL, char* ws, con
   if (tc && tcq) {
     const __nv_bfloat16* abf = (const __nv_bfloat16*)(ws + BL.abf);
     if (pr.d == 64)
-      rc = launch_k7(*tc, P, Q, dO, W, a32, weight, abf, dQ, da, db, pr.BH(), smh, pr.N, pr.p(), (int*)(ws + L.status), st,
+      rc = launch_k7(*tc, P, Q, dO, W, weight, abf, dQ, da, ei, pr.BH(), smh, pr.N, pr.p(), (int*)(ws + L.status), st,
                      &cuda_err);
     else
-      rc = launch_k4(*tc, P, Q, dO, W, a32, weight, abf, dQ, da, db, pr.BH(), smh, pr.N, pr.d, pr.p(),
+      rc = launch_k4(*tc, P, Q, dO, W, weight, abf, dQ, da, ei, pr.BH(), smh, pr.N, pr.d, pr.p(),
                      (int*)(ws + L.status), st, &cuda_err, ws + BL.rowstat);
     if (rc) { g_last_cuda_error = cuda_err; return rc; }
     ++*launches;
@@ -980,17 +987,17 @@ int backward_pipeline(const Problem& pr, const BackwardLayout& BL, char* ws, con
     if ((e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess)
       return cuda_fail(e);
     dim3 grid((pr.N + 31) / 32, pr.BH());
-    fn<<<grid, 256, smem, st>>>((const T*)Q, (const T*)W, (const T*)dO, weight, a32, (T*)dQ, da, db, pr.N, pr.d,
+    fn<<<grid, 256, smem, st>>>((const T*)Q, (const T*)W, (const T*)dO, weight, a32, (T*)dQ, da, ei, pr.N, pr.d,
                                 pr.p(), smh);
     ++*launches;
   }
   __nv_bfloat16* split = tc ? (__nv_bfloat16*)(ws + BL.split) : nullptr;
   if (tc && P && pr.d == 64) {
-    rc = launch_k6(*tc, W, kpvp, weight, a32, da, db, split, pr.BH(), pr.k, pr.p(), (int*)(ws + L.status), st, &cuda_err);
+    rc = launch_k6(*tc, W, kpvp, weight, da, ei, split, pr.BH(), pr.k, pr.p(), (int*)(ws + L.status), st, &cuda_err);
     if (rc) { g_last_cuda_error = cuda_err; return rc; }
     ++*launches;
   } else {
-    rc = launch_simt_bwd_key_side<T, P>(pr, kpvp, W, weight, a32, da, db, dkpvp, split, st);
+    rc = launch_simt_bwd_key_side<T, P>(pr, kpvp, W, weight, da, ei, dkpvp, split, st);
     if (rc) return rc;
     ++*launches;
   }

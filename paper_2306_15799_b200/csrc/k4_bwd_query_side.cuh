@@ -36,10 +36,9 @@ struct K4Params {
   int d;                        // 64, or 128 (PERFORMER only: see the kernel's header)
   int tiles_per_head, total_tiles;
   const float* weight;          // [BH][p]      b_i
-  const float* a32;             // [BH][p][d]   a_i (fp32)
   __nv_bfloat16* dQ;
   float* da;                    // [BH][p][d]   added to
-  float* db;                    // [BH][p]      added to
+  float* ei;                    // [BH][p]      e_i = db_i - a_i . da_i = -sum_n P_ni delta_n, added to
   float2* rowstat;              // d = 128: [total_tiles * 128] (log-sum-exp, delta) of every row, kept from a
                                 // tile's first visit for its second
   int* status;
@@ -64,19 +63,6 @@ __device__ __forceinline__ float k4_ex2(float x) {
   float y;
   asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
   return y;
-}
-
-// a [BH][p][d] fp32 -> two bf16 terms, [BH][2][p][d]
-__global__ void k4_split_a(const float* __restrict__ a32, __nv_bfloat16* __restrict__ abf, int BH, int p, int d) {
-  const long long per_head = (long long)p * d;
-  const long long total = (long long)BH * per_head;
-  for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += (long long)gridDim.x * blockDim.x) {
-    const long long h = i / per_head, r = i % per_head;
-    const float x = a32[i];
-    const __nv_bfloat16 hi = __float2bfloat16_rn(x);
-    abf[(h * 2) * per_head + r] = hi;
-    abf[(h * 2 + 1) * per_head + r] = __float2bfloat16_rn(x - __bfloat162float(hi));
-  }
 }
 
 template <bool kPerformer, bool kStream>
@@ -187,7 +173,7 @@ k4_bwd_query_side(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
     }
   };
 
-  // da, P^T delta of one head leave TMEM: thread = feature; db from the identity in the header
+  // da, P^T delta of one head leave TMEM: thread = feature; see the header of k7
   auto flush = [&](int hkey) {
     const int head = hkey % prm.BH, dh = hkey / prm.BH;     // dh: which 64 columns of da these accumulators are
     if (!owner || fh >= nh) return;
@@ -199,29 +185,19 @@ k4_bwd_query_side(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
       tmem_wait_ld(dd);
       const int feat = hh * 128 + row;
       const bool live = feat < p;            // (the TMEM loads below are warp-wide: every lane takes them)
-      const float* arow = prm.a32 + ((size_t)head * p + (live ? feat : 0)) * d + dh * 64;
       float* darow = prm.da + ((size_t)head * p + (live ? feat : 0)) * d + dh * 64;
-      float dot = 0.f;
 #pragma unroll 1
       for (int c = 0; c < 64; c += 32) {
         uint32_t r[32];
         tmem_ld32(tmem + lane_off + kK4ColDA + hh * 64 + c, r);
         tmem_wait_ld(r);
 #pragma unroll
-        for (int e = 0; e < 32; e += 4) {
-          const float4 av = *reinterpret_cast<const float4*>(arow + c + e);
-          dot = fmaf(av.x, __uint_as_float(r[e]), dot);
-          dot = fmaf(av.y, __uint_as_float(r[e + 1]), dot);
-          dot = fmaf(av.z, __uint_as_float(r[e + 2]), dot);
-          dot = fmaf(av.w, __uint_as_float(r[e + 3]), dot);
-        }
-#pragma unroll
         for (int e = 0; e < 32; ++e)
           if (live) atomicAdd(darow + c + e, __uint_as_float(r[e]));
       }
       // (both column halves accumulate P^T delta; it is subtracted once)
       const float pd = dh == 0 ? __uint_as_float(dd[0]) + __uint_as_float(dd[1]) + __uint_as_float(dd[2]) : 0.f;
-      if (live) atomicAdd(prm.db + (size_t)head * p + feat, dot - pd);
+      if (live) atomicAdd(prm.ei + (size_t)head * p + feat, -pd);
     }
     tcgen05_fence_before();
   };

@@ -2,7 +2,7 @@
 //
 // Forward (arxiv 2306.15799, Eq. (2) with Appendix D's normaliser, per feature i in the log domain):
 //     L_ij = w_i . k'_j - |k'_j|^2 / 2,   b_i = log sum_j exp(L_ij),   A_ij = exp(L_ij - b_i),   a_i = sum_j A_ij v'_j.
-// Given da_i, db_i (from the query side), by the chain rule
+// Given da_i and e_i (from the query side, which has it as -sum_n P_ni delta_n), by the chain rule
 //     g_ij = da_i . v'_j + e_i  with  e_i = db_i - da_i . a_i,        dL_ij = A_ij g_ij,
 //     dv'_j = sum_i A_ij da_i,        dk'_j = sum_i dL_ij w_i - k'_j sum_i dL_ij.
 // One CTA owns 128 projected keys of one head and walks the features 128 at a time; every product is a
@@ -26,9 +26,8 @@ struct K6Params {
   int k, p, BH;                 // d = 64
   const float* kpvp;            // [2][BH][k][64]  K', V'
   const float* weight;          // [BH][p]         b_i
-  const float* a32;             // [BH][p][64]
   const float* da;              // [BH][p][64]
-  const float* db;              // [BH][p]
+  const float* ei;              // [BH][p]         db_i - da_i . a_i
   __nv_bfloat16* split;         // [2][2 terms][k][BH][64]  dK', dV' as two bf16 terms
   int* status;
 };
@@ -185,15 +184,7 @@ k6_bwd_key_side(const __grid_constant__ CUtensorMap tmW, const K6Params prm) {
     const int feat = i0 + (warp & 3) * 32 + lane;
     const bool feat_live = warp < 4 && feat < p;
     if (feat_live) {
-      const float4* dr = reinterpret_cast<const float4*>(prm.da + ((size_t)head * p + feat) * 64);
-      const float4* ar = reinterpret_cast<const float4*>(prm.a32 + ((size_t)head * p + feat) * 64);
-      float dot = 0.f;
-#pragma unroll 4
-      for (int c = 0; c < 16; ++c) {
-        const float4 x = dr[c], y = ar[c];
-        dot = fmaf(x.x, y.x, fmaf(x.y, y.y, fmaf(x.z, y.z, fmaf(x.w, y.w, dot))));
-      }
-      e_i = prm.db[(size_t)head * p + feat] - dot;
+      e_i = prm.ei[(size_t)head * p + feat];
       b_i = prm.weight[(size_t)head * p + feat];
     }
     fence_proxy_async_smem();

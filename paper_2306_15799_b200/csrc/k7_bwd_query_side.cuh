@@ -16,8 +16,8 @@
 // cycles per tile.)  What a row needs from the other half of the features, its maximum, sum and weighted sum, crosses
 // the cluster through shared memory (st.async), and so does the half of dQ the other CTA stores, one tile later; S, G
 // of tile i+1 are computed under tile i's arithmetic.
-// da and P^T delta stay in TMEM over all the tiles of a head; they are added to global memory when it changes; db
-// comes from them there.
+// da and P^T delta stay in TMEM over all the tiles of a head; they are added to global memory when it changes.  The
+// key side wants e_i = db_i - a_i . da_i, which is -sum_n P_ni delta_n: db itself is never formed.
 // RNN (kPerformer = false): l_ni = log((elu(q_ni) + 1) z_i), so the weights come from the Q tile in shared memory, no S
 // product, no exponent, and dq_ni = c_ni elu'(q_ni) / (elu(q_ni) + 1) needs no product either.
 // K7_FIG
@@ -35,10 +35,9 @@ struct K7Params {
   int N, p, BH, H;              // H > 0: Q, dO, dQ are [B,N,H,d]; H == 0: [BH,N,d]; d = 64
   int tiles_per_head, total_tiles;
   const float* weight;          // [BH][p]      b_i (RNN: z_i)
-  const float* a32;             // [BH][p][64]  a_i (fp32)
   __nv_bfloat16* dQ;
   float* da;                    // [BH][p][64]  added to
-  float* db;                    // [BH][p]      added to
+  float* ei;                    // [BH][p]      e_i, added to
   int* status;
 };
 
@@ -328,19 +327,13 @@ k7_bwd_query_side(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
         tmem_wait_ld(r);
         const int feat = f0 + row;
         if (feat >= p) return;
-        const float4* arow = reinterpret_cast<const float4*>(prm.a32 + ((size_t)head * p + feat) * 64 + fh * 32);
         float4* darow = reinterpret_cast<float4*>(prm.da + ((size_t)head * p + feat) * 64 + fh * 32);
-        float dot = 0.f;
 #pragma unroll
-        for (int e = 0; e < 8; ++e) {
-          const float4 av = __ldcg(arow + e);
-          const float4 v = make_float4(__uint_as_float(r[4 * e]), __uint_as_float(r[4 * e + 1]), __uint_as_float(r[4 * e + 2]),
-                                       __uint_as_float(r[4 * e + 3]));
-          dot = fmaf(av.x, v.x, fmaf(av.y, v.y, fmaf(av.z, v.z, fmaf(av.w, v.w, dot))));
-          atomicAdd(darow + e, v);
-        }
-        if (fh == 0) dot -= __uint_as_float(dd[0]) + __uint_as_float(dd[1]) + __uint_as_float(dd[2]);
-        atomicAdd(prm.db + (size_t)head * p + feat, dot);
+        for (int e = 0; e < 8; ++e)
+          atomicAdd(darow + e, make_float4(__uint_as_float(r[4 * e]), __uint_as_float(r[4 * e + 1]),
+                                           __uint_as_float(r[4 * e + 2]), __uint_as_float(r[4 * e + 3])));
+        if (fh == 0)
+          atomicAdd(prm.ei + (size_t)head * p + feat, -(__uint_as_float(dd[0]) + __uint_as_float(dd[1]) + __uint_as_float(dd[2])));
       };
       auto dq_row = [&](int head, int row0) {
         return prm.dQ + (prm.H > 0 ? (((size_t)(head / prm.H) * prm.N + row0 + row) * prm.H + (size_t)(head % prm.H)) * 64

@@ -11,7 +11,8 @@
 //                dq_n = sum_i c_ni w_i  (PERFORMER; the -q_n sum_i c_ni term vanishes),
 //                dq_ni = c_ni elu'(q_ni)/(elu(q_ni)+1)  (RNN)
 //                da_i = sum_n P_ni dO_n,   db_i = sum_n c_ni
-//   key side     g_ij = da_i.(v'_j - a_i) + db_i,   dL_ji = A_ij g_ij,   dv'_j = sum_i A_ij da_i,
+//   key side     g_ij = da_i.v'_j + e_i with e_i = db_i - da_i.a_i = -sum_n P_ni (O_n.dO_n) (db itself is never formed),
+//                 dL_ji = A_ij g_ij,   dv'_j = sum_i A_ij da_i,
 //                dk'_j = sum_i dL_ji (w_i - k'_j)  (PERFORMER),  dk'_ji = dL_ji elu'(k'_ji)/(elu(k'_ji)+1)  (RNN)
 //   projections  dK = E^T dK',  dV = F^T dV',  dE = sum_heads dK' K^T,  dF = sum_heads dV' V^T.
 #pragma once
@@ -26,7 +27,7 @@ __device__ __forceinline__ float elu1_slope(float x) { return x > 0.f ? 1.f : ex
 // ---------------------------------------------------------------------------------------------
 // Query side.  grid = (ceil(N/32), B*H); block = 256: warp w owns rows 4w..4w+3 of the tile.
 // Two sweeps over the features in chunks of 32: the first is the forward (running maximum, sum,
-// O_n); the second forms c_ni and accumulates dq_n, da_i, db_i.  da, db (fp32, zeroed before) are
+// O_n); the second forms c_ni and accumulates dq_n, da_i, e_i.  da, e (fp32, zeroed before) are
 // added to with atomics: every row tile of a head contributes.
 // Dynamic shared memory: 2 * 32 * (d+1) floats (W chunk, a chunk) + 32 * 33 (P tile) + 32 * d (dO tile).
 // ---------------------------------------------------------------------------------------------
@@ -34,7 +35,7 @@ template <typename T, bool kPerformer>
 __global__ void __launch_bounds__(256)
 simt_bwd_query_side(const T* __restrict__ Q, const T* __restrict__ W, const T* __restrict__ dO,
                     const float* __restrict__ weight, const float* __restrict__ a32, T* __restrict__ dQ,
-                    float* __restrict__ da, float* __restrict__ db, int N, int d, int p, int seq_major_heads) {
+                    float* __restrict__ da, float* __restrict__ ei, int N, int d, int p, int seq_major_heads) {
   extern __shared__ float smem[];
   float* Ws = smem;                          // [32][d+1]
   float* As = Ws + 32 * (d + 1);             // [32][d+1]
@@ -42,7 +43,7 @@ simt_bwd_query_side(const T* __restrict__ Q, const T* __restrict__ W, const T* _
   float* Gs = Ps + 32 * 33;                  // [32 rows][d]   dO tile
   __shared__ float qs[32][128];
   __shared__ float ws[32];
-  __shared__ float dbs[8][32];
+  __shared__ float es[8][32];
 
   const int bh = blockIdx.y;
   const int n0 = blockIdx.x * 32;
@@ -137,11 +138,11 @@ simt_bwd_query_side(const T* __restrict__ Q, const T* __restrict__ W, const T* _
     t[r] = s;
   }
 
-  // ---- sweep 2: c_ni, dq_n, da_i, db_i
+  // ---- sweep 2: c_ni, dq_n, da_i, e_i
   for (int i0 = 0; i0 < p; i0 += 32) {
     stage_chunk(i0);
     const bool live = (i0 + lane) < p;
-    float db_part = 0.f;
+    float e_part = 0.f;
 #pragma unroll
     for (int r = 0; r < 4; ++r) {
       const int row = warp * 4 + r;
@@ -152,7 +153,7 @@ simt_bwd_query_side(const T* __restrict__ Q, const T* __restrict__ W, const T* _
       float u = 0.f;
       for (int c = 0; c < d; ++c) u = fmaf(As[lane * (d + 1) + c], Gs[row * d + c], u);
       const float cv = P * (u - t[r]);
-      db_part += cv;
+      e_part -= P * t[r];
       Ps[row * 33 + lane] = P;
       if (kPerformer) {
         for (int ii = 0; ii < 32; ++ii) {
@@ -169,7 +170,7 @@ simt_bwd_query_side(const T* __restrict__ Q, const T* __restrict__ W, const T* _
         store_out(dQ + hv.base + (size_t)(n0 + row) * hv.row_stride + i0 + lane, cv * elu1_slope(x) / elu1(x));
       }
     }
-    dbs[warp][lane] = db_part;
+    es[warp][lane] = e_part;
     __syncthreads();
     // da_i[c] += sum over the tile's rows of P_ri dO_r[c]: warp w takes features 4w..4w+3 of the chunk
 #pragma unroll
@@ -194,8 +195,8 @@ simt_bwd_query_side(const T* __restrict__ Q, const T* __restrict__ W, const T* _
     if (warp == 0 && live) {
       float s = 0.f;
 #pragma unroll
-      for (int w8 = 0; w8 < 8; ++w8) s += dbs[w8][lane];
-      atomicAdd(db + (size_t)bh * p + i0 + lane, s);
+      for (int w8 = 0; w8 < 8; ++w8) s += es[w8][lane];
+      atomicAdd(ei + (size_t)bh * p + i0 + lane, s);
     }
   }
   if (kPerformer) {
@@ -217,98 +218,154 @@ simt_bwd_query_side(const T* __restrict__ Q, const T* __restrict__ W, const T* _
 // projected keys and walks the features 64 at a time: the exponents k'_j . w_i and the products v'_j . da_i are dot
 // products of rows, the weights A and dL go through shared memory, and dv'_j = sum_i A_ij da_i,
 // dk'_j = sum_i dL_ij w_i - k'_j sum_i dL_ij are register-tile products that read da and W where the dot products left
-// them.  Inputs: K', V' (KpVp), W, a, b (weight), da, db.  Outputs: dKpVp [2][B*H][k][d] fp32 (dK' then dV').
-// Bound by shared memory reads (R = 2: six 16-byte reads per 32 FMA).  RNN, B H = 96, k = 256, d = 64: BKR_FIG;
-// PERFORMER, B H = 8, k = 512, m = 256, d = 128: BKP_FIG (a warp with four keys, scalar reads, before).
+// them.  Inputs: K', V' (KpVp), W, b (weight), da, e.  Outputs: dK', dV' as two bf16 terms into `split`
+// ([2][2 terms][k][BH][d], what k5_bwd_projections reads), or, split == NULL, as fp32 into dKpVp [2][B*H][k][d].
+// kD: the head dimension where it is known at compile time (all loads of a step are then in flight together, and
+// the next step's travel in registers under this step's products), or 0.
 // ---------------------------------------------------------------------------------------------
 inline size_t simt_bwd_key_side_smem(int R, int d) {
   return ((size_t)(2 * 64 + 2 * 16 * R) * simt_ld(d) + (size_t)2 * 16 * R * 68 + 128 + 128) * 4;
 }
-template <typename T, bool kPerformer, int R, int NB>
-__global__ void __launch_bounds__(kSimtThreads, NB == 1 ? 2 : 1)
+// four consecutive values of a row of dK' or dV'
+__device__ __forceinline__ void simt_put4(float* f32, __nv_bfloat16* hi, size_t term, const float (&v)[4], int live, bool vec) {
+  if (hi) {
+    uint32_t h[2], l[2];
+#pragma unroll
+    for (int e = 0; e < 2; ++e) {
+      const __nv_bfloat162 h2 = __floats2bfloat162_rn(v[2 * e], v[2 * e + 1]);
+      const __nv_bfloat162 l2 = __floats2bfloat162_rn(v[2 * e] - __low2float(h2), v[2 * e + 1] - __high2float(h2));
+      h[e] = *reinterpret_cast<const uint32_t*>(&h2);
+      l[e] = *reinterpret_cast<const uint32_t*>(&l2);
+    }
+    *reinterpret_cast<uint2*>(hi) = make_uint2(h[0], h[1]);            // (only for d = 64, 128: live is 4 or <= 0)
+    *reinterpret_cast<uint2*>(hi + term) = make_uint2(l[0], l[1]);
+  } else if (vec && live >= 4) {
+    *reinterpret_cast<float4*>(f32) = make_float4(v[0], v[1], v[2], v[3]);
+  } else {
+#pragma unroll
+    for (int e = 0; e < 4; ++e)
+      if (e < live) f32[e] = v[e];
+  }
+}
+
+template <typename T, bool kPerformer, int R, int NB, int kD>
+__global__ void __launch_bounds__(256, NB == 1 && kD > 0 && !kPerformer ? 3 : (NB == 1 ? 2 : 1))
 simt_bwd_key_side(const float* __restrict__ KpVp, const T* __restrict__ W, const float* __restrict__ weight,
-                  const float* __restrict__ a32, const float* __restrict__ da, const float* __restrict__ db,
-                  float* __restrict__ dKpVp, __nv_bfloat16* __restrict__ split, int BH, int d, int k, int p) {
-  // split != NULL: the results leave as two bf16 terms, [2][2 terms][k][BH][d] (what k5_bwd_projections reads), else
-  // as fp32 into dKpVp
+                  const float* __restrict__ da, const float* __restrict__ ei, float* __restrict__ dKpVp,
+                  __nv_bfloat16* __restrict__ split, int BH, int d_rt, int k, int p) {
   extern __shared__ __align__(16) float smem[];
   constexpr int kRows = 16 * R, kLd = 68;
-  const int ld = simt_ld(d), cols = (d + 3) & ~3;
+  const int d = kD > 0 ? kD : d_rt;
+  const int ld = kD > 0 ? kD + 4 : simt_ld(d), cols = (d + 3) & ~3, pieces = cols >> 2;
   float* Ks = smem;                        // [16R][ld]
   float* Vs = Ks + kRows * ld;             // [16R][ld]
   float* Ws = Vs + kRows * ld;             // [64][ld]
   float* Ds = Ws + 64 * ld;                // [64][ld]  da (the products below may read past its end: columns nobody keeps)
   float* As = Ds + 64 * ld;                // [16R][68] A
-  float* Ls = As + kRows * kLd;            // [16R][68] dL
+  float* Ls = As + kRows * kLd;            // [16R][68] dL (RNN: dk')
   float* bs = Ls + kRows * kLd;            // [64] b_i (RNN: 1 / z_i)
-  float* es = bs + 64;                     // [64] db_i - da_i . a_i
-  float* nrm = es + 64;                    // [16R <= 128] |k'_j|^2 / 2
+  float* es = bs + 64;                     // [64] e_i
+  float* nrm = es + 64;                    // [16R] |k'_j|^2 / 2
   const int bh = blockIdx.y, j0 = blockIdx.x * kRows;
   const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
-  const bool vec = (d & 3) == 0;
+  const bool vec = kD > 0 || (d & 3) == 0;
   const float* __restrict__ Kp = KpVp + (size_t)bh * k * d;
   const float* __restrict__ Vp = KpVp + ((size_t)BH + bh) * (size_t)k * d;
+  const float* __restrict__ dah = da + (size_t)bh * p * d;
   tc::grid_launch_dependents();
   tc::grid_dependency_wait();
 
-  const size_t hd = (size_t)BH * d, term = (size_t)k * hd;
-  auto put = [&](int z, int j, int c, float v) {       // element (j, c) of dK' (z = 0) or dV'
-    if (split) {
-      __nv_bfloat16* o = split + (size_t)z * 2 * term + (size_t)j * hd + (size_t)bh * d + c;
-      const __nv_bfloat16 hi = __float2bfloat16_rn(v);
-      o[0] = hi;
-      o[term] = __float2bfloat16_rn(v - __bfloat162float(hi));
-    } else {
-      dKpVp[(((size_t)z * BH + bh) * k + j) * d + c] = v;
+  // the step's W and da: into registers first where d is known
+  constexpr int kPre = kD > 0 ? 64 * (kD / 4) / kSimtThreads : 1;
+  float4 rw[kPre], rd[kPre];
+  float rb = 0.f, re = 0.f;
+  auto fetch = [&](int i0) {
+    if constexpr (kD > 0) {
+#pragma unroll
+      for (int u = 0; u < kPre; ++u) {
+        const int idx = threadIdx.x + u * kSimtThreads, r = idx / (kD / 4), c = (idx % (kD / 4)) * 4;
+        const int live = i0 + r < p ? 4 : 0;
+        rd[u] = simt_load_row4(dah + (size_t)(i0 + r) * kD + c, live, true);
+        if (kPerformer) rw[u] = simt_load_row4(W + (size_t)(i0 + r) * kD + c, live, true);
+      }
+    }
+    if (threadIdx.x < 64) {
+      const bool in = i0 + threadIdx.x < p;
+      rb = in ? weight[(size_t)bh * p + i0 + threadIdx.x] : 1.f;
+      re = in ? ei[(size_t)bh * p + i0 + threadIdx.x] : 0.f;
     }
   };
-  for (int idx = threadIdx.x; idx < kRows * (cols >> 2); idx += kSimtThreads) {
-    const int r = idx / (cols >> 2), c = (idx % (cols >> 2)) * 4;
-    const int live = j0 + r < k ? d - c : 0;
-    *reinterpret_cast<float4*>(Ks + r * ld + c) = simt_load_row4(Kp + (size_t)(j0 + r) * d + c, live, vec);
-    *reinterpret_cast<float4*>(Vs + r * ld + c) = simt_load_row4(Vp + (size_t)(j0 + r) * d + c, live, vec);
+  if constexpr (kD > 0) {
+    constexpr int kKV = kRows * (kD / 4) / kSimtThreads;
+    float4 rk[kKV], rv[kKV];
+#pragma unroll
+    for (int u = 0; u < kKV; ++u) {
+      const int idx = threadIdx.x + u * kSimtThreads, r = idx / (kD / 4), c = (idx % (kD / 4)) * 4;
+      const int live = j0 + r < k ? 4 : 0;
+      rk[u] = simt_load_row4(Kp + (size_t)(j0 + r) * kD + c, live, true);
+      rv[u] = simt_load_row4(Vp + (size_t)(j0 + r) * kD + c, live, true);
+    }
+    fetch(0);
+#pragma unroll
+    for (int u = 0; u < kKV; ++u) {
+      const int idx = threadIdx.x + u * kSimtThreads, r = idx / (kD / 4), c = (idx % (kD / 4)) * 4;
+      *reinterpret_cast<float4*>(Ks + r * ld + c) = rk[u];
+      *reinterpret_cast<float4*>(Vs + r * ld + c) = rv[u];
+    }
+  } else {
+    for (int idx = threadIdx.x; idx < kRows * pieces; idx += kSimtThreads) {
+      const int r = idx / pieces, c = (idx % pieces) * 4;
+      const int live = j0 + r < k ? d - c : 0;
+      *reinterpret_cast<float4*>(Ks + r * ld + c) = simt_load_row4(Kp + (size_t)(j0 + r) * d + c, live, vec);
+      *reinterpret_cast<float4*>(Vs + r * ld + c) = simt_load_row4(Vp + (size_t)(j0 + r) * d + c, live, vec);
+    }
+    fetch(0);
   }
-  float dk[R][NB * 4], dv[R][NB * 4], dl_sum[R];
+  float dk[kPerformer ? R : 1][NB * 4], dv[R][NB * 4], dl_sum[R];
 #pragma unroll
   for (int r = 0; r < R; ++r) {
     dl_sum[r] = 0.f;
 #pragma unroll
-    for (int c = 0; c < NB * 4; ++c) dk[r][c] = dv[r][c] = 0.f;
+    for (int c = 0; c < NB * 4; ++c) {
+      dv[r][c] = 0.f;
+      if (kPerformer) dk[r][c] = 0.f;
+    }
   }
-  __syncthreads();
-  if (kPerformer && threadIdx.x < kRows) {
-    float s = 0.f;
-    for (int c = 0; c < cols; ++c) s = fmaf(Ks[threadIdx.x * ld + c], Ks[threadIdx.x * ld + c], s);
-    nrm[threadIdx.x] = 0.5f * s;
+  const size_t hd = (size_t)BH * d, term = (size_t)k * hd;
+  if (kPerformer) {
+    __syncthreads();
+    if (threadIdx.x < kRows) {
+      float s = 0.f;
+      for (int c = 0; c < cols; c += 4) {
+        const float4 v = *reinterpret_cast<const float4*>(Ks + threadIdx.x * ld + c);
+        s = fmaf(v.x, v.x, fmaf(v.y, v.y, fmaf(v.z, v.z, fmaf(v.w, v.w, s))));
+      }
+      nrm[threadIdx.x] = 0.5f * s;
+    }
   }
   for (int i0 = 0; i0 < p; i0 += 64) {
-    __syncthreads();
-    for (int idx = threadIdx.x; idx < 64 * (cols >> 2); idx += kSimtThreads) {
-      const int r = idx / (cols >> 2), c = (idx % (cols >> 2)) * 4;
-      const int live = i0 + r < p ? d - c : 0;
-      if (kPerformer) *reinterpret_cast<float4*>(Ws + r * ld + c) = simt_load_row4(W + (size_t)(i0 + r) * d + c, live, vec);
-      *reinterpret_cast<float4*>(Ds + r * ld + c) = simt_load_row4(da + ((size_t)bh * p + i0 + r) * d + c, live, vec);
-    }
-    __syncthreads();
-    {
-      // e_i, four threads per feature
-      const int r = threadIdx.x >> 2;
-      const bool in = i0 + r < p;
-      float s = 0.f;
-      for (int c = (threadIdx.x & 3) * 4; c < cols; c += 16) {
-        const float4 x = *reinterpret_cast<const float4*>(Ds + r * ld + c);
-        const float4 y = simt_load_row4(a32 + ((size_t)bh * p + i0 + r) * d + c, in ? d - c : 0, vec);
-        s = fmaf(x.x, y.x, fmaf(x.y, y.y, fmaf(x.z, y.z, fmaf(x.w, y.w, s))));
+    if (i0 > 0) __syncthreads();
+    if constexpr (kD > 0) {
+#pragma unroll
+      for (int u = 0; u < kPre; ++u) {
+        const int idx = threadIdx.x + u * kSimtThreads, r = idx / (kD / 4), c = (idx % (kD / 4)) * 4;
+        *reinterpret_cast<float4*>(Ds + r * ld + c) = rd[u];
+        if (kPerformer) *reinterpret_cast<float4*>(Ws + r * ld + c) = rw[u];
       }
-      s += __shfl_xor_sync(0xffffffffu, s, 1);
-      s += __shfl_xor_sync(0xffffffffu, s, 2);
-      if ((threadIdx.x & 3) == 0) {
-        es[r] = in ? db[(size_t)bh * p + i0 + r] - s : 0.f;
-        const float w = in ? weight[(size_t)bh * p + i0 + r] : 0.f;
-        bs[r] = kPerformer ? w : (in ? 1.f / w : 0.f);
+    } else {
+      for (int idx = threadIdx.x; idx < 64 * pieces; idx += kSimtThreads) {
+        const int r = idx / pieces, c = (idx % pieces) * 4;
+        const int live = i0 + r < p ? d - c : 0;
+        if (kPerformer) *reinterpret_cast<float4*>(Ws + r * ld + c) = simt_load_row4(W + (size_t)(i0 + r) * d + c, live, vec);
+        *reinterpret_cast<float4*>(Ds + r * ld + c) = simt_load_row4(dah + (size_t)(i0 + r) * d + c, live, vec);
       }
     }
+    if (threadIdx.x < 64) {
+      bs[threadIdx.x] = kPerformer ? rb : 1.f / rb;
+      es[threadIdx.x] = re;
+    }
     __syncthreads();
+    if (i0 + 64 < p) fetch(i0 + 64);
     float s[R][4], t[R][4];
 #pragma unroll
     for (int r = 0; r < R; ++r)
@@ -322,26 +379,39 @@ simt_bwd_key_side(const float* __restrict__ KpVp, const T* __restrict__ W, const
 #pragma unroll
       for (int f = 0; f < 4; ++f) {
         const int i = tx + 16 * f;
-        float A = 0.f, x = 0.f;
-        if (i0 + i < p && j0 + row < k) {
-          if (kPerformer) {
-            A = expf(s[r][f] - nrm[row] - bs[i]);       // b_i = log sum_j exp(L_ji): A <= 1
-          } else {
-            x = Ks[row * ld + i0 + i];
-            A = elu1(x) * bs[i];
-          }
+        const bool live = i0 + i < p && j0 + row < k;
+        float A, factor = 1.f;
+        if (kPerformer) {
+          A = expf(s[r][f] - nrm[row] - bs[i]);         // b_i = log sum_j exp(L_ji): A <= 1
+        } else {
+          // RNN: feature i is column i0 + i (p = d); d log(elu(x) + 1) / dx = elu'(x) / (elu(x) + 1)
+          const float x = live ? Ks[row * ld + i0 + i] : 0.f;
+          A = (fmaxf(x, 0.f) + expf(fminf(x, 0.f))) * bs[i];
+          factor = x > 0.f ? 1.f / (x + 1.f) : 1.f;
         }
+        if (!live) A = 0.f;
         const float dL = A * (t[r][f] + es[i]);
         dl_sum[r] += dL;
         As[row * kLd + i] = A;
-        Ls[row * kLd + i] = dL;
-        if (!kPerformer && i0 + i < p && j0 + row < k) put(0, j0 + row, i0 + i, dL * elu1_slope(x) / elu1(x));
+        Ls[row * kLd + i] = dL * factor;
       }
     }
     __syncthreads();
     const int kk = min(64, (p - i0 + 3) & ~3);
+    if constexpr (!kPerformer) {
+      // dk' of these 64 columns, four at a time
+#pragma unroll
+      for (int u = 0; u < R; ++u) {
+        const int row = ty + 16 * u, c = tx * 4;
+        const float4 x = *reinterpret_cast<const float4*>(Ls + row * kLd + c);
+        const float v[4] = {x.x, x.y, x.z, x.w};
+        if (j0 + row < k && i0 + c < d)
+          simt_put4(dKpVp + ((size_t)bh * k + j0 + row) * d + i0 + c,
+                    split ? split + (size_t)(j0 + row) * hd + (size_t)bh * d + i0 + c : nullptr, term, v, d - i0 - c, vec);
+      }
+    }
     simt_product<R, NB>(dv, As, kLd, Ds, ld, kk);
-    if (kPerformer) simt_product<R, NB>(dk, Ls, kLd, Ws, ld, kk);
+    if constexpr (kPerformer) simt_product<R, NB>(dk, Ls, kLd, Ws, ld, kk);
   }
 #pragma unroll
   for (int r = 0; r < R; ++r) {
@@ -353,12 +423,17 @@ simt_bwd_key_side(const float* __restrict__ KpVp, const T* __restrict__ W, const
 #pragma unroll
     for (int q = 0; q < NB; ++q) {
       const int c0 = q * 64 + tx * 4;
+      if (c0 >= d) continue;
+      __nv_bfloat16* sp = split ? split + (size_t)(j0 + row) * hd + (size_t)bh * d + c0 : nullptr;
+      float v[4];
+      if constexpr (kPerformer) {
 #pragma unroll
-      for (int e = 0; e < 4; ++e) {
-        if (c0 + e >= d) continue;
-        if (kPerformer) put(0, j0 + row, c0 + e, dk[r][q * 4 + e] - Ks[row * ld + c0 + e] * ds);
-        put(1, j0 + row, c0 + e, dv[r][q * 4 + e]);
+        for (int e = 0; e < 4; ++e) v[e] = dk[r][q * 4 + e] - Ks[row * ld + c0 + e] * ds;
+        simt_put4(dKpVp + ((size_t)bh * k + j0 + row) * d + c0, sp, term, v, d - c0, vec);
       }
+#pragma unroll
+      for (int e = 0; e < 4; ++e) v[e] = dv[r][q * 4 + e];
+      simt_put4(dKpVp + (((size_t)BH + bh) * k + j0 + row) * d + c0, sp ? sp + 2 * term : nullptr, term, v, d - c0, vec);
     }
   }
 }

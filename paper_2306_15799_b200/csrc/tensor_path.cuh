@@ -487,10 +487,10 @@ inline int launch_k3(TensorContext& tc, bool performer, const void* Q, const voi
   return 0;
 }
 
-// ---- backward of the query side, d = 64: dQ, and da, db added to ---------------------------------------
+// ---- backward of the query side, d = 64: dQ, and da, e added to ---------------------------------------
 // abf: the two bf16 terms of a, [BH][2][p][64]
-inline int launch_k7(TensorContext& tc, bool performer, const void* Q, const void* dO, const void* W, const float* a32,
-                     const float* weight, const __nv_bfloat16* abf, void* dQ, float* da, float* db, int BH, int H, int N,
+inline int launch_k7(TensorContext& tc, bool performer, const void* Q, const void* dO, const void* W,
+                     const float* weight, const __nv_bfloat16* abf, void* dQ, float* da, float* ei, int BH, int H, int N,
                      int p, int* status, cudaStream_t st, int* cuda_err) {
   TensorMaps& tm = tc.maps;
   const unsigned long long dQd[3] = {(unsigned long long)(H > 0 ? H * 64 : 64), (unsigned long long)N,
@@ -509,9 +509,9 @@ inline int launch_k7(TensorContext& tc, bool performer, const void* Q, const voi
   prm.N = N; prm.p = p; prm.BH = BH; prm.H = H;
   prm.tiles_per_head = (N + 127) / 128;
   prm.total_tiles = prm.tiles_per_head * BH;
-  prm.weight = weight; prm.a32 = a32;
+  prm.weight = weight;
   prm.dQ = reinterpret_cast<__nv_bfloat16*>(dQ);
-  prm.da = da; prm.db = db; prm.status = status;
+  prm.da = da; prm.ei = ei; prm.status = status;
   const int parts = (p + 127) / 128;                      // 1 or 2 CTAs share a tile
   auto fn = !performer ? k7_bwd_query_side<false, 1> : (parts == 2 ? k7_bwd_query_side<true, 2> : k7_bwd_query_side<true, 1>);
   const int smem = performer ? K7Smem<true>::bytes : K7Smem<false>::bytes;
@@ -525,10 +525,10 @@ inline int launch_k7(TensorContext& tc, bool performer, const void* Q, const voi
   return 0;
 }
 
-// ---- backward of the query side (PERFORMER, d = 64, p = 64, 128, 192 or 256): dQ, and da, db added to --
+// ---- backward of the query side (PERFORMER, d = 64, p = 64, 128, 192 or 256): dQ, and da, e added to --
 // abf: scratch for the two bf16 terms of a, [BH][2][p][64]
-inline int launch_k4(TensorContext& tc, bool performer, const void* Q, const void* dO, const void* W, const float* a32,
-                     const float* weight, const __nv_bfloat16* abf, void* dQ, float* da, float* db, int BH, int H, int N,
+inline int launch_k4(TensorContext& tc, bool performer, const void* Q, const void* dO, const void* W,
+                     const float* weight, const __nv_bfloat16* abf, void* dQ, float* da, float* ei, int BH, int H, int N,
                      int d, int p, int* status, cudaStream_t st, int* cuda_err, void* rowstat = nullptr) {
   // rowstat: d = 128 only, 8 bytes per query row of every 128-row tile (BH * ceil(N / 128) * 128 rows)
   TensorMaps& tm = tc.maps;
@@ -552,9 +552,9 @@ inline int launch_k4(TensorContext& tc, bool performer, const void* Q, const voi
   prm.N = N; prm.p = p; prm.BH = BH; prm.H = H; prm.d = d;
   prm.tiles_per_head = (N + 127) / 128;
   prm.total_tiles = prm.tiles_per_head * BH;
-  prm.weight = weight; prm.a32 = a32;
+  prm.weight = weight;
   prm.dQ = reinterpret_cast<__nv_bfloat16*>(dQ);
-  prm.da = da; prm.db = db; prm.status = status;
+  prm.da = da; prm.ei = ei; prm.status = status;
   prm.rowstat = reinterpret_cast<float2*>(rowstat);
   auto fn = stream ? k4_bwd_query_side<true, true> : (performer ? k4_bwd_query_side<true, false> : k4_bwd_query_side<false, false>);
   cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, kK4SmemBytes);
@@ -626,9 +626,9 @@ inline int launch_k5(TensorContext& tc, const void* E, const void* F, const void
   return 0;
 }
 
-// ---- backward of the key side (PERFORMER, d = 64): dK', dV' from da, db ---------------------------------
-inline int launch_k6(TensorContext& tc, const void* W, const float* kpvp, const float* weight, const float* a32,
-                     const float* da, const float* db, __nv_bfloat16* split, int BH, int k, int p, int* status,
+// ---- backward of the key side (PERFORMER, d = 64): dK', dV' from da, e ----------------------------------
+inline int launch_k6(TensorContext& tc, const void* W, const float* kpvp, const float* weight,
+                     const float* da, const float* ei, __nv_bfloat16* split, int BH, int k, int p, int* status,
                      cudaStream_t st, int* cuda_err) {
   TensorMaps& tm = tc.maps;
   const unsigned long long dW[2] = {64ull, (unsigned long long)p};
@@ -639,7 +639,7 @@ inline int launch_k6(TensorContext& tc, const void* W, const float* kpvp, const 
   }
   K6Params prm;
   prm.k = k; prm.p = p; prm.BH = BH;
-  prm.kpvp = kpvp; prm.weight = weight; prm.a32 = a32; prm.da = da; prm.db = db; prm.split = split; prm.status = status;
+  prm.kpvp = kpvp; prm.weight = weight; prm.da = da; prm.ei = ei; prm.split = split; prm.status = status;
   cudaError_t e = cudaFuncSetAttribute(k6_bwd_key_side, cudaFuncAttributeMaxDynamicSharedMemorySize, kK6SmemBytes);
   if (e != cudaSuccess) { *cuda_err = (int)e; (void)cudaGetLastError(); return -6; }
   e = launch_after_predecessor(k6_bwd_key_side, BH * ((k + 127) / 128), kK6Threads, kK6SmemBytes, st, tm.W2.map, prm);
