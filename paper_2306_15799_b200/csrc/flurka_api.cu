@@ -866,7 +866,7 @@ namespace {
 // range to clear), then dK', dV' [2][BH][k][d]; all fp32.
 struct BackwardLayout {
   Layout L;
-  size_t da, dae_bytes, ei, dkpvp, abf, split, rowstat, efpad, total;
+  size_t da, dae_bytes, ei, dkpvp, abf, split, efpad, total;
 };
 
 // the query side of the backward has a tensor-core kernel for d = 64 (PERFORMER: any feature count the
@@ -888,9 +888,6 @@ BackwardLayout make_backward_layout(const Problem& pr) {
   b.dkpvp = off; off = align256(off + (size_t)2 * pr.BH() * pr.k * pr.d * 4);
   b.abf = off;
   if (backward_tensor_ok(pr)) off = align256(off + (size_t)2 * pr.BH() * pr.p() * pr.d * 2);   // a as two bf16 terms
-  b.rowstat = off;
-  if (backward_tensor_ok(pr) && pr.d == 128)             // (log-sum-exp, delta) of every row of every 128-row tile
-    off = align256(off + (size_t)pr.BH() * ((pr.N + 127) / 128) * 128 * 8);
   b.split = off;
   if (tensor_path_ok(pr)) off = align256(off + (size_t)2 * pr.k * 2 * pr.BH() * pr.d * 2);      // dK', dV' as two bf16 terms
   b.efpad = off;
@@ -973,12 +970,8 @@ int backward_pipeline(const Problem& pr, const BackwardLayout& BL, char* ws, con
   }
   if (tc && tcq) {
     const __nv_bfloat16* abf = (const __nv_bfloat16*)(ws + BL.abf);
-    if (pr.d == 64)
-      rc = launch_k7(*tc, P, Q, dO, W, weight, abf, dQ, da, ei, pr.BH(), smh, pr.N, pr.p(), (int*)(ws + L.status), st,
-                     &cuda_err);
-    else
-      rc = launch_k4(*tc, P, Q, dO, W, weight, abf, dQ, da, ei, pr.BH(), smh, pr.N, pr.d, pr.p(),
-                     (int*)(ws + L.status), st, &cuda_err, ws + BL.rowstat);
+    rc = launch_bwd_query(*tc, P, Q, dO, W, weight, abf, dQ, da, ei, pr.BH(), smh, pr.N, pr.d, pr.p(),
+                          (int*)(ws + L.status), st, &cuda_err);
     if (rc) { g_last_cuda_error = cuda_err; return rc; }
     ++*launches;
   } else {

@@ -1,0 +1,522 @@
+// Backward of the query side on tensor cores for d = 128 (bf16, PERFORMER with up to 256 features): the formulas and the
+// division of the features over a cluster of CTAs are those of k7_bwd_query_side.cuh.
+//
+// What d = 128 changes is room.  W and the two terms of a take 96 KB for a CTA's 128 features, P 32 KB, a Q or dO tile
+// 32 KB each, so there are two tile buffers in all, and TMEM is full with S, G, dQ and da (128 columns each):
+//   * Q(i) is free once S(i) is formed, dO(i) only after da(i).  dO(i+1) therefore goes where Q(i) was and G(i+1) is formed
+//     under tile i's arithmetic; Q(i+1) goes where dO(i) was, and S(i+1) follows it: the one load that is waited for.
+//   * c as bf16 pairs lies over S in TMEM and is the A operand of dQ = C W from there.
+//   * What the other CTA adds to this CTA's half of dQ arrives in the P tile, which is free between da and the next
+//     tile's P: thread (row, half) finds its 32 columns in the 128 bytes that it will write its part of P to.  Both
+//     CTAs' commits for a tile arrive at both (tcgen05.commit with multicast), so both know that both P tiles are read.
+//   * sum_n P_ni delta_n is added up by the row owners, 32 rows at a time across a warp (the same rounded P that da
+//     uses), while they would wait for the products: it needs no operand, no product and no TMEM.
+// Per tile and CTA 2304 cycles of MMA; the row owners' chain is about three times that (see K4_FIG).
+#pragma once
+
+#include <cuda_bf16.h>
+
+#include "k1_down_project_pair.cuh"
+#include "tc_common.cuh"
+
+namespace flurka {
+
+// the backward kernels of the query side
+struct K7Params {
+  int N, p, BH, H;              // H > 0: Q, dO, dQ are [B,N,H,d]; H == 0: [BH,N,d]
+  int tiles_per_head, total_tiles;
+  const float* weight;          // [BH][p]     b_i (RNN: z_i)
+  __nv_bfloat16* dQ;
+  float* da;                    // [BH][p][d]  added to
+  float* ei;                    // [BH][p]     e_i, added to
+  int* status;
+};
+
+constexpr int kK7Threads = 384;      // loader, MMA issuer, head operands, an idle warp; two warpgroups of row owners
+// registers: 384 threads x 168 at launch = 128 x 72 + 256 x 216
+constexpr int kK7RegsFew = 72, kK7RegsMany = 216;
+
+__device__ __forceinline__ uint32_t k4_bf16x2(float lo, float hi) {
+  uint32_t r;
+  asm("cvt.rn.bf16x2.f32 %0, %2, %1;" : "=r"(r) : "f"(lo), "f"(hi));
+  return r;
+}
+__device__ __forceinline__ float k4_ex2(float x) {
+  float y;
+  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+  return y;
+}
+// 16 bf16 values, 32-byte aligned
+__device__ __forceinline__ void k4_store16(__nv_bfloat16* o, const uint32_t (&v)[8]) {
+  asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(o), "r"(v[0]), "r"(v[1]), "r"(v[2]),
+               "r"(v[3]), "r"(v[4]), "r"(v[5]), "r"(v[6]), "r"(v[7]) : "memory");
+}
+
+// shared memory
+struct K4Smem {
+  static constexpr uint32_t w = 0, a_hi = 32768, a_lo = 65536, p = 98304, x = 131072;    // x: two buffers of 32 KB
+  static constexpr uint32_t stat = x + 65536;                                            // [2 parities][3][4 parts][128] floats
+  static constexpr uint32_t bias = stat + 12288;                                         // b_i log2 e
+  static constexpr uint32_t bars = bias + 512;
+  static constexpr int bytes = (int)bars + 256 + 1024;
+};
+// TMEM columns: S 0..127 (c over 0..63), G, dQ, da
+constexpr uint32_t kK4ColG = 128, kK4ColDQ = 256, kK4ColDA = 384;
+
+// kParts: CTAs per cluster (1 or 2), 128 features each
+template <int kParts>
+__global__ void __launch_bounds__(kK7Threads, 1)
+k4_bwd_query_wide(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmDO,
+                  const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUtensorMap tmA,
+                  const K7Params prm) {
+  using namespace tc;
+  using L = K4Smem;
+  extern __shared__ uint8_t smem_raw[];
+  const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u;
+  uint8_t* base_ptr = smem_raw + (base - smem_u32(smem_raw));
+  const uint32_t bars = base + L::bars;
+  const uint32_t bar_w = bars;               // W landed
+  const uint32_t bar_q = bars + 8;           // [2] Q of a tile landed
+  const uint32_t bar_qfree = bars + 24;      // [2] ... S formed
+  const uint32_t bar_do = bars + 40;         // [2] dO landed
+  const uint32_t bar_dofree = bars + 56;     // [2] ... da added to
+  const uint32_t bar_head = bars + 72;       // a, b of a new head in place
+  const uint32_t bar_sg = bars + 80;         // S (and before it G) ready
+  const uint32_t bar_sgfree = bars + 88;     // S, G and b read out (8 warps)
+  const uint32_t bar_pc = bars + 96;         // P, C written (8 warps)
+  const uint32_t bar_c = bars + 104;         // this CTA's dQ complete (C is no longer needed)
+  const uint32_t bar_out = bars + 112;       // dQ, da complete in all CTAs of the cluster
+  const uint32_t bar_x = bars + 120;         // [2] the row sums of all parts are here (8 local warps, the others by their bytes)
+  const uint32_t bar_y = bars + 136;         // the other CTA's part of this CTA's half of dQ is here
+  const uint32_t tmem_slot = bars + 144;
+  __shared__ int abort_flag;
+  __shared__ uint32_t tmem_base_shared;
+
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int p = prm.p;
+  const uint32_t rank = kParts == 2 ? cluster_ctarank() : 0u;
+  const int f0 = (int)rank * 128;                             // first feature of this CTA
+  const int group = blockIdx.x / kParts, groups = gridDim.x / kParts;
+  const int t_begin = (int)(((long long)group * prm.total_tiles) / groups);
+  const int nt = (int)(((long long)(group + 1) * prm.total_tiles) / groups) - t_begin;
+
+  if (tid == 0) {
+    abort_flag = 0;
+    mbar_init(bar_w, 1);
+    for (int s = 0; s < 2; ++s) {
+      mbar_init(bar_q + 8 * s, 1);
+      mbar_init(bar_qfree + 8 * s, 1);
+      mbar_init(bar_do + 8 * s, 1);
+      mbar_init(bar_dofree + 8 * s, 1);
+      mbar_init(bar_x + 8 * s, 8);
+    }
+    mbar_init(bar_head, 33);
+    mbar_init(bar_sg, 1);
+    mbar_init(bar_sgfree, 8);
+    mbar_init(bar_pc, 8);
+    mbar_init(bar_c, 1);
+    mbar_init(bar_out, kParts);
+    mbar_init(bar_y, 1);
+    fence_mbar_init();
+  }
+  if (warp == 1) {
+    tmem_alloc(tmem_slot, 512);
+    tmem_relinquish();
+  }
+  tcgen05_fence_before();
+  __syncthreads();
+  tcgen05_fence_after();
+  if (tid == 0) {
+    uint32_t v;
+    asm volatile("ld.shared.u32 %0, [%1];" : "=r"(v) : "r"(tmem_slot));
+    tmem_base_shared = v;
+  }
+  if (kParts == 2) cluster_sync_all();       // the other CTA's barriers exist before anything is sent to them
+  else __syncthreads();
+  const uint32_t tmem = tmem_base_shared;
+  const float kLog2e = 1.4426950408889634f;
+  // tile i: Q in buffer i & 1, dO in the other; the n-th use of a barrier of a pair has parity (n >> 1) & 1
+  auto q_buf = [&](int i) { return base + L::x + (uint32_t)(i & 1) * 32768u; };
+  auto do_buf = [&](int i) { return base + L::x + (uint32_t)(~i & 1) * 32768u; };
+
+  if (nt > 0) {
+    if (warp < 4) {
+      asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kK7RegsFew));
+      if (warp == 0 && elect_one()) {
+        // ============================================================ loader
+        prefetch_tmap(&tmQ);
+        prefetch_tmap(&tmDO);
+        prefetch_tmap(&tmW);
+        mbar_arrive_expect_tx(bar_w, 32768u);
+        for (int kb = 0; kb < 2; ++kb) tma_load_2d(base + L::w + kb * 16384, &tmW, bar_w, kb * 64, f0);   // rows past p: zero
+        int head = t_begin / prm.tiles_per_head, tih = t_begin % prm.tiles_per_head;
+        bool ok = true;
+        int nq = 0, nd = 0;                                    // Q and dO loads issued
+        for (int i = 0; i < nt; ++i) {
+          const int x = prm.H > 0 ? (head % prm.H) * 128 : 0, z = prm.H > 0 ? head / prm.H : head;
+          // dO(i) where Q(i-1) was, then Q(i) where dO(i-1) was
+          if (i > 0) ok = mbar_wait(bar_qfree + 8 * ((i - 1) & 1), (uint32_t)((i - 1) >> 1) & 1u, prm.status, &abort_flag);
+          if (!ok) break;
+          mbar_arrive_expect_tx(bar_do + 8 * (i & 1), 32768u);
+          for (int kb = 0; kb < 2; ++kb) tma_load_3d(do_buf(i) + kb * 16384, &tmDO, bar_do + 8 * (i & 1), x + kb * 64, tih * 128, z);
+          ++nd;
+          if (i > 0) ok = mbar_wait(bar_dofree + 8 * ((i - 1) & 1), (uint32_t)((i - 1) >> 1) & 1u, prm.status, &abort_flag);
+          if (!ok) break;
+          mbar_arrive_expect_tx(bar_q + 8 * (i & 1), 32768u);
+          for (int kb = 0; kb < 2; ++kb) tma_load_3d(q_buf(i) + kb * 16384, &tmQ, bar_q + 8 * (i & 1), x + kb * 64, tih * 128, z);
+          ++nq;
+          if (++tih == prm.tiles_per_head) { tih = 0; ++head; }
+          // the next tile's Q is loaded when it is wanted: let it wait in L2
+          if (i + 1 < nt) {
+            const int x1 = prm.H > 0 ? (head % prm.H) * 128 : 0, z1 = prm.H > 0 ? head / prm.H : head;
+            for (int kb = 0; kb < 2; ++kb) tma_prefetch_3d(&tmQ, x1 + kb * 64, tih * 128, z1);
+          }
+        }
+        if (!ok) {
+          // loads in flight still land in this CTA's shared memory: wait for them (bounded)
+          if (nd > 0) (void)mbar_wait(bar_do + 8 * ((nd - 1) & 1), (uint32_t)((nd - 1) >> 1) & 1u, prm.status, &abort_flag);
+          if (nq > 0) (void)mbar_wait(bar_q + 8 * ((nq - 1) & 1), (uint32_t)((nq - 1) >> 1) & 1u, prm.status, &abort_flag);
+        }
+      } else if (warp == 1 && elect_one()) {
+        // ============================================================ MMA issuer
+        const uint32_t idescS = make_idesc(kFmtBF16, 0, 0, 128, 128);    // S, G: both operands K-major
+        const uint32_t idescQ = make_idesc(kFmtBF16, 0, 1, 128, 128);    // dQ: C from TMEM, W MN-major
+        const uint32_t idescA = make_idesc(kFmtBF16, 1, 1, 128, 128);    // da: P^T (MN-major A) x dO (MN-major B)
+        bool ok = mbar_wait(bar_w, 0, prm.status, &abort_flag);
+        int head = -1, events = 0;
+        auto form_g = [&](int i) {      // once dO and a are in place and G of the tile before is read out
+          const int h = (t_begin + i) / prm.tiles_per_head;
+          if (h != head) {
+            ok = mbar_wait(bar_head, (uint32_t)(events++) & 1u, prm.status, &abort_flag);
+            head = h;
+          }
+          if (ok) ok = mbar_wait(bar_do + 8 * (i & 1), (uint32_t)(i >> 1) & 1u, prm.status, &abort_flag);
+          if (ok && i > 0) ok = mbar_wait(bar_sgfree, (uint32_t)(i - 1) & 1u, prm.status, &abort_flag);
+          if (!ok) return;
+          tcgen05_fence_after();
+          for (int kb = 0; kb < 2; ++kb) {
+            const uint64_t ag = make_sdesc(do_buf(i) + kb * 16384, 16, 1024, kSwizzle128);
+            mma_ss_x4(tmem + kK4ColG, ag, make_sdesc(base + L::a_hi + kb * 16384, 16, 1024, kSwizzle128), 2, 2, idescS, kb > 0 ? 1u : 0u);
+            mma_ss_x4(tmem + kK4ColG, ag, make_sdesc(base + L::a_lo + kb * 16384, 16, 1024, kSwizzle128), 2, 2, idescS, 1u);
+          }
+        };
+        auto form_s = [&](int i) {
+          ok = mbar_wait(bar_q + 8 * (i & 1), (uint32_t)(i >> 1) & 1u, prm.status, &abort_flag);
+          if (ok && i > 0) ok = mbar_wait(bar_c, (uint32_t)(i - 1) & 1u, prm.status, &abort_flag);     // c lies over S
+          if (!ok) return;
+          tcgen05_fence_after();
+          for (int kb = 0; kb < 2; ++kb)
+            mma_ss_x4(tmem, make_sdesc(q_buf(i) + kb * 16384, 16, 1024, kSwizzle128),
+                      make_sdesc(base + L::w + kb * 16384, 16, 1024, kSwizzle128), 2, 2, idescS, kb > 0 ? 1u : 0u);
+          mma_commit(bar_sg);
+          mma_commit(bar_qfree + 8 * (i & 1));
+        };
+        if (ok) form_g(0);
+        if (ok) form_s(0);
+        int acc_head = -1;
+        for (int i = 0; i < nt && ok; ++i) {
+          const int this_head = (t_begin + i) / prm.tiles_per_head;
+          if (i + 1 < nt) {
+            form_g(i + 1);
+            if (!ok) break;
+          }
+          ok = mbar_wait(bar_pc, (uint32_t)i & 1u, prm.status, &abort_flag);
+          if (!ok) break;
+          tcgen05_fence_after();
+          const uint32_t first = this_head != acc_head ? 0u : 1u;
+          acc_head = this_head;
+          for (int j = 0; j < 2; ++j)        // 64 rows: 16 rows of P and of dO per step; 64-wide slabs 16384 B apart
+            mma_ss_x4(tmem + kK4ColDA, make_sdesc(base + L::p + j * 8192, 16384, 1024, kSwizzle128),
+                      make_sdesc(do_buf(i) + j * 8192, 16384, 1024, kSwizzle128), 128, 128, idescA, j > 0 ? 1u : first);
+          mma_commit(bar_dofree + 8 * (i & 1));
+          for (int j = 0; j < 2; ++j)        // 64 features: 8 columns of C and 16 rows of W per step
+            mma_ts_x4(tmem + kK4ColDQ, tmem + j * 32, make_sdesc(base + L::w + j * 8192, 16384, 1024, kSwizzle128), 128, idescQ,
+                      j > 0 ? 1u : 0u);
+          mma_commit(bar_c);
+          if (kParts == 2) mma_commit_cluster(bar_out, 3);
+          else mma_commit(bar_out);
+          if (i + 1 < nt) form_s(i + 1);
+        }
+      } else if (warp == 2) {
+        // ============================================================ a and b of a new head, once the old head's last tile
+        // is read out (every tile is waited for: a parity wait sees one bit of the phase count)
+        if (lane == 0) prefetch_tmap(&tmA);
+        grid_dependency_wait_async();
+        int head_prev = -1;
+        bool ok = true;
+        for (int i = 0; i < nt && ok; ++i) {
+          const int head = (t_begin + i) / prm.tiles_per_head;
+          if (i > 0) ok = mbar_wait(bar_sgfree, (uint32_t)(i - 1) & 1u, prm.status, &abort_flag);
+          if (!ok || head == head_prev) continue;
+          head_prev = head;
+          if (lane == 0) {
+            mbar_arrive_expect_tx(bar_head, 65536u);
+            for (int kb = 0; kb < 2; ++kb) {
+              tma_load_3d(base + L::a_hi + kb * 16384, &tmA, bar_head, kb * 64, f0, head * 2);
+              tma_load_3d(base + L::a_lo + kb * 16384, &tmA, bar_head, kb * 64, f0, head * 2 + 1);
+            }
+          }
+          const float* wv = prm.weight + (size_t)head * p;
+          float mx = -INFINITY;
+          for (int f = lane; f < p; f += 32) mx = fmaxf(mx, __ldcg(wv + f));
+#pragma unroll
+          for (int o = 16; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+          float* bs = reinterpret_cast<float*>(base_ptr + L::bias);
+          for (int f = lane; f < 128; f += 32) bs[f] = f0 + f < p ? (__ldcg(wv + f0 + f) - mx) * kLog2e : 0.f;
+          mbar_arrive(bar_head);
+        }
+      }
+    } else {
+      // ============================================================ row owners: two threads per row, 64 features each
+      asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(kK7RegsMany));
+      constexpr int kStat = 2 * kParts * 128;                      // floats of one kind of row sum
+      const int q4 = warp & 3, row = q4 * 32 + lane, fh = (warp - 4) >> 2;
+      const uint32_t lane_base = tmem + ((uint32_t)(q4 * 32) << 16);
+      const bool live = f0 + fh * 64 < p;                          // features past p: weight zero
+      const uint32_t peer = kParts == 2 ? (rank ^ 1u) : 0u;
+      const uint32_t x_peer = map_to_cta(bar_x, peer), y_peer = map_to_cta(bar_y, peer);
+      float* stat = reinterpret_cast<float*>(base_ptr + L::stat);
+      const uint32_t stat_peer = map_to_cta(base + L::stat, peer);
+      // this thread's 128 bytes of the P tile: 16-byte piece e at (e ^ (row & 7)) * 16
+      const uint32_t prow = base + L::p + (uint32_t)fh * 16384u + (uint32_t)row * 128u, prow_peer = map_to_cta(prow, peer);
+      const uint32_t swz = (uint32_t)(row & 7);
+      const float* bs = reinterpret_cast<const float*>(base_ptr + L::bias) + fh * 64;
+      float esum0 = 0.f, esum1 = 0.f;          // -sum P delta of features 2 lane, 2 lane + 1 of this half, this warp's rows
+      bool ok = true;
+      grid_dependency_wait();
+
+      // da of one head leaves TMEM: lane = feature, 64 of the 128 columns per thread; and e
+      auto flush = [&](int head) {
+        const int feat = f0 + row;
+#pragma unroll 1
+        for (int c = 0; c < 64; c += 32) {
+          uint32_t r[32];
+          tmem_ld32(lane_base + kK4ColDA + fh * 64 + c, r);
+          tmem_wait_ld(r);
+          if (feat < p) {
+            float4* darow = reinterpret_cast<float4*>(prm.da + ((size_t)head * p + feat) * 128 + fh * 64 + c);
+#pragma unroll
+            for (int e = 0; e < 8; ++e)
+              atomicAdd(darow + e, make_float4(__uint_as_float(r[4 * e]), __uint_as_float(r[4 * e + 1]),
+                                               __uint_as_float(r[4 * e + 2]), __uint_as_float(r[4 * e + 3])));
+          }
+        }
+        if (live) {
+          float* e = prm.ei + (size_t)head * p + f0 + fh * 64 + 2 * lane;
+          atomicAdd(e, esum0);
+          atomicAdd(e + 1, esum1);
+        }
+        esum0 = esum1 = 0.f;
+      };
+      auto store32 = [&](__nv_bfloat16* o, const uint32_t (&r)[32]) {
+#pragma unroll
+        for (int g = 0; g < 2; ++g) {
+          uint32_t v[8];
+#pragma unroll
+          for (int e = 0; e < 8; ++e)
+            v[e] = k4_bf16x2(__uint_as_float(r[16 * g + 2 * e]), __uint_as_float(r[16 * g + 2 * e + 1]));
+          k4_store16(o + 16 * g, v);
+        }
+      };
+
+      int head = t_begin / prm.tiles_per_head, tih = t_begin % prm.tiles_per_head;
+      for (int i = 0; i < nt; ++i) {
+        const int row0 = tih * 128;
+        const uint32_t par = (uint32_t)(i & 1);
+        ok = mbar_wait(bar_sg, par, prm.status, &abort_flag);
+        if (!ok) break;
+        tcgen05_fence_after();
+        uint64_t w2[32], g2[32];                                   // weights exp(l - own maximum), g, as pairs
+        float mx;
+        uint64_t den2 = 0ull, num2 = 0ull;
+        {
+          uint32_t ga[32], gb[32], sa[32], sb[32];
+          tmem_ld32(lane_base + fh * 64, sa);
+          tmem_ld32(lane_base + fh * 64 + 32, sb);
+          tmem_ld32(lane_base + kK4ColG + fh * 64, ga);
+          tmem_ld32(lane_base + kK4ColG + fh * 64 + 32, gb);
+          tmem_wait_ld(sa);
+          tmem_wait_ld(sb);
+          tmem_wait_ld(ga);
+          tmem_wait_ld(gb);
+          const uint64_t l2 = pack2(kLog2e, kLog2e);
+          float m0 = -INFINITY, m1 = -INFINITY;
+#pragma unroll
+          for (int e = 0; e < 16; ++e) {
+            g2[e] = pack2u(ga[2 * e], ga[2 * e + 1]);
+            g2[16 + e] = pack2u(gb[2 * e], gb[2 * e + 1]);
+          }
+#pragma unroll
+          for (int e = 0; e < 32; e += 2) {
+            const ulonglong2 b4 = *reinterpret_cast<const ulonglong2*>(bs + 2 * e);
+            w2[e] = fma2(e < 16 ? pack2u(sa[2 * e & 31], sa[(2 * e + 1) & 31]) : pack2u(sb[2 * e & 31], sb[(2 * e + 1) & 31]), l2, b4.x);
+            w2[e + 1] = fma2(e < 16 ? pack2u(sa[(2 * e + 2) & 31], sa[(2 * e + 3) & 31]) : pack2u(sb[(2 * e + 2) & 31], sb[(2 * e + 3) & 31]), l2, b4.y);
+            float x0, x1, x2, x3;
+            unpack2(w2[e], x0, x1);
+            unpack2(w2[e + 1], x2, x3);
+            m0 = fmax3(m0, x0, x1);
+            m1 = fmax3(m1, x2, x3);
+          }
+          mx = live ? fmaxf(m0, m1) : -INFINITY;
+          tcgen05_fence_before();
+          __syncwarp();
+          if (lane == 0) mbar_arrive(bar_sgfree);
+          if (live) {
+            const uint64_t nm2 = pack2(-mx, -mx);
+#pragma unroll
+            for (int e = 0; e < 32; ++e) {
+              float x0, x1;
+              unpack2(add2(w2[e], nm2), x0, x1);
+              w2[e] = pack2(k4_ex2(x0), k4_ex2(x1));
+              den2 = add2(den2, w2[e]);
+              num2 = fma2(w2[e], g2[e], num2);
+            }
+          }
+        }
+        // ---- the sums to everyone who shares the row
+        {
+          float d0, d1, n0, n1;
+          unpack2(den2, d0, d1);
+          unpack2(num2, n0, n1);
+          const uint32_t at = par * (3 * kStat) + (rank * 2 + (uint32_t)fh) * 128 + (uint32_t)row;
+          stat[at] = mx;
+          stat[at + kStat] = d0 + d1;
+          stat[at + 2 * kStat] = n0 + n1;
+          if (kParts == 2) {
+            const uint32_t bar = x_peer + par * 8u;
+            st_async_b32(stat_peer + at * 4u, __float_as_uint(mx), bar);
+            st_async_b32(stat_peer + (at + kStat) * 4u, __float_as_uint(d0 + d1), bar);
+            st_async_b32(stat_peer + (at + 2 * kStat) * 4u, __float_as_uint(n0 + n1), bar);
+          }
+          __syncwarp();
+          if (lane == 0) {
+            if (kParts == 2 && warp == 4) mbar_arrive_expect_tx(bar_x + par * 8u, 256u * 12u);
+            else mbar_arrive(bar_x + par * 8u);
+          }
+        }
+        ok = mbar_wait(bar_x + par * 8u, (uint32_t)(i >> 1) & 1u, prm.status, &abort_flag);
+        if (!ok) break;
+        tcgen05_fence_after();
+        float delta, scale;
+        {
+          const float* st0 = stat + par * (3 * kStat) + row;
+          float m[2 * kParts], all = -INFINITY, dsum = 0.f, nsum = 0.f;
+#pragma unroll
+          for (int q = 0; q < 2 * kParts; ++q) {
+            m[q] = st0[q * 128];
+            all = fmaxf(all, m[q]);
+          }
+#pragma unroll
+          for (int q = 0; q < 2 * kParts; ++q) {
+            const float f = k4_ex2(m[q] - all);
+            dsum = fmaf(st0[kStat + q * 128], f, dsum);
+            nsum = fmaf(st0[2 * kStat + q * 128], f, nsum);
+          }
+          const float inv = __fdividef(1.f, dsum);
+          delta = nsum * inv;
+          scale = live ? k4_ex2(mx - all) * inv : 0.f;               // (features past p: finite values times zero)
+        }
+        // ---- P into shared memory, C over S (already read by every thread whose columns these are: lane and half own them)
+        uint32_t pw[32];
+        {
+          uint32_t cw[32];
+          const uint64_t sc2 = pack2(scale, scale), nd2 = pack2(-delta, -delta);
+#pragma unroll
+          for (int j = 0; j < 32; ++j) {
+            const uint64_t pp = mul2(w2[j], sc2);
+            float p0, p1, c0, c1;
+            unpack2(pp, p0, p1);
+            unpack2(mul2(pp, add2(g2[j], nd2)), c0, c1);
+            pw[j] = k4_bf16x2(p0, p1);
+            cw[j] = k4_bf16x2(c0, c1);
+          }
+          // features 0..63 -> columns 0..31, 64..127 -> 32..63; both halves of a row have read S by now (bar_x)
+          tmem_st16(lane_base + fh * 32, *reinterpret_cast<const uint32_t (*)[16]>(&cw[0]));
+          tmem_st16(lane_base + fh * 32 + 16, *reinterpret_cast<const uint32_t (*)[16]>(&cw[16]));
+#pragma unroll
+          for (int e = 0; e < 8; ++e)
+            asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(prow + (((uint32_t)e ^ swz) << 4)), "r"(pw[4 * e]),
+                         "r"(pw[4 * e + 1]), "r"(pw[4 * e + 2]), "r"(pw[4 * e + 3]) : "memory");
+          tmem_wait_st();
+          fence_proxy_async_smem();
+          tcgen05_fence_before();
+          __syncwarp();
+          if (lane == 0) mbar_arrive(bar_pc);
+        }
+        // ---- while the products run: -sum over the warp's rows of P_ni delta_n, the number of features per lane halved
+        //      and the number of rows doubled at each step; lane l ends with features 2 l, 2 l + 1
+        {
+          float v[32];
+          const bool up = (lane & 16) != 0;
+#pragma unroll
+          for (int j = 0; j < 16; ++j) {
+            const float l0 = __uint_as_float(pw[j] << 16), l1 = __uint_as_float(pw[j] & 0xffff0000u);
+            const float h0 = __uint_as_float(pw[16 + j] << 16), h1 = __uint_as_float(pw[16 + j] & 0xffff0000u);
+            v[2 * j] = -delta * (up ? h0 : l0) + __shfl_xor_sync(0xffffffffu, -delta * (up ? l0 : h0), 16);
+            v[2 * j + 1] = -delta * (up ? h1 : l1) + __shfl_xor_sync(0xffffffffu, -delta * (up ? l1 : h1), 16);
+          }
+#pragma unroll
+          for (int o = 8; o > 0; o >>= 1) {
+            const bool hi = (lane & o) != 0;
+#pragma unroll
+            for (int j = 0; j < 2 * o; ++j) v[j] = (hi ? v[2 * o + j] : v[j]) + __shfl_xor_sync(0xffffffffu, hi ? v[j] : v[2 * o + j], o);
+          }
+          esum0 += v[0];
+          esum1 += v[1];
+        }
+        // ---- dQ: with two CTAs each stores 64 of the 128 columns, its own sums plus the other CTA's
+        ok = mbar_wait(bar_out, par, prm.status, &abort_flag);
+        if (!ok) break;
+        tcgen05_fence_after();
+        const bool last_of_head = i + 1 == nt || tih + 1 == prm.tiles_per_head;
+        __nv_bfloat16* orow = prm.dQ + (prm.H > 0 ? (((size_t)(head / prm.H) * prm.N + row0 + row) * prm.H + (size_t)(head % prm.H)) * 128
+                                                  : ((size_t)head * prm.N + row0 + row) * 128);
+        const bool in_range = row0 + row < prm.N;
+        if constexpr (kParts == 2) {
+          uint32_t own[32], other[32];
+          tmem_ld32(lane_base + kK4ColDQ + peer * 64 + fh * 32, other);
+          tmem_ld32(lane_base + kK4ColDQ + rank * 64 + fh * 32, own);
+          tmem_wait_ld(other);
+          tmem_wait_ld(own);
+#pragma unroll
+          for (int e = 0; e < 8; ++e)
+            st_async_v4(prow_peer + (((uint32_t)e ^ swz) << 4), other[4 * e], other[4 * e + 1], other[4 * e + 2], other[4 * e + 3], y_peer);
+          if (tid == 128) mbar_arrive_expect_tx(bar_y, 32768u);
+          if (last_of_head) flush(head);
+          tcgen05_fence_before();
+          ok = mbar_wait(bar_y, par, prm.status, &abort_flag);
+          if (!ok) break;
+#pragma unroll
+          for (int e = 0; e < 8; ++e) {
+            float a, b, c, d;
+            asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(a), "=f"(b), "=f"(c), "=f"(d)
+                         : "r"(prow + (((uint32_t)e ^ swz) << 4)) : "memory");
+            own[4 * e] = __float_as_uint(__uint_as_float(own[4 * e]) + a);
+            own[4 * e + 1] = __float_as_uint(__uint_as_float(own[4 * e + 1]) + b);
+            own[4 * e + 2] = __float_as_uint(__uint_as_float(own[4 * e + 2]) + c);
+            own[4 * e + 3] = __float_as_uint(__uint_as_float(own[4 * e + 3]) + d);
+          }
+          if (in_range) store32(orow + rank * 64 + fh * 32, own);
+        } else {
+#pragma unroll 1
+          for (int c = 0; c < 64; c += 32) {
+            uint32_t own[32];
+            tmem_ld32(lane_base + kK4ColDQ + fh * 64 + c, own);
+            tmem_wait_ld(own);
+            if (in_range) store32(orow + fh * 64 + c, own);
+          }
+          if (last_of_head) flush(head);
+          tcgen05_fence_before();
+        }
+        if (++tih == prm.tiles_per_head) { tih = 0; ++head; }
+      }
+      if (warp == 4 && lane == 0) grid_launch_dependents();
+    }
+  }
+  tcgen05_fence_before();
+  __syncthreads();
+  if (kParts == 2) cluster_sync_all();       // nothing is sent to a CTA that has left
+  if (warp == 1) tmem_dealloc(tmem, 512);
+}
+
+}  // namespace flurka

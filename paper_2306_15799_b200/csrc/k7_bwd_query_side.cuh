@@ -26,24 +26,11 @@
 #include <cuda_bf16.h>
 
 #include "k1_down_project_pair.cuh"
-#include "k4_bwd_query_side.cuh"
+#include "k4_bwd_query_wide.cuh"
 #include "tc_common.cuh"
 
 namespace flurka {
 
-struct K7Params {
-  int N, p, BH, H;              // H > 0: Q, dO, dQ are [B,N,H,d]; H == 0: [BH,N,d]; d = 64
-  int tiles_per_head, total_tiles;
-  const float* weight;          // [BH][p]      b_i (RNN: z_i)
-  __nv_bfloat16* dQ;
-  float* da;                    // [BH][p][64]  added to
-  float* ei;                    // [BH][p]      e_i, added to
-  int* status;
-};
-
-constexpr int kK7Threads = 384;      // loader, MMA issuer, head operands, an idle warp; two warpgroups of row owners
-// registers: 384 threads x 168 at launch = 128 x 72 + 256 x 216
-constexpr int kK7RegsFew = 72, kK7RegsMany = 216;
 // Shared memory.  PERFORMER: a Q tile is free as soon as S is formed, a dO tile only after da, so three stages of it.
 // RNN (bound by the traffic of Q, dO, dQ): no W, C, dQ exchange, so four of each.
 template <bool kPerformer>
@@ -60,36 +47,6 @@ struct K7Smem {
 };
 // TMEM columns: S 0..127, G 128..255, dQ 256..383 (two tiles of 64), da 384..447, P^T delta 448..463
 constexpr uint32_t kK7ColG = 128, kK7ColDQ = 256, kK7ColDA = 384, kK7ColDD = 448;
-
-namespace tc {
-// Stores to a CTA of the cluster that count their bytes on a barrier there: whoever waits for that barrier sees the
-// data, and the sender needs no fence (a release at cluster scope would wait for its global stores too: 1400 cycles
-// per tile here).
-__device__ __forceinline__ void st_async_b32(uint32_t addr, uint32_t v, uint32_t bar) {
-  asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.b32 [%0], %1, [%2];" ::"r"(addr), "r"(v), "r"(bar) : "memory");
-}
-__device__ __forceinline__ void st_async_v4(uint32_t addr, uint32_t a, uint32_t b, uint32_t c, uint32_t d, uint32_t bar) {
-  asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.v4.b32 [%0], {%1, %2, %3, %4}, [%5];"
-               ::"r"(addr), "r"(a), "r"(b), "r"(c), "r"(d), "r"(bar) : "memory");
-}
-__device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t (&r)[16]) {
-  asm volatile(
-      "tcgen05.ld.sync.aligned.32x32b.x16.b32 "
-      "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"
-      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
-        "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
-      : "r"(taddr)
-      : "memory");
-}
-__device__ __forceinline__ void tmem_wait_ld16(uint32_t (&r)[16]) {
-  asm volatile(
-      "tcgen05.wait::ld.sync.aligned;"
-      : "+r"(r[0]), "+r"(r[1]), "+r"(r[2]), "+r"(r[3]), "+r"(r[4]), "+r"(r[5]), "+r"(r[6]), "+r"(r[7]),
-        "+r"(r[8]), "+r"(r[9]), "+r"(r[10]), "+r"(r[11]), "+r"(r[12]), "+r"(r[13]), "+r"(r[14]), "+r"(r[15])
-      :
-      : "memory");
-}
-}  // namespace tc
 
 // kParts: CTAs per cluster (1 or 2), 128 features each
 template <bool kPerformer, int kParts>
@@ -339,11 +296,6 @@ k7_bwd_query_side(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
         return prm.dQ + (prm.H > 0 ? (((size_t)(head / prm.H) * prm.N + row0 + row) * prm.H + (size_t)(head % prm.H)) * 64
                                    : ((size_t)head * prm.N + row0 + row) * 64);
       };
-      // 16 bf16 values, 32-byte aligned
-      auto store16 = [&](__nv_bfloat16* o, const uint32_t (&v)[8]) {
-        asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(o), "r"(v[0]), "r"(v[1]), "r"(v[2]),
-                     "r"(v[3]), "r"(v[4]), "r"(v[5]), "r"(v[6]), "r"(v[7]) : "memory");
-      };
       // dQ of a tile: with two CTAs each stores 32 of the 64 columns, its own sums plus the other CTA's.  The other CTA's
       // part of a thread's values comes from the thread of the same row and columns there, which sends it only after
       // this thread's row sums of the next tile have arrived there, i.e. after this thread has read the part before.
@@ -392,7 +344,7 @@ k7_bwd_query_side(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
 #pragma unroll
               for (int e = 0; e < 8; ++e)
                 v[e] = k4_bf16x2(__uint_as_float(own[16 * g + 2 * e]), __uint_as_float(own[16 * g + 2 * e + 1]));
-              store16(o + 16 * g, v);
+              k4_store16(o + 16 * g, v);
             }
           }
         }
@@ -589,8 +541,8 @@ k7_bwd_query_side(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
           if constexpr (!kPerformer) {
             if (row0 + row < prm.N) {
               __nv_bfloat16* o = dq_row(head, row0) + fh * 32;
-              store16(o, *reinterpret_cast<const uint32_t (*)[8]>(&dqv[0]));
-              store16(o + 16, *reinterpret_cast<const uint32_t (*)[8]>(&dqv[8]));
+              k4_store16(o, *reinterpret_cast<const uint32_t (*)[8]>(&dqv[0]));
+              k4_store16(o + 16, *reinterpret_cast<const uint32_t (*)[8]>(&dqv[8]));
             }
           }
         }

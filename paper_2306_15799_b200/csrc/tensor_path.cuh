@@ -14,7 +14,7 @@
 #include "k1_down_project_pair.cuh"
 #include "k2_key_side.cuh"
 #include "k3_query_side.cuh"
-#include "k4_bwd_query_side.cuh"
+#include "k4_bwd_query_wide.cuh"
 #include "k5_bwd_projections.cuh"
 #include "k6_bwd_key_side.cuh"
 #include "k7_bwd_query_side.cuh"
@@ -487,18 +487,18 @@ inline int launch_k3(TensorContext& tc, bool performer, const void* Q, const voi
   return 0;
 }
 
-// ---- backward of the query side, d = 64: dQ, and da, e added to ---------------------------------------
-// abf: the two bf16 terms of a, [BH][2][p][64]
-inline int launch_k7(TensorContext& tc, bool performer, const void* Q, const void* dO, const void* W,
-                     const float* weight, const __nv_bfloat16* abf, void* dQ, float* da, float* ei, int BH, int H, int N,
-                     int p, int* status, cudaStream_t st, int* cuda_err) {
+// ---- backward of the query side (d = 64, or PERFORMER with d = 128): dQ, and da, e added to ---------------
+// abf: the two bf16 terms of a, [BH][2][p][d]
+inline int launch_bwd_query(TensorContext& tc, bool performer, const void* Q, const void* dO, const void* W,
+                            const float* weight, const __nv_bfloat16* abf, void* dQ, float* da, float* ei, int BH, int H,
+                            int N, int d, int p, int* status, cudaStream_t st, int* cuda_err) {
   TensorMaps& tm = tc.maps;
-  const unsigned long long dQd[3] = {(unsigned long long)(H > 0 ? H * 64 : 64), (unsigned long long)N,
+  const unsigned long long dQd[3] = {(unsigned long long)(H > 0 ? H * d : d), (unsigned long long)N,
                                      (unsigned long long)(H > 0 ? BH / H : BH)};
   const unsigned bQ[3] = {64, 128, 1};
-  const unsigned long long dW[2] = {64ull, (unsigned long long)p};
+  const unsigned long long dW[2] = {(unsigned long long)d, (unsigned long long)p};
   const unsigned bW[2] = {64, 128};                       // 128 features of a CTA; rows past p read as zero
-  const unsigned long long dA[3] = {64ull, (unsigned long long)p, (unsigned long long)BH * 2};
+  const unsigned long long dA[3] = {(unsigned long long)d, (unsigned long long)p, (unsigned long long)BH * 2};
   const CUtensorMapDataType bf = CU_TENSOR_MAP_DATA_TYPE_BFLOAT16;
   if (!encode_map(&tm.Q, bf, 2, 3, Q, dQd, bQ) || !encode_map(&tm.dO, bf, 2, 3, dO, dQd, bQ) ||
       (performer && !encode_map(&tm.W2, bf, 2, 2, W, dW, bW)) || !encode_map(&tm.abf, bf, 2, 3, abf, dA, bQ)) {
@@ -513,8 +513,10 @@ inline int launch_k7(TensorContext& tc, bool performer, const void* Q, const voi
   prm.dQ = reinterpret_cast<__nv_bfloat16*>(dQ);
   prm.da = da; prm.ei = ei; prm.status = status;
   const int parts = (p + 127) / 128;                      // 1 or 2 CTAs share a tile
-  auto fn = !performer ? k7_bwd_query_side<false, 1> : (parts == 2 ? k7_bwd_query_side<true, 2> : k7_bwd_query_side<true, 1>);
-  const int smem = performer ? K7Smem<true>::bytes : K7Smem<false>::bytes;
+  auto fn = d == 128 ? (parts == 2 ? k4_bwd_query_wide<2> : k4_bwd_query_wide<1>)
+                     : (!performer ? k7_bwd_query_side<false, 1>
+                                   : (parts == 2 ? k7_bwd_query_side<true, 2> : k7_bwd_query_side<true, 1>));
+  const int smem = d == 128 ? K4Smem::bytes : (performer ? K7Smem<true>::bytes : K7Smem<false>::bytes);
   cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
   if (e != cudaSuccess) { *cuda_err = (int)e; (void)cudaGetLastError(); return -6; }
   const int groups = std::max(1, std::min(tc.sm_count() / parts, prm.total_tiles));
@@ -522,49 +524,6 @@ inline int launch_k7(TensorContext& tc, bool performer, const void* Q, const voi
   e = launch_cluster_after_predecessor(parts, fn, groups * parts, kK7Threads, smem, st, tm.Q.map, tm.dO.map,
                                        performer ? tm.W2.map : tm.Q.map, tm.abf.map, prm);
   if (e != cudaSuccess) { *cuda_err = (int)e; (void)cudaGetLastError(); return -6; }
-  return 0;
-}
-
-// ---- backward of the query side (PERFORMER, d = 64, p = 64, 128, 192 or 256): dQ, and da, e added to --
-// abf: scratch for the two bf16 terms of a, [BH][2][p][64]
-inline int launch_k4(TensorContext& tc, bool performer, const void* Q, const void* dO, const void* W,
-                     const float* weight, const __nv_bfloat16* abf, void* dQ, float* da, float* ei, int BH, int H, int N,
-                     int d, int p, int* status, cudaStream_t st, int* cuda_err, void* rowstat = nullptr) {
-  // rowstat: d = 128 only, 8 bytes per query row of every 128-row tile (BH * ceil(N / 128) * 128 rows)
-  TensorMaps& tm = tc.maps;
-  const bool stream = d == 128;      // W and a come in per step of 128 features (boxes of 128 rows)
-  const unsigned long long dQd[3] = {(unsigned long long)(H > 0 ? H * d : d), (unsigned long long)N,
-                                     (unsigned long long)(H > 0 ? BH / H : BH)};
-  const unsigned bQ[3] = {64, 128, 1};
-  const unsigned long long dW[2] = {(unsigned long long)d, (unsigned long long)p};
-  const unsigned prows = stream ? 128u : (unsigned)((p + 127) / 128) * 128;   // whole 128-feature tiles; rows past p read as zero
-  const unsigned bW[2] = {64, prows};
-  const unsigned long long dA[3] = {(unsigned long long)d, (unsigned long long)p, (unsigned long long)BH * 2};
-  const unsigned bA[3] = {64, prows, 1};
-  if (!encode_map(&tm.Q, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, 3, Q, dQd, bQ) ||
-      !encode_map(&tm.dO, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, 3, dO, dQd, bQ) ||
-      (performer && !encode_map(&tm.W, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, 2, W, dW, bW)) ||
-      !encode_map(&tm.abf, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, 3, abf, dA, bA)) {
-    *cuda_err = (int)cudaErrorInvalidValue;
-    return -6;
-  }
-  K4Params prm;
-  prm.N = N; prm.p = p; prm.BH = BH; prm.H = H; prm.d = d;
-  prm.tiles_per_head = (N + 127) / 128;
-  prm.total_tiles = prm.tiles_per_head * BH;
-  prm.weight = weight;
-  prm.dQ = reinterpret_cast<__nv_bfloat16*>(dQ);
-  prm.da = da; prm.ei = ei; prm.status = status;
-  prm.rowstat = reinterpret_cast<float2*>(rowstat);
-  auto fn = stream ? k4_bwd_query_side<true, true> : (performer ? k4_bwd_query_side<true, false> : k4_bwd_query_side<false, false>);
-  cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, kK4SmemBytes);
-  if (e != cudaSuccess) { *cuda_err = (int)e; (void)cudaGetLastError(); return -6; }
-  int grid = tc.sm_count();
-  if (grid > prm.total_tiles) grid = prm.total_tiles;
-  // the RNN kernel ignores tmW; pass any valid map
-  fn<<<grid, kK4Threads, kK4SmemBytes, st>>>(tm.Q.map, tm.dO.map, performer ? tm.W.map : tm.Q.map, tm.abf.map, prm);
-  e = cudaGetLastError();
-  if (e != cudaSuccess) { *cuda_err = (int)e; return -6; }
   return 0;
 }
 
