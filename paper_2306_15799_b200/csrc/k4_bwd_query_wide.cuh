@@ -6,9 +6,12 @@
 //   * Q(i) is free once S(i) is formed, dO(i) only after da(i).  dO(i+1) therefore goes where Q(i) was and G(i+1) is formed
 //     under tile i's arithmetic; Q(i+1) goes where dO(i) was, and S(i+1) follows it: the one load that is waited for.
 //   * c as bf16 pairs lies over S in TMEM and is the A operand of dQ = C W from there.
-//   * What the other CTA adds to this CTA's half of dQ arrives in the P tile, which is free between da and the next
-//     tile's P: thread (row, half) finds its 32 columns in the 128 bytes that it will write its part of P to.  Both
-//     CTAs' commits for a tile arrive at both (tcgen05.commit with multicast), so both know that both P tiles are read.
+//   * What the other CTA adds to this CTA's half of dQ (32 KB, which cross the cluster at about 24 bytes a cycle) arrives
+//     half in a buffer of its own, under da, and half in the P tile, which is free between da and the next tile's P: a
+//     warp finds its rows' columns in the 4 KB that it will write its part of P to, in 16-byte pieces, 32 rows of a
+//     piece side by side (a warp's stores to the other CTA are then runs of 512 bytes; row by row, 128 bytes apart, they
+//     took 3000 cycles per tile).  Both CTAs' commits of da arrive at both (tcgen05.commit with multicast), so both know
+//     that both P tiles are read.
 //   * sum_n P_ni delta_n is added up by the row owners, 32 rows at a time across a warp (the same rounded P that da
 //     uses), while they would wait for the products: it needs no operand, no product and no TMEM.
 // Per tile and CTA 2304 cycles of MMA; the row owners' chain is about three times that (see K4_FIG).
@@ -55,7 +58,8 @@ __device__ __forceinline__ void k4_store16(__nv_bfloat16* o, const uint32_t (&v)
 // shared memory
 struct K4Smem {
   static constexpr uint32_t w = 0, a_hi = 32768, a_lo = 65536, p = 98304, x = 131072;    // x: two buffers of 32 KB
-  static constexpr uint32_t stat = x + 65536;                                            // [2 parities][3][4 parts][128] floats
+  static constexpr uint32_t dq = x + 65536;                                              // received: 8 warps x 2 KB
+  static constexpr uint32_t stat = dq + 16384;                                           // [2 parities][3][4 parts][128] floats
   static constexpr uint32_t bias = stat + 12288;                                         // b_i log2 e
   static constexpr uint32_t bars = bias + 512;
   static constexpr int bytes = (int)bars + 256 + 1024;
@@ -85,7 +89,7 @@ k4_bwd_query_wide(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
   const uint32_t bar_sgfree = bars + 88;     // S, G and b read out (8 warps)
   const uint32_t bar_pc = bars + 96;         // P, C written (8 warps)
   const uint32_t bar_c = bars + 104;         // this CTA's dQ complete (C is no longer needed)
-  const uint32_t bar_out = bars + 112;       // dQ, da complete in all CTAs of the cluster
+  const uint32_t bar_out = bars + 112;       // da complete in all CTAs of the cluster
   const uint32_t bar_x = bars + 120;         // [2] the row sums of all parts are here (8 local warps, the others by their bytes)
   const uint32_t bar_y = bars + 136;         // the other CTA's part of this CTA's half of dQ is here
   const uint32_t tmem_slot = bars + 144;
@@ -225,14 +229,14 @@ k4_bwd_query_wide(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
           tcgen05_fence_after();
           const uint32_t first = this_head != acc_head ? 0u : 1u;
           acc_head = this_head;
-          for (int j = 0; j < 2; ++j)        // 64 rows: 16 rows of P and of dO per step; 64-wide slabs 16384 B apart
-            mma_ss_x4(tmem + kK4ColDA, make_sdesc(base + L::p + j * 8192, 16384, 1024, kSwizzle128),
-                      make_sdesc(do_buf(i) + j * 8192, 16384, 1024, kSwizzle128), 128, 128, idescA, j > 0 ? 1u : first);
-          mma_commit(bar_dofree + 8 * (i & 1));
           for (int j = 0; j < 2; ++j)        // 64 features: 8 columns of C and 16 rows of W per step
             mma_ts_x4(tmem + kK4ColDQ, tmem + j * 32, make_sdesc(base + L::w + j * 8192, 16384, 1024, kSwizzle128), 128, idescQ,
                       j > 0 ? 1u : 0u);
           mma_commit(bar_c);
+          for (int j = 0; j < 2; ++j)        // 64 rows: 16 rows of P and of dO per step; 64-wide slabs 16384 B apart
+            mma_ss_x4(tmem + kK4ColDA, make_sdesc(base + L::p + j * 8192, 16384, 1024, kSwizzle128),
+                      make_sdesc(do_buf(i) + j * 8192, 16384, 1024, kSwizzle128), 128, 128, idescA, j > 0 ? 1u : first);
+          mma_commit(bar_dofree + 8 * (i & 1));
           if (kParts == 2) mma_commit_cluster(bar_out, 3);
           else mma_commit(bar_out);
           if (i + 1 < nt) form_s(i + 1);
@@ -278,7 +282,11 @@ k4_bwd_query_wide(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
       float* stat = reinterpret_cast<float*>(base_ptr + L::stat);
       const uint32_t stat_peer = map_to_cta(base + L::stat, peer);
       // this thread's 128 bytes of the P tile: 16-byte piece e at (e ^ (row & 7)) * 16
-      const uint32_t prow = base + L::p + (uint32_t)fh * 16384u + (uint32_t)row * 128u, prow_peer = map_to_cta(prow, peer);
+      const uint32_t prow = base + L::p + (uint32_t)fh * 16384u + (uint32_t)row * 128u;
+      // ... and of the dQ columns that arrive in it and in the buffer: piece e of four at e * 512
+      const uint32_t drow[2] = {base + L::dq + (uint32_t)(fh * 4 + q4) * 2048u + (uint32_t)lane * 16u,
+                                base + L::p + (uint32_t)fh * 16384u + (uint32_t)q4 * 4096u + (uint32_t)lane * 16u};
+      const uint32_t drow_peer[2] = {map_to_cta(drow[0], peer), map_to_cta(drow[1], peer)};
       const uint32_t swz = (uint32_t)(row & 7);
       const float* bs = reinterpret_cast<const float*>(base_ptr + L::bias) + fh * 64;
       float esum0 = 0.f, esum1 = 0.f;          // -sum P delta of features 2 lane, 2 lane + 1 of this half, this warp's rows
@@ -465,7 +473,7 @@ k4_bwd_query_wide(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
           esum1 += v[1];
         }
         // ---- dQ: with two CTAs each stores 64 of the 128 columns, its own sums plus the other CTA's
-        ok = mbar_wait(bar_out, par, prm.status, &abort_flag);
+        ok = mbar_wait(bar_c, par, prm.status, &abort_flag);
         if (!ok) break;
         tcgen05_fence_after();
         const bool last_of_head = i + 1 == nt || tih + 1 == prm.tiles_per_head;
@@ -478,10 +486,18 @@ k4_bwd_query_wide(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
           tmem_ld32(lane_base + kK4ColDQ + rank * 64 + fh * 32, own);
           tmem_wait_ld(other);
           tmem_wait_ld(own);
-#pragma unroll
-          for (int e = 0; e < 8; ++e)
-            st_async_v4(prow_peer + (((uint32_t)e ^ swz) << 4), other[4 * e], other[4 * e + 1], other[4 * e + 2], other[4 * e + 3], y_peer);
           if (tid == 128) mbar_arrive_expect_tx(bar_y, 32768u);
+#pragma unroll
+          for (int h = 0; h < 2; ++h) {
+            if (h == 1) ok = mbar_wait(bar_out, par, prm.status, &abort_flag);
+            if (!ok) break;
+#pragma unroll
+            for (int e = 0; e < 4; ++e)
+              st_async_v4(drow_peer[h] + (uint32_t)e * 512u, other[16 * h + 4 * e], other[16 * h + 4 * e + 1],
+                          other[16 * h + 4 * e + 2], other[16 * h + 4 * e + 3], y_peer);
+          }
+          if (!ok) break;
+          tcgen05_fence_after();
           if (last_of_head) flush(head);
           tcgen05_fence_before();
           ok = mbar_wait(bar_y, par, prm.status, &abort_flag);
@@ -490,12 +506,13 @@ k4_bwd_query_wide(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
           for (int e = 0; e < 8; ++e) {
             float a, b, c, d;
             asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(a), "=f"(b), "=f"(c), "=f"(d)
-                         : "r"(prow + (((uint32_t)e ^ swz) << 4)) : "memory");
+                         : "r"(drow[e >> 2] + (uint32_t)(e & 3) * 512u) : "memory");
             own[4 * e] = __float_as_uint(__uint_as_float(own[4 * e]) + a);
             own[4 * e + 1] = __float_as_uint(__uint_as_float(own[4 * e + 1]) + b);
             own[4 * e + 2] = __float_as_uint(__uint_as_float(own[4 * e + 2]) + c);
             own[4 * e + 3] = __float_as_uint(__uint_as_float(own[4 * e + 3]) + d);
           }
+          __syncwarp();                        // the warp has read its 4 KB: P may be written there again
           if (in_range) store32(orow + rank * 64 + fh * 32, own);
         } else {
 #pragma unroll 1
@@ -505,6 +522,9 @@ k4_bwd_query_wide(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
             tmem_wait_ld(own);
             if (in_range) store32(orow + fh * 64 + c, own);
           }
+          ok = mbar_wait(bar_out, par, prm.status, &abort_flag);
+          if (!ok) break;
+          tcgen05_fence_after();
           if (last_of_head) flush(head);
           tcgen05_fence_before();
         }
