@@ -9,6 +9,7 @@
 
 #include "simt_backward.cuh"
 #include "simt_kernels.cuh"
+#include "simt_small.cuh"
 #include "tensor_path.cuh"
 
 namespace {
@@ -376,6 +377,37 @@ int run_pipeline(const Problem& pr, const Layout& L, char* ws, const void* Q, co
   return run_pipeline_with<T>(pr, L, ws, Q, W, out, st, tc2, tc3, tc, timer, keep_status, launches, stage1, phases);
 }
 
+// Whether the one-kernel forward pass takes the problem: everything fits the shared memory of a cluster of eight CTAs per
+// head, all heads run at once, and a thread has at most kSmallFma multiply-adds (padding included).  Measured against the
+// four launches, us per call: fp32, two heads, d = 32, k = 32, m = 64: N = 128 13.0 / 17.8, N = 256 (2048 multiply-adds)
+// 13.4 / 17.7, N = 512 (3328) 18.3 / 17.9; d = 64, k = 64, N = 256: RNN, four heads (2048) 16.3 / 17.3, m = 64 (3072) 18.5 / 19.2.
+constexpr long long kSmallFma = 2100;
+bool small_forward_ok(const Problem& pr) {
+  if ((long long)pr.BH() * kSmallCtas > 148 || pr.d > 64 || pr.k > 1024) return false;
+  const SmallShape S = small_shape(pr.N, pr.d, pr.k, pr.p());
+  if (S.total * 4 > 200 * 1024) return false;
+  const long long n = S.n32, f = (S.fpc + 31) & ~31, k32 = (pr.k + 31) & ~31, k64 = (pr.k + 63) & ~63,
+                  p64 = (pr.p() + 63) & ~63, per_item = 64 + (pr.kernel == FLURKA_PERFORMER ? pr.d : 0);
+  return (2 * n * k32 * 64 + f * k64 * per_item + n * p64 * per_item) / kSmallThreads <= kSmallFma;
+}
+
+template <typename T>
+int launch_small_forward(const Problem& pr, const Layout& L, char* ws, const void* Q, const void* K, const void* V,
+                         const void* E, const void* F, const void* W, void* out, cudaStream_t st, bool keep_status,
+                         int* launches) {
+  const size_t smem = small_shape(pr.N, pr.d, pr.k, pr.p()).total * 4;
+  auto fn = pr.kernel == FLURKA_PERFORMER ? simt_small_forward<T, true> : simt_small_forward<T, false>;
+  cudaError_t e = cudaSuccess;
+  if (smem > 48 * 1024) e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (e == cudaSuccess)
+    e = launch_after_predecessor(fn, pr.BH() * kSmallCtas, kSmallThreads, smem, st, (const T*)Q, (const T*)K, (const T*)V,
+                                 (const T*)E, (const T*)F, (const T*)W, (float*)(ws + L.kpvp), (float*)(ws + L.weight),
+                                 (float*)(ws + L.a32), (int*)(ws + L.status), (T*)out, pr.BH(), pr.N, pr.d, pr.k, pr.p(),
+                                 pr.seq_major_heads(), pr.ef_heads(), keep_status ? 1 : 0);
+  ++*launches;
+  return e == cudaSuccess ? FLURKA_OK : cuda_fail(e);
+}
+
 int validate_pointers(const Problem& pr, const void* Q, const void* K, const void* V, const void* E,
                       const void* F, const void* W, const void* out) {
   if (!Q || !K || !V || !E || !F || !out) return FLURKA_ERR_NULL;
@@ -443,7 +475,10 @@ int forward_device(const void* Q, const void* K, const void* V, const void* E, c
     rc = timer->create();
     if (rc != cudaSuccess) return cuda_fail((cudaError_t)rc);
   }
-  if (pr.fp32) {
+  if (path == FLURKA_PATH_SIMT && g_path == FLURKA_PATH_AUTO && phases == 3 && !timer && small_forward_ok(pr)) {
+    rc = pr.fp32 ? launch_small_forward<float>(pr, L, ws, Q, K, V, E, F, W, out, st, keep_status, &launches)
+                 : launch_small_forward<__nv_bfloat16>(pr, L, ws, Q, K, V, E, F, W, out, st, keep_status, &launches);
+  } else if (pr.fp32) {
     rc = run_pipeline<float>(pr, L, ws, Q, K, V, E, F, W, out, st, false, false, false, &ds.tc, timer, keep_status,
                              &launches, phases);
   } else {

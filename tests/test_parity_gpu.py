@@ -501,3 +501,23 @@ def test_ragged_lengths_on_the_tensor_path(w, layout, per_head):
 ], ids=lambda w: w.name)
 def test_simt_path_at_the_edges_of_its_tiles(w):
     pu.check_all_heads(w, path=binding.PATH_SIMT)
+
+
+@pytest.mark.parametrize("w", [
+    # one position and one key; fewer positions, keys, features than CTAs; remainders of every tile
+    _wl("small_n1", PERFORMER, "fp32", 1, 2, 1, 8, 1, 1, 161),
+    _wl("small_few", PERFORMER, "fp32", 1, 3, 5, 7, 3, 5, 162),
+    _wl("small_odd", PERFORMER, "fp32", 2, 2, 250, 31, 30, 61, 163),
+    _wl("small_rnn", RNN, "fp32", 1, 4, 256, 64, 63, 0, 164),
+    _wl("small_m33", PERFORMER, "fp32", 1, 2, 60, 12, 17, 33, 165),
+    _wl("small_bf16", PERFORMER, "bf16", 1, 2, 123, 32, 32, 64, 166),
+], ids=lambda w: w.name)
+def test_small_forward_in_one_kernel(w):
+    pu.check_all_heads(w)
+    assert binding.flurka_last_path() == binding.PATH_SIMT and binding.flurka_last_launches() == 1
+    Kp = binding.flurka_debug_copy(0, (w.B, w.H, w.k, w.d)).cpu().double().numpy()
+    inputs = synth.make_inputs(w)
+    for h in range(w.H):
+        _, inter = pu.oracle_head(inputs, w, w.B - 1, h, rows=[0], intermediates=True)
+        # fp32 sums of at most 256 terms in another order: 256 * 2^-24 of the largest term's scale
+        assert np.abs(Kp[w.B - 1, h] - inter["Kp"]).max() < 2e-5 * max(1.0, np.abs(inter["Kp"]).max())
