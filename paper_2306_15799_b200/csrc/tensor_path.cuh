@@ -14,6 +14,7 @@
 #include "k1_down_project_pair.cuh"
 #include "k2_key_side.cuh"
 #include "k3_query_side.cuh"
+#include "k3_query_units.cuh"
 #include "k4_bwd_query_wide.cuh"
 #include "k5_bwd_projections.cuh"
 #include "k6_bwd_key_side.cuh"
@@ -472,14 +473,16 @@ inline int launch_k3(TensorContext& tc, bool performer, const void* Q, const voi
   prm.weight = weight;
   prm.out = reinterpret_cast<__nv_bfloat16*>(out);
   prm.status = status;
-  const K3Smem L = k3_smem_plan(d, p, performer);
-  auto fn = performer ? k3_query_side<true> : k3_query_side<false>;
-  cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)L.total);
+  // PERFORMER, d = 64: four tiles at a time (64 columns of S and 64 of O each fill TMEM; with d = 128 O alone would)
+  const bool units = performer && d == 64;
+  const uint32_t smem = units ? k3u_smem_plan(p).total : k3_smem_plan(d, p, performer).total;
+  auto fn = units ? k3_query_units : (performer ? k3_query_side<true> : k3_query_side<false>);
+  cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) { *cuda_err = (int)e; (void)cudaGetLastError(); return -6; }
   int grid = tc.sm_count();
   if (grid > prm.total_tiles) grid = prm.total_tiles;
   // the RNN kernel ignores tmW and only d = 64 stores through tmO; pass any valid map otherwise
-  e = launch_after_predecessor(fn, grid, kK3Threads, L.total, st, tm.Q.map, performer ? tm.W.map : tm.Q.map,
+  e = launch_after_predecessor(fn, grid, units ? kK3UThreads : kK3Threads, smem, st, tm.Q.map, performer ? tm.W.map : tm.Q.map,
                                tm.aT.map, d == 64 ? tm.O.map : tm.Q.map, prm);
   if (e != cudaSuccess) { *cuda_err = (int)e; (void)cudaGetLastError(); return -6; }
   e = cudaGetLastError();
