@@ -11,14 +11,12 @@
 // The per-feature summaries a_i, b_i (or z_i) come from stage 2.  A persistent CTA walks a
 // contiguous range of 128-row tiles; warp 0 feeds Q tiles by TMA, warps 1 and 3 issue the first and the second
 // products, warp 2 reloads a^T and rebuilds the bias operand when the head changes, and two groups of four warps
-// alternate tiles.  TMEM holds S/p and O of the tiles in flight: two 256-column buffers in general, four
-// 128-column buffers when d = 64 and p <= 128.  p overwrites S at half the width, block by block of 64
-// features, and the row owners hand every finished block to the second product.  With d = 64, O sits in
-// columns 64..127 of its buffer, which pass 2 has consumed after the first 128 features (blocks 2 and 3 of
-// p go to columns 128.. instead), so at m = 256 the second product of a tile runs under the second half
-// of its pass 2 and only its last block is left when the row owners start waiting for O.  With four
-// buffers each group has two tiles in flight and reads tile i-2 out after it has handed tile i to the
-// second product.  Every thread of a group owns one output row and writes it with 32-byte stores.
+// alternate tiles.  TMEM holds S/p and O of the tiles in flight: two 256-column buffers with d = 128, four
+// 128-column buffers with d = 64.  p overwrites S at half the width, block by block of 64 features, and the row
+// owners hand every finished block to the second product.  With four buffers each group has two tiles in flight
+// and reads tile i-2 out after it has handed tile i to the second product.
+// PERFORMER with d = 64 has a kernel of its own (k3_query_units.cuh), which keeps four tiles at work at a time;
+// with d = 128 O alone would fill TMEM for four tiles.
 #pragma once
 
 #include <cuda_bf16.h>
@@ -56,7 +54,7 @@ struct K3Smem {
 __host__ __device__ inline K3Smem k3_smem_plan(int d, int p, bool performer) {
   K3Smem s;
   uint32_t off = 0;
-  s.w = off;    off += performer ? (uint32_t)p * d * 2 : 0;        // W: d/64 K-blocks of [p rows x 128 B]
+  s.w = off;    off += performer ? (uint32_t)p * d * 2 : 0;        // W (PERFORMER, d = 128): 2 K-blocks of [p rows x 128 B]
   s.ones = off; off += performer ? 4096 : 0;                       // [128 x 16] bf16, no swizzle
   s.bias = off; off += performer ? 8192 : 0;                       // [256 x 16] bf16, no swizzle
   off = (off + 1023u) & ~1023u;
@@ -160,7 +158,7 @@ k3_query_side(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ C
   const int kq = d >> 6;      // 64-wide K-blocks of the Q / W tiles
   const int kp = p >> 6;      // 64-wide K-blocks of a^T
   // TMEM buffers: tile i uses buffer i % NB, its barriers flip once per NB tiles
-  const int NB = (d == 64 && p <= 128) ? 4 : 2;
+  const int NB = d == 64 ? 4 : 2;
   const int nb_shift = NB == 4 ? 2 : 1;
   const uint32_t buf_cols = 512u / NB;
   const uint32_t o_col = d == 64 ? 64u : 128u;
@@ -169,9 +167,7 @@ k3_query_side(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ C
   // of 64 features whose completion its issuer waits for (the blocks before it need no signal).
   int q_first = 0;
   if (kPerformer && (int)o_col < p) q_first = (min(p, (int)o_col + d) - 1) >> 6;
-  // p's block kb of 64 features (32 columns of fp16 pairs) sits at column pcol(kb): side by side from
-  // column 0, except that with d = 64 blocks 2 and 3 skip over O to columns 128 and 160
-  auto pcol = [&](int kb) -> uint32_t { return (uint32_t)(32 * kb + ((d == 64 && kb >= 2) ? 64 : 0)); };
+  // p's block kb of 64 features (32 columns of fp16 pairs) sits at column 32 kb
 
   if (ntiles > 0 && warp == 0 && lane == 0) {
     // W is an input, not a result of stage 2: its load starts before the dependency wait
@@ -281,7 +277,7 @@ k3_query_side(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ C
           tcgen05_fence_after();
           for (int kk = (kb == q_first ? 0 : kb); kk <= kb; ++kk) {
             const uint64_t bd = make_sdesc(base + L.aT + kk * (d * 128), 16, 1024, kSwizzle128);
-            mma_ts_x4(tb + o_col, tb + pcol(kk), bd, 2, idesc2, kk > 0 ? 1u : 0u);
+            mma_ts_x4(tb + o_col, tb + 32 * kk, bd, 2, idesc2, kk > 0 ? 1u : 0u);
           }
         }
         if (!ok) break;
@@ -507,7 +503,7 @@ k3_query_side(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ C
             tmem_wait_ld(ra);
             tmem_ld32(tb + c + 32, rb);
             exp_block(ra, h);
-            const uint32_t pc = pcol(c >> 6);
+            const uint32_t pc = (uint32_t)(c >> 1);
             tmem_st16(tb + pc, h);
             tmem_wait_ld(rb);
             if (c + 64 < p) tmem_ld32(tb + c + 64, ra);

@@ -13,7 +13,11 @@
 // barrier round trips and read-outs of the others.  Two groups with 256 features at a time (k3_query_side) left them
 // half idle: a group's tile took 7390 cycles at m = 256, 3160 of which were exponentials, at 12 cycles each because one
 // warp alone does not overlap them (7 with two).  Two groups with 128 features in registers took 7900.
-// K3U_FIG
+// Measured, two groups -> this kernel: 120 -> 107 us at 64 heads x N = 16384 with m = 256, 64.5 -> 56 us at 96 heads x
+// N = 8192 with m = 128, 8.1 -> 7.4 us at 2 heads x N = 1024.  A tile with m = 256 takes 3200 cycles of an SM, 1480 of them
+// tensor (N = 64 costs 48 cycles per step with A in shared memory and 32 with A in TMEM: the reads of A bind), 1800
+// special-function; what is left is latency: a block's round trip through two chains of products is 1000 cycles.  Three groups
+// with S of the next block formed under the exponentials of this one came out the same (108 us).
 #pragma once
 
 #include "k3_query_side.cuh"
@@ -249,14 +253,15 @@ k3_query_units(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
       const uint32_t slab = base + L.ostage + (uint32_t)(warp - 8) * 4096u;
       const float kLog2e = 1.4426950408889634f;
       const uint64_t l2 = pack2(kLog2e, kLog2e);
-      // 32 columns: x = 2^(S log2e - r) as fp16 pairs and the row sum.  Three pairs in eight take their exponential as a
-      // cubic on the FMA pipe, the others on the special-function unit.
+      // 32 columns: x = 2^(S log2e - r) as fp16 pairs and the row sum.  One pair in eight takes its exponential as a
+      // cubic on the FMA pipe, the others on the special-function unit (three in eight, the mix of k3_query_side, is 2.5 %
+      // slower here, where issue slots are the scarcer: 110.3 against 107.2 us; none at all 112.7).
       auto exp_block = [&](const uint32_t (&r)[32], uint32_t (&hh)[16], uint64_t ms2, uint64_t& den2) {
 #pragma unroll
         for (int e = 0; e < 16; ++e) {
           float x0, x1, e0, e1;
           unpack2(fma2(pack2u(r[2 * e], r[2 * e + 1]), l2, ms2), x0, x1);
-          if ((e & 7) == 1 || (e & 7) == 4 || (e & 7) == 6) {
+          if ((e & 7) == 4) {
             // far below what fp16 can hold the result is 0 either way; the cubic needs its exponent in range
             exp2_cubic2(pack2(fmaxf(x0, -60.f), fmaxf(x1, -60.f)), e0, e1);
           } else {

@@ -521,3 +521,33 @@ def test_small_forward_in_one_kernel(w):
         _, inter = pu.oracle_head(inputs, w, w.B - 1, h, rows=[0], intermediates=True)
         # fp32 sums of at most 256 terms in another order: 256 * 2^-24 of the largest term's scale
         assert np.abs(Kp[w.B - 1, h] - inter["Kp"]).max() < 2e-5 * max(1.0, np.abs(inter["Kp"]).max())
+
+
+@pytest.mark.parametrize("limit", [0, 2])
+@pytest.mark.parametrize("w", [
+    # one to four blocks of 64 features; fewer tiles than groups, a ragged last tile, heads that change inside a CTA's range
+    _wl("units_m64", PERFORMER, "bf16", 1, 3, 520, 64, 64, 64, 171),
+    _wl("units_m128_one_tile", PERFORMER, "bf16", 1, 5, 128, 64, 128, 128, 172),
+    _wl("units_m192", PERFORMER, "bf16", 2, 2, 776, 64, 64, 192, 173),
+    _wl("units_m256", PERFORMER, "bf16", 1, 3, 520, 64, 128, 256, 174),
+], ids=lambda w: w.name)
+def test_query_side_in_blocks_of_64_features(w, limit):
+    """Q is scaled by 2 so that, with more than one block, some rows find their maximum more than 15 above (base 2) the one of
+    the block that the kernel takes first (the one with the largest log-weight) and have to raise their reference."""
+    inputs = synth.make_inputs(w)
+    inputs["Q"] = (inputs["Q"].double() * 2.0).to(inputs["Q"].dtype)
+    prev = binding.flurka_set_cta_limit(limit)
+    try:
+        out = pu.run_gpu(w, inputs, binding.PATH_TENSOR).cpu().double().numpy()
+    finally:
+        binding.flurka_set_cta_limit(prev)
+    raised = 0
+    for b in range(w.B):
+        for h in range(w.H):
+            ref, inter = pu.oracle_head(inputs, w, b, h, intermediates=True)
+            pu.assert_close(out[b, h], ref, "bf16", "%s head (%d,%d)" % (w.name, b, h))
+            log_z = np.log(inter["z"])
+            s = inputs["Q"][b, h].double().numpy() @ inputs["W"].double().numpy().T + log_z
+            blocks = s.reshape(w.N, -1, 64).max(2) / np.log(2.0)
+            raised += int((blocks.max(1) > blocks[:, int(np.argmax(log_z)) // 64] + 15.0).sum())
+    assert raised > 0 or w.m < 256
