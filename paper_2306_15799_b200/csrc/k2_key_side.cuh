@@ -18,7 +18,7 @@
 // weights are the fp16 f tile as it lies ([key][feature], the MN-major A operand), and z_i comes from the same tile
 // times a column of ones.
 // One block of 256 keys takes about 10 k cycles; the earlier form (eight warps, a staging copy and a block barrier per
-// 128 keys, one thread per row) took 17 us after stage 1's end at B H = 64, k = m = 256, d = 64, this one K2_FIG.
+// 128 keys, one thread per row) took 17 us after stage 1's end at B H = 64, k = m = 256, d = 64, this one 9.
 //
 // With few heads and several blocks the blocks are divided over `nsplit` CTAs per (head, feature tile): each keeps its
 // own maximum, sum and unnormalised accumulator, writes them to a scratch area, and the CTA that arrives
