@@ -87,8 +87,8 @@ typedef enum {
  *
  * Shape limits: B, H, N >= 1, B*H <= 65535; 1 <= d <= 128; 1 <= k <= 4096; PERFORMER: m >= 1.
  * Pointers 16-byte aligned.  The tensor-core path additionally needs bf16, d in {64, 128},
- * N % 8 == 0, k % 64 == 0 with k <= 512, and (PERFORMER) m in {64, 128, 192, 256}; other shapes run
- * on the SIMT path.  The call enqueues work and returns; it never synchronises.  Scratch comes from the
+ * N % 8 == 0 or N >= 256 (other N: E, F are copied once into rows on 16-byte boundaries, in the workspace),
+ * k % 64 == 0 with k <= 512, and (PERFORMER) m in {64, 128, 192, 256}; other shapes run on the SIMT path.  The call enqueues work and returns; it never synchronises.  Scratch comes from the
  * workspace set by flurka_set_workspace(), or from one the library obtains on first need and re-uses:
  * when a later problem needs more, the old block is released and a larger one obtained in stream order
  * on `stream` (cudaFreeAsync / cudaMallocAsync), so calls that share the library-owned workspace must
@@ -176,7 +176,7 @@ int flurka_forward_finish(const void* Q, const void* W, int variant, int B, int 
  * The forward's key-side summaries are recomputed inside the call, so nothing has to be kept from the
  * forward pass.  No output may overlap an input or another output.
  * Kernels: where flurka_forward's tensor-core path takes the shape (bf16, the rules below) the two
- * down-projections, the key-side summaries and, with E, F shared by the heads, the gradients dK, dV, dE, dF
+ * down-projections, the key-side summaries and the gradients dK, dV, dE, dF
  * (products with E, F, K, V: dK', dV' enter as two bf16 terms) run on tcgen05 kernels; so does the query side
  * (dQ and the gradients of the key-side summaries) for d = 64 and, PERFORMER only, d = 128, and the key side's
  * backward half (dK', dV' from those gradients) for PERFORMER with d = 64.
