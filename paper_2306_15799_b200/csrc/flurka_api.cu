@@ -1042,13 +1042,22 @@ int backward_pipeline(const Problem& pr, const BackwardLayout& BL, char* ws, con
       ++*launches;
     }
   } else {
-    dim3 grid((pr.N + 31) / 32, pr.BH(), 2);
-    simt_bwd_inputs<T><<<grid, 256, 0, st>>>((const T*)E, (const T*)F, dkpvp, (T*)dK, (T*)dV, pr.BH(), pr.N, pr.d,
-                                             pr.k, smh, efh);
+    // tiles of 128 rows where they are at least as many as SMs, else of 32
+    const int zi = 2 * ((pr.d + 63) / 64), zp = 2 * (efh > 0 ? efh : 1);
+    auto blocks = [](int n, int per) { return (n + per - 1) / per; };
+    if ((long long)blocks(pr.N, 128) * pr.BH() * zi >= 148)
+      simt_bwd_inputs<T, 8><<<dim3(blocks(pr.N, 128), pr.BH(), zi), kSimtThreads, 0, st>>>(
+          (const T*)E, (const T*)F, dkpvp, (T*)dK, (T*)dV, pr.BH(), pr.N, pr.d, pr.k, smh, efh);
+    else
+      simt_bwd_inputs<T, 2><<<dim3(blocks(pr.N, 32), pr.BH(), zi), kSimtThreads, 0, st>>>(
+          (const T*)E, (const T*)F, dkpvp, (T*)dK, (T*)dV, pr.BH(), pr.N, pr.d, pr.k, smh, efh);
     ++*launches;
-    dim3 grid2((pr.N + 31) / 32, (pr.k + 31) / 32, 2 * (efh > 0 ? efh : 1));
-    simt_bwd_projections<T><<<grid2, 256, 0, st>>>((const T*)K, (const T*)V, dkpvp, (T*)dE, (T*)dF, pr.BH(), pr.N,
-                                                   pr.d, pr.k, smh, efh);
+    if ((long long)blocks(pr.N, 64) * blocks(pr.k, 128) * zp >= 148)
+      simt_bwd_projections<T, 8><<<dim3(blocks(pr.N, 64), blocks(pr.k, 128), zp), kSimtThreads, 0, st>>>(
+          (const T*)K, (const T*)V, dkpvp, (T*)dE, (T*)dF, pr.BH(), pr.N, pr.d, pr.k, smh, efh);
+    else
+      simt_bwd_projections<T, 2><<<dim3(blocks(pr.N, 64), blocks(pr.k, 32), zp), kSimtThreads, 0, st>>>(
+          (const T*)K, (const T*)V, dkpvp, (T*)dE, (T*)dF, pr.BH(), pr.N, pr.d, pr.k, smh, efh);
     ++*launches;
   }
   e = cudaGetLastError();

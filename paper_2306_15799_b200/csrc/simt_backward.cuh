@@ -439,98 +439,154 @@ simt_bwd_key_side(const float* __restrict__ KpVp, const T* __restrict__ W, const
 }
 
 // ---------------------------------------------------------------------------------------------
-// dK = E^T dK', dV = F^T dV'.  grid = (ceil(N/32), B*H, 2); block = 256: warp w owns positions
-// 4w..4w+3 of the tile, lane owns columns lane + 32 b.  E, F: [k][N] (or [H][k][N], ef_heads = H).
+// dK = E^T dK', dV = F^T dV'.  grid = (ceil(N / 16R), B*H, 2 ceil(d / 64)); block = 256.  E, F: [k][N] (or [H][k][N],
+// ef_heads = H).  Both operands lie [j][..], so a thread's R consecutive positions x 4 columns are an outer product per
+// projected key, read from shared memory in 16-byte pieces (3 per 32 FFMA with R = 8; FFMA-bound, as stage 1); the next
+// 32 keys travel in registers under this step's products.  B = 2, H = 8, N = 4096, d = 64, k = 256, fp32, against scalar
+// reads and four rows per warp: 335 -> 115 us (B = 1, H = 2, N = 1024, k = 128: 20.5 -> 6.6).  R = 2 keeps more blocks busy where 128-row tiles would be fewer than SMs.
 // ---------------------------------------------------------------------------------------------
-template <typename T>
-__global__ void __launch_bounds__(256)
+template <typename T, int R>
+__global__ void __launch_bounds__(kSimtThreads)
 simt_bwd_inputs(const T* __restrict__ E, const T* __restrict__ F, const float* __restrict__ dKpVp,
                 T* __restrict__ dK, T* __restrict__ dV, int BH, int N, int d, int k, int seq_major_heads,
                 int ef_heads) {
-  __shared__ float Ps[32][33];     // [j][n]
-  __shared__ float Gs[32][128];    // [j][c]
-  const int t = blockIdx.z, bh = blockIdx.y, n0 = blockIdx.x * 32;
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  constexpr int kRows = 16 * R, kA = kRows / 32;   // 16-byte pieces of the E tile per thread
+  __shared__ __align__(16) float Ps[32][kRows];    // [j][n]
+  __shared__ __align__(16) float Gs[32][64];       // [j][c]
+  const int cb = (d + 63) / 64;
+  const int t = blockIdx.z / cb, c0 = (blockIdx.z % cb) * 64, bh = blockIdx.y, n0 = blockIdx.x * kRows;
+  const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
   const T* __restrict__ P = (t ? F : E) + (ef_heads > 0 ? (size_t)(bh % ef_heads) * k * N : 0);
   const float* __restrict__ G = dKpVp + ((size_t)t * BH + bh) * (size_t)k * d;
   const HeadView hv = head_view(bh, seq_major_heads, N, d);
   T* __restrict__ out = (t ? dV : dK) + hv.base;
-  float acc[4][4];
+  const bool vec_n = (N & 3) == 0, vec_d = (d & 3) == 0;
+  float4 pa[kA], pg[2];
+  auto fetch = [&](int j0) {
 #pragma unroll
-  for (int r = 0; r < 4; ++r)
+    for (int q = 0; q < kA; ++q) {
+      const int e = threadIdx.x + q * kSimtThreads, jj = e / (kRows / 4), n = n0 + (e % (kRows / 4)) * 4;
+      pa[q] = simt_load_row4(P + (size_t)(j0 + jj) * N + n, j0 + jj < k ? N - n : 0, vec_n);
+    }
+#pragma unroll
+    for (int q = 0; q < 2; ++q) {
+      const int e = threadIdx.x + q * kSimtThreads, jj = e >> 4, c = c0 + (e & 15) * 4;
+      pg[q] = simt_load_row4(G + (size_t)(j0 + jj) * d + c, j0 + jj < k ? d - c : 0, vec_d);
+    }
+  };
+  float acc[R][4];
+#pragma unroll
+  for (int r = 0; r < R; ++r)
 #pragma unroll
     for (int b = 0; b < 4; ++b) acc[r][b] = 0.f;
+  fetch(0);
   for (int j0 = 0; j0 < k; j0 += 32) {
     __syncthreads();
-    for (int idx = threadIdx.x; idx < 32 * 32; idx += 256) {
-      const int jj = idx >> 5, nn = idx & 31;
-      Ps[jj][nn] = (j0 + jj < k && n0 + nn < N) ? to_f32(P[(size_t)(j0 + jj) * N + n0 + nn]) : 0.f;
-    }
-    for (int idx = threadIdx.x; idx < 32 * 128; idx += 256) {
-      const int jj = idx >> 7, c = idx & 127;
-      Gs[jj][c] = (j0 + jj < k && c < d) ? G[(size_t)(j0 + jj) * d + c] : 0.f;
-    }
+#pragma unroll
+    for (int q = 0; q < kA; ++q) reinterpret_cast<float4*>(&Ps[0][0])[threadIdx.x + q * kSimtThreads] = pa[q];
+#pragma unroll
+    for (int q = 0; q < 2; ++q) reinterpret_cast<float4*>(&Gs[0][0])[threadIdx.x + q * kSimtThreads] = pg[q];
     __syncthreads();
+    if (j0 + 32 < k) fetch(j0 + 32);
+#pragma unroll 4
     for (int jj = 0; jj < 32; ++jj) {
+      const float4 g = *reinterpret_cast<const float4*>(&Gs[jj][tx * 4]);
+      float p[R];
 #pragma unroll
-      for (int r = 0; r < 4; ++r) {
-        const float e = Ps[jj][warp * 4 + r];
+      for (int r = 0; r < R; r += 2) {
+        const float2 v = *reinterpret_cast<const float2*>(&Ps[jj][ty * R + r]);
+        p[r] = v.x;
+        p[r + 1] = v.y;
+      }
 #pragma unroll
-        for (int b = 0; b < 4; ++b) acc[r][b] = fmaf(e, Gs[jj][lane + 32 * b], acc[r][b]);
+      for (int r = 0; r < R; ++r) {
+        acc[r][0] = fmaf(p[r], g.x, acc[r][0]);
+        acc[r][1] = fmaf(p[r], g.y, acc[r][1]);
+        acc[r][2] = fmaf(p[r], g.z, acc[r][2]);
+        acc[r][3] = fmaf(p[r], g.w, acc[r][3]);
       }
     }
   }
 #pragma unroll
-  for (int r = 0; r < 4; ++r) {
-    const int n = n0 + warp * 4 + r;
+  for (int r = 0; r < R; ++r) {
+    const int n = n0 + ty * R + r;
     if (n >= N) continue;
 #pragma unroll
     for (int b = 0; b < 4; ++b) {
-      const int c = lane + 32 * b;
+      const int c = c0 + tx * 4 + b;
       if (c < d) store_out(out + (size_t)n * hv.row_stride + c, acc[r][b]);
     }
   }
 }
 
 // ---------------------------------------------------------------------------------------------
-// dE = sum over heads of dK' K^T, dF = sum over heads of dV' V^T.  grid = (ceil(N/32), ceil(k/32),
-// 2 * max(ef_heads, 1)); block = 256 (a 32 x 32 tile of dE, four rows per thread).  With shared E, F
-// the sum runs over all B*H heads; with one pair per head over the batch only.
+// dE = sum over heads of dK' K^T, dF = sum over heads of dV' V^T.  grid = (ceil(N / 64), ceil(k / 16R),
+// 2 * max(ef_heads, 1)); block = 256.  With shared E, F the sum runs over all B*H heads; with one pair per head over the
+// batch only.  Both operands are rows of d values: dot products 32 columns at a time (simt_dots), the next step's
+// operands in registers.  B = 2, H = 8, N = 4096, d = 64, k = 256, fp32, against scalar reads and four outputs per
+// thread: 431 -> 128 us (small as above: 12.9 -> 6.1).  R as above.
 // ---------------------------------------------------------------------------------------------
-template <typename T>
-__global__ void __launch_bounds__(256)
+template <typename T, int R>
+__global__ void __launch_bounds__(kSimtThreads)
 simt_bwd_projections(const T* __restrict__ Kin, const T* __restrict__ Vin, const float* __restrict__ dKpVp,
                      T* __restrict__ dE, T* __restrict__ dF, int BH, int N, int d, int k, int seq_major_heads,
                      int ef_heads) {
-  __shared__ float Gs[32][129];    // [j][c]
-  __shared__ float Xs[32][129];    // [n][c]
+  constexpr int kLd = 36, kG = (16 * R) / 32 > 0 ? (16 * R) / 32 : 1;   // simt_ld(32); pieces of dK' per thread
+  __shared__ __align__(16) float Gs[16 * R][kLd];  // [j][c]
+  __shared__ __align__(16) float Xs[64][kLd];      // [n][c]
   const int groups = ef_heads > 0 ? ef_heads : 1;
   const int t = blockIdx.z / groups, eh = blockIdx.z % groups;
-  const int n0 = blockIdx.x * 32, j0 = blockIdx.y * 32;
-  const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
-  float acc[4] = {0.f, 0.f, 0.f, 0.f};
-  for (int bh = eh; bh < BH; bh += groups) {
+  const int n0 = blockIdx.x * 64, j0 = blockIdx.y * (16 * R);
+  const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
+  const int row8 = threadIdx.x >> 3, col4 = (threadIdx.x & 7) * 4;
+  const bool vec_d = (d & 3) == 0;
+  const T* __restrict__ Xin = t ? Vin : Kin;
+  float4 pg[kG], px[2];
+  auto fetch = [&](int bh, int c0) {
     const float* __restrict__ G = dKpVp + ((size_t)t * BH + bh) * (size_t)k * d;
     const HeadView hv = head_view(bh, seq_major_heads, N, d);
-    const T* __restrict__ X = (t ? Vin : Kin) + hv.base;
-    __syncthreads();
-    for (int idx = threadIdx.x; idx < 32 * 128; idx += 256) {
-      const int rr = idx >> 7, c = idx & 127;
-      Gs[rr][c] = (j0 + rr < k && c < d) ? G[(size_t)(j0 + rr) * d + c] : 0.f;
-      Xs[rr][c] = (n0 + rr < N && c < d) ? to_f32(X[(size_t)(n0 + rr) * hv.row_stride + c]) : 0.f;
-    }
-    __syncthreads();
-    for (int c = 0; c < d; ++c) {
-      const float x = Xs[tx][c];
+    const int c = c0 + col4;
 #pragma unroll
-      for (int r = 0; r < 4; ++r) acc[r] = fmaf(Gs[ty + 8 * r][c], x, acc[r]);
+    for (int q = 0; q < kG; ++q) {
+      const int j = j0 + row8 + 32 * q;
+      pg[q] = simt_load_row4(G + (size_t)j * d + c, j < k ? d - c : 0, vec_d);
     }
+#pragma unroll
+    for (int q = 0; q < 2; ++q) {
+      const int n = n0 + row8 + 32 * q;
+      px[q] = simt_load_row4(Xin + hv.base + (size_t)n * hv.row_stride + c, n < N ? d - c : 0, vec_d);
+    }
+  };
+  float acc[R][4];
+#pragma unroll
+  for (int r = 0; r < R; ++r)
+#pragma unroll
+    for (int f = 0; f < 4; ++f) acc[r][f] = 0.f;
+  int bh = eh, c0 = 0;
+  fetch(bh, c0);
+  while (bh < BH) {
+    __syncthreads();
+#pragma unroll
+    for (int q = 0; q < kG; ++q)
+      if (row8 + 32 * q < 16 * R) *reinterpret_cast<float4*>(&Gs[row8 + 32 * q][col4]) = pg[q];
+#pragma unroll
+    for (int q = 0; q < 2; ++q) *reinterpret_cast<float4*>(&Xs[row8 + 32 * q][col4]) = px[q];
+    __syncthreads();
+    const int cols = min(32, (d - c0 + 3) & ~3);
+    c0 += 32;
+    if (c0 >= d) { c0 = 0; bh += groups; }
+    if (bh < BH) fetch(bh, c0);
+    simt_dots<R>(acc, &Gs[0][0], &Xs[0][0], kLd, cols);
   }
   T* __restrict__ out = (t ? dF : dE) + (size_t)eh * k * N;
 #pragma unroll
-  for (int r = 0; r < 4; ++r) {
-    const int j = j0 + ty + 8 * r;
-    if (j < k && n0 + tx < N) store_out(out + (size_t)j * N + n0 + tx, acc[r]);
+  for (int r = 0; r < R; ++r) {
+    const int j = j0 + ty + 16 * r;
+#pragma unroll
+    for (int f = 0; f < 4; ++f) {
+      const int n = n0 + tx + 16 * f;
+      if (j < k && n < N) store_out(out + (size_t)j * N + n, acc[r][f]);
+    }
   }
 }
 

@@ -240,3 +240,19 @@ def test_backward_of_ragged_lengths_on_the_tensor_path(w, layout, per_head):
     """N no multiple of 8: E, F are read from padded copies, dE, dF leave through them."""
     _check(w, layout=layout, per_head=per_head)
     assert binding.flurka_last_path() == binding.PATH_TENSOR
+
+
+@pytest.mark.parametrize("w,layout,per_head", [
+    # tiles of 32 rows: one row, remainders of every tile, more than 64 columns.  (One row with ONE key has dQ = 0 exactly: every
+    # a_i is that key's v', so the row's output does not depend on q, and a relative bound on dQ would have to be 0 / 0.)
+    (Workload("bwd_cc_n1", PERFORMER, "fp32", 1, 1, 1, 8, 5, 8, 331), "bhnd", False),
+    (Workload("bwd_cc_odd", PERFORMER, "fp32", 1, 2, 97, 33, 31, 24, 332), "bnhd", False),
+    (Workload("bwd_cc_d100", RNN, "bf16", 1, 2, 66, 100, 65, 0, 333), "bhnd", True),
+    # tiles of 128 rows (at least 148 blocks): remainders of them, one and two column blocks
+    (Workload("bwd_cc_big", RNN, "fp32", 2, 3, 1601, 20, 300, 0, 334), "bhnd", False),
+    (Workload("bwd_cc_big_d100", RNN, "fp32", 1, 4, 1281, 100, 400, 0, 335), "bnhd", False),
+    (Workload("bwd_cc_big_per_head", RNN, "bf16", 1, 6, 1604, 36, 129, 0, 336), "bhnd", True),
+], ids=lambda v: v.name if hasattr(v, "name") else str(v))
+def test_backward_products_with_inputs_on_cuda_cores(w, layout, per_head):
+    _check(w, layout=layout, per_head=per_head)
+    assert binding.flurka_last_path() == binding.PATH_SIMT
