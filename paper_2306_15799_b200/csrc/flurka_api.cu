@@ -1010,13 +1010,16 @@ int backward_pipeline(const Problem& pr, const BackwardLayout& BL, char* ws, con
     if (rc) { g_last_cuda_error = cuda_err; return rc; }
     ++*launches;
   } else {
-    auto fn = simt_bwd_query_side<T, P>;
-    const size_t smem = ((size_t)2 * 32 * (pr.d + 1) + 32 * 33 + 32 * pr.d) * 4;
+    // tiles of 64 rows where they are at least as many as SMs, else of 32
+    const bool big = (long long)((pr.N + 63) / 64) * pr.BH() >= 148;
+    auto fn = pr.d > 64 ? (big ? simt_bwd_query_side<T, P, 4, 2> : simt_bwd_query_side<T, P, 2, 2>)
+                        : (big ? simt_bwd_query_side<T, P, 4, 1> : simt_bwd_query_side<T, P, 2, 1>);
+    const int rows = big ? 64 : 32;
+    const size_t smem = simt_bwd_query_floats(pr.d, rows / 16, P) * 4;
     if ((e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess)
       return cuda_fail(e);
-    dim3 grid((pr.N + 31) / 32, pr.BH());
-    fn<<<grid, 256, smem, st>>>((const T*)Q, (const T*)W, (const T*)dO, weight, a32, (T*)dQ, da, ei, pr.N, pr.d,
-                                pr.p(), smh);
+    fn<<<dim3((pr.N + rows - 1) / rows, pr.BH()), kSimtThreads, smem, st>>>((const T*)Q, (const T*)W, (const T*)dO, weight, a32,
+                                                                           (T*)dQ, da, ei, pr.N, pr.d, pr.p(), smh);
     ++*launches;
   }
   __nv_bfloat16* split = tc ? (__nv_bfloat16*)(ws + BL.split) : nullptr;

@@ -25,190 +25,200 @@ __device__ __forceinline__ float elu1(float x) { return x > 0.f ? x + 1.f : expf
 __device__ __forceinline__ float elu1_slope(float x) { return x > 0.f ? 1.f : expf(x); }
 
 // ---------------------------------------------------------------------------------------------
-// Query side.  grid = (ceil(N/32), B*H); block = 256: warp w owns rows 4w..4w+3 of the tile.
-// Two sweeps over the features in chunks of 32: the first is the forward (running maximum, sum,
-// O_n); the second forms c_ni and accumulates dq_n, da_i, e_i.  da, e (fp32, zeroed before) are
-// added to with atomics: every row tile of a head contributes.
-// Dynamic shared memory: 2 * 32 * (d+1) floats (W chunk, a chunk) + 32 * 33 (P tile) + 32 * d (dO tile).
+// Query side.  grid = (ceil(N / 16R), B*H); block = 256 (the building blocks of simt_kernels.cuh); 64 features at a time.
+// With g_ni = a_i . dO_n, O_n . dO_n = sum_i P_ni g_ni: sweep 1 is the dot products l and g with a running maximum, sum and
+// weighted sum; sweep 2 forms them again, then c_ni, dq += C W, da += P^T dO (C and P^T through shared memory), e_i.
+// RNN: the weights come from the Q tile, no l, no dq product.  da, e (fp32, zeroed before) are added to with atomics: every
+// row tile of a head contributes.  Six units of 2 N m d operations (RNN: three) at the FFMA rate of the register tiles.
+// fp32, B = 2, H = 8, N = 4096, d = 64, m = 256, against one feature per lane and scalar reads: 1667 -> 543 us
+// (B = 1, H = 2, N = 1024, m = 128: 78 -> 30; RNN, first sizes: 250 -> 109; RNN, bf16, d = 128: 655 -> 399).
+// R = 2 (tiles of 32 rows) where tiles of 64 would be fewer than SMs.
 // ---------------------------------------------------------------------------------------------
-template <typename T, bool kPerformer>
-__global__ void __launch_bounds__(256)
+// floats of shared memory; a product reads up to 64 NB columns of a row, so a tile it reads has another one behind it
+__host__ __device__ inline size_t simt_bwd_query_floats(int d, int R, bool performer) {
+  return (size_t)simt_ld(d) * (2 * 16 * R + (performer ? 2 : 1) * 64) + 64 * (16 * R + 4) + (performer ? 16 * R * 68 : 0) + 128;
+}
+template <typename T, bool kPerformer, int R, int NB>
+__global__ void __launch_bounds__(kSimtThreads, NB == 1 ? 2 : 1)
 simt_bwd_query_side(const T* __restrict__ Q, const T* __restrict__ W, const T* __restrict__ dO,
                     const float* __restrict__ weight, const float* __restrict__ a32, T* __restrict__ dQ,
                     float* __restrict__ da, float* __restrict__ ei, int N, int d, int p, int seq_major_heads) {
-  extern __shared__ float smem[];
-  float* Ws = smem;                          // [32][d+1]
-  float* As = Ws + 32 * (d + 1);             // [32][d+1]
-  float* Ps = As + 32 * (d + 1);             // [32 rows][33]
-  float* Gs = Ps + 32 * 33;                  // [32 rows][d]   dO tile
-  __shared__ float qs[32][128];
-  __shared__ float ws[32];
-  __shared__ float es[8][32];
+  extern __shared__ __align__(16) float smem[];
+  constexpr int kRows = 16 * R, kLdP = kRows + 4, kLdC = 68;
+  const int ld = simt_ld(d), cols = (d + 3) & ~3;
+  float* Gs = smem;                          // [kRows][ld]  dO tile
+  float* Qs = Gs + kRows * ld;               // [kRows][ld]
+  float* As = Qs + kRows * ld;               // [64][ld]     a of the chunk's features
+  float* Ws = As + 64 * ld;                  // [64][ld]     PERFORMER: W of the chunk's features
+  float* Pt = Ws + (kPerformer ? 64 * ld : 0);   // [64 features][kRows]
+  float* Cs = Pt + 64 * kLdP;                // [kRows][64]  PERFORMER
+  __shared__ float ws[64];
+  __shared__ float es[8][64];
 
-  const int bh = blockIdx.y;
-  const int n0 = blockIdx.x * 32;
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int bh = blockIdx.y, n0 = blockIdx.x * kRows;
+  const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4, warp = tid >> 5, lane = tid & 31;
   const HeadView hv = head_view(bh, seq_major_heads, N, d);
   const float* __restrict__ ah = a32 + (size_t)bh * p * d;
   const float* __restrict__ wh = weight + (size_t)bh * p;
+  const bool vec_d = (d & 3) == 0;
+  const int pieces = ld >> 2;
 
-  for (int idx = threadIdx.x; idx < 32 * d; idx += 256) {
-    const int r = idx / d, c = idx % d;
-    const bool in = n0 + r < N;
-    qs[r][c] = in ? to_f32(Q[hv.base + (size_t)(n0 + r) * hv.row_stride + c]) : 0.f;
-    Gs[r * d + c] = in ? to_f32(dO[hv.base + (size_t)(n0 + r) * hv.row_stride + c]) : 0.f;
-  }
-  float run_max[4], run_sum[4], acc[4][4];
-#pragma unroll
-  for (int r = 0; r < 4; ++r) {
-    run_max[r] = kPerformer ? -INFINITY : 0.f;
-    run_sum[r] = 0.f;
-#pragma unroll
-    for (int b = 0; b < 4; ++b) acc[r][b] = 0.f;
+  for (int e = tid; e < kRows * pieces; e += kSimtThreads) {
+    const int r = e / pieces, c = (e % pieces) * 4, live = n0 + r < N ? d - c : 0;
+    const size_t at = hv.base + (size_t)(n0 + r) * hv.row_stride + c;
+    *reinterpret_cast<float4*>(Qs + r * ld + c) = simt_load_row4(Q + at, live, vec_d);
+    *reinterpret_cast<float4*>(Gs + r * ld + c) = simt_load_row4(dO + at, live, vec_d);
   }
   auto stage_chunk = [&](int i0) {
     __syncthreads();
-    for (int idx = threadIdx.x; idx < 32 * d; idx += 256) {
-      const int ii = idx / d, c = idx % d;
-      const bool in = i0 + ii < p;
-      if (kPerformer) Ws[ii * (d + 1) + c] = in ? to_f32(W[(size_t)(i0 + ii) * d + c]) : 0.f;
-      As[ii * (d + 1) + c] = in ? ah[(size_t)(i0 + ii) * d + c] : 0.f;
+    for (int e = tid; e < 64 * pieces; e += kSimtThreads) {
+      const int i = e / pieces, c = (e % pieces) * 4, live = i0 + i < p ? d - c : 0;
+      const size_t at = (size_t)(i0 + i) * d + c;
+      if (kPerformer) *reinterpret_cast<float4*>(Ws + i * ld + c) = simt_load_row4(W + at, live, vec_d);
+      *reinterpret_cast<float4*>(As + i * ld + c) = simt_load_row4(ah + at, live, vec_d);
     }
-    if (threadIdx.x < 32) ws[threadIdx.x] = (i0 + threadIdx.x < p) ? wh[i0 + threadIdx.x] : 0.f;
+    if (tid < 64) ws[tid] = i0 + tid < p ? wh[i0 + tid] : 0.f;
     __syncthreads();
   };
-  // unnormalised weight of (row, feature lane) and its logit: PERFORMER exp(s - max) with s = q.w + b
-  auto logit = [&](int row, int i0, bool live) -> float {
-    if (kPerformer) {
-      float s = 0.f;
-      for (int c = 0; c < d; ++c) s = fmaf(qs[row][c], Ws[lane * (d + 1) + c], s);
-      return live ? s + ws[lane] : -INFINITY;
-    }
-    return live ? elu1(qs[row][i0 + lane]) * ws[lane] : 0.f;     // RNN: the weight itself, no exponent
+  // this thread's rows ty + 16 r x features i0 + tx + 16 f: PERFORMER the logit, RNN the weight itself; and g
+  auto form = [&](int i0, float (&s)[R][4], float (&g)[R][4]) {
+#pragma unroll
+    for (int r = 0; r < R; ++r)
+#pragma unroll
+      for (int f = 0; f < 4; ++f) s[r][f] = g[r][f] = 0.f;
+    if (kPerformer) simt_dots<R>(s, Qs, Ws, ld, cols);
+    simt_dots<R>(g, Gs, As, ld, cols);
+#pragma unroll
+    for (int r = 0; r < R; ++r)
+#pragma unroll
+      for (int f = 0; f < 4; ++f) {
+        const int i = tx + 16 * f;
+        const bool live = i0 + i < p;
+        if (kPerformer) s[r][f] = live ? s[r][f] + ws[i] : -INFINITY;
+        else s[r][f] = live ? elu1(Qs[(ty + 16 * r) * ld + i0 + i]) * ws[i] : 0.f;
+      }
   };
 
-  // ---- sweep 1: the forward (O_n, the row maximum and sum)
-  for (int i0 = 0; i0 < p; i0 += 32) {
+  // ---- sweep 1: row maximum, sum and weighted sum of g
+  float run_max[R], sum[R], t[R];
+#pragma unroll
+  for (int r = 0; r < R; ++r) {
+    run_max[r] = kPerformer ? -INFINITY : 0.f;
+    sum[r] = t[r] = 0.f;
+  }
+  for (int i0 = 0; i0 < p; i0 += 64) {
     stage_chunk(i0);
-    const bool live = (i0 + lane) < p;
+    float s[R][4], g[R][4];
+    form(i0, s, g);
 #pragma unroll
-    for (int r = 0; r < 4; ++r) {
-      const int row = warp * 4 + r;
-      float pv = logit(row, i0, live);
+    for (int r = 0; r < R; ++r) {
       if (kPerformer) {
-        float cm = pv;
+        float cm = fmaxf(fmaxf(s[r][0], s[r][1]), fmaxf(s[r][2], s[r][3]));
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) cm = fmaxf(cm, __shfl_xor_sync(0xffffffffu, cm, o));
+        for (int o = 8; o > 0; o >>= 1) cm = fmaxf(cm, __shfl_xor_sync(0xffffffffu, cm, o));
         const float new_max = fmaxf(run_max[r], cm);
         const float rescale = expf(run_max[r] - new_max);
         run_max[r] = new_max;
-        run_sum[r] *= rescale;
-#pragma unroll
-        for (int b = 0; b < 4; ++b) acc[r][b] *= rescale;
-        pv = live ? expf(pv - new_max) : 0.f;
+        sum[r] *= rescale;
+        t[r] *= rescale;
       }
-      float psum = pv;
 #pragma unroll
-      for (int o = 16; o > 0; o >>= 1) psum += __shfl_xor_sync(0xffffffffu, psum, o);
-      run_sum[r] += psum;
-      for (int ii = 0; ii < 32; ++ii) {
-        const float pi = __shfl_sync(0xffffffffu, pv, ii);
-#pragma unroll
-        for (int b = 0; b < 4; ++b) {
-          const int c = lane + 32 * b;
-          if (c < d) acc[r][b] = fmaf(pi, As[ii * (d + 1) + c], acc[r][b]);
-        }
+      for (int f = 0; f < 4; ++f) {
+        const float pv = kPerformer ? expf(s[r][f] - run_max[r]) : s[r][f];
+        sum[r] += pv;
+        t[r] = fmaf(pv, g[r][f], t[r]);
       }
     }
   }
-  // t_r = O_r . dO_r
-  float inv_sum[4], t[4], dq[4][4];
+  float inv_sum[R];
 #pragma unroll
-  for (int r = 0; r < 4; ++r) {
-    inv_sum[r] = 1.f / fmaxf(run_sum[r], 1.17549435e-38f);
-    float s = 0.f;
+  for (int r = 0; r < R; ++r) {
 #pragma unroll
-    for (int b = 0; b < 4; ++b) {
-      const int c = lane + 32 * b;
-      if (c < d) s = fmaf(acc[r][b] * inv_sum[r], Gs[(warp * 4 + r) * d + c], s);
-      dq[r][b] = 0.f;
+    for (int o = 8; o > 0; o >>= 1) {
+      sum[r] += __shfl_xor_sync(0xffffffffu, sum[r], o);
+      t[r] += __shfl_xor_sync(0xffffffffu, t[r], o);
     }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-    t[r] = s;
+    const bool row_live = n0 + ty + 16 * r < N;
+    inv_sum[r] = row_live ? 1.f / fmaxf(sum[r], 1.17549435e-38f) : 0.f;     // rows past the end weigh nothing
+    t[r] *= inv_sum[r];
   }
 
   // ---- sweep 2: c_ni, dq_n, da_i, e_i
-  for (int i0 = 0; i0 < p; i0 += 32) {
+  float dq[R][NB * 4];
+#pragma unroll
+  for (int r = 0; r < R; ++r)
+#pragma unroll
+    for (int c = 0; c < NB * 4; ++c) dq[r][c] = 0.f;
+  for (int i0 = 0; i0 < p; i0 += 64) {
     stage_chunk(i0);
-    const bool live = (i0 + lane) < p;
-    float e_part = 0.f;
-#pragma unroll
-    for (int r = 0; r < 4; ++r) {
-      const int row = warp * 4 + r;
-      const bool row_live = n0 + row < N;
-      float pv = logit(row, i0, live);
-      if (kPerformer) pv = live ? expf(pv - run_max[r]) : 0.f;
-      const float P = row_live ? pv * inv_sum[r] : 0.f;
-      float u = 0.f;
-      for (int c = 0; c < d; ++c) u = fmaf(As[lane * (d + 1) + c], Gs[row * d + c], u);
-      const float cv = P * (u - t[r]);
-      e_part -= P * t[r];
-      Ps[row * 33 + lane] = P;
-      if (kPerformer) {
-        for (int ii = 0; ii < 32; ++ii) {
-          const float ci = __shfl_sync(0xffffffffu, cv, ii);
-#pragma unroll
-          for (int b = 0; b < 4; ++b) {
-            const int c = lane + 32 * b;
-            if (c < d) dq[r][b] = fmaf(ci, Ws[ii * (d + 1) + c], dq[r][b]);
-          }
-        }
-      } else if (live && row_live) {
-        // feature i is column i of the row: d log(elu(x)+1)/dx = elu'(x)/(elu(x)+1)
-        const float x = qs[row][i0 + lane];
-        store_out(dQ + hv.base + (size_t)(n0 + row) * hv.row_stride + i0 + lane, cv * elu1_slope(x) / elu1(x));
-      }
-    }
-    es[warp][lane] = e_part;
-    __syncthreads();
-    // da_i[c] += sum over the tile's rows of P_ri dO_r[c]: warp w takes features 4w..4w+3 of the chunk
+    float s[R][4], g[R][4];
+    form(i0, s, g);
 #pragma unroll
     for (int f = 0; f < 4; ++f) {
-      const int ii = warp * 4 + f;
-      if (i0 + ii >= p) continue;
-      float s4[4] = {0.f, 0.f, 0.f, 0.f};
-      for (int r = 0; r < 32; ++r) {
-        const float pr = Ps[r * 33 + ii];
+      const int i = tx + 16 * f;
+      float e_part = 0.f;
 #pragma unroll
-        for (int b = 0; b < 4; ++b) {
-          const int c = lane + 32 * b;
-          if (c < d) s4[b] = fmaf(pr, Gs[r * d + c], s4[b]);
+      for (int r = 0; r < R; ++r) {
+        const int row = ty + 16 * r;
+        const float P = (kPerformer ? expf(s[r][f] - run_max[r]) : s[r][f]) * inv_sum[r];
+        const float cv = P * (g[r][f] - t[r]);
+        e_part = fmaf(-P, t[r], e_part);
+        Pt[i * kLdP + row] = P;
+        if (kPerformer) {
+          Cs[row * kLdC + i] = cv;
+        } else if (i0 + i < p && n0 + row < N) {
+          // feature i is column i of the row: d log(elu(x)+1)/dx = elu'(x)/(elu(x)+1)
+          const float x = Qs[row * ld + i0 + i];
+          store_out(dQ + hv.base + (size_t)(n0 + row) * hv.row_stride + i0 + i, cv * elu1_slope(x) / elu1(x));
         }
       }
+      e_part += __shfl_xor_sync(0xffffffffu, e_part, 16);
+      if (lane < 16) es[warp][i] = e_part;
+    }
+    __syncthreads();
+    if (kPerformer) simt_product<R, NB>(dq, Cs, kLdC, Ws, ld, 64);
+    float acc[4][NB * 4];
 #pragma unroll
-      for (int b = 0; b < 4; ++b) {
-        const int c = lane + 32 * b;
-        if (c < d) atomicAdd(da + ((size_t)bh * p + i0 + ii) * d + c, s4[b]);
+    for (int r = 0; r < 4; ++r)
+#pragma unroll
+      for (int c = 0; c < NB * 4; ++c) acc[r][c] = 0.f;
+    simt_product<4, NB>(acc, Pt, kLdP, Gs, ld, kRows);
+#pragma unroll
+    for (int r = 0; r < 4; ++r) {
+      const int i = i0 + ty + 16 * r;
+      if (i >= p) continue;
+#pragma unroll
+      for (int q = 0; q < NB; ++q) {
+        const int c = q * 64 + tx * 4;
+        float* at = da + ((size_t)bh * p + i) * d + c;
+        if (vec_d && c < d) {
+          atomicAdd(reinterpret_cast<float4*>(at), make_float4(acc[r][q * 4], acc[r][q * 4 + 1], acc[r][q * 4 + 2], acc[r][q * 4 + 3]));
+        } else {
+#pragma unroll
+          for (int x = 0; x < 4; ++x)
+            if (c + x < d) atomicAdd(at + x, acc[r][q * 4 + x]);
+        }
       }
     }
-    if (warp == 0 && live) {
-      float s = 0.f;
+    if (tid < 64 && i0 + tid < p) {
+      float e = 0.f;
 #pragma unroll
-      for (int w8 = 0; w8 < 8; ++w8) s += es[w8][lane];
-      atomicAdd(ei + (size_t)bh * p + i0 + lane, s);
+      for (int w8 = 0; w8 < 8; ++w8) e += es[w8][tid];
+      atomicAdd(ei + (size_t)bh * p + i0 + tid, e);
     }
   }
   if (kPerformer) {
 #pragma unroll
-    for (int r = 0; r < 4; ++r) {
-      const int n = n0 + warp * 4 + r;
+    for (int r = 0; r < R; ++r) {
+      const int n = n0 + ty + 16 * r;
       if (n >= N) continue;
 #pragma unroll
-      for (int b = 0; b < 4; ++b) {
-        const int c = lane + 32 * b;
-        if (c < d) store_out(dQ + hv.base + (size_t)n * hv.row_stride + c, dq[r][b]);
-      }
+      for (int q = 0; q < NB; ++q)
+#pragma unroll
+        for (int x = 0; x < 4; ++x) {
+          const int c = q * 64 + tx * 4 + x;
+          if (c < d) store_out(dQ + hv.base + (size_t)n * hv.row_stride + c, dq[r][q * 4 + x]);
+        }
     }
   }
 }

@@ -252,6 +252,9 @@ def test_backward_of_ragged_lengths_on_the_tensor_path(w, layout, per_head):
     (Workload("bwd_cc_big", RNN, "fp32", 2, 3, 1601, 20, 300, 0, 334), "bhnd", False),
     (Workload("bwd_cc_big_d100", RNN, "fp32", 1, 4, 1281, 100, 400, 0, 335), "bnhd", False),
     (Workload("bwd_cc_big_per_head", RNN, "bf16", 1, 6, 1604, 36, 129, 0, 336), "bhnd", True),
+    # query side: tiles of 64 rows, remainders of 64 features, one and two column blocks; a last tile of one row
+    (Workload("bwd_cc_query_big", PERFORMER, "fp32", 1, 8, 1217, 30, 20, 70, 337), "bhnd", False),
+    (Workload("bwd_cc_query_big_d97", PERFORMER, "fp32", 2, 6, 833, 97, 12, 129, 338), "bnhd", False),
 ], ids=lambda v: v.name if hasattr(v, "name") else str(v))
 def test_backward_products_with_inputs_on_cuda_cores(w, layout, per_head):
     _check(w, layout=layout, per_head=per_head)
