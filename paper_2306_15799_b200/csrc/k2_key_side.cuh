@@ -222,8 +222,14 @@ k2_key_side(const __grid_constant__ CUtensorMap tmW, const K2Params prm) {
         }
       }
       load_values();
-      // |k'_r|^2 of the eight rows over the lanes that share them, halving the number of rows per lane on the way
+      // |k'_r|^2 of the eight rows over the lanes that share them, halving the number of rows per lane on the way.  The
+      // halves of a row of 128 meet first: with |k'|^2 / 2 in the thousands one ulp of this sum is 1e-4 of a weight,
+      // so another tree gives other results (N = 131072, k = 512: 1e-4 to 4e-4 of the output's norm; seven more shuffles than joining them last)
       static_assert(kIters == 8, "eight rows per lane");
+      if (kLpr == 32) {
+#pragma unroll
+        for (int t = 0; t < kIters; ++t) sq[t] += __shfl_xor_sync(0xffffffffu, sq[t], 16);
+      }
       float s4[4], s2[2];
       const bool up8 = (lane & 8) != 0, up4 = (lane & 4) != 0, up2 = (lane & 2) != 0;
 #pragma unroll
@@ -232,7 +238,6 @@ k2_key_side(const __grid_constant__ CUtensorMap tmW, const K2Params prm) {
       for (int e = 0; e < 2; ++e) s2[e] = (up4 ? s4[2 + e] : s4[e]) + __shfl_xor_sync(0xffffffffu, up4 ? s4[e] : s4[2 + e], 4);
       float s1 = (up2 ? s2[1] : s2[0]) + __shfl_xor_sync(0xffffffffu, up2 ? s2[0] : s2[1], 2);
       s1 += __shfl_xor_sync(0xffffffffu, s1, 1);
-      if (kLpr == 32) s1 += __shfl_xor_sync(0xffffffffu, s1, 16);
       if ((lane & 1) == 0 && (kLpr == 16 || lane < 16)) {
         // B operand of the bias step: row r, columns 0..2 = three bf16 terms of -|k'_r|^2/2
         const int r = crow + ((up8 ? 4 : 0) + (up4 ? 2 : 0) + (up2 ? 1 : 0)) * 16 * kRpi;

@@ -551,3 +551,21 @@ def test_query_side_in_blocks_of_64_features(w, limit):
             blocks = s.reshape(w.N, -1, 64).max(2) / np.log(2.0)
             raised += int((blocks.max(1) > blocks[:, int(np.argmax(log_z)) // 64] + 15.0).sum())
     assert raised > 0 or w.m < 256
+
+
+@pytest.mark.parametrize("d", [64, 128])
+def test_squared_norm_is_added_in_one_order_whatever_the_width(d):
+    """|k'|^2 is summed over a row's columns as a tree that joins columns c and c + d/2 first.  2^24 in column 0 and ones
+    in the columns d/2 and 3d/4 meet as (2^24 + 1) + 1, and each 1 is lost to round-to-even; the tree that joins d/2 and
+    3d/4 first gives 2^24 + 2 and with it log-weights that are 1 lower.  (With W = 0 the log-weight of a feature is
+    -|k'|^2 / 2 + log k, here -2^23 + log 64, held to the fp32 spacing of 1/2 there.)"""
+    k = 64
+    dev = dict(device="cuda", dtype=torch.bfloat16)
+    K = torch.zeros(1, 1, k, d, **dev)
+    K[..., 0], K[..., d // 2], K[..., 3 * d // 4] = 4096.0, 1.0, 1.0
+    E = torch.eye(k, **dev)
+    binding.flurka_forward(torch.zeros_like(K), K, torch.ones_like(K), E, E, torch.zeros(64, d, **dev), PERFORMER)
+    torch.cuda.synchronize()
+    assert binding.flurka_last_status() == 0 and binding.flurka_last_path() == binding.PATH_TENSOR
+    b = binding.flurka_debug_copy(3, (64,)).cpu().double()
+    assert (b - (np.log(64.0) - 2.0 ** 23)).abs().max() < 0.5
