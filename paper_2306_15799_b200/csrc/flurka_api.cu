@@ -59,6 +59,10 @@ bool tensor_path_ok(const Problem& pr) {
   return true;
 }
 
+// Whether a path that the caller forces may take the problem: ragged lengths need a copy of E, F first, which only the
+// library's own choice of path makes.
+bool forced_tensor_ok(const Problem& pr) { return tensor_path_ok(pr) && pr.N % 8 == 0; }
+
 // Elements between the rows of E, F as the tensor-core kernels read them: N, or whole 128-byte lines above it
 // where N is ragged and the rows are copied.
 int ef_pitch(const Problem& pr) { return pr.N % 8 ? (pr.N + 63) & ~63 : pr.N; }
@@ -448,7 +452,7 @@ int forward_device(const void* Q, const void* K, const void* V, const void* E, c
   if (rc) return rc;
   int path = g_path;
   const bool tensor_ok = tensor_path_ok(pr);
-  if (path >= FLURKA_PATH_TENSOR && !tensor_ok) return FLURKA_ERR_SHAPE;
+  if (path >= FLURKA_PATH_TENSOR && !forced_tensor_ok(pr)) return FLURKA_ERR_SHAPE;
   if (path == FLURKA_PATH_AUTO) path = tensor_ok ? FLURKA_PATH_TENSOR : FLURKA_PATH_SIMT;
   rc = check_device();
   if (rc) return rc;
@@ -859,7 +863,7 @@ int flurka_forward_fused(const void* Xq, const void* Xk, const void* Xv, const v
     return FLURKA_ERR_OVERLAP;
   int path = g_path;
   const bool tensor_ok = fused_tensor_ok(pr, dm);
-  if (path >= FLURKA_PATH_TENSOR && !tensor_ok) return FLURKA_ERR_SHAPE;
+  if (path >= FLURKA_PATH_TENSOR && !(tensor_ok && forced_tensor_ok(pr))) return FLURKA_ERR_SHAPE;
   if (path == FLURKA_PATH_AUTO) path = tensor_ok ? FLURKA_PATH_TENSOR : FLURKA_PATH_SIMT;
   if (path != FLURKA_PATH_TENSOR && path != FLURKA_PATH_SIMT) return FLURKA_ERR_VARIANT;   // no bisecting paths here
   rc = check_device();
@@ -1111,7 +1115,7 @@ int flurka_backward(const void* Q, const void* K, const void* V, const void* E, 
   // tensor-core kernels for stage 1 and the query side where the shape allows (and the path knob does not
   // force the CUDA-core kernels); a forced tensor path with another shape is refused
   const bool tensor_ok = backward_tensor_ok(pr);
-  if (g_path >= FLURKA_PATH_TENSOR && !tensor_ok) return FLURKA_ERR_SHAPE;
+  if (g_path >= FLURKA_PATH_TENSOR && !(tensor_ok && forced_tensor_ok(pr))) return FLURKA_ERR_SHAPE;
   TensorContext* tc = (tensor_path_ok(pr) && g_path != FLURKA_PATH_SIMT) ? &ds.tc : nullptr;
   const bool tcq = tc && tensor_ok;
   if (pr.fp32)

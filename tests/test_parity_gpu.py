@@ -569,3 +569,32 @@ def test_squared_norm_is_added_in_one_order_whatever_the_width(d):
     assert binding.flurka_last_status() == 0 and binding.flurka_last_path() == binding.PATH_TENSOR
     b = binding.flurka_debug_copy(3, (64,)).cpu().double()
     assert (b - (np.log(64.0) - 2.0 ** 23)).abs().max() < 0.5
+
+
+def test_forced_tensor_paths_refuse_ragged_lengths():
+    """The rows of E, F start on 16-byte boundaries only where N is a multiple of 8: a path the caller forces makes no
+    copies of them.  Forward, fused and backward call; the library's own choice of path takes the same shapes."""
+    w = _wl("forced_ragged", PERFORMER, "bf16", 1, 2, 267, 64, 64, 64, 181)
+    x = pu.to_device(synth.make_inputs(w))
+    X = torch.zeros(1, w.N, 128, dtype=torch.bfloat16, device="cuda")
+    Wq = torch.zeros(128, 128, dtype=torch.bfloat16, device="cuda")
+    calls = [
+        lambda: binding.flurka_forward(x["Q"], x["K"], x["V"], x["E"], x["F"], x["W"], w.variant),
+        lambda: binding.flurka_forward_fused(X, X, X, x["E"], x["F"], Wq, Wq, Wq, x["W"], w.variant, w.H),
+        lambda: binding.flurka_backward(x["Q"], x["K"], x["V"], x["E"], x["F"], x["W"], x["Q"], w.variant),
+    ]
+    prev = binding.flurka_set_path(binding.PATH_TENSOR)
+    try:
+        for path in (binding.PATH_TENSOR, binding.PATH_TENSOR_STAGE1, binding.PATH_TENSOR_STAGE3, binding.PATH_TENSOR_STAGE23):
+            binding.flurka_set_path(path)
+            for call in calls:
+                with pytest.raises(binding.FlurkaError) as ei:
+                    call()
+                assert ei.value.code == -3
+        binding.flurka_set_path(binding.PATH_AUTO)
+        for call in calls:
+            call()
+            torch.cuda.synchronize()
+            assert binding.flurka_last_status() == 0
+    finally:
+        binding.flurka_set_path(prev)
