@@ -87,9 +87,10 @@ typedef enum {
  *
  * Shape limits: B, H, N >= 1, B*H <= 65535; 1 <= d <= 128; 1 <= k <= 4096; PERFORMER: m >= 1.
  * Pointers 16-byte aligned.  The tensor-core path additionally needs bf16, d in {64, 128},
- * N % 8 == 0 or N >= 256 (other N: E, F are copied once into rows on 16-byte boundaries, in the workspace;
- * FLURKA_PATH_AUTO only, a forced tensor-core path refuses them), k % 64 == 0 with k <= 512, and (PERFORMER)
- * m in {64, 128, 192, 256}; other shapes run on the SIMT path.  The call enqueues work and returns; it never
+ * N % 8 == 0, k % 64 == 0 with k <= 512, and (PERFORMER) m in {64, 128, 192, 256}; other shapes run on the
+ * SIMT path.  Under FLURKA_PATH_AUTO it also takes other N >= 256, with E, F copied once into rows on 16-byte
+ * boundaries (in the workspace) and with weights of 32-bit precision: all three stages for PERFORMER with
+ * d = 64, else stage 1 alone (FLURKA_PATH_TENSOR_STAGE1).  The call enqueues work and returns; it never
  * synchronises.  Scratch comes from the workspace set by flurka_set_workspace(), or from one the library obtains on first need and re-uses:
  * when a later problem needs more, the old block is released and a larger one obtained in stream order
  * on `stream` (cudaFreeAsync / cudaMallocAsync), so calls that share the library-owned workspace must

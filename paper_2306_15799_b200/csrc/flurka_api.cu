@@ -38,7 +38,8 @@ struct Problem {
 //   kpvp    fp32 [2][BH][k][d]     K' then V'
 //           (status and kpvp are adjacent: one range to clear per forward)
 //   weight  fp32 [BH][p]           b_i (PERFORMER) or z_i (RNN)
-//   a32     fp32 [BH][p][d]        key-side summary, feature-major
+//   a32     fp32 [BH][p][d]        key-side summary, feature-major (ragged lengths on tensor cores: two bf16 terms,
+//                                  [BH][2][p][d], in the same bytes)
 //   aT16    fp16 [BH][d][p]        the same, transposed, as the tensor-core B operand
 //   part    fp32 partial results of a key-split stage 2 (tensor-core path only)
 //   efpad   E, F with padded rows (tensor-core path, N no multiple of 8); last, the only part that depends on N
@@ -59,15 +60,33 @@ bool tensor_path_ok(const Problem& pr) {
   return true;
 }
 
+// Ragged lengths keep 32-bit weights: they came to the tensor cores from the CUDA-core kernels, whose weights, a and V' are
+// fp32, while the kernels of the other lengths round weights and a to fp16 (the backward: P, c to bf16).  Stage 1 gives
+// fp32 sums of exact products either way.  Stages 2 and 3 of PERFORMER with d = 64 have a form with two bf16 terms of
+// everything (fp32's range; error of the output against 64 bits as with fp32 weights, 1.649e-3 at B H = 8, N = 3001,
+// k = m = 256, all of it the output's own rounding, where fp16 weights give 1.667e-3); the rest runs on CUDA cores.
+bool ragged(const Problem& pr) { return pr.N % 8 != 0; }
+bool tensor_stages23_ok(const Problem& pr) {
+  return !ragged(pr) || (pr.kernel == FLURKA_PERFORMER && pr.d == 64);
+}
+// With stages 2 and 3 on CUDA cores, stage 1 on tensor cores (and the copy of E, F) pays from about 2^24 multiply-adds on.
+// us per call, stage 1 on tensor cores / on CUDA cores: 10.5 M (BH = 2, N = 643, k = 64, PERFORMER d = 128) 44.6 / 43.5, 12.6 M
+// (2, 385, 256, RNN d = 64) 37.5 / 36.2, 16.8 M (16, 257, 64, RNN d = 64) 21.5 / 25.2, 21 M (2, 643, 256, RNN d = 64) 37.8 / 42.6.
+int auto_path(const Problem& pr) {
+  if (!tensor_path_ok(pr)) return FLURKA_PATH_SIMT;
+  if (tensor_stages23_ok(pr)) return FLURKA_PATH_TENSOR;
+  return (double)pr.BH() * pr.N * pr.k * pr.d >= (double)(1 << 24) ? FLURKA_PATH_TENSOR_STAGE1 : FLURKA_PATH_SIMT;
+}
+
 // Whether a path that the caller forces may take the problem: ragged lengths need a copy of E, F first, which only the
 // library's own choice of path makes.
-bool forced_tensor_ok(const Problem& pr) { return tensor_path_ok(pr) && pr.N % 8 == 0; }
+bool forced_tensor_ok(const Problem& pr) { return tensor_path_ok(pr) && !ragged(pr); }
 
 // Elements between the rows of E, F as the tensor-core kernels read them: N, or whole 128-byte lines above it
 // where N is ragged and the rows are copied.
-int ef_pitch(const Problem& pr) { return pr.N % 8 ? (pr.N + 63) & ~63 : pr.N; }
+int ef_pitch(const Problem& pr) { return ragged(pr) ? (pr.N + 63) & ~63 : pr.N; }
 size_t efpad_bytes(const Problem& pr) {
-  return pr.N % 8 && tensor_path_ok(pr) ? (size_t)2 * pr.k * (pr.ef_per_head ? pr.H : 1) * ef_pitch(pr) * 2 : 0;
+  return ragged(pr) && tensor_path_ok(pr) ? (size_t)2 * pr.k * (pr.ef_per_head ? pr.H : 1) * ef_pitch(pr) * 2 : 0;
 }
 
 size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }
@@ -202,7 +221,7 @@ int check_device() {
 
 // Copies E, F into `pad` with padded rows where the tensor-core kernels need that, and points *E, *F there.
 int pad_projections(const Problem& pr, char* pad, const void** E, const void** F, cudaStream_t st, int* launches) {
-  if (pr.N % 8 == 0) return FLURKA_OK;
+  if (!ragged(pr)) return FLURKA_OK;
   const int rows = pr.k * (pr.ef_per_head ? pr.H : 1);
   char* Fp = pad + efpad_bytes(pr) / 2;
   int cuda_err = 0;
@@ -333,10 +352,12 @@ int run_pipeline_with(const Problem& pr, const Layout& L, char* ws, const void* 
     e = cudaGetLastError();
     return e == cudaSuccess ? FLURKA_OK : cuda_fail(e);
   }
+  // ragged lengths: a as two bf16 terms, which together are as large as the fp32 a they lie in place of
+  __nv_bfloat16* abf = tc2 && ragged(pr) ? (__nv_bfloat16*)a32 : nullptr;
   if (tc2) {
     float* part = L.total > L.part ? (float*)(ws + L.part) : nullptr;
-    rc = launch_k2(*tc, performer, kpvp, W, weight, aT16, part, status + 4, pr.BH(), pr.d, pr.k, pr.p(), status, st,
-                   &cuda_err);
+    rc = launch_k2(*tc, performer, kpvp, W, weight, abf ? nullptr : aT16, part, status + 4, pr.BH(), pr.d, pr.k, pr.p(), status,
+                   st, &cuda_err, nullptr, abf, abf != nullptr);
     if (rc) { g_last_cuda_error = cuda_err; return rc; }
     ++*launches;
   } else {
@@ -345,7 +366,7 @@ int run_pipeline_with(const Problem& pr, const Layout& L, char* ws, const void* 
   }
   if (timer) timer->mark(2, st);
   if (tc3) {
-    rc = launch_k3(*tc, performer, Q, W, aT16, weight, out, pr.BH(), pr.seq_major_heads(), pr.N, pr.d, pr.p(),
+    rc = launch_k3(*tc, performer, Q, W, aT16, abf, weight, out, pr.BH(), pr.seq_major_heads(), pr.N, pr.d, pr.p(),
                    status, st, &cuda_err);
     if (rc) { g_last_cuda_error = cuda_err; return rc; }
     ++*launches;
@@ -451,9 +472,8 @@ int forward_device(const void* Q, const void* K, const void* V, const void* E, c
   }
   if (rc) return rc;
   int path = g_path;
-  const bool tensor_ok = tensor_path_ok(pr);
   if (path >= FLURKA_PATH_TENSOR && !forced_tensor_ok(pr)) return FLURKA_ERR_SHAPE;
-  if (path == FLURKA_PATH_AUTO) path = tensor_ok ? FLURKA_PATH_TENSOR : FLURKA_PATH_SIMT;
+  if (path == FLURKA_PATH_AUTO) path = auto_path(pr);
   rc = check_device();
   if (rc) return rc;
   DeviceState& ds = dev_state();
@@ -827,7 +847,8 @@ int fused_pipeline(const Problem& pr, int dm, const FusedLayout& FL, char* ws, c
                           st, n))) return rc;
     return simt_map<T>(Xq, Wq, qp, false, sizeof(T) == 4, pr.B * pr.N, dm, pr.H * pr.d, 1, 0, 0, 0, 0, st, n);
   };
-  return run_pipeline_with<T>(pr, FL.L, ws, qp, W, out, st, tensor, tensor, tc, timer, /*keep_status=*/false, launches,
+  const bool tensor23 = tensor && tensor_stages23_ok(pr);
+  return run_pipeline_with<T>(pr, FL.L, ws, qp, W, out, st, tensor23, tensor23, tc, timer, /*keep_status=*/false, launches,
                               stage1, 3, tensor ? kt : nullptr, tensor ? FL.kt_bytes : 0);
 }
 
@@ -889,7 +910,7 @@ int flurka_forward_fused(const void* Xq, const void* Xk, const void* Xv, const v
   if (rc) return rc;
   ds.timer.have = g_stage_timing;
   ds.partial_pending = false;
-  ds.last_path = path;
+  ds.last_path = path == FLURKA_PATH_TENSOR && !tensor_stages23_ok(pr) ? FLURKA_PATH_TENSOR_STAGE1 : path;
   ds.last_launches = launches;
   ds.have_last = true;
   ds.last_problem = pr;

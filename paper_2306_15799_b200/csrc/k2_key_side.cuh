@@ -17,6 +17,9 @@
 // second product reads the weights from TMEM.  Several blocks: running maximum, accumulator in registers.  RNN: the
 // weights are the fp16 f tile as it lies ([key][feature], the MN-major A operand), and z_i comes from the same tile
 // times a column of ones.
+// kSplit (PERFORMER, d = 64) serves sequence lengths whose weights are kept in 32 bits: weights and V' are two bf16 terms each,
+// the low weights where L was read from, three products instead of two (low x low is 2^-18), and a leaves as the two bf16
+// terms that the query side reads.  bf16 has fp32's range, so V' may be as large as it may be on CUDA cores.
 // One block of 256 keys takes about 10 k cycles; the earlier form (eight warps, a staging copy and a block barrier per
 // 128 keys, one thread per row) took 17 us after stage 1's end at B H = 64, k = m = 256, d = 64, this one 9.
 //
@@ -88,10 +91,12 @@ __device__ __forceinline__ void k2_store_split(__nv_bfloat16* dst, size_t term, 
 }
 __device__ __forceinline__ uint32_t half2_bits(__half2 h) { return *reinterpret_cast<const uint32_t*>(&h); }
 
-template <bool kPerformer, int kD>
+// kSplit: weights and V' as two bf16 terms each, without the low x low product (see the header)
+template <bool kPerformer, int kD, bool kSplit = false>
 __global__ void __launch_bounds__(kK2Threads, 1)
 k2_key_side(const __grid_constant__ CUtensorMap tmW, const K2Params prm) {
   using namespace tc;
+  static_assert(!kSplit || kPerformer, "the RNN weights are one fp16 tile");
   constexpr int KB = kK2BlockElems / kD;                  // keys per block
   constexpr int kq = kD / 64;                             // 64-wide blocks of the head dimension
   constexpr uint32_t kSlab = KB * 128;                    // bytes of one 64-column slab of a term
@@ -282,16 +287,23 @@ k2_key_side(const __grid_constant__ CUtensorMap tmW, const K2Params prm) {
         st_shared_v2(base + kK2K3 + coff + r * 128 + ((cchunk ^ (r & 7)) << 4), half2_bits(h0), half2_bits(h1));
       }
     }
-    // ---- V' = hi + lo in fp16 (the MN-major B operand of the second product), under the first product's MMAs
+    // ---- V' = hi + lo in fp16 (kSplit: bf16) as the MN-major B operand of the second product, under the first product's MMAs
 #pragma unroll
     for (int t = 0; t < kIters; ++t) {
       const int r = crow + t * 16 * kRpi;
-      const __half2 hi0 = __floats2half2_rn(vx[t].x, vx[t].y), hi1 = __floats2half2_rn(vx[t].z, vx[t].w);
-      const float2 b0 = __half22float2(hi0), b1 = __half22float2(hi1);
       const uint32_t off = base + kK2V2 + coff + r * 128 + ((cchunk ^ (r & 7)) << 4);
-      st_shared_v2(off, half2_bits(hi0), half2_bits(hi1));
-      st_shared_v2(off + 32768, half2_bits(__floats2half2_rn(vx[t].x - b0.x, vx[t].y - b0.y)),
-                   half2_bits(__floats2half2_rn(vx[t].z - b1.x, vx[t].w - b1.y)));
+      if constexpr (kSplit) {
+        const uint32_t h0 = pack_bf16x2(vx[t].x, vx[t].y), h1 = pack_bf16x2(vx[t].z, vx[t].w);
+        st_shared_v2(off, h0, h1);
+        st_shared_v2(off + 32768, pack_bf16x2(vx[t].x - __uint_as_float(h0 << 16), vx[t].y - __uint_as_float(h0 & 0xffff0000u)),
+                     pack_bf16x2(vx[t].z - __uint_as_float(h1 << 16), vx[t].w - __uint_as_float(h1 & 0xffff0000u)));
+      } else {
+        const __half2 hi0 = __floats2half2_rn(vx[t].x, vx[t].y), hi1 = __floats2half2_rn(vx[t].z, vx[t].w);
+        const float2 b0 = __half22float2(hi0), b1 = __half22float2(hi1);
+        st_shared_v2(off, half2_bits(hi0), half2_bits(hi1));
+        st_shared_v2(off + 32768, half2_bits(__floats2half2_rn(vx[t].x - b0.x, vx[t].y - b0.y)),
+                     half2_bits(__floats2half2_rn(vx[t].z - b1.x, vx[t].w - b1.y)));
+      }
     }
     fence_proxy_async_smem();
 
@@ -327,13 +339,28 @@ k2_key_side(const __grid_constant__ CUtensorMap tmW, const K2Params prm) {
       if (have) {
         auto weigh = [&](const uint32_t (&r)[32], uint32_t col) {
           uint32_t h[16];
+          if constexpr (kSplit) {
+            uint32_t lo[16];
 #pragma unroll
-          for (int e = 0; e < 16; ++e) {
-            const __half2 hh = __floats2half2_rn(k2_ex2(fmaf(__uint_as_float(r[2 * e]), kLog2e, -shift)),
-                                                 k2_ex2(fmaf(__uint_as_float(r[2 * e + 1]), kLog2e, -shift)));
-            const float2 back = __half22float2(hh);
-            part += back.x + back.y;
-            h[e] = half2_bits(hh);
+            for (int e = 0; e < 16; ++e) {
+              // (the difference first: the rounding of max * log2 e would go into b_i)
+              const float w0 = k2_ex2((__uint_as_float(r[2 * e]) - new_max) * kLog2e);
+              const float w1 = k2_ex2((__uint_as_float(r[2 * e + 1]) - new_max) * kLog2e);
+              h[e] = pack_bf16x2(w0, w1);
+              const float h0 = __uint_as_float(h[e] << 16), h1 = __uint_as_float(h[e] & 0xffff0000u);
+              lo[e] = pack_bf16x2(w0 - h0, w1 - h1);
+              part += (h0 + __uint_as_float(lo[e] << 16)) + (h1 + __uint_as_float(lo[e] & 0xffff0000u));
+            }
+            tmem_st16(lane_base + KB / 2 + col, lo);          // (L has been read by everybody: there is room for both)
+          } else {
+#pragma unroll
+            for (int e = 0; e < 16; ++e) {
+              const __half2 hh = __floats2half2_rn(k2_ex2(fmaf(__uint_as_float(r[2 * e]), kLog2e, -shift)),
+                                                   k2_ex2(fmaf(__uint_as_float(r[2 * e + 1]), kLog2e, -shift)));
+              const float2 back = __half22float2(hh);
+              part += back.x + back.y;
+              h[e] = half2_bits(hh);
+            }
           }
           tmem_st16(lane_base + col, h);
         };
@@ -353,7 +380,11 @@ k2_key_side(const __grid_constant__ CUtensorMap tmW, const K2Params prm) {
         for (int s2 = 0; s2 < 2; ++s2) {
           const uint64_t bd = make_sdesc(base + kK2V2 + s2 * 32768 + q4 * 8192, kSlab, 1024, kSwizzle128);
           const uint32_t add = (q4 > 0 || s2 > 0) ? 1u : first;
-          if (kPerformer) {
+          if constexpr (kSplit) {
+            constexpr uint32_t idesc = make_idesc(kFmtBF16, 0, /*B MN-major*/ 1, 128, kD);
+            mma_ts_x4(tmem + kK2OCol, tmem + q4 * 32, bd, 128, idesc, add);
+            if (s2 == 0) mma_ts_x4(tmem + kK2OCol, tmem + KB / 2 + q4 * 32, bd, 128, idesc, 1u);
+          } else if (kPerformer) {
             mma_ts_x4(tmem + kK2OCol, tmem + q4 * 32, bd, 128, make_idesc(kFmtF16, 0, /*B MN-major*/ 1, 128, kD), add);
           } else {
             const uint64_t ad = make_sdesc(base + kK2K3 + q4 * 8192, kSlab, 1024, kSwizzle128);
@@ -402,7 +433,7 @@ k2_key_side(const __grid_constant__ CUtensorMap tmW, const K2Params prm) {
     // a^T leaves in whole 128- or 256-byte runs
     if (ok) {
       const float inv = 1.f / zsum;
-      if (qd == 0 && feat < p) prm.weight[(size_t)head * p + feat] = kPerformer ? run_max + __logf(zsum) : zsum;
+      if (qd == 0 && feat < p) prm.weight[(size_t)head * p + feat] = kPerformer ? run_max + (kSplit ? logf(zsum) : __logf(zsum)) : zsum;
       __half* tile = reinterpret_cast<__half*>(base_ptr + kK2K3) + (size_t)(qd * kColsPer) * 128 + frow;
 #pragma unroll
       for (int c = 0; c < kColsPer; ++c) {
@@ -466,7 +497,7 @@ k2_key_side(const __grid_constant__ CUtensorMap tmW, const K2Params prm) {
             acc[c] = fmaf(scale, __ldcg(all + q * part_stride + (size_t)(2 + qd * kColsPer + c) * 128 + frow), acc[c]);
         }
       }
-      if (qd == 0 && feat < p) prm.weight[(size_t)head * p + feat] = m_all + __logf(z_all);
+      if (qd == 0 && feat < p) prm.weight[(size_t)head * p + feat] = m_all + (kSplit ? logf(z_all) : __logf(z_all));
       const float inv = 1.f / z_all;
       __half* dst = prm.aT16 + ((size_t)head * kD + qd * kColsPer) * p + feat;
       if (feat < p) {

@@ -18,8 +18,14 @@
 // tensor (N = 64 costs 48 cycles per step with A in shared memory and 32 with A in TMEM: the reads of A bind), 1800
 // special-function; what is left is latency: a block's round trip through two chains of products is 1000 cycles.  Three groups
 // with S of the next block formed under the exponentials of this one came out the same (108 us).
+//
+// kSplit: lengths whose weights are kept in 32 bits (ragged N).  p as two bf16 terms, which fill S's 64 columns, times a as two
+// bf16 terms ([feature][column], as stage 2 leaves them for the backward as well): three products instead of one (low x low
+// is 2^-18).  a's second term takes the room of the output slabs, so every thread stores its own row.  2 x 8 heads x N = 6001,
+// k = m = 256: the call 60.3 us, 51.9 with fp16 weights, 281 with stages 2 and 3 on CUDA cores.
 #pragma once
 
+#include "k2_key_side.cuh"
 #include "k3_query_side.cuh"
 
 namespace flurka {
@@ -30,13 +36,14 @@ constexpr int kK3URegsFew = 32, kK3URegsMany = 104;     // 768 threads x 80 at l
 struct K3USmem {
   uint32_t w, aT, q, ostage, ones, bias, bars, total;
 };
-__host__ __device__ inline K3USmem k3u_smem_plan(int p) {
+__host__ __device__ inline K3USmem k3u_smem_plan(int p, bool split) {
   K3USmem s;
   uint32_t off = 0;
   s.w = off;      off += (uint32_t)p * 128;              // W: [p rows x 128 B]
   s.aT = off;     off += (uint32_t)p * 128;              // a^T: p/64 K-blocks of [64 rows x 128 B]
+  if (split) off += (uint32_t)p * 128;                   // (split: a, two terms of [p rows x 128 B] each)
   s.q = off;      off += 4 * 16384;                      // one Q tile per group
-  s.ostage = off; off += 16 * 4096;                      // a [32 x 64] bf16 output slab per row-owner warp
+  s.ostage = off; off += split ? 0 : 16 * 4096;          // a [32 x 64] bf16 output slab per row-owner warp
   s.ones = off;   off += 4096;                           // [128 x 16] bf16, no swizzle
   s.bias = off;   off += 8192;                           // [256 x 16] bf16, no swizzle
   s.bars = off;   off += 512;
@@ -44,6 +51,7 @@ __host__ __device__ inline K3USmem k3u_smem_plan(int p) {
   return s;
 }
 
+template <bool kSplit>
 __global__ void __launch_bounds__(kK3UThreads, 1)
 k3_query_units(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmW,
                const __grid_constant__ CUtensorMap tmAT, const __grid_constant__ CUtensorMap tmO,
@@ -53,7 +61,7 @@ k3_query_units(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
   const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u;
   uint8_t* base_ptr = smem_raw + (base - smem_u32(smem_raw));
   const int p = prm.p;
-  const K3USmem L = k3u_smem_plan(p);
+  const K3USmem L = k3u_smem_plan(p, kSplit);
   const int U = p >> 6;                       // blocks of 64 features
 
   const uint32_t bars = base + L.bars;
@@ -153,7 +161,8 @@ k3_query_units(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
         // ============================================================ MMA issuer of group g
         const int g = warp;
         const uint32_t ts = tmem + g * 128, to = ts + 64;
-        const uint32_t idescS = make_idesc(kFmtBF16, 0, 0, 128, 64), idescO = make_idesc(kFmtF16, 0, 0, 128, 64);
+        const uint32_t idescS = make_idesc(kFmtBF16, 0, 0, 128, 64);
+        const uint32_t idescO = kSplit ? make_idesc(kFmtBF16, 0, 1, 128, 64) : make_idesc(kFmtF16, 0, 0, 128, 64);
         const uint64_t qd = make_sdesc(base + L.q + g * 16384, 16, 1024, kSwizzle128);
         const uint64_t od = make_sdesc(base + L.ones, 128, 256, kSwizzleNone);
         bool ok = mbar_wait(bar_wfull, 0, prm.status, &abort_flag);
@@ -184,7 +193,16 @@ k3_query_units(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
               ok = mbar_wait(bar_pfull + 8 * g, n & 1u, prm.status, &abort_flag);
               if (!ok) break;
               tcgen05_fence_after();
-              mma_ts_x4(to, ts, make_sdesc(base + L.aT + block(u) * 8192, 16, 1024, kSwizzle128), 2, idescO, u > 0 ? 1u : 0u);
+              const uint32_t blk = base + L.aT + block(u) * 8192;
+              if constexpr (kSplit) {
+                // hi hi + lo hi + hi lo; a lies [feature][column]: an MN-major operand, 16 features = 2048 B per step
+                const uint64_t ah = make_sdesc(blk, 8192, 1024, kSwizzle128);
+                mma_ts_x4(to, ts, ah, 128, idescO, u > 0 ? 1u : 0u);
+                mma_ts_x4(to, ts + 32, ah, 128, idescO, 1u);
+                mma_ts_x4(to, ts, make_sdesc(blk + p * 128, 8192, 1024, kSwizzle128), 128, idescO, 1u);
+              } else {
+                mma_ts_x4(to, ts, make_sdesc(blk, 16, 1024, kSwizzle128), 2, idescO, u > 0 ? 1u : 0u);
+              }
               if (u + 1 < U) {
                 form_s(block(u + 1));
                 if (u + 2 == U) mma_commit(bar_qempty + 8 * g);
@@ -212,8 +230,15 @@ k3_query_units(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
           for (int g = 0; g < 4 && e > 0 && ok; ++g) ok = mbar_wait(bar_drained + 8 * g, (uint32_t)(e - 1) & 1u, prm.status, &abort_flag);
           if (!ok) break;
           if (lane == 0) {
-            mbar_arrive_expect_tx(bar_head, (uint32_t)p * 128);
-            for (int kb = 0; kb < U; ++kb) tma_load_3d(base + L.aT + kb * 8192, &tmAT, bar_head, kb * 64, 0, head);
+            mbar_arrive_expect_tx(bar_head, (uint32_t)p * (kSplit ? 256 : 128));
+            for (int kb = 0; kb < U; ++kb) {
+              if constexpr (kSplit) {
+                tma_load_3d(base + L.aT + kb * 8192, &tmAT, bar_head, 0, kb * 64, head * 2);
+                tma_load_3d(base + L.aT + p * 128 + kb * 8192, &tmAT, bar_head, 0, kb * 64, head * 2 + 1);
+              } else {
+                tma_load_3d(base + L.aT + kb * 8192, &tmAT, bar_head, kb * 64, 0, head);
+              }
+            }
           }
           const float* wv = prm.weight + (size_t)head * p;
           float mx = -INFINITY;
@@ -256,6 +281,18 @@ k3_query_units(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
       // 32 columns: x = 2^(S log2e - r) as fp16 pairs and the row sum.  One pair in eight takes its exponential as a
       // cubic on the FMA pipe, the others on the special-function unit (three in eight, the mix of k3_query_side, is 2.5 %
       // slower here, where issue slots are the scarcer: 110.3 against 107.2 us; none at all 112.7).
+      // kSplit: as two bf16 terms, all exponentials on the special-function unit (the cubic is good for fp16 only).
+      auto exp_split = [&](const uint32_t (&r)[32], uint32_t (&hi)[16], uint32_t (&lo)[16], uint64_t ms2, uint64_t& den2) {
+#pragma unroll
+        for (int e = 0; e < 16; ++e) {
+          float x0, x1;
+          unpack2(fma2(pack2u(r[2 * e], r[2 * e + 1]), l2, ms2), x0, x1);
+          const float e0 = ex2_approx(x0), e1 = ex2_approx(x1);
+          den2 = add2(den2, pack2(e0, e1));
+          hi[e] = pack_bf16x2(e0, e1);
+          lo[e] = pack_bf16x2(e0 - __uint_as_float(hi[e] << 16), e1 - __uint_as_float(hi[e] & 0xffff0000u));
+        }
+      };
       auto exp_block = [&](const uint32_t (&r)[32], uint32_t (&hh)[16], uint64_t ms2, uint64_t& den2) {
 #pragma unroll
         for (int e = 0; e < 16; ++e) {
@@ -319,10 +356,20 @@ k3_query_units(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
             }
           }
           const uint64_t ms2 = pack2(-r, -r);
-          exp_block(ra, hh, ms2, den2);
-          tmem_st16(ts, hh);
-          exp_block(rb, hh, ms2, den2);
-          tmem_st16(ts + 16, hh);
+          if constexpr (kSplit) {
+            uint32_t lo[16];
+            exp_split(ra, hh, lo, ms2, den2);
+            tmem_st16(ts, hh);
+            tmem_st16(ts + 32, lo);
+            exp_split(rb, hh, lo, ms2, den2);
+            tmem_st16(ts + 16, hh);
+            tmem_st16(ts + 48, lo);
+          } else {
+            exp_block(ra, hh, ms2, den2);
+            tmem_st16(ts, hh);
+            exp_block(rb, hh, ms2, den2);
+            tmem_st16(ts + 16, hh);
+          }
           tmem_wait_st();
           tcgen05_fence_before();
           __syncwarp();
@@ -336,8 +383,13 @@ k3_query_units(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
         ok = mbar_wait(bar_ofull + 8 * g, t & 1u, prm.status, &abort_flag);
         if (!ok) break;
         tcgen05_fence_after();
-        if (lane == 0) bulk_wait_group_read0();          // the slab's previous store has been read
+        if (!kSplit && lane == 0) bulk_wait_group_read0();   // the slab's previous store has been read
         __syncwarp();
+        const int row = tih * 128 + q4 * 32 + lane;
+        __nv_bfloat16* orow = nullptr;
+        if constexpr (kSplit)
+          orow = prm.out + (prm.H > 0 ? (((size_t)(head / prm.H) * prm.N + row) * prm.H + (size_t)(head % prm.H)) * 64
+                                      : ((size_t)head * prm.N + row) * 64);
 #pragma unroll
         for (int c = 0; c < 2; ++c) {
           uint32_t o[32];
@@ -351,14 +403,19 @@ k3_query_units(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
               const __nv_bfloat162 o2 = __floats2bfloat162_rn(__uint_as_float(o[e * 8 + 2 * x]) * inv, __uint_as_float(o[e * 8 + 2 * x + 1]) * inv);
               w[x] = *reinterpret_cast<const uint32_t*>(&o2);
             }
-            asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(slab + lane * 128 + (((4 * c + e) ^ (lane & 7)) << 4)),
-                         "r"(w[0]), "r"(w[1]), "r"(w[2]), "r"(w[3]) : "memory");
+            if constexpr (kSplit) {
+              // (the second term of a has the slabs' room: a thread stores its own row)
+              if (row < prm.N) reinterpret_cast<uint4*>(orow)[4 * c + e] = make_uint4(w[0], w[1], w[2], w[3]);
+            } else {
+              asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(slab + lane * 128 + (((4 * c + e) ^ (lane & 7)) << 4)),
+                           "r"(w[0]), "r"(w[1]), "r"(w[2]), "r"(w[3]) : "memory");
+            }
           }
         }
         tcgen05_fence_before();
-        fence_proxy_async_smem();
+        if (!kSplit) fence_proxy_async_smem();
         __syncwarp();
-        if (lane == 0 && tih * 128 + q4 * 32 < prm.N) {  // rows past the end are clipped by the tensor map
+        if (!kSplit && lane == 0 && tih * 128 + q4 * 32 < prm.N) {  // rows past the end are clipped by the tensor map
           if (prm.H > 0) tma_store_3d(&tmO, slab, (head % prm.H) * 64, tih * 128 + q4 * 32, head / prm.H);
           else tma_store_3d(&tmO, slab, 0, tih * 128 + q4 * 32, head);
           bulk_commit_group();
@@ -366,7 +423,7 @@ k3_query_units(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
         tih += 4;
         while (tih >= prm.tiles_per_head) { tih -= prm.tiles_per_head; ++head; }
       }
-      if (lane == 0) bulk_wait_group0();                // this warp's output stores are complete
+      if (!kSplit && lane == 0) bulk_wait_group0();     // this warp's output stores are complete
     }
   }
   tcgen05_fence_before();

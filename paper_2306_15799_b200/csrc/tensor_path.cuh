@@ -142,7 +142,7 @@ inline bool encode_map(CachedMap* cm, CUtensorMapDataType dt, int esize, int ran
 }
 
 struct TensorMaps {
-  CachedMap E, F, K, V, kpvp, Q, W, W2, aT, O;
+  CachedMap E, F, K, V, kpvp, Q, W, W2, aT, aS, O;
   CachedMap dO, abf;                            // backward of the query side
   CachedMap bE, bF, bK, bV, split64, split128, gK, gV, gE, gF;   // backward of the down-projection
   CachedMap A3, Wk, Wv, Xq, Wq, Qp, kpvp2;      // the linear maps of the entry point with un-projected inputs
@@ -401,9 +401,10 @@ inline size_t k2_part_floats(bool performer, int BH, int d, int k, int p) {
 }
 
 // ---- stage 2: per-feature summaries a (fp16, transposed) and weights b / z from K', V' --------
+// split: PERFORMER with d = 64, the weights inside as two bf16 terms (32-bit precision in the forward of ragged lengths)
 inline int launch_k2(TensorContext& tc, bool performer, const float* kpvp, const void* W, float* weight,
                      __half* aT16, float* part, int* counters, int BH, int d, int k, int p, int* status,
-                     cudaStream_t st, int* cuda_err, float* a32 = nullptr, __nv_bfloat16* abf = nullptr) {
+                     cudaStream_t st, int* cuda_err, float* a32 = nullptr, __nv_bfloat16* abf = nullptr, bool split = false) {
   TensorMaps& tm = tc.maps;
   if (performer) {
     const unsigned long long dW[2] = {(unsigned long long)d, (unsigned long long)p};
@@ -425,7 +426,8 @@ inline int launch_k2(TensorContext& tc, bool performer, const float* kpvp, const
   prm.nsplit = (part && counters) ? k2_nsplit(tc.sm_total(), performer, BH, d, k, p) : 1;
   prm.part = part;
   prm.counters = counters;
-  auto fn = d == 64 ? (performer ? k2_key_side<true, 64> : k2_key_side<false, 64>)
+  auto fn = split ? k2_key_side<true, 64, true>
+          : d == 64 ? (performer ? k2_key_side<true, 64> : k2_key_side<false, 64>)
                     : (performer ? k2_key_side<true, 128> : k2_key_side<false, 128>);
   cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, kK2SmemBytes);
   if (e != cudaSuccess) { *cuda_err = (int)e; (void)cudaGetLastError(); return -6; }
@@ -439,9 +441,10 @@ inline int launch_k2(TensorContext& tc, bool performer, const float* kpvp, const
 }
 
 // ---- stage 3: O from Q, W and the key-side summaries ------------------------------------------
+// abf != NULL (PERFORMER, d = 64): a as two bf16 terms, [BH][2][p][64], in place of aT16; weights as two terms too
 inline int launch_k3(TensorContext& tc, bool performer, const void* Q, const void* W, const __half* aT16,
-                     const float* weight, void* out, int BH, int H, int N, int d, int p, int* status, cudaStream_t st,
-                     int* cuda_err) {
+                     const __nv_bfloat16* abf, const float* weight, void* out, int BH, int H, int N, int d, int p,
+                     int* status, cudaStream_t st, int* cuda_err) {
   TensorMaps& tm = tc.maps;
   const unsigned long long dQ[3] = {(unsigned long long)(H > 0 ? H * d : d), (unsigned long long)N,
                                     (unsigned long long)(H > 0 ? BH / H : BH)};
@@ -453,8 +456,11 @@ inline int launch_k3(TensorContext& tc, bool performer, const void* Q, const voi
     *cuda_err = (int)cudaErrorInvalidValue;
     return -6;
   }
+  const unsigned long long dS[3] = {64ull, (unsigned long long)p, (unsigned long long)BH * 2};
+  const unsigned bS[3] = {64, 64, 1};
   if (!encode_map(&tm.Q, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, 3, Q, dQ, bQ) ||
-      !encode_map(&tm.aT, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 2, 3, aT16, dA, bA)) {
+      !(abf ? encode_map(&tm.aS, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, 3, abf, dS, bS)
+            : encode_map(&tm.aT, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 2, 3, aT16, dA, bA))) {
     *cuda_err = (int)cudaErrorInvalidValue;
     return -6;
   }
@@ -475,15 +481,15 @@ inline int launch_k3(TensorContext& tc, bool performer, const void* Q, const voi
   prm.status = status;
   // PERFORMER, d = 64: four tiles at a time (64 columns of S and 64 of O each fill TMEM; with d = 128 O alone would)
   const bool units = performer && d == 64;
-  const uint32_t smem = units ? k3u_smem_plan(p).total : k3_smem_plan(d, p, performer).total;
-  auto fn = units ? k3_query_units : (performer ? k3_query_side<true> : k3_query_side<false>);
+  const uint32_t smem = units ? k3u_smem_plan(p, abf != nullptr).total : k3_smem_plan(d, p, performer).total;
+  auto fn = units ? (abf ? k3_query_units<true> : k3_query_units<false>) : (performer ? k3_query_side<true> : k3_query_side<false>);
   cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) { *cuda_err = (int)e; (void)cudaGetLastError(); return -6; }
   int grid = tc.sm_count();
   if (grid > prm.total_tiles) grid = prm.total_tiles;
   // the RNN kernel ignores tmW and only d = 64 stores through tmO; pass any valid map otherwise
   e = launch_after_predecessor(fn, grid, units ? kK3UThreads : kK3Threads, smem, st, tm.Q.map, performer ? tm.W.map : tm.Q.map,
-                               tm.aT.map, d == 64 ? tm.O.map : tm.Q.map, prm);
+                               abf ? tm.aS.map : tm.aT.map, d == 64 ? tm.O.map : tm.Q.map, prm);
   if (e != cudaSuccess) { *cuda_err = (int)e; (void)cudaGetLastError(); return -6; }
   e = cudaGetLastError();
   if (e != cudaSuccess) { *cuda_err = (int)e; return -6; }
