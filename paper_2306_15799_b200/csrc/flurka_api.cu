@@ -72,10 +72,11 @@ bool tensor_stages23_ok(const Problem& pr) {
 // With stages 2 and 3 on CUDA cores, stage 1 on tensor cores (and the copy of E, F) pays from about 2^24 multiply-adds on.
 // us per call, stage 1 on tensor cores / on CUDA cores: 10.5 M (BH = 2, N = 643, k = 64, PERFORMER d = 128) 44.6 / 43.5, 12.6 M
 // (2, 385, 256, RNN d = 64) 37.5 / 36.2, 16.8 M (16, 257, 64, RNN d = 64) 21.5 / 25.2, 21 M (2, 643, 256, RNN d = 64) 37.8 / 42.6.
+double projection_fmas(const Problem& pr) { return (double)pr.BH() * pr.N * pr.k * pr.d; }
 int auto_path(const Problem& pr) {
   if (!tensor_path_ok(pr)) return FLURKA_PATH_SIMT;
   if (tensor_stages23_ok(pr)) return FLURKA_PATH_TENSOR;
-  return (double)pr.BH() * pr.N * pr.k * pr.d >= (double)(1 << 24) ? FLURKA_PATH_TENSOR_STAGE1 : FLURKA_PATH_SIMT;
+  return projection_fmas(pr) >= (double)(1 << 24) ? FLURKA_PATH_TENSOR_STAGE1 : FLURKA_PATH_SIMT;
 }
 
 // Whether a path that the caller forces may take the problem: ragged lengths need a copy of E, F first, which only the
@@ -931,10 +932,16 @@ struct BackwardLayout {
 
 // the query side of the backward has a tensor-core kernel for d = 64 (PERFORMER: any feature count the
 // forward's tensor path takes, 64 to 256; RNN: its 64 features are the head dimension) and for PERFORMER
-// with d = 128
+// with d = 128.  P and c are bf16 there: not for ragged lengths
 bool backward_tensor_ok(const Problem& pr) {
-  return tensor_path_ok(pr) && (pr.d == 64 || pr.kernel == FLURKA_PERFORMER);
+  return tensor_path_ok(pr) && !ragged(pr) && (pr.d == 64 || pr.kernel == FLURKA_PERFORMER);
 }
+
+// Whether a ragged backward pass takes the tensor-core kernels for its products with E, F, K, V (and the copies of E, F and of
+// dE, dF): from about 2^22 multiply-adds per product on.  us per call, tensor cores / CUDA cores: 2.6 M (one head, N = 643,
+// k = 64, PERFORMER d = 64) 76 / 72, 5.3 M (two heads) 76 / 76, 4.2 M (one head, N = 257, k = 256) 97 / 105, RNN 66 / 74,
+// 10.5 M (two heads, N = 1283, k = 64) 76 / 82, RNN 49 / 53; 16 heads, N = 257, k = 64: 84 / 123.
+bool ragged_backward_pays(const Problem& pr) { return projection_fmas(pr) >= (double)(1 << 22); }
 
 BackwardLayout make_backward_layout(const Problem& pr) {
   BackwardLayout b;
@@ -991,8 +998,9 @@ template <typename T, bool P>
 int backward_pipeline(const Problem& pr, const BackwardLayout& BL, char* ws, const void* Q, const void* K,
                       const void* V, const void* E, const void* F, const void* W, const void* dO, void* dQ, void* dK,
                       void* dV, void* dE, void* dF, cudaStream_t st, int* launches, TensorContext* tc, bool tcq) {
-  // tc != NULL: stage 1 and (with shared E, F) the projection gradients run on the tensor-core kernels;
-  // tcq: so does the query side (bf16 PERFORMER, d = 64, 128 or 256 features)
+  // tc != NULL: stage 1 and the gradients that are products with E, F, K, V run on the tensor-core kernels (exact
+  // products of bf16 inputs, fp32 sums; dK', dV' as two bf16 terms), and but for ragged lengths the key side's forward
+  // half does; tcq: so do the query side and, PERFORMER with d = 64, the key side's backward half
   const Layout& L = BL.L;
   float* kpvp = (float*)(ws + L.kpvp);
   float* weight = (float*)(ws + L.weight);
@@ -1018,7 +1026,7 @@ int backward_pipeline(const Problem& pr, const BackwardLayout& BL, char* ws, con
     rc = launch_simt_down_project<T>(pr, K, V, E, F, kpvp, st, launches);
     if (rc) return rc;
   }
-  if (tc) {
+  if (tc && !ragged(pr)) {
     // the key side on its tensor-core kernel, one CTA per (head, feature tile), with a in fp32 as well
     rc = launch_k2(*tc, P, kpvp, W, weight, nullptr, nullptr, nullptr, pr.BH(), pr.d, pr.k, pr.p(),
                    (int*)(ws + L.status), st, &cuda_err, tcq ? nullptr : a32, tcq ? (__nv_bfloat16*)(ws + BL.abf) : nullptr);
@@ -1028,7 +1036,7 @@ int backward_pipeline(const Problem& pr, const BackwardLayout& BL, char* ws, con
     rc = launch_simt_key_side<T, P>(pr, kpvp, W, weight, a32, nullptr, st, launches);
     if (rc) return rc;
   }
-  if (tc && tcq) {
+  if (tcq) {
     const __nv_bfloat16* abf = (const __nv_bfloat16*)(ws + BL.abf);
     rc = launch_bwd_query(*tc, P, Q, dO, W, weight, abf, dQ, da, ei, pr.BH(), smh, pr.N, pr.d, pr.p(),
                           (int*)(ws + L.status), st, &cuda_err);
@@ -1048,7 +1056,7 @@ int backward_pipeline(const Problem& pr, const BackwardLayout& BL, char* ws, con
     ++*launches;
   }
   __nv_bfloat16* split = tc ? (__nv_bfloat16*)(ws + BL.split) : nullptr;
-  if (tc && P && pr.d == 64) {
+  if (tcq && P && pr.d == 64) {
     rc = launch_k6(*tc, W, kpvp, weight, da, ei, split, pr.BH(), pr.k, pr.p(), (int*)(ws + L.status), st, &cuda_err);
     if (rc) { g_last_cuda_error = cuda_err; return rc; }
     ++*launches;
@@ -1137,7 +1145,8 @@ int flurka_backward(const void* Q, const void* K, const void* V, const void* E, 
   // force the CUDA-core kernels); a forced tensor path with another shape is refused
   const bool tensor_ok = backward_tensor_ok(pr);
   if (g_path >= FLURKA_PATH_TENSOR && !(tensor_ok && forced_tensor_ok(pr))) return FLURKA_ERR_SHAPE;
-  TensorContext* tc = (tensor_path_ok(pr) && g_path != FLURKA_PATH_SIMT) ? &ds.tc : nullptr;
+  const bool use_tc = tensor_path_ok(pr) && g_path != FLURKA_PATH_SIMT && (!ragged(pr) || ragged_backward_pays(pr));
+  TensorContext* tc = use_tc ? &ds.tc : nullptr;
   const bool tcq = tc && tensor_ok;
   if (pr.fp32)
     rc = perf ? backward_pipeline<float, true>(pr, BL, ws, Q, K, V, E, F, W, dO, dQ, dK, dV, dE, dF, st, &launches, nullptr, false)

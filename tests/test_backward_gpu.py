@@ -42,8 +42,10 @@ def _oracle_grads(w, x, dO, per_head):
     return g
 
 
-def _check(w, layout="bhnd", per_head=False):
+def _check(w, layout="bhnd", per_head=False, tol=None, v_scale=1.0):
+    """The relative Frobenius error of each gradient, and the share of its elements that are not the oracle's rounded."""
     x = synth.make_inputs(w)
+    x["V"] = (x["V"].double() * v_scale).to(x["V"].dtype)
     gen = torch.Generator().manual_seed(w.seed + 5)
     if per_head:
         for name in ("E", "F"):
@@ -56,12 +58,15 @@ def _check(w, layout="bhnd", per_head=False):
     torch.cuda.synchronize()
     assert binding.flurka_last_status() == 0
     ref = _oracle_grads(w, x, dO, per_head)
+    moved = {}
     for name, tensor in zip(("dQ", "dK", "dV", "dE", "dF"), got):
         arr = tensor.transpose(1, 2) if (layout == "bnhd" and tensor.dim() == 4) else tensor
+        moved[name] = float((arr.cpu() != torch.from_numpy(ref[name]).to(arr.dtype)).double().mean())
         arr = arr.cpu().double().numpy()
         assert np.isfinite(arr).all(), name
         rel = np.linalg.norm(arr - ref[name]) / max(np.linalg.norm(ref[name]), 1e-300)
-        assert rel <= TOL[w.io], "%s %s: rel-Fro %.3e > %.0e" % (w.name, name, rel, TOL[w.io])
+        assert rel <= (tol or TOL[w.io]), "%s %s: rel-Fro %.3e > %.1e" % (w.name, name, rel, tol or TOL[w.io])
+    return moved
 
 
 CASES = [
@@ -237,9 +242,11 @@ def test_backward_argument_errors():
     (Workload("bwd_odd_per_head", PERFORMER, "bf16", 2, 2, 301, 64, 64, 128, 355), "bhnd", True),
 ], ids=lambda v: v.name if hasattr(v, "name") else str(v))
 def test_backward_of_ragged_lengths_on_the_tensor_path(w, layout, per_head):
-    """N no multiple of 8: E, F are read from padded copies, dE, dF leave through them."""
+    """N no multiple of 8: E, F are read from padded copies, dE, dF leave through them.  (The key and query side, whose
+    tensor-core kernels round weights to 16 bits, run on CUDA cores.)"""
     _check(w, layout=layout, per_head=per_head)
-    assert binding.flurka_last_path() == binding.PATH_TENSOR
+    products = w.B * w.H * w.N * w.k * w.d >= 1 << 22
+    assert binding.flurka_last_path() == (binding.PATH_TENSOR_STAGE1 if products else binding.PATH_SIMT)
 
 
 @pytest.mark.parametrize("w,layout,per_head", [
@@ -259,3 +266,21 @@ def test_backward_of_ragged_lengths_on_the_tensor_path(w, layout, per_head):
 def test_backward_products_with_inputs_on_cuda_cores(w, layout, per_head):
     _check(w, layout=layout, per_head=per_head)
     assert binding.flurka_last_path() == binding.PATH_SIMT
+
+
+@pytest.mark.parametrize("v_scale", [1.0, 2.0 ** 20])
+@pytest.mark.parametrize("w,layout,per_head", [
+    (Workload("bwd_exact_k256", PERFORMER, "bf16", 2, 2, 643, 64, 256, 256, 361), "bhnd", False),
+    (Workload("bwd_exact_d128", PERFORMER, "bf16", 1, 2, 390, 128, 128, 128, 362), "bnhd", False),
+    (Workload("bwd_exact_rnn", RNN, "bf16", 1, 3, 1001, 64, 192, 0, 363), "bhnd", False),
+    (Workload("bwd_exact_rnn_d128", RNN, "bf16", 1, 2, 771, 128, 192, 0, 364), "bnhd", False),
+    (Workload("bwd_exact_per_head", PERFORMER, "bf16", 2, 2, 301, 64, 64, 128, 365), "bhnd", True),
+], ids=lambda v: v.name if hasattr(v, "name") else str(v))
+def test_gradients_of_ragged_lengths_keep_32_bit_weights(w, layout, per_head, v_scale):
+    """Rounding to bf16 costs an element at most 2^-9 of itself: gradients that are the rounding of fp32 results are within
+    2^-9 of the oracle's in norm.  (With P, c and the key side's weights in bf16 dK, dE were 2.2e-3 to 2.9e-3 off, with fp16
+    weights the RNN's dQ 1.7e-3.)  Elements moved: an error of 2^-16 crosses a rounding boundary with a probability of at most
+    2^-8, twice that for elements below the rms; dK, dE add a cancelling difference (g - delta), again twice (measured: at
+    most 0.4 %, the RNN's dQ with fp16 weights 19 %)."""
+    moved = _check(w, layout=layout, per_head=per_head, tol=2.0 ** -9, v_scale=v_scale)
+    assert max(moved.values()) <= 2.0 ** -6, moved
