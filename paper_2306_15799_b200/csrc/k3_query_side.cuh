@@ -33,6 +33,7 @@ struct K3Params {
   int total_tiles;
   const float* weight;      // [BH][p]  b_i or z_i
   __nv_bfloat16* out;       // [BH][N][d]
+  int wide;                 // out is 32-byte aligned
   int* status;
 };
 
@@ -411,10 +412,15 @@ k3_query_side(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ C
                                                               __uint_as_float(src[(g8 & 1) * 16 + 2 * e + 1]) * inv);
               v[e] = *reinterpret_cast<const uint32_t*>(&o2);
             }
-            if (in_range)
-            asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(orow + c + g8 * 16),
-                         "r"(v[0]), "r"(v[1]), "r"(v[2]), "r"(v[3]), "r"(v[4]), "r"(v[5]), "r"(v[6]), "r"(v[7])
-                         : "memory");
+            // out is 16-byte aligned, or 32 as well; every offset into it is a multiple of 32 bytes
+            __nv_bfloat16* o = orow + c + g8 * 16;
+            if (in_range && prm.wide) {
+              asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(o), "r"(v[0]), "r"(v[1]),
+                           "r"(v[2]), "r"(v[3]), "r"(v[4]), "r"(v[5]), "r"(v[6]), "r"(v[7]) : "memory");
+            } else if (in_range) {
+              reinterpret_cast<uint4*>(o)[0] = make_uint4(v[0], v[1], v[2], v[3]);
+              reinterpret_cast<uint4*>(o)[1] = make_uint4(v[4], v[5], v[6], v[7]);
+            }
           }
         }
         return true;

@@ -32,6 +32,7 @@ struct K7Params {
   int tiles_per_head, total_tiles;
   const float* weight;          // [BH][p]     b_i (RNN: z_i)
   __nv_bfloat16* dQ;
+  int wide;                     // dQ is 32-byte aligned
   float* da;                    // [BH][p][d]  added to
   float* ei;                    // [BH][p]     e_i, added to
   int* status;
@@ -51,10 +52,15 @@ __device__ __forceinline__ float k4_ex2(float x) {
   asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
   return y;
 }
-// 16 bf16 values, 32-byte aligned
-__device__ __forceinline__ void k4_store16(__nv_bfloat16* o, const uint32_t (&v)[8]) {
-  asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(o), "r"(v[0]), "r"(v[1]), "r"(v[2]),
-               "r"(v[3]), "r"(v[4]), "r"(v[5]), "r"(v[6]), "r"(v[7]) : "memory");
+// 16 bf16 values; `wide`: 32-byte aligned (the caller's buffers are 16-byte aligned, every offset into them is a multiple of 32)
+__device__ __forceinline__ void k4_store16(__nv_bfloat16* o, const uint32_t (&v)[8], bool wide) {
+  if (wide) {
+    asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(o), "r"(v[0]), "r"(v[1]), "r"(v[2]),
+                 "r"(v[3]), "r"(v[4]), "r"(v[5]), "r"(v[6]), "r"(v[7]) : "memory");
+  } else {
+    reinterpret_cast<uint4*>(o)[0] = make_uint4(v[0], v[1], v[2], v[3]);
+    reinterpret_cast<uint4*>(o)[1] = make_uint4(v[4], v[5], v[6], v[7]);
+  }
 }
 
 // shared memory
@@ -318,6 +324,7 @@ k4_bwd_query_wide(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
         }
         esum0 = esum1 = 0.f;
       };
+      const bool wide = prm.wide != 0;
       auto store32 = [&](__nv_bfloat16* o, const uint32_t (&r)[32]) {
 #pragma unroll
         for (int g = 0; g < 2; ++g) {
@@ -325,7 +332,7 @@ k4_bwd_query_wide(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
 #pragma unroll
           for (int e = 0; e < 8; ++e)
             v[e] = k4_bf16x2(__uint_as_float(r[16 * g + 2 * e]), __uint_as_float(r[16 * g + 2 * e + 1]));
-          k4_store16(o + 16 * g, v);
+          k4_store16(o + 16 * g, v, wide);
         }
       };
 

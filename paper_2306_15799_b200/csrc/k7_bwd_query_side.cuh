@@ -346,7 +346,7 @@ k7_bwd_query_side(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
 #pragma unroll
               for (int e = 0; e < 8; ++e)
                 v[e] = k4_bf16x2(__uint_as_float(own[16 * g + 2 * e]), __uint_as_float(own[16 * g + 2 * e + 1]));
-              k4_store16(o + 16 * g, v);
+              k4_store16(o + 16 * g, v, prm.wide != 0);
             }
           }
         }
@@ -543,8 +543,8 @@ k7_bwd_query_side(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
           if constexpr (!kPerformer) {
             if (row0 + row < prm.N) {
               __nv_bfloat16* o = dq_row(head, row0) + fh * 32;
-              k4_store16(o, *reinterpret_cast<const uint32_t (*)[8]>(&dqv[0]));
-              k4_store16(o + 16, *reinterpret_cast<const uint32_t (*)[8]>(&dqv[8]));
+              k4_store16(o, *reinterpret_cast<const uint32_t (*)[8]>(&dqv[0]), prm.wide != 0);
+              k4_store16(o + 16, *reinterpret_cast<const uint32_t (*)[8]>(&dqv[8]), prm.wide != 0);
             }
           }
         }

@@ -478,6 +478,7 @@ inline int launch_k3(TensorContext& tc, bool performer, const void* Q, const voi
   prm.total_tiles = prm.tiles_per_head * BH;
   prm.weight = weight;
   prm.out = reinterpret_cast<__nv_bfloat16*>(out);
+  prm.wide = ((uintptr_t)out & 31) == 0;
   prm.status = status;
   // PERFORMER, d = 64: four tiles at a time (64 columns of S and 64 of O each fill TMEM; with d = 128 O alone would)
   const bool units = performer && d == 64;
@@ -520,6 +521,7 @@ inline int launch_bwd_query(TensorContext& tc, bool performer, const void* Q, co
   prm.total_tiles = prm.tiles_per_head * BH;
   prm.weight = weight;
   prm.dQ = reinterpret_cast<__nv_bfloat16*>(dQ);
+  prm.wide = ((uintptr_t)dQ & 31) == 0;
   prm.da = da; prm.ei = ei; prm.status = status;
   const int parts = (p + 127) / 128;                      // 1 or 2 CTAs share a tile
   auto fn = d == 128 ? (parts == 2 ? k4_bwd_query_wide<2> : k4_bwd_query_wide<1>)

@@ -284,3 +284,42 @@ def test_gradients_of_ragged_lengths_keep_32_bit_weights(w, layout, per_head, v_
     most 0.4 %, the RNN's dQ with fp16 weights 19 %)."""
     moved = _check(w, layout=layout, per_head=per_head, tol=2.0 ** -9, v_scale=v_scale)
     assert max(moved.values()) <= 2.0 ** -6, moved
+
+
+def _at_16_mod_32(t):
+    """A copy of t that starts 16 bytes past a 32-byte boundary, the least alignment the library asks for."""
+    skip = 16 // t.element_size()
+    u = torch.empty(t.numel() + skip, dtype=t.dtype, device="cuda")[skip:].view(t.shape)
+    assert u.data_ptr() % 32 == 16
+    return u.copy_(t)
+
+
+@pytest.mark.parametrize("w,layout", [
+    # every kernel that stores dQ or out row by row: one and two CTAs per tile (64, 256 features), RNN, d = 128
+    (Workload("off16_m256", PERFORMER, "bf16", 1, 2, 392, 64, 64, 256, 371), "bhnd"),
+    (Workload("off16_m64", PERFORMER, "bf16", 2, 2, 136, 64, 64, 64, 372), "bnhd"),
+    (Workload("off16_rnn", RNN, "bf16", 1, 3, 264, 64, 64, 0, 373), "bnhd"),
+    (Workload("off16_d128_m64", PERFORMER, "bf16", 1, 2, 200, 128, 64, 64, 374), "bhnd"),
+    (Workload("off16_d128_m256", PERFORMER, "bf16", 2, 2, 392, 128, 64, 256, 375), "bnhd"),
+    (Workload("off16_rnn_d128", RNN, "bf16", 1, 2, 200, 128, 64, 0, 376), "bhnd"),
+    (Workload("off16_ragged", PERFORMER, "bf16", 1, 2, 301, 64, 64, 128, 377), "bhnd"),
+    (Workload("off16_fp32", PERFORMER, "fp32", 1, 2, 100, 64, 33, 40, 378), "bhnd"),
+], ids=lambda v: v.name if hasattr(v, "name") else str(v))
+def test_buffers_that_are_16_byte_aligned_only(w, layout):
+    """Forward and backward with every input and output 16 bytes past a 32-byte boundary give what aligned buffers give."""
+    x = synth.make_inputs(w)
+    gen = torch.Generator().manual_seed(w.seed)
+    dO = torch.randn(w.B, w.H, w.N, w.d, generator=gen, dtype=torch.float64).to(x["Q"].dtype)
+    t = (lambda a: a.transpose(1, 2).contiguous()) if layout == "bnhd" else (lambda a: a)
+    ins = [t(x[n].cuda()) for n in ("Q", "K", "V")] + [x["E"].cuda(), x["F"].cuda(), x["W"].cuda() if x["W"] is not None else None]
+    off = [_at_16_mod_32(a) if a is not None else None for a in ins]
+    want = [binding.flurka_forward(*ins, w.variant, layout=layout), *binding.flurka_backward(*ins, t(dO.cuda()), w.variant, layout=layout)]
+    out, *grads = [_at_16_mod_32(torch.full_like(a, 7.0)) for a in want]
+    got = [binding.flurka_forward(*off, w.variant, out=out, layout=layout),
+           *binding.flurka_backward(*off, _at_16_mod_32(t(dO.cuda())), w.variant, layout=layout, out=grads)]
+    torch.cuda.synchronize()
+    assert binding.flurka_last_status() == 0
+    for name, a, b in zip(("out", "dQ", "dK", "dV", "dE", "dF"), got, want):
+        # partial sums meet in any order: the two may differ by that, not by a row or a piece of one
+        rel = float((a.double() - b.double()).norm() / b.double().norm())
+        assert rel <= 2e-3, "%s %s: %.3e" % (w.name, name, rel)
