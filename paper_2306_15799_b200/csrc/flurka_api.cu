@@ -270,7 +270,7 @@ int launch_simt_down_project(const Problem& pr, const void* K, const void* V, co
 
 template <typename T, bool P, bool kKeySide, int R, int NB>
 int launch_simt_attend_as(const Problem& pr, const void* Q, const void* W, const float* kpvp, float* weight, float* a32,
-                          __half* aT16, void* out, cudaStream_t st) {
+                          __half* aT16, void* out, cudaStream_t st, bool chained) {
   const size_t smem = simt_attend_smem(R, NB, pr.d);
   auto fn = simt_attend<T, P, kKeySide, R, NB>;
   if (smem > 48 * 1024) {
@@ -278,43 +278,45 @@ int launch_simt_attend_as(const Problem& pr, const void* Q, const void* W, const
     if (e != cudaSuccess) return cuda_fail(e);
   }
   dim3 grid(((kKeySide ? pr.p() : pr.N) + 16 * R - 1) / (16 * R), pr.BH());
-  cudaError_t e = launch_after_predecessor(fn, grid, kSimtThreads, smem, st, (const T*)Q, (const T*)W, kpvp, weight, a32,
-                                           aT16, (T*)out, pr.BH(), pr.N, pr.d, pr.k, pr.p(), pr.seq_major_heads());
+  cudaError_t e = launch_chained(chained, fn, grid, kSimtThreads, smem, st, (const T*)Q, (const T*)W, kpvp, weight, a32,
+                                 aT16, (T*)out, pr.BH(), pr.N, pr.d, pr.k, pr.p(), pr.seq_major_heads());
   if (e != cudaSuccess) return cuda_fail(e);
   return FLURKA_OK;
 }
 
+// chained: everything that the kernel and the query side after it read before they wait (their rows: W, and Q) was complete
+// when the call's chain of launches began.  Otherwise it is launched ordinarily and starts when all before it is complete.
 template <typename T, bool P, bool kKeySide>
 int launch_simt_attend(const Problem& pr, const void* Q, const void* W, const float* kpvp, float* weight, float* a32,
-                       __half* aT16, void* out, cudaStream_t st, int* launches) {
+                       __half* aT16, void* out, cudaStream_t st, int* launches, bool chained) {
   // 128 rows per block as soon as that gives every SM a block; 32 below, where the length of one block is the time
   const bool big = (long long)(((kKeySide ? pr.p() : pr.N) + 127) / 128) * pr.BH() >= 148;
   ++*launches;
   if (pr.d > 64)
-    return big ? launch_simt_attend_as<T, P, kKeySide, 8, 2>(pr, Q, W, kpvp, weight, a32, aT16, out, st)
-               : launch_simt_attend_as<T, P, kKeySide, 2, 2>(pr, Q, W, kpvp, weight, a32, aT16, out, st);
-  return big ? launch_simt_attend_as<T, P, kKeySide, 8, 1>(pr, Q, W, kpvp, weight, a32, aT16, out, st)
-             : launch_simt_attend_as<T, P, kKeySide, 2, 1>(pr, Q, W, kpvp, weight, a32, aT16, out, st);
+    return big ? launch_simt_attend_as<T, P, kKeySide, 8, 2>(pr, Q, W, kpvp, weight, a32, aT16, out, st, chained)
+               : launch_simt_attend_as<T, P, kKeySide, 2, 2>(pr, Q, W, kpvp, weight, a32, aT16, out, st, chained);
+  return big ? launch_simt_attend_as<T, P, kKeySide, 8, 1>(pr, Q, W, kpvp, weight, a32, aT16, out, st, chained)
+             : launch_simt_attend_as<T, P, kKeySide, 2, 1>(pr, Q, W, kpvp, weight, a32, aT16, out, st, chained);
 }
 
 template <typename T, bool P>
 int launch_simt_key_side(const Problem& pr, const float* kpvp, const void* W, float* weight, float* a32,
-                         __half* aT16, cudaStream_t st, int* launches) {
-  return launch_simt_attend<T, P, true>(pr, nullptr, W, kpvp, weight, a32, aT16, nullptr, st, launches);
+                         __half* aT16, cudaStream_t st, int* launches, bool chained = true) {
+  return launch_simt_attend<T, P, true>(pr, nullptr, W, kpvp, weight, a32, aT16, nullptr, st, launches, chained);
 }
 
 template <typename T, bool P>
 int launch_simt_query_side(const Problem& pr, const void* Q, const void* W, float* weight, float* a32, void* out,
                            cudaStream_t st, int* launches) {
-  return launch_simt_attend<T, P, false>(pr, Q, W, nullptr, weight, a32, nullptr, out, st, launches);
+  return launch_simt_attend<T, P, false>(pr, Q, W, nullptr, weight, a32, nullptr, out, st, launches, true);
 }
 
 template <typename T>
 int key_side_dispatch(const Problem& pr, const float* kpvp, const void* W, float* weight, float* a32,
-                      __half* aT16, cudaStream_t st, int* launches) {
+                      __half* aT16, cudaStream_t st, int* launches, bool chained) {
   return pr.kernel == FLURKA_PERFORMER
-             ? launch_simt_key_side<T, true>(pr, kpvp, W, weight, a32, aT16, st, launches)
-             : launch_simt_key_side<T, false>(pr, kpvp, W, weight, a32, aT16, st, launches);
+             ? launch_simt_key_side<T, true>(pr, kpvp, W, weight, a32, aT16, st, launches, chained)
+             : launch_simt_key_side<T, false>(pr, kpvp, W, weight, a32, aT16, st, launches, chained);
 }
 
 // The three stages in order.  tc1 / tc3 choose the tensor-core kernel for stage 1 / stage 3
@@ -326,8 +328,10 @@ int key_side_dispatch(const Problem& pr, const float* kpvp, const void* W, float
 template <typename T, typename Stage1>
 int run_pipeline_with(const Problem& pr, const Layout& L, char* ws, const void* Q, const void* W, void* out,
                       cudaStream_t st, bool tc2, bool tc3, TensorContext* tc, StageTimer* timer, bool keep_status,
-                      int* launches, Stage1&& stage1, int phases = 3, void* more = nullptr, size_t more_bytes = 0) {
+                      int* launches, Stage1&& stage1, int phases = 3, void* more = nullptr, size_t more_bytes = 0,
+                      bool own_queries = false) {
   // more: one further range of the workspace that has to start at zero
+  // own_queries: Q is a result of stage 1, written by a kernel that the last one of stage 1 does not wait for
   // phases: bit 0 = clear the accumulators and run stage 1, bit 1 = run stages 2 and 3 (a sequence-sharded
   // forward does the two halves in separate calls, with the sum over the shards in between)
   float* kpvp = (float*)(ws + L.kpvp);
@@ -353,16 +357,20 @@ int run_pipeline_with(const Problem& pr, const Layout& L, char* ws, const void* 
     e = cudaGetLastError();
     return e == cudaSuccess ? FLURKA_OK : cuda_fail(e);
   }
+  // The kernels of stages 2 and 3 read W and Q before they wait: inputs that were complete before the clearing kernel let
+  // the chain begin.  Without that kernel (phases without bit 0), or with Q computed by an ordinary launch in the call, stage
+  // 2 starts a chain of its own.
+  const bool chained = (phases & 1) && !own_queries;
   // ragged lengths: a as two bf16 terms, which together are as large as the fp32 a they lie in place of
   __nv_bfloat16* abf = tc2 && ragged(pr) ? (__nv_bfloat16*)a32 : nullptr;
   if (tc2) {
     float* part = L.total > L.part ? (float*)(ws + L.part) : nullptr;
     rc = launch_k2(*tc, performer, kpvp, W, weight, abf ? nullptr : aT16, part, status + 4, pr.BH(), pr.d, pr.k, pr.p(), status,
-                   st, &cuda_err, nullptr, abf, abf != nullptr);
+                   st, &cuda_err, nullptr, abf, abf != nullptr, chained);
     if (rc) { g_last_cuda_error = cuda_err; return rc; }
     ++*launches;
   } else {
-    rc = key_side_dispatch<T>(pr, kpvp, W, weight, tc3 ? nullptr : a32, tc3 ? aT16 : nullptr, st, launches);
+    rc = key_side_dispatch<T>(pr, kpvp, W, weight, tc3 ? nullptr : a32, tc3 ? aT16 : nullptr, st, launches, chained);
     if (rc) return rc;
   }
   if (timer) timer->mark(2, st);
@@ -850,7 +858,7 @@ int fused_pipeline(const Problem& pr, int dm, const FusedLayout& FL, char* ws, c
   };
   const bool tensor23 = tensor && tensor_stages23_ok(pr);
   return run_pipeline_with<T>(pr, FL.L, ws, qp, W, out, st, tensor23, tensor23, tc, timer, /*keep_status=*/false, launches,
-                              stage1, 3, tensor ? kt : nullptr, tensor ? FL.kt_bytes : 0);
+                              stage1, 3, tensor ? kt : nullptr, tensor ? FL.kt_bytes : 0, /*own_queries=*/!tensor);
 }
 
 }  // namespace

@@ -250,7 +250,8 @@ simt_attend(const T* __restrict__ Q, const T* __restrict__ W, const float* __res
       *reinterpret_cast<float4*>(Xs + r * ld + c) = simt_load_row4(src + c, row0 + r < rows ? d - c : 0, vec);
     }
   }
-  tc::grid_dependency_wait();          // rows are inputs of the call; everything else comes from the kernels before
+  // rows are inputs of the call, or complete because the key side was an ordinary launch; the rest comes from the kernels before
+  tc::grid_dependency_wait();
   float run_max[R], run_sum[R], acc[R][NB * 4];
 #pragma unroll
   for (int r = 0; r < R; ++r) {

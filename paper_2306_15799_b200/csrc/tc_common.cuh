@@ -45,9 +45,12 @@ __device__ __forceinline__ void grid_dependency_wait_async() {
   grid_dependency_wait();
   asm volatile("fence.proxy.async.global;" ::: "memory");
 }
-// Lets the next kernel in the stream be scheduled once every CTA of this grid has said so or has
-// exited.  Called late in a CTA's life: when the last CTA calls it, every CTA of this grid already
-// holds its SM, so the successor's CTAs can never keep one of ours from starting.
+// Lets the next kernel in the stream be scheduled once every CTA of this grid has said so or has exited: by then every
+// CTA of this grid holds its SM, so the successor's CTAs can never keep one of ours from starting.
+// clear_ranges, the first kernel of a call, waits and then says so at once; the kernels after it say so late (only their
+// epilogue is left) or, where their CTAs are small, at their start, before they have waited themselves.  A kernel that has
+// started therefore knows only that everything before the call's first kernel is complete: before its own wait it may read
+// the call's inputs and nothing that a kernel of the call writes.  A call without clear_ranges starts with an ordinary launch.
 __device__ __forceinline__ void grid_launch_dependents() {
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }

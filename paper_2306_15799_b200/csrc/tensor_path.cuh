@@ -27,9 +27,10 @@ namespace flurka {
 // kernel in the stream is finishing (its CTAs call griddepcontrol.launch_dependents) and waits in
 // griddepcontrol.wait before it touches that kernel's results.  Every kernel of a chain waits somewhere before it
 // ends, so that the completion of one says that all before it are complete.
+// chained = false: an ordinary launch, which starts when everything before it in the stream is complete.
 template <typename... KArgs, typename... Args>
 inline cudaError_t launch_cluster_after_predecessor(int cluster, void (*fn)(KArgs...), dim3 grid, int block, size_t smem,
-                                                    cudaStream_t st, Args... args) {
+                                                    cudaStream_t st, bool chained, Args... args) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = grid;
   cfg.blockDim = dim3((unsigned)block, 1, 1);
@@ -37,7 +38,7 @@ inline cudaError_t launch_cluster_after_predecessor(int cluster, void (*fn)(KArg
   cfg.stream = st;
   cudaLaunchAttribute attr[2];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  attr[0].val.programmaticStreamSerializationAllowed = chained ? 1 : 0;
   attr[1].id = cudaLaunchAttributeClusterDimension;
   attr[1].val.clusterDim.x = (unsigned)cluster;
   attr[1].val.clusterDim.y = 1;
@@ -50,7 +51,12 @@ inline cudaError_t launch_cluster_after_predecessor(int cluster, void (*fn)(KArg
 template <typename... KArgs, typename... Args>
 inline cudaError_t launch_after_predecessor(void (*fn)(KArgs...), dim3 grid, int block, size_t smem, cudaStream_t st,
                                             Args... args) {
-  return launch_cluster_after_predecessor(1, fn, grid, block, smem, st, args...);
+  return launch_cluster_after_predecessor(1, fn, grid, block, smem, st, true, args...);
+}
+template <typename... KArgs, typename... Args>
+inline cudaError_t launch_chained(bool chained, void (*fn)(KArgs...), dim3 grid, int block, size_t smem, cudaStream_t st,
+                                  Args... args) {
+  return launch_cluster_after_predecessor(1, fn, grid, block, smem, st, chained, args...);
 }
 
 // Zeroes [p0, p0 + n0) and [p1, p1 + n1) (16-byte aligned; lengths are rounded up to 16 bytes).
@@ -402,9 +408,11 @@ inline size_t k2_part_floats(bool performer, int BH, int d, int k, int p) {
 
 // ---- stage 2: per-feature summaries a (fp16, transposed) and weights b / z from K', V' --------
 // split: PERFORMER with d = 64, the weights inside as two bf16 terms (32-bit precision in the forward of ragged lengths)
+// chained: W is an input of a call whose chain of launches began before this kernel (it is read before the wait)
 inline int launch_k2(TensorContext& tc, bool performer, const float* kpvp, const void* W, float* weight,
                      __half* aT16, float* part, int* counters, int BH, int d, int k, int p, int* status,
-                     cudaStream_t st, int* cuda_err, float* a32 = nullptr, __nv_bfloat16* abf = nullptr, bool split = false) {
+                     cudaStream_t st, int* cuda_err, float* a32 = nullptr, __nv_bfloat16* abf = nullptr, bool split = false,
+                     bool chained = true) {
   TensorMaps& tm = tc.maps;
   if (performer) {
     const unsigned long long dW[2] = {(unsigned long long)d, (unsigned long long)p};
@@ -432,8 +440,8 @@ inline int launch_k2(TensorContext& tc, bool performer, const float* kpvp, const
   cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, kK2SmemBytes);
   if (e != cudaSuccess) { *cuda_err = (int)e; (void)cudaGetLastError(); return -6; }
   // the RNN kernel ignores tmW; pass any valid map
-  e = launch_after_predecessor(fn, BH * prm.ftiles * prm.nsplit, kK2Threads, kK2SmemBytes, st,
-                               performer ? tm.W2.map : tm.kpvp.map, prm);
+  e = launch_chained(chained, fn, BH * prm.ftiles * prm.nsplit, kK2Threads, kK2SmemBytes, st,
+                     performer ? tm.W2.map : tm.kpvp.map, prm);
   if (e != cudaSuccess) { *cuda_err = (int)e; (void)cudaGetLastError(); return -6; }
   e = cudaGetLastError();
   if (e != cudaSuccess) { *cuda_err = (int)e; return -6; }
@@ -532,7 +540,7 @@ inline int launch_bwd_query(TensorContext& tc, bool performer, const void* Q, co
   if (e != cudaSuccess) { *cuda_err = (int)e; (void)cudaGetLastError(); return -6; }
   const int groups = std::max(1, std::min(tc.sm_count() / parts, prm.total_tiles));
   // the RNN kernel ignores tmW; pass any valid map
-  e = launch_cluster_after_predecessor(parts, fn, groups * parts, kK7Threads, smem, st, tm.Q.map, tm.dO.map,
+  e = launch_cluster_after_predecessor(parts, fn, groups * parts, kK7Threads, smem, st, true, tm.Q.map, tm.dO.map,
                                        performer ? tm.W2.map : tm.Q.map, tm.abf.map, prm);
   if (e != cudaSuccess) { *cuda_err = (int)e; (void)cudaGetLastError(); return -6; }
   return 0;

@@ -148,3 +148,40 @@ def test_fused_argument_errors():
     assert lib.flurka_forward_fused(*bad, RNN, 1, 1, 256, 64, 64, 64, 0, out.data_ptr(), None) == -1
     assert binding.flurka_fused_workspace_bytes(RNN, torch.bfloat16, 1, 1, 256, 64, 64, 64, 0) > \
         binding.flurka_workspace_bytes(RNN, torch.bfloat16, 1, 1, 256, 64, 64, 0)
+
+
+@pytest.mark.parametrize("w", [
+    _fw("fused_order_fp32", PERFORMER, "fp32", 2, 4, 2048, 64, 32, 32, 64, 81, shared_x=False),
+    _fw("fused_order_bf16", RNN, "bf16", 1, 8, 4000, 64, 32, 48, 0, 82, shared_x=False),
+], ids=lambda w: w.name)
+def test_fused_on_cuda_cores_reads_its_own_query_map(w):
+    """The query side reads the rows that the query map of the same call wrote, two kernels earlier, before it waits for
+    the key side: the key side has to start after that map is complete.  (Inputs change from pass to pass, so rows of the
+    pass before would show.)"""
+    dev = {n: (t.cuda() if t is not None else None) for n, t in synth.make_fused_inputs(w).items()}
+    X = torch.empty_like(dev["Xq"])
+    prev = binding.flurka_set_path(binding.PATH_SIMT)
+    try:
+        for i in range(6):
+            torch.mul(dev["Xq"], (-1.0) ** i * (1.0 + 0.5 * i), out=X)
+            out = binding.flurka_forward_fused(X, dev["Xk"], dev["Xv"], dev["E"], dev["F"], dev["Wq"], dev["Wk"], dev["Wv"],
+                                               dev["W"], w.variant, w.H)
+            Q = (X.double() @ dev["Wq"].double()).to(X.dtype).view(w.B, w.N, w.H, w.d)
+            Kp = binding.flurka_debug_copy(0, (w.B, w.H, w.k, w.d)).double()
+            Vp = binding.flurka_debug_copy(1, (w.B, w.H, w.k, w.d)).double()
+            torch.cuda.synchronize()
+            Qd = Q.double().transpose(1, 2)
+            if w.variant == PERFORMER:
+                L = dev["W"].double() @ Kp.transpose(-1, -2) - 0.5 * (Kp * Kp).sum(-1)[..., None, :]
+                P = torch.softmax(Qd @ dev["W"].double().T + torch.logsumexp(L, -1)[..., None, :], -1)
+                a = torch.softmax(L, -1) @ Vp
+            else:
+                elu = lambda t: torch.where(t > 0, t + 1, torch.exp(t.clamp(max=0)))
+                f = elu(Kp).transpose(-1, -2)
+                a, P = (f / f.sum(-1, keepdim=True)) @ Vp, elu(Qd) * f.sum(-1)[..., None, :]
+                P = P / P.sum(-1, keepdim=True)
+            ref = (P @ a).transpose(1, 2)
+            rel = float((out.double() - ref).norm() / ref.norm())
+            assert rel <= (1e-4 if w.io == "fp32" else 1e-2), (i, rel)
+    finally:
+        binding.flurka_set_path(prev)

@@ -72,3 +72,31 @@ def test_finish_without_partial_is_refused():
     with pytest.raises(binding.FlurkaError) as err:
         binding.flurka_forward_finish(dev["Q"], None, w.variant, w.k)
     assert err.value.code == -5
+
+
+@pytest.mark.parametrize("w", [
+    Workload("shard_order_simt", PERFORMER, "fp32", 2, 8, 4096, 64, 64, 128, 96),
+    Workload("shard_order_tensor", PERFORMER, "bf16", 2, 8, 8192, 64, 128, 128, 97),
+    Workload("shard_order_ragged_rnn", RNN, "bf16", 2, 8, 8001, 64, 64, 0, 98),
+], ids=lambda w: w.name)
+def test_finish_reads_queries_that_the_kernel_before_it_writes(w):
+    """The caller's last kernel before the second half writes Q and W: the second half's kernels read both before they wait
+    for one another, so its first launch has to wait for everything before it.  (The order cannot be provoked from here:
+    this runs the sequence with data that changes from pass to pass, against the same call after a synchronisation.)"""
+    x = pu.to_device(synth.make_inputs(w))
+    binding.flurka_forward_partial(x["K"], x["V"], x["E"], x["F"], w.variant, m=w.m)
+    total = binding.flurka_partial_sums().clone()
+    Q = torch.empty_like(x["Q"])
+    W = torch.empty_like(x["W"]) if x["W"] is not None else None
+    for i in range(8):
+        sign = -1.0 if i & 1 else 1.0
+        binding.flurka_partial_sums().copy_(total)
+        if W is not None:
+            torch.mul(x["W"], sign, out=W)
+        torch.mul(x["Q"], sign * (1.0 + 0.25 * i), out=Q)
+        got = binding.flurka_forward_finish(Q, W, w.variant, w.k)
+        torch.cuda.synchronize()
+        want = binding.flurka_forward_finish(Q, W, w.variant, w.k)
+        torch.cuda.synchronize()
+        assert binding.flurka_last_status() == 0 and torch.equal(got, want)
+        Q.fill_(float("nan"))
