@@ -193,7 +193,10 @@ int flurka_backward(const void* Q, const void* K, const void* V, const void* E, 
 size_t flurka_backward_workspace_bytes(int variant, int B, int H, int N, int d, int k, int m);
 
 /* Bytes of device scratch flurka_forward needs for this problem (0 on invalid arguments). Holds the
- * fp32 projections K', V' (Eq. (2)'s E K and F V), the key-side feature summaries and a status word. */
+ * fp32 projections K', V' (Eq. (2)'s E K and F V), the key-side feature summaries and a status word; N no
+ * multiple of 8 adds the copies of E, F that the tensor-core kernels want.  Only those depend on N: a caller's
+ * workspace that was sized at another N, without room for them, still serves such a call, on CUDA cores
+ * (the same holds for flurka_backward and flurka_forward_fused). */
 size_t flurka_workspace_bytes(int variant, int B, int H, int N, int d, int k, int m);
 
 /* Hands the library a caller-owned device workspace (256-byte aligned) for the current device.

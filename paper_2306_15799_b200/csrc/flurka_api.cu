@@ -79,6 +79,8 @@ int auto_path(const Problem& pr) {
   return projection_fmas(pr) >= (double)(1 << 24) ? FLURKA_PATH_TENSOR_STAGE1 : FLURKA_PATH_SIMT;
 }
 
+int path_without_copies(const Problem& pr, int path) { return ragged(pr) ? FLURKA_PATH_SIMT : path; }
+
 // Whether a path that the caller forces may take the problem: ragged lengths need a copy of E, F first, which only the
 // library's own choice of path makes.
 bool forced_tensor_ok(const Problem& pr) { return tensor_path_ok(pr) && !ragged(pr); }
@@ -207,6 +209,11 @@ int get_workspace(DeviceState& ds, size_t need, cudaStream_t st, char** ws) {
   *ws = (char*)ds.own_ws;
   return FLURKA_OK;
 }
+
+// Whether the workspace of the next call holds (the library's own: will hold) that much.  A caller's workspace that is large
+// enough but for the copies of E, F of a ragged length gets the CUDA-core kernels, which make none: without the copies the
+// size does not depend on N, and a workspace may have been sized at another N.
+bool workspace_holds(const DeviceState& ds, size_t need) { return !ds.user_ws || ds.user_ws_bytes >= need; }
 
 int check_device() {
   int dev = 0;
@@ -498,7 +505,8 @@ int forward_device(const void* Q, const void* K, const void* V, const void* E, c
       return FLURKA_ERR_WORKSPACE;
     ws = ds.last_ws;
   } else {
-    rc = get_workspace(ds, std::max(L.total, reserve), st, &ws);
+    if (g_path == FLURKA_PATH_AUTO && !workspace_holds(ds, std::max(L.total, reserve))) path = path_without_copies(pr, path);
+    rc = get_workspace(ds, std::max(path == FLURKA_PATH_SIMT ? L.efpad : L.total, reserve), st, &ws);
     if (rc) return rc;
   }
   int launches = 0;
@@ -625,13 +633,16 @@ int flurka_forward_host(const void* Q, const void* K, const void* V, const void*
   // The groups need not be equal (12 heads in 8 groups: 1, 2, 1, 2, ...).  One workspace that fits the
   // largest group is obtained before the first group runs, so it never moves between groups; the
   // status words sit at its start for every group size.
-  size_t reserve = 0;
+  size_t reserve = 0, without_copies = 0;
   for (int gi = 0; gi < groups; ++gi) {
     const int cnt = (int)((long long)heads * (gi + 1) / groups) - (int)((long long)heads * gi / groups);
     Problem sub = pr;
     if (by_batch) sub.B = cnt; else { sub.B = 1; sub.H = cnt; }
-    reserve = std::max(reserve, make_layout(sub).total);
+    const Layout L = make_layout(sub);
+    reserve = std::max(reserve, L.total);
+    without_copies = std::max(without_copies, L.efpad);
   }
+  if (!workspace_holds(ds, reserve)) reserve = without_copies;      // (ragged lengths: see workspace_holds)
   const size_t head_bytes = (size_t)N * d * pr.esize() * (by_batch ? H : 1);
   rc = FLURKA_OK;
   for (int gi = 0; gi < groups && rc == FLURKA_OK; ++gi) {
@@ -789,10 +800,10 @@ struct FusedLayout {
   size_t kt, kt_bytes, a3, qp, total;
 };
 
-FusedLayout make_fused_layout(const Problem& pr, int dm) {
+FusedLayout make_fused_layout(const Problem& pr, int dm, bool copies = true) {
   FusedLayout f;
   f.L = make_layout(pr);
-  size_t off = f.L.total;
+  size_t off = copies ? f.L.total : f.L.efpad;             // (room for copies of E, F: ragged lengths on tensor cores)
   f.kt_bytes = (size_t)2 * pr.B * pr.k * dm * 4;
   f.kt = off; off = align256(off + f.kt_bytes);
   f.a3 = off; off = align256(off + (pr.fp32 ? 0 : (size_t)2 * pr.B * pr.k * 3 * dm * 2));
@@ -899,7 +910,8 @@ int flurka_forward_fused(const void* Xq, const void* Xk, const void* Xv, const v
   rc = check_device();
   if (rc) return rc;
   DeviceState& ds = dev_state();
-  const FusedLayout FL = make_fused_layout(pr, dm);
+  if (g_path == FLURKA_PATH_AUTO && !workspace_holds(ds, make_fused_layout(pr, dm).total)) path = path_without_copies(pr, path);
+  const FusedLayout FL = make_fused_layout(pr, dm, /*copies=*/path != FLURKA_PATH_SIMT);
   cudaStream_t st = (cudaStream_t)stream;
   char* ws = nullptr;
   rc = get_workspace(ds, FL.total, st, &ws);
@@ -1145,17 +1157,19 @@ int flurka_backward(const void* Q, const void* K, const void* V, const void* E, 
   const BackwardLayout BL = make_backward_layout(pr);
   cudaStream_t st = (cudaStream_t)stream;
   char* ws = nullptr;
-  rc = get_workspace(ds, BL.total, st, &ws);
-  if (rc) return rc;
-  int launches = 0;
-  const bool perf = pr.kernel == FLURKA_PERFORMER;
   // tensor-core kernels for stage 1 and the query side where the shape allows (and the path knob does not
   // force the CUDA-core kernels); a forced tensor path with another shape is refused
   const bool tensor_ok = backward_tensor_ok(pr);
   if (g_path >= FLURKA_PATH_TENSOR && !(tensor_ok && forced_tensor_ok(pr))) return FLURKA_ERR_SHAPE;
-  const bool use_tc = tensor_path_ok(pr) && g_path != FLURKA_PATH_SIMT && (!ragged(pr) || ragged_backward_pays(pr));
+  const bool use_tc = tensor_path_ok(pr) && g_path != FLURKA_PATH_SIMT &&
+                      (!ragged(pr) || (ragged_backward_pays(pr) && workspace_holds(ds, BL.total)));
   TensorContext* tc = use_tc ? &ds.tc : nullptr;
   const bool tcq = tc && tensor_ok;
+  // (a ragged length on CUDA cores: neither copies nor the two-term gradients)
+  rc = get_workspace(ds, use_tc ? BL.total : (ragged(pr) ? BL.split : BL.efpad), st, &ws);
+  if (rc) return rc;
+  int launches = 0;
+  const bool perf = pr.kernel == FLURKA_PERFORMER;
   if (pr.fp32)
     rc = perf ? backward_pipeline<float, true>(pr, BL, ws, Q, K, V, E, F, W, dO, dQ, dK, dV, dE, dF, st, &launches, nullptr, false)
               : backward_pipeline<float, false>(pr, BL, ws, Q, K, V, E, F, W, dO, dQ, dK, dV, dE, dF, st, &launches,

@@ -641,3 +641,51 @@ def test_ragged_lengths_keep_32_bit_weights(w, limit, scale):
             moved += int((out[b, h] != ref.to(torch.bfloat16)).sum())
             total += ref.numel()
     assert moved <= 2.0 ** -7 * total, "%s: %.5f of the elements moved" % (w.name, moved / total)
+
+
+@pytest.mark.parametrize("per_head", [False, True])
+def test_ragged_call_in_a_workspace_sized_at_another_length(per_head):
+    """Scratch without the copies of E, F does not depend on N (and not on whether E, F are shared): a block of the size
+    asked for at a multiple of 8 serves a ragged length too.  Forward, host, fused and backward call; nothing is written
+    past the block, and a quarter of it is refused."""
+    w = _wl("ws_other_n", PERFORMER, "bf16", 2, 2, 999, 64, 256, 128, 185)
+    x = synth.make_inputs(w)
+    if per_head:
+        gen = torch.Generator().manual_seed(w.seed)
+        for name in ("E", "F"):
+            x[name] = (torch.randn(w.H, w.k, w.N, generator=gen, dtype=torch.float64) * float(w.k) ** -0.5).bfloat16()
+    dev = pu.to_device(x)
+    args = [dev[n] for n in ("Q", "K", "V", "E", "F", "W")]
+    sizes = (w.variant, torch.bfloat16, w.B, w.H, 1000)
+    dm = 128
+    X = torch.randn(w.B, w.N, dm, device="cuda").bfloat16()
+    Wq = torch.randn(dm, w.H * w.d, device="cuda").mul_(dm ** -0.5 * w.d ** -0.25).bfloat16()
+    calls = {
+        "forward": (binding.flurka_workspace_bytes(*sizes, w.d, w.k, w.m), lambda: binding.flurka_forward(*args, w.variant)),
+        "host": (binding.flurka_workspace_bytes(*sizes, w.d, w.k, w.m),
+                 lambda: binding.flurka_forward_host(*[x[n].pin_memory() for n in ("Q", "K", "V", "E", "F", "W")], w.variant)),
+        "backward": (binding.flurka_backward_workspace_bytes(*sizes, w.d, w.k, w.m),
+                     lambda: binding.flurka_backward(*args, dev["Q"], w.variant)),
+    }
+    if not per_head:
+        calls["fused"] = (binding.flurka_fused_workspace_bytes(*sizes, dm, w.d, w.k, w.m),
+                          lambda: binding.flurka_forward_fused(X, X, X, dev["E"], dev["F"], Wq, Wq, Wq, dev["W"], w.variant, w.H))
+    for name, (need, call) in calls.items():
+        own = call()
+        torch.cuda.synchronize()
+        buf = torch.full((need + 4096,), 0xA5, dtype=torch.uint8, device="cuda")
+        try:
+            binding.flurka_set_workspace(buf[:need])
+            got = call()
+            torch.cuda.synchronize()
+            assert binding.flurka_last_status() == 0 and binding.flurka_last_path() == binding.PATH_SIMT, name
+            binding.flurka_set_workspace(buf[:need // 4])
+            with pytest.raises(binding.FlurkaError) as ei:
+                call()
+            assert ei.value.code == -5, name
+        finally:
+            binding.flurka_set_workspace(None)
+        assert bool((buf[need:] == 0xA5).all()), name
+        for a, b in zip(got if isinstance(got, tuple) else (got,), own if isinstance(own, tuple) else (own,)):
+            rel = float((a.double().cpu() - b.double().cpu()).norm() / b.double().cpu().norm())
+            assert rel <= 2e-3, (name, rel)
