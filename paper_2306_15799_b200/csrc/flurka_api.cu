@@ -261,10 +261,14 @@ cudaError_t launch_simt_down_project_as(const Problem& pr, const void* K, const 
 template <typename T>
 int launch_simt_down_project(const Problem& pr, const void* K, const void* V, const void* E,
                              const void* F, float* kpvp, cudaStream_t st, int* launches) {
-  // rows per block: the largest tile that k fills (the larger the tile, the fewer shared memory reads per FMA)
+  // rows per block: the largest tile that k fills (the larger the tile, the fewer shared memory reads per FMA).
   const bool wide = pr.d > 64;
   cudaError_t e;
-  if (pr.k > 64) e = wide ? launch_simt_down_project_as<T, 8, 2>(pr, K, V, E, F, kpvp, st)
+  // (bf16 with more than 64 columns: 64 rows, two blocks per SM, which hide the conversions and, with N no multiple of 4, the
+  // element-wise loads; RNN, 24 heads, k = 1024, the call, us, 64 / 128 rows: N = 4096, d = 128 2284 / 2628, N = 4097, d = 127
+  // 2759 / 3490, N = 4097, d = 66 2472 / 3025; fp32 N = 4096, d = 128 1897 / 1813)
+  constexpr int kWideRows = sizeof(T) == 2 ? 4 : 8;
+  if (pr.k > 64) e = wide ? launch_simt_down_project_as<T, kWideRows, 2>(pr, K, V, E, F, kpvp, st)
                           : launch_simt_down_project_as<T, 8, 1>(pr, K, V, E, F, kpvp, st);
   else if (pr.k > 32) e = wide ? launch_simt_down_project_as<T, 4, 2>(pr, K, V, E, F, kpvp, st)
                                : launch_simt_down_project_as<T, 4, 1>(pr, K, V, E, F, kpvp, st);
