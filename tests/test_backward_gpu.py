@@ -240,6 +240,9 @@ def test_backward_argument_errors():
     (Workload("bwd_odd_d128", PERFORMER, "bf16", 1, 2, 390, 128, 128, 128, 353), "bhnd", False),
     (Workload("bwd_odd_rnn", RNN, "bf16", 1, 3, 1001, 64, 192, 0, 354), "bhnd", False),
     (Workload("bwd_odd_per_head", PERFORMER, "bf16", 2, 2, 301, 64, 64, 128, 355), "bhnd", True),
+    # enough tiles for 256 x 256 ones in both products (at least a third of the SMs), shared and one pair E, F per head
+    (Workload("bwd_odd_wide", PERFORMER, "bf16", 1, 2, 6147, 64, 256, 64, 356), "bnhd", False),
+    (Workload("bwd_odd_wide_per_head", RNN, "bf16", 2, 2, 3333, 64, 256, 0, 357), "bhnd", True),
 ], ids=lambda v: v.name if hasattr(v, "name") else str(v))
 def test_backward_of_ragged_lengths_on_the_tensor_path(w, layout, per_head):
     """N no multiple of 8: E, F are read from padded copies, dE, dF leave through them.  (The key and query side, whose

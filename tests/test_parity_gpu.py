@@ -476,6 +476,9 @@ def _ragged_path(w):
     (_wl("odd_perf_d128", PERFORMER, "bf16", 1, 3, 1003, 128, 128, 128, 143), "bhnd", False),
     (_wl("odd_rnn_n262", RNN, "bf16", 2, 2, 262, 64, 128, 0, 144), "bnhd", False),
     (_wl("odd_perf_per_head", PERFORMER, "bf16", 2, 2, 519, 64, 64, 128, 145), "bhnd", True),
+    # more than one block of the copying kernel per row (2048 elements), stage 1 as pairs; the same with one pair E, F per head
+    (_wl("odd_perf_n4099", PERFORMER, "bf16", 1, 4, 4099, 64, 256, 64, 146), "bnhd", False),
+    (_wl("odd_rnn_n2051_per_head", RNN, "bf16", 1, 3, 2051, 64, 128, 0, 147), "bhnd", True),
 ], ids=lambda v: v.name if hasattr(v, "name") else str(v))
 def test_ragged_lengths_on_the_tensor_path(w, layout, per_head):
     """N no multiple of 8: E, F are read from copies whose rows start on 16-byte boundaries.  (The key and query side of
