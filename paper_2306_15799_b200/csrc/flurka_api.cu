@@ -423,17 +423,24 @@ int run_pipeline(const Problem& pr, const Layout& L, char* ws, const void* Q, co
 }
 
 // Whether the one-kernel forward pass takes the problem: everything fits the shared memory of a cluster of eight CTAs per
-// head, all heads run at once, and a thread has at most kSmallFma multiply-adds (padding included).  Measured against the
-// four launches, us per call: fp32, two heads, d = 32, k = 32, m = 64: N = 128 13.0 / 17.8, N = 256 (2048 multiply-adds)
-// 13.4 / 17.7, N = 512 (3328) 18.3 / 17.9; d = 64, k = 64, N = 256: RNN, four heads (2048) 16.3 / 17.3, m = 64 (3072) 18.5 / 19.2.
-constexpr long long kSmallFma = 2100;
-bool small_forward_ok(const Problem& pr) {
-  if ((long long)pr.BH() * kSmallCtas > 148 || pr.d > 64 || pr.k > 1024) return false;
+// head, and a thread has few enough multiply-adds (padding included) that no shape measured is slower than as four launches.
+// us per call, one kernel / four launches, on 170 shapes:
+//   up to 15 heads (that many clusters of eight run at once with an SM per CTA): 2048 multiply-adds 12.6 / 18.0 (d = 32, k = m =
+//   32, N = 256) to 17.5 / 18.0; 2304 14.7 / 18.5 (d = 16, k = m = 64, N = 200); 2432 20.4 / 22.4; 2560 15.0 / 18.4 (d = 32, k = 64,
+//   m = 32, N = 128) but also 19.2 / 17.2 (RNN, bf16, d = 64, k = 32, N = 384); 3072 17.5 / 18.3 to 20.8 / 19.8; 3584 19.0 / 17.2;
+//   16 heads, RNN, d = k = 48, N = 64 (131 KB of shared memory: one CTA on an SM) 26.7 / 17.3, 15 heads 14.4 / 17.4;
+//   16 heads, two CTAs on an SM: 1536 12.7 / 17.7, 1792 16.5 / 18.4, 2048 16.2 / 18.0 to 18.6 / 17.3, 2304 20.3 / 18.2.
+constexpr int kSmallHeads = 15;
+constexpr long long kSmallFma = 2500, kSmallFmaTwo = 1800;
+constexpr size_t kSmallSmem = 200 * 1024, kSmallSmemTwo = 112 * 1024;
+bool small_forward_ok(const Problem& pr, int sms) {
+  if ((long long)pr.BH() * kSmallCtas > sms || pr.d > 64 || pr.k > 1024) return false;
   const SmallShape S = small_shape(pr.N, pr.d, pr.k, pr.p());
-  if (S.total * 4 > 200 * 1024) return false;
+  const bool two = pr.BH() > kSmallHeads;
+  if (S.total * 4 > (two ? kSmallSmemTwo : kSmallSmem)) return false;
   const long long n = S.n32, f = (S.fpc + 31) & ~31, k32 = (pr.k + 31) & ~31, k64 = (pr.k + 63) & ~63,
                   p64 = (pr.p() + 63) & ~63, per_item = 64 + (pr.kernel == FLURKA_PERFORMER ? pr.d : 0);
-  return (2 * n * k32 * 64 + f * k64 * per_item + n * p64 * per_item) / kSmallThreads <= kSmallFma;
+  return (2 * n * k32 * 64 + f * k64 * per_item + n * p64 * per_item) / kSmallThreads <= (two ? kSmallFmaTwo : kSmallFma);
 }
 
 template <typename T>
@@ -520,7 +527,8 @@ int forward_device(const void* Q, const void* K, const void* V, const void* E, c
     rc = timer->create();
     if (rc != cudaSuccess) return cuda_fail((cudaError_t)rc);
   }
-  if (path == FLURKA_PATH_SIMT && g_path == FLURKA_PATH_AUTO && phases == 3 && !timer && small_forward_ok(pr)) {
+  if (path == FLURKA_PATH_SIMT && g_path == FLURKA_PATH_AUTO && phases == 3 && !timer &&
+      small_forward_ok(pr, ds.tc.sm_total())) {
     rc = pr.fp32 ? launch_small_forward<float>(pr, L, ws, Q, K, V, E, F, W, out, st, keep_status, &launches)
                  : launch_small_forward<__nv_bfloat16>(pr, L, ws, Q, K, V, E, F, W, out, st, keep_status, &launches);
   } else if (pr.fp32) {

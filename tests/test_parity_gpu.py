@@ -692,3 +692,18 @@ def test_ragged_call_in_a_workspace_sized_at_another_length(per_head):
         for a, b in zip(got if isinstance(got, tuple) else (got,), own if isinstance(own, tuple) else (own,)):
             rel = float((a.double().cpu() - b.double().cpu()).norm() / b.double().cpu().norm())
             assert rel <= 2e-3, (name, rel)
+
+
+@pytest.mark.parametrize("w,launches", [
+    # as many heads as clusters of eight run at once with an SM per CTA, one more, and one more where two CTAs fit an SM
+    (_wl("limit_15_heads", RNN, "fp32", 1, 15, 64, 48, 48, 0, 201), 1),
+    (_wl("limit_16_heads", RNN, "fp32", 1, 16, 64, 48, 48, 0, 202), 3),
+    (_wl("limit_16_small_heads", RNN, "fp32", 2, 8, 200, 32, 16, 0, 203), 1),
+    (_wl("limit_16_heads_more_work", PERFORMER, "fp32", 2, 8, 128, 48, 32, 64, 204), 3),
+    # 2432 and 2560 multiply-adds per thread
+    (_wl("limit_2432", PERFORMER, "fp32", 1, 4, 200, 16, 32, 128, 205), 1),
+    (_wl("limit_2560", PERFORMER, "fp32", 1, 4, 128, 32, 64, 32, 206), 3),
+], ids=lambda v: v.name if hasattr(v, "name") else str(v))
+def test_limits_of_the_one_kernel_forward(w, launches):
+    pu.check_all_heads(w)
+    assert binding.flurka_last_path() == binding.PATH_SIMT and binding.flurka_last_launches() == launches
