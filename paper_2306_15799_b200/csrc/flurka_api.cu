@@ -155,6 +155,9 @@ DeviceState& dev_state() {
   return g_dev[dev];
 }
 
+// SMs of the current device
+int device_sms() { return dev_state().tc.sm_total(); }
+
 int cuda_fail(cudaError_t e) {
   g_last_cuda_error = (int)e;
   (void)cudaGetLastError();
@@ -246,7 +249,7 @@ cudaError_t launch_simt_down_project_as(const Problem& pr, const void* K, const 
                                  float* kpvp, cudaStream_t st) {
   // enough sequence splits for about four blocks per SM; a split is a multiple of one step
   const int jt = (pr.k + 16 * R - 1) / (16 * R);
-  int nsplit = 4 * 148 / (jt * pr.BH() * 2);
+  int nsplit = 4 * device_sms() / (jt * pr.BH() * 2);
   const int max_split = (pr.N + kSimtTN - 1) / kSimtTN;
   nsplit = std::max(1, std::min(nsplit, std::min(max_split, 16384)));
   int chunk = (pr.N + nsplit - 1) / nsplit;
@@ -301,7 +304,7 @@ template <typename T, bool P, bool kKeySide>
 int launch_simt_attend(const Problem& pr, const void* Q, const void* W, const float* kpvp, float* weight, float* a32,
                        __half* aT16, void* out, cudaStream_t st, int* launches, bool chained) {
   // 128 rows per block as soon as that gives every SM a block; 32 below, where the length of one block is the time
-  const bool big = (long long)(((kKeySide ? pr.p() : pr.N) + 127) / 128) * pr.BH() >= 148;
+  const bool big = (long long)(((kKeySide ? pr.p() : pr.N) + 127) / 128) * pr.BH() >= device_sms();
   ++*launches;
   if (pr.d > 64)
     return big ? launch_simt_attend_as<T, P, kKeySide, 8, 2>(pr, Q, W, kpvp, weight, a32, aT16, out, st, chained)
@@ -357,7 +360,7 @@ int run_pipeline_with(const Problem& pr, const Layout& L, char* ws, const void* 
   cudaError_t e = cudaSuccess;
   int rc = FLURKA_OK;
   if (phases & 1) {
-    e = launch_clear(ws + clear_from, L.kpvp_end - clear_from, more, more_bytes, st);
+    e = launch_clear(ws + clear_from, L.kpvp_end - clear_from, more, more_bytes, device_sms(), st);
     if (e != cudaSuccess) return cuda_fail(e);
     if (timer) timer->mark(0, st);
     rc = stage1(kpvp, status, launches);
@@ -433,8 +436,8 @@ int run_pipeline(const Problem& pr, const Layout& L, char* ws, const void* Q, co
 constexpr int kSmallHeads = 15;
 constexpr long long kSmallFma = 2500, kSmallFmaTwo = 1800;
 constexpr size_t kSmallSmem = 200 * 1024, kSmallSmemTwo = 112 * 1024;
-bool small_forward_ok(const Problem& pr, int sms) {
-  if ((long long)pr.BH() * kSmallCtas > sms || pr.d > 64 || pr.k > 1024) return false;
+bool small_forward_ok(const Problem& pr) {
+  if ((long long)pr.BH() * kSmallCtas > device_sms() || pr.d > 64 || pr.k > 1024) return false;
   const SmallShape S = small_shape(pr.N, pr.d, pr.k, pr.p());
   const bool two = pr.BH() > kSmallHeads;
   if (S.total * 4 > (two ? kSmallSmemTwo : kSmallSmem)) return false;
@@ -528,7 +531,7 @@ int forward_device(const void* Q, const void* K, const void* V, const void* E, c
     if (rc != cudaSuccess) return cuda_fail((cudaError_t)rc);
   }
   if (path == FLURKA_PATH_SIMT && g_path == FLURKA_PATH_AUTO && phases == 3 && !timer &&
-      small_forward_ok(pr, ds.tc.sm_total())) {
+      small_forward_ok(pr)) {
     rc = pr.fp32 ? launch_small_forward<float>(pr, L, ws, Q, K, V, E, F, W, out, st, keep_status, &launches)
                  : launch_small_forward<__nv_bfloat16>(pr, L, ws, Q, K, V, E, F, W, out, st, keep_status, &launches);
   } else if (pr.fp32) {
@@ -1019,7 +1022,7 @@ template <typename T, bool P>
 int launch_simt_bwd_key_side(const Problem& pr, const float* kpvp, const void* W, const float* weight, const float* da,
                              const float* ei, float* dkpvp, __nv_bfloat16* split, cudaStream_t st) {
   // 64 keys per block where that still gives every SM a block, else 32
-  const bool big = (long long)((pr.k + 63) / 64) * pr.BH() >= 148;
+  const bool big = (long long)((pr.k + 63) / 64) * pr.BH() >= device_sms();
   if (pr.d > 64) return big ? launch_simt_bwd_key_side_as<T, P, 4, 2>(pr, kpvp, W, weight, da, ei, dkpvp, split, st)
                             : launch_simt_bwd_key_side_as<T, P, 2, 2>(pr, kpvp, W, weight, da, ei, dkpvp, split, st);
   return big ? launch_simt_bwd_key_side_as<T, P, 4, 1>(pr, kpvp, W, weight, da, ei, dkpvp, split, st)
@@ -1041,7 +1044,7 @@ int backward_pipeline(const Problem& pr, const BackwardLayout& BL, char* ws, con
   float* ei = (float*)(ws + BL.ei);
   float* dkpvp = (float*)(ws + BL.dkpvp);
   const int smh = pr.seq_major_heads(), efh = pr.ef_heads();
-  cudaError_t e = launch_clear(ws + L.status, L.kpvp_end - L.status, da, BL.dae_bytes, st);
+  cudaError_t e = launch_clear(ws + L.status, L.kpvp_end - L.status, da, BL.dae_bytes, device_sms(), st);
   if (e != cudaSuccess) return cuda_fail(e);
   // the forward's stages 1 and 2 again: K', V', a_i, b_i (or z_i)
   int rc = FLURKA_OK;
@@ -1076,7 +1079,7 @@ int backward_pipeline(const Problem& pr, const BackwardLayout& BL, char* ws, con
     ++*launches;
   } else {
     // tiles of 64 rows where they are at least as many as SMs, else of 32
-    const bool big = (long long)((pr.N + 63) / 64) * pr.BH() >= 148;
+    const bool big = (long long)((pr.N + 63) / 64) * pr.BH() >= device_sms();
     auto fn = pr.d > 64 ? (big ? simt_bwd_query_side<T, P, 4, 2> : simt_bwd_query_side<T, P, 2, 2>)
                         : (big ? simt_bwd_query_side<T, P, 4, 1> : simt_bwd_query_side<T, P, 2, 1>);
     const int rows = big ? 64 : 32;
@@ -1113,14 +1116,15 @@ int backward_pipeline(const Problem& pr, const BackwardLayout& BL, char* ws, con
     // tiles of 128 rows where they are at least as many as SMs, else of 32
     const int zi = 2 * ((pr.d + 63) / 64), zp = 2 * (efh > 0 ? efh : 1);
     auto blocks = [](int n, int per) { return (n + per - 1) / per; };
-    if ((long long)blocks(pr.N, 128) * pr.BH() * zi >= 148)
+    const int sms = device_sms();
+    if ((long long)blocks(pr.N, 128) * pr.BH() * zi >= sms)
       simt_bwd_inputs<T, 8><<<dim3(blocks(pr.N, 128), pr.BH(), zi), kSimtThreads, 0, st>>>(
           (const T*)E, (const T*)F, dkpvp, (T*)dK, (T*)dV, pr.BH(), pr.N, pr.d, pr.k, smh, efh);
     else
       simt_bwd_inputs<T, 2><<<dim3(blocks(pr.N, 32), pr.BH(), zi), kSimtThreads, 0, st>>>(
           (const T*)E, (const T*)F, dkpvp, (T*)dK, (T*)dV, pr.BH(), pr.N, pr.d, pr.k, smh, efh);
     ++*launches;
-    if ((long long)blocks(pr.N, 64) * blocks(pr.k, 128) * zp >= 148)
+    if ((long long)blocks(pr.N, 64) * blocks(pr.k, 128) * zp >= sms)
       simt_bwd_projections<T, 8><<<dim3(blocks(pr.N, 64), blocks(pr.k, 128), zp), kSimtThreads, 0, st>>>(
           (const T*)K, (const T*)V, dkpvp, (T*)dE, (T*)dF, pr.BH(), pr.N, pr.d, pr.k, smh, efh);
     else

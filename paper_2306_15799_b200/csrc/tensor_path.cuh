@@ -60,7 +60,7 @@ inline cudaError_t launch_chained(bool chained, void (*fn)(KArgs...), dim3 grid,
 }
 
 // Zeroes [p0, p0 + n0) and [p1, p1 + n1) (16-byte aligned; lengths are rounded up to 16 bytes).
-inline cudaError_t launch_clear(void* p0, size_t n0, void* p1, size_t n1, cudaStream_t st) {
+inline cudaError_t launch_clear(void* p0, size_t n0, void* p1, size_t n1, int sms, cudaStream_t st) {
   ClearRanges r;
   r.ptr[0] = reinterpret_cast<uint4*>(p0);
   r.ptr[1] = reinterpret_cast<uint4*>(p1);
@@ -68,7 +68,7 @@ inline cudaError_t launch_clear(void* p0, size_t n0, void* p1, size_t n1, cudaSt
   r.count[1] = (n1 + 15) >> 4;
   // four 16-byte words per thread, at most eight blocks per SM
   size_t blocks = (std::max(r.count[0], r.count[1]) + 1023) / 1024;
-  blocks = std::max<size_t>(1, std::min<size_t>(blocks, 148 * 8));
+  blocks = std::max<size_t>(1, std::min<size_t>(blocks, (size_t)sms * 8));
   return launch_after_predecessor(clear_ranges, dim3((unsigned)blocks), 256, 0, st, r);
 }
 
