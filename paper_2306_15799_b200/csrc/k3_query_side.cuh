@@ -61,7 +61,7 @@ __host__ __device__ inline K3Smem k3_smem_plan(int d, int p, bool performer) {
   off = (off + 1023u) & ~1023u;
   s.aT = off;   off += (uint32_t)d * p * 2;                        // a^T: p/64 K-blocks of [d rows x 128 B]
   off = (off + 1023u) & ~1023u;
-  s.q_stages = (d == 64) ? 4 : 2;
+  s.q_stages = (d == 64) ? 4 : 2;                                 // (RNN)
   s.q = off;    off += (uint32_t)s.q_stages * 128 * d * 2;
   s.ostage = off; off += (d == 64) ? 8 * 4096 : 0;                 // d = 64: a [32 x 64] bf16 output slab per row-owner warp
   s.scale = off; off += 1024;                                      // RNN: z_i / max z as floats
@@ -79,7 +79,7 @@ k3_query_side(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ C
   extern __shared__ uint8_t smem_raw[];
   const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u;
   uint8_t* base_ptr = smem_raw + (base - smem_u32(smem_raw));
-  const int d = prm.d, p = prm.p;
+  const int d = kPerformer ? 128 : prm.d, p = prm.p;   // (PERFORMER with d = 64: k3_query_units)
   const K3Smem L = k3_smem_plan(d, p, kPerformer);
   const int NS = L.q_stages;
   const uint32_t q_stage_bytes = 128u * d * 2u;

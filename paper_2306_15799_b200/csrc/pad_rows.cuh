@@ -5,7 +5,7 @@
 // E K of arxiv 2306.15799, Section 2.1 / Eq. (2), runs along their rows) have a pitch of N elements.  They
 // are shared by all heads, so a copy moves 2 k N elements against the 2 B H d N of K and V; the tensor maps
 // keep the true extent N, so the padding is never read.  Bound by memory traffic; measured at B H = 16, N = 6001,
-// d = 64, k = m = 256: the forward 1678 us (fp32 CUDA-core kernels) -> 66 us, of which the copy is 4.
+// d = 64, k = m = 256: the forward 449 us on the CUDA-core kernels, 60 on tensor cores, of which the copy is 4.
 #pragma once
 
 #include <cuda_bf16.h>

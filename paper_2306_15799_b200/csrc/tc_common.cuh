@@ -142,9 +142,6 @@ __device__ __forceinline__ void tcgen05_fence_before() {
 __device__ __forceinline__ void tcgen05_fence_after() {
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
 }
-__device__ __forceinline__ void named_barrier_sync(uint32_t id, uint32_t threads) {
-  asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(threads) : "memory");
-}
 
 // ------------------------------------------------------------------------------ TMA
 __device__ __forceinline__ void prefetch_tmap(const CUtensorMap* m) {
@@ -176,12 +173,6 @@ __device__ __forceinline__ void tma_store_3d(const CUtensorMap* m, uint32_t src,
 __device__ __forceinline__ void tma_reduce_add_3d(const CUtensorMap* m, uint32_t src, int x, int y, int z) {
   asm volatile("cp.reduce.async.bulk.tensor.3d.global.shared::cta.add.tile.bulk_group [%0, {%2, %3, %4}], [%1];"
                ::"l"(reinterpret_cast<uint64_t>(m)), "r"(src), "r"(x), "r"(y), "r"(z)
-               : "memory");
-}
-// Untiled bulk copy global -> shared (both 16-byte aligned, size a multiple of 16 bytes); completes on `bar`.
-__device__ __forceinline__ void bulk_load(uint32_t dst, const void* src, uint32_t bytes, uint32_t bar) {
-  asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
-               ::"r"(dst), "l"(src), "r"(bytes), "r"(bar)
                : "memory");
 }
 __device__ __forceinline__ void bulk_commit_group() { asm volatile("cp.async.bulk.commit_group;" ::: "memory"); }
@@ -321,10 +312,9 @@ __device__ __forceinline__ uint64_t sub2(uint64_t a, uint64_t b) {
   return r;
 }
 
-// 2^x for a pair of x in [-100, 1] on the FMA pipe instead of the special-function unit: n = round(x)
-// (by adding 1.5 * 2^23, which leaves n in the low mantissa bits), f = x - n in [-1/2, 1/2], a cubic in
-// f (relative error below 8e-5, well under the rounding of the fp16 result), n added to the exponent
-// field as an integer.
+// 2^x for a pair of x in [-100, 100] (k3_query_units: up to 15) on the FMA pipe instead of the special-function unit: n =
+// round(x) (by adding 1.5 * 2^23, which leaves n in the low mantissa bits), f = x - n in [-1/2, 1/2], a cubic in f (relative
+// error below 8e-5, well under the rounding of the fp16 result), n added to the exponent field as an integer.
 __device__ __forceinline__ void exp2_cubic2(uint64_t x2, float& e0, float& e1) {
   const uint64_t magic = pack2(12582912.f, 12582912.f);
   const uint64_t t2 = add2(x2, magic);
@@ -348,16 +338,6 @@ __device__ __forceinline__ void mma_ss(uint32_t d_tmem, uint64_t a_desc, uint64_
       "setp.ne.b32 p, %4, 0;\n\t"
       "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}"
       ::"r"(d_tmem), "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate)
-      : "memory");
-}
-// D[tmem] (+)= A[tmem] * B[smem]
-__device__ __forceinline__ void mma_ts(uint32_t d_tmem, uint32_t a_tmem, uint64_t b_desc, uint32_t idesc,
-                                       uint32_t accumulate) {
-  asm volatile(
-      "{\n\t.reg .pred p;\n\t"
-      "setp.ne.b32 p, %4, 0;\n\t"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n\t}"
-      ::"r"(d_tmem), "r"(a_tmem), "l"(b_desc), "r"(idesc), "r"(accumulate)
       : "memory");
 }
 // Four consecutive 16-wide contraction steps in one go.  Queuing an MMA costs the issuing thread
