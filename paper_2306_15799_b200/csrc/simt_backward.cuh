@@ -345,12 +345,17 @@ simt_bwd_key_side(const float* __restrict__ KpVp, const T* __restrict__ W, const
   if (kPerformer) {
     __syncthreads();
     if (threadIdx.x < kRows) {
-      float s = 0.f;
-      for (int c = 0; c < cols; c += 4) {
-        const float4 v = *reinterpret_cast<const float4*>(Ks + threadIdx.x * ld + c);
-        s = fmaf(v.x, v.x, fmaf(v.y, v.y, fmaf(v.z, v.z, fmaf(v.w, v.w, s))));
+      // as the forward's key side adds them up, rounding for rounding: its error then cancels between L_ij and b_i
+      float s[4] = {0.f, 0.f, 0.f, 0.f};
+      for (int c = 0; c < cols; c += 16) {
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+          if (c + 4 * q >= cols) break;
+          const float4 v = *reinterpret_cast<const float4*>(Ks + threadIdx.x * ld + c + 4 * q);
+          s[q] = fmaf(v.x, v.x, fmaf(v.y, v.y, fmaf(v.z, v.z, fmaf(v.w, v.w, s[q]))));
+        }
       }
-      nrm[threadIdx.x] = 0.5f * s;
+      nrm[threadIdx.x] = 0.5f * ((s[0] + s[1]) + (s[2] + s[3]));
     }
   }
   for (int i0 = 0; i0 < p; i0 += 64) {

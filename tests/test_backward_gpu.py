@@ -326,3 +326,20 @@ def test_buffers_that_are_16_byte_aligned_only(w, layout):
         # partial sums meet in any order: the two may differ by that, not by a row or a piece of one
         rel = float((a.double() - b.double()).norm() / b.double().norm())
         assert rel <= 2e-3, "%s %s: %.3e" % (w.name, name, rel)
+
+
+@pytest.mark.parametrize("seed", [381, 382, 383])
+def test_key_weights_of_the_backward_share_the_forwards_norms(seed):
+    """A_ij = exp(w_i.k'_j - |k'_j|^2/2 - b_i) with |k'|^2/2 around 130, where the fp32 spacing is 1.5e-5: an error of that norm
+    cancels between the exponent and b_i only if both have the same one.  dV is linear in A: with norms of two roundings it
+    was 0.5e-5 to 3e-5 off; the rest is a sum of 64 fp32 terms and one of 128 (about 2e-6)."""
+    w = Workload("bwd_norms", PERFORMER, "fp32", 1, 1, 3000, 128, 128, 64, seed)
+    x = synth.make_inputs(w)
+    dO = torch.randn(w.B, w.H, w.N, w.d, generator=torch.Generator().manual_seed(seed))
+    dev = pu.to_device(x)
+    dV = binding.flurka_backward(dev["Q"], dev["K"], dev["V"], dev["E"], dev["F"], dev["W"], dO.cuda(), w.variant)[2]
+    torch.cuda.synchronize()
+    assert binding.flurka_last_status() == 0
+    ref = torch.from_numpy(_oracle_grads(w, x, dO, False)["dV"])
+    rel = float((dV.cpu().double() - ref).norm() / ref.norm())
+    assert rel <= 6e-6, rel
