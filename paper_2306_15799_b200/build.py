@@ -31,25 +31,29 @@ def is_stale() -> bool:
     return any(os.path.getmtime(p) > t for p in _deps())
 
 
-def build_marshal(force: bool = False) -> str:
-    """g++ against torch's headers -> paper_2306_15799_b200/_marshal.so"""
-    if not force and os.path.exists(MARSHAL) and os.path.getmtime(MARSHAL) >= os.path.getmtime(MARSHAL_SOURCE):
-        return MARSHAL
+def compile_marshal(source: str, target: str) -> None:
+    """g++ against torch's headers: marshal.cpp -> a Python module"""
     import sysconfig
     import torch
     root = os.path.join(os.path.dirname(os.path.abspath(torch.__file__)))
-    tmp = MARSHAL + ".tmp.%d" % os.getpid()
+    tmp = target + ".tmp.%d" % os.getpid()
     cmd = [os.environ.get("CXX", "g++"), "-O2", "-std=c++17", "-shared", "-fPIC",
            "-D_GLIBCXX_USE_CXX11_ABI=%d" % int(torch._C._GLIBCXX_USE_CXX11_ABI),
            "-isystem", os.path.join(root, "include"), "-isystem", os.path.join(root, "include", "torch", "csrc", "api", "include"),
            "-isystem", os.path.join(os.environ.get("CUDA_HOME", "/usr/local/cuda"), "include"),
-           "-isystem", sysconfig.get_paths()["include"], MARSHAL_SOURCE, "-o", tmp,
+           "-isystem", sysconfig.get_paths()["include"], source, "-o", tmp,
            "-L", os.path.join(root, "lib"), "-lc10", "-lc10_cuda", "-ltorch_cpu", "-ltorch", "-ltorch_python"]
     res = subprocess.run(cmd, capture_output=True, text=True)
     if res.returncode != 0:
         sys.stderr.write(res.stdout + res.stderr)
         raise RuntimeError("g++ failed building _marshal.so")
-    os.replace(tmp, MARSHAL)
+    os.replace(tmp, target)
+
+
+def build_marshal(force: bool = False) -> str:
+    """paper_2306_15799_b200/_marshal.so"""
+    if force or not os.path.exists(MARSHAL) or os.path.getmtime(MARSHAL) < os.path.getmtime(MARSHAL_SOURCE):
+        compile_marshal(MARSHAL_SOURCE, MARSHAL)
     return MARSHAL
 
 

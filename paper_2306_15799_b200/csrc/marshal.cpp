@@ -27,11 +27,25 @@ struct Problem {
   int variant, B, H, N, d, k, m;
 };
 
-// the tensor of an exact torch.Tensor on the device that Q is like: contiguous, on CUDA, of Q's type
+// What of a call may throw (addresses, the stream) is taken while the interpreter is held: an exception that left a block
+// without it would be caught by code that uses the interpreter.
+class WithoutInterpreter {
+ public:
+  WithoutInterpreter() : state_(PyEval_SaveThread()) {}
+  ~WithoutInterpreter() { PyEval_RestoreThread(state_); }
+  WithoutInterpreter(const WithoutInterpreter&) = delete;
+  WithoutInterpreter& operator=(const WithoutInterpreter&) = delete;
+
+ private:
+  PyThreadState* state_;
+};
+
+// the tensor of an exact torch.Tensor on the device that Q is like: contiguous, on CUDA, of Q's type, with memory of its own
+// (the wrapped tensors of torch.func's transforms have the type, device and strides of what they wrap, but no memory)
 const at::Tensor* plain(PyObject* o, const at::Tensor* like) {
   if (!THPVariable_CheckExact(o)) return nullptr;
   const at::Tensor& t = THPVariable_Unpack(o);
-  if (!t.is_cuda() || t.layout() != at::kStrided || !t.is_contiguous()) return nullptr;
+  if (!t.has_storage() || !t.is_cuda() || t.layout() != at::kStrided || !t.is_contiguous()) return nullptr;
   if (like && t.scalar_type() != like->scalar_type()) return nullptr;
   return &t;
 }
@@ -92,12 +106,14 @@ PyObject* forward(PyObject*, PyObject* const* a, Py_ssize_t n) {
     if (n != 8 || !g_forward || !parse(a, &p)) Py_RETURN_NONE;
     at::Tensor out = at::empty_like(*p.Q);
     if (out.sizes() != p.Q->sizes() || !out.is_contiguous()) Py_RETURN_NONE;
-    void* stream = stream_of_current_device();
+    const void* const in[6] = {address(p.Q), address(p.K), address(p.V), address(p.E), address(p.F), address(p.W)};
+    void* const to = out.data_ptr();
+    void* const stream = stream_of_current_device();
     int rc;
-    Py_BEGIN_ALLOW_THREADS
-    rc = g_forward(address(p.Q), address(p.K), address(p.V), address(p.E), address(p.F), address(p.W), p.variant, p.B, p.H,
-                   p.N, p.d, p.k, p.m, out.data_ptr(), stream);
-    Py_END_ALLOW_THREADS
+    {
+      WithoutInterpreter released;
+      rc = g_forward(in[0], in[1], in[2], in[3], in[4], in[5], p.variant, p.B, p.H, p.N, p.d, p.k, p.m, to, stream);
+    }
     return Py_BuildValue("(iN)", rc, THPVariable_Wrap(std::move(out)));
   } catch (...) {
     Py_RETURN_NONE;                                        // (out of memory and the like: the Python path says so)
@@ -110,19 +126,22 @@ PyObject* backward(PyObject*, PyObject* const* a, Py_ssize_t n) {
   try {
     if (n != 9 || !g_backward || !parse(a, &p)) Py_RETURN_NONE;
     if (!(p.dO = plain(a[8], p.Q)) || p.dO->sizes() != p.Q->sizes()) Py_RETURN_NONE;
-    const at::Tensor* in[5] = {p.Q, p.K, p.V, p.E, p.F};
+    const at::Tensor* like[5] = {p.Q, p.K, p.V, p.E, p.F};
     at::Tensor g[5];
+    void* to[5];
     for (int i = 0; i < 5; ++i) {
-      g[i] = at::empty_like(*in[i]);
+      g[i] = at::empty_like(*like[i]);
       if (!g[i].is_contiguous()) Py_RETURN_NONE;
+      to[i] = g[i].data_ptr();
     }
-    void* stream = stream_of_current_device();
+    const void* const in[7] = {address(p.Q), address(p.K), address(p.V), address(p.E), address(p.F), address(p.W), address(p.dO)};
+    void* const stream = stream_of_current_device();
     int rc;
-    Py_BEGIN_ALLOW_THREADS
-    rc = g_backward(address(p.Q), address(p.K), address(p.V), address(p.E), address(p.F), address(p.W), address(p.dO),
-                    p.variant, p.B, p.H, p.N, p.d, p.k, p.m, g[0].data_ptr(), g[1].data_ptr(), g[2].data_ptr(),
-                    g[3].data_ptr(), g[4].data_ptr(), stream);
-    Py_END_ALLOW_THREADS
+    {
+      WithoutInterpreter released;
+      rc = g_backward(in[0], in[1], in[2], in[3], in[4], in[5], in[6], p.variant, p.B, p.H, p.N, p.d, p.k, p.m, to[0], to[1],
+                      to[2], to[3], to[4], stream);
+    }
     return Py_BuildValue("(iNNNNN)", rc, THPVariable_Wrap(std::move(g[0])), THPVariable_Wrap(std::move(g[1])),
                          THPVariable_Wrap(std::move(g[2])), THPVariable_Wrap(std::move(g[3])), THPVariable_Wrap(std::move(g[4])));
   } catch (...) {

@@ -1,6 +1,7 @@
 """The C-ABI library loads without a GPU, exports every declared symbol, and rejects bad arguments
 before touching the device."""
 import ctypes
+import importlib.util
 import os
 import re
 
@@ -88,6 +89,73 @@ def test_binding_rejects_bad_tensors():
                                     out=torch.zeros_like(Q).half())
 
 
+@pytest.fixture(scope="module")
+def cpu_marshal(tmp_path_factory):
+    """csrc/marshal.cpp for tensors on the CPU, in front of functions that record what they are given: (module, calls)."""
+    text = open(build.MARSHAL_SOURCE).read()
+    for old, new in (("t.is_cuda()", "t.is_cpu()"), ("c10::cuda::getCurrentCUDAStream().stream()", "nullptr")):
+        assert text.count(old) == 1
+        text = text.replace(old, new)
+    folder = tmp_path_factory.mktemp("marshal")
+    source, target = str(folder / "marshal.cpp"), str(folder / "_marshal.so")
+    open(source, "w").write(text)
+    build.compile_marshal(source, target)
+    spec = importlib.util.spec_from_file_location("_marshal", target)
+    module = importlib.util.module_from_spec(spec)
+    spec.loader.exec_module(module)
+    calls = []
+    vp, ci = ctypes.c_void_p, ctypes.c_int
+    record = lambda *a: calls.append(a) or 0
+    forward = ctypes.CFUNCTYPE(ci, *[vp] * 6, *[ci] * 7, vp, vp)(record)
+    backward = ctypes.CFUNCTYPE(ci, *[vp] * 7, *[ci] * 7, *[vp] * 6)(record)
+    module.init(ctypes.cast(forward, vp).value, ctypes.cast(backward, vp).value)
+    yield module, calls
+    del forward, backward
+
+
+def _small_call(layout="bhnd", per_head=False, dtype=torch.float32):
+    B, H, N, d, k, m = 2, 3, 12, 8, 5, 7
+    shape = (B, N, H, d) if layout == "bnhd" else (B, H, N, d)
+    r = lambda *s: torch.randn(*s).to(dtype)
+    ef = (H, k, N) if per_head else (k, N)
+    return (B, H, N, d, k, m), [r(*shape), r(*shape), r(*shape), r(*ef), r(*ef), r(m, d)], r(*shape)
+
+
+@pytest.mark.parametrize("transform", ["vmap", "grad", "jvp", "grad of others"])
+def test_tensors_without_memory_are_left_to_the_python_path(cpu_marshal, transform):
+    """Inside torch.func's transforms a tensor has a type, a device and strides but no memory: the module declines such a
+    call (binding.py then raises RuntimeError) with the interpreter in hand."""
+    module, calls = cpu_marshal
+    _, (Q, *rest), dO = _small_call()
+    seen = []
+
+    def call(q):
+        del calls[:]
+        seen.append(module.forward(q, *rest, PERFORMER, False))
+        seen.append(module.backward(q, *rest, PERFORMER, False, dO))
+        seen.append(module.backward(Q, *rest, PERFORMER, False, q))
+        assert not calls
+        with pytest.raises(RuntimeError):
+            q.data_ptr()
+        return q.sum()
+
+    def others(q):                             # (what is allocated inside has no memory either)
+        del calls[:]
+        seen.append(module.forward(Q, *rest, PERFORMER, False))
+        assert not calls
+        return q.sum()
+
+    if transform == "vmap":
+        torch.func.vmap(call)(torch.stack([Q, Q]))
+    elif transform == "grad":
+        torch.func.grad(call)(Q)
+    elif transform == "jvp":
+        torch.func.jvp(call, (Q,), (torch.ones_like(Q),))
+    else:
+        torch.func.grad(others)(Q.clone())
+    assert seen and all(s is None for s in seen)
+
+
 @pytest.mark.gpu
 @pytest.mark.parametrize("dtype", [torch.float32, torch.bfloat16])
 @pytest.mark.parametrize("layout", ["bhnd", "bnhd"])
@@ -131,3 +199,8 @@ def test_plain_calls_and_calls_with_outputs_agree(lib, dtype, layout, per_head):
     assert ei.value.code == -2
     with pytest.raises(ValueError):
         binding.flurka_forward(Q, K, V, E, F, W, PERFORMER, layout="nbhd")
+    with pytest.raises(RuntimeError):
+        torch.func.vmap(lambda q: binding.flurka_forward(q, K, V, E, F, W, PERFORMER, layout=layout))(torch.stack([Q, Q]))
+    for q, do in ((Q, dO), (dO, Q)):
+        with pytest.raises(RuntimeError):
+            torch.func.grad(lambda x: binding.flurka_backward(x, K, V, E, F, W, do, PERFORMER, layout=layout)[0].sum())(q)
