@@ -73,8 +73,8 @@ __device__ __forceinline__ float k2_ex2(float x) {
 __device__ __forceinline__ void st_shared_v2(uint32_t addr, uint32_t a, uint32_t b) {
   asm volatile("st.shared.v2.b32 [%0], {%1, %2};" ::"r"(addr), "r"(a), "r"(b) : "memory");
 }
-// kCols consecutive values of a feature's a, as two bf16 terms `term` elements apart
-template <int kCols>
+// kCols consecutive values of a feature's a, as two bf16 terms `term` elements apart (kInf: an infinite one has no low term)
+template <int kCols, bool kInf = false>
 __device__ __forceinline__ void k2_store_split(__nv_bfloat16* dst, size_t term, const float (&v)[kCols]) {
 #pragma unroll
   for (int c = 0; c < kCols; c += 8) {
@@ -83,7 +83,12 @@ __device__ __forceinline__ void k2_store_split(__nv_bfloat16* dst, size_t term, 
     for (int e = 0; e < 4; ++e) {
       const float x = v[c + 2 * e], y = v[c + 2 * e + 1];
       hi[e] = pack_bf16x2(x, y);
-      lo[e] = pack_bf16x2(x - __uint_as_float(hi[e] << 16), y - __uint_as_float(hi[e] & 0xffff0000u));
+      float rx = x - __uint_as_float(hi[e] << 16), ry = y - __uint_as_float(hi[e] & 0xffff0000u);
+      if (kInf) {
+        rx = isnan(rx) ? 0.f : rx;
+        ry = isnan(ry) ? 0.f : ry;
+      }
+      lo[e] = pack_bf16x2(rx, ry);
     }
     *reinterpret_cast<uint4*>(dst + c) = make_uint4(hi[0], hi[1], hi[2], hi[3]);
     *reinterpret_cast<uint4*>(dst + term + c) = make_uint4(lo[0], lo[1], lo[2], lo[3]);
@@ -438,6 +443,25 @@ k2_key_side(const __grid_constant__ CUtensorMap tmW, const K2Params prm) {
     tmem_wait_ld(r);
 #pragma unroll
     for (int c = 0; c < kColsPer; ++c) acc[c] = __uint_as_float(r[c]);
+    if constexpr (kSplit) {
+      // an infinite V' has no low term (inf - inf), and times a low weight it may have either sign: such a sum is formed in fp32
+      bool odd = false;
+#pragma unroll
+      for (int c = 0; c < kColsPer; ++c) odd |= isnan(acc[c]);
+      if (odd && i0 + frow < p) {
+        float sum[kColsPer];
+#pragma unroll
+        for (int c = 0; c < kColsPer; ++c) sum[c] = 0.f;
+#pragma unroll 1
+        for (int j = 0; j < k; ++j) {
+          const float x = __ldcg(Kp + (size_t)j * kD + i0 + frow), f = fmaxf(x, 0.f) + __expf(fminf(x, 0.f));
+#pragma unroll
+          for (int c = 0; c < kColsPer; ++c) sum[c] = fmaf(f, __ldcg(Vp + (size_t)j * kD + qd * kColsPer + c), sum[c]);
+        }
+#pragma unroll
+        for (int c = 0; c < kColsPer; ++c) acc[c] = isnan(acc[c]) ? sum[c] : acc[c];
+      }
+    }
   }
 
   if (tid == 0) grid_launch_dependents();   // only the write-out (and the merge) is left
@@ -447,7 +471,8 @@ k2_key_side(const __grid_constant__ CUtensorMap tmW, const K2Params prm) {
     // through shared memory (the K' terms are free by now): a [d][128] fp16 tile, then 16 bytes at a time, so that
     // a^T leaves in whole 128- or 256-byte runs
     if (ok) {
-      const float inv = 1.f / zsum;
+      // (RNN: z_i = 0 where every weight has underflowed; ragged lengths then have a_i = 0, as the CUDA-core kernels do)
+      const float inv = 1.f / (kSplit ? fmaxf(zsum, 1.17549435e-38f) : zsum);
       if (qd == 0 && feat < p) prm.weight[(size_t)head * p + feat] = kPerformer ? run_max + (kSplit ? logf(zsum) : __logf(zsum)) : zsum;
       __half* tile = reinterpret_cast<__half*>(base_ptr + kK2K3) + (size_t)(qd * kColsPer) * 128 + frow;
 #pragma unroll
@@ -461,7 +486,7 @@ k2_key_side(const __grid_constant__ CUtensorMap tmW, const K2Params prm) {
         for (int c = 0; c < kColsPer; c += 4) arow[c >> 2] = make_float4(acc[c], acc[c + 1], acc[c + 2], acc[c + 3]);
       }
       if (prm.abf && feat < p)
-        k2_store_split(prm.abf + ((size_t)head * 2 * p + feat) * kD + qd * kColsPer, (size_t)p * kD, acc);
+        k2_store_split<kColsPer, kSplit && !kPerformer>(prm.abf + ((size_t)head * 2 * p + feat) * kD + qd * kColsPer, (size_t)p * kD, acc);
     }
     __syncthreads();
     if (ok && prm.aT16) {

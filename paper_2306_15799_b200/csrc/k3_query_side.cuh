@@ -40,6 +40,7 @@ struct K3Params {
   const float* weight;      // [BH][p]  b_i or z_i
   __nv_bfloat16* out;       // [BH][N][d]
   int wide;                 // out is 32-byte aligned
+  const __nv_bfloat16* abf; // [BH][2][p][d]  a as two bf16 terms (kSplit)
   int* status;
 };
 
@@ -72,7 +73,7 @@ __host__ __device__ inline K3Smem k3_smem_plan(int d, int p, bool performer, boo
   s.q_stages = k3_groups(d);
   s.q = off;    off += (uint32_t)s.q_stages * 128 * d * 2;
   s.ostage = off; off += (d == 64) ? 16 * 4096 : 0;                // d = 64: a [32 x 64] bf16 output slab per row-owner warp
-  s.scale = off; off += 1024;                                      // RNN: z_i / max z as floats
+  s.scale = off; off += 1024;                                      // RNN: z_i / max z as floats; split: infinite columns of a
   s.bars = off; off += 512;
   s.total = off + 1024;                                            // alignment slack
   return s;
@@ -330,6 +331,11 @@ k3_query_side(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ C
           }
         }
         const float* wv = prm.weight + (size_t)head * p;
+        [[maybe_unused]] float a0[kSplit ? kD / 32 : 1];           // a of the first feature
+        if constexpr (kSplit) {
+#pragma unroll
+          for (int q = 0; q < kD / 32; ++q) a0[q] = __bfloat162float(__ldcg(prm.abf + (size_t)head * 2 * p * d + q * 32 + lane));
+        }
         float mx = -INFINITY;
         for (int f = lane; f < p; f += 32) mx = fmaxf(mx, wv[f]);
 #pragma unroll
@@ -354,6 +360,27 @@ k3_query_side(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ C
           float* sc = reinterpret_cast<float*>(base_ptr + L.scale);
           const float inv = 1.f / mx;
           for (int f = lane; f < p; f += 32) sc[f] = wv[f] * inv;
+          if constexpr (kSplit) {
+            uint32_t* odd = reinterpret_cast<uint32_t*>(sc) + 128 + events % (2 * kGroups) * (d / 8);
+            uint32_t any = 0u;
+#pragma unroll
+            for (int q = 0; q < kD / 32; ++q) {
+              uint32_t plus = 0u, minus = 0u;
+              if (__ballot_sync(0xffffffffu, isinf(a0[q]))) {
+                const __nv_bfloat16* ah = prm.abf + (size_t)head * 2 * p * d + q * 32 + lane;
+                bool all = isinf(a0[q]);
+                for (int f = 1; f < p; ++f) all = all && __bfloat162float(__ldcg(ah + (size_t)f * d)) == a0[q];
+                plus = __ballot_sync(0xffffffffu, all && a0[q] > 0.f);
+                minus = __ballot_sync(0xffffffffu, all && a0[q] < 0.f);
+              }
+              if (lane == 0) {
+                odd[4 + 2 * q] = plus;
+                odd[5 + 2 * q] = minus;
+              }
+              any |= plus | minus;
+            }
+            if (lane == 0) odd[0] = any;
+          }
           __syncwarp();
           if (lane == 0) {
             __threadfence_block();
@@ -376,7 +403,25 @@ k3_query_side(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ C
       // read-out of tile j: O / sum -> bf16 -> the output rows
       // (head and first row of the tile are tracked by the caller: no divisions on this path)
       const uint32_t slab = base + L.ostage + (uint32_t)(warp - 4) * 4096u;
-      auto read_out = [&](int j, float inv, int head, int row0) -> bool {
+      // kSplit: columns in which a is infinite, for an infinite V' has (all features with one sign: every weight is > 0).  The low
+      // terms' products make them NaN, here they become infinite again, but for rows whose sum of weights is no number.
+      // Words of the head, behind the scales: any; 4 + 2 q, 5 + 2 q: +, - of column block q.  As many heads as the tiles
+      // in flight can belong to, twice.
+      auto infinite_columns = [&](uint32_t (&ra)[32], uint32_t (&rb)[32], int c, float sum) {
+        if constexpr (kSplit) {
+          const uint32_t* odd = reinterpret_cast<const uint32_t*>(base_ptr + L.scale) + 128 + (events - 1) % (2 * kGroups) * (d / 8);
+          if (odd[0] != 0u && sum < INFINITY) {
+            const uint4 w = *reinterpret_cast<const uint4*>(odd + 4 + (c >> 4));
+#pragma unroll
+            for (int e = 0; e < 32; ++e) {
+              ra[e] = (w.x >> e & 1u) ? 0x7f800000u : ((w.y >> e & 1u) ? 0xff800000u : ra[e]);
+              rb[e] = (w.z >> e & 1u) ? 0x7f800000u : ((w.w >> e & 1u) ? 0xff800000u : rb[e]);
+            }
+          }
+        }
+      };
+      auto read_out = [&](int j, float sum, int head, int row0) -> bool {
+        const float inv = 1.f / fmaxf(sum, 1.17549435e-38f);
         const int buf = j & (NB - 1);
         const uint32_t tb = tmem + buf * buf_cols + lane_off + o_col;
         if (!mbar_wait(bar_ofull + 8 * buf, (j >> nb_shift) & 1, prm.status, &abort_flag)) return false;
@@ -393,6 +438,7 @@ k3_query_side(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ C
           tmem_wait_ld(ra);
           tmem_wait_ld(rb);
           tcgen05_fence_before();
+          infinite_columns(ra, rb, 0, sum);
 #pragma unroll
           for (int g = 0; g < 8; ++g) {
             const uint32_t* src = g < 4 ? ra : rb;
@@ -430,6 +476,7 @@ k3_query_side(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ C
             tcgen05_fence_before();
             mbar_arrive(bar_sfree + 8 * buf);
           }
+          infinite_columns(ra, rb, c, sum);
 #pragma unroll
           for (int g8 = 0; g8 < 4; ++g8) {
             const uint32_t* src = g8 < 2 ? ra : rb;
@@ -613,8 +660,7 @@ k3_query_side(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ C
         hand_over(buf, kp - 1);                         // the last block of the tile
         if (kArrivals == 4 && lane == 0) mbar_arrive(bar_qempty + 8 * st);     // this warp is done with it
 
-        const float inv = 1.f / fmaxf(denom + denom1, 1.17549435e-38f);
-        ok = read_out(i, inv, head, row0);
+        ok = read_out(i, denom + denom1, head, row0);
         tih += kGroups;
         while (tih >= prm.tiles_per_head) { tih -= prm.tiles_per_head; ++head_i; }
       }

@@ -491,6 +491,7 @@ inline int launch_k3(TensorContext& tc, bool performer, const void* Q, const voi
   prm.total_tiles = prm.tiles_per_head * BH;
   prm.weight = weight;
   prm.out = reinterpret_cast<__nv_bfloat16*>(out);
+  prm.abf = abf;
   prm.wide = ((uintptr_t)out & 31) == 0;
   prm.status = status;
   // PERFORMER, d = 64: four tiles at a time (64 columns of S and 64 of O each fill TMEM; with d = 128 O alone would)

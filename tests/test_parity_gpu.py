@@ -662,6 +662,38 @@ def test_ragged_lengths_keep_32_bit_weights(w, limit, scale):
     assert moved <= 2.0 ** -7 * total, "%s: %.5f of the elements moved" % (w.name, moved / total)
 
 
+@pytest.mark.parametrize("limit", [0, 2])
+@pytest.mark.parametrize("d,H,k", [(64, 5, 64), (128, 4, 64)])
+def test_infinities_at_ragged_lengths_stay_in_their_columns(d, H, k, limit):
+    """RNN, weights and values as two bf16 terms on tensor cores: an infinite V (under projections that are positive) makes its
+    column of the output infinite, in its head; K = -inf takes its feature out (weight 0)."""
+    from paper_2306_15799_b200.configs import Workload
+    w = Workload("rnn_infinities_d%d" % d, RNN, "bf16", 1, H, 1027, d, k, 0, 471)
+    x = synth.make_inputs(w)
+    for name in ("E", "F"):
+        x[name] = (x[name].abs() + 0.01) / 16
+    x["V"][0, 0, 7, 3], x["V"][0, H - 1, 1020, d - 1], x["V"][0, 1, 500, 33] = float("inf"), float("-inf"), float("-inf")
+    x["K"][0, 2, 100, 5] = float("-inf")
+    prev = binding.flurka_set_cta_limit(limit)
+    try:
+        got = pu.run_gpu(w, x).cpu().double()[0]
+        assert binding.flurka_last_path() == binding.PATH_TENSOR_STAGE1
+    finally:
+        binding.flurka_set_cta_limit(prev)
+    E, F = x["E"].double(), x["F"].double()
+    for h in range(H):
+        Q, K, V = (x[n][0, h].double() for n in ("Q", "K", "V"))
+        inf = torch.isinf(V).any(0)
+        assert inf.sum() == (1 if h in (0, 1, H - 1) else 0)
+        keep = ~torch.isinf(K).any(0)
+        phi = lambda t: torch.nn.functional.elu(t) + 1
+        f, q = phi(E @ K)[:, keep], phi(Q)[:, keep]
+        ref = q @ (f.T @ (F @ torch.where(torch.isinf(V), 0.0, V))) / (q @ f.sum(0, keepdim=True).T)
+        want = torch.where(torch.isinf(V), V, 0.0).sum(0)[inf]
+        assert (got[h][:, inf] == want).all(), h
+        pu.assert_close(got[h][:, ~inf].numpy(), ref[:, ~inf].numpy(), "bf16", "head %d" % h)
+
+
 @pytest.mark.parametrize("per_head", [False, True])
 def test_ragged_call_in_a_workspace_sized_at_another_length(per_head):
     """Scratch without the copies of E, F does not depend on N (and not on whether E, F are shared): a block of the size
