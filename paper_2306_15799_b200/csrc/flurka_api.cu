@@ -1108,15 +1108,11 @@ int backward_pipeline(const Problem& pr, const BackwardLayout& BL, char* ws, con
     ++*launches;
   }
   __nv_bfloat16* split = tc ? (__nv_bfloat16*)(ws + BL.split) : nullptr;
-  // d = 64 with at most two blocks of features and few keys: the CUDA-core kernel's CTAs of 32 keys are one wave, and its chain
-  // is shorter (us per call, CUDA cores / k10: 8 heads, k = 128, m = 64, N = 5695 68.2 / 70.2, 4 heads, k = 128, m = 64, N = 1283
-  // 48.7 / 50.6; two waves, 96 heads, k = m = 64, N = 515 84.7 / 80.6; four blocks, 16 heads, k = m = 256, N = 6001 158 / 148)
-  const bool few_keys = pr.d == 64 && pr.p() <= 128 && pr.BH() * (pr.k / 32) <= device_sms();
   if (tcq && P && pr.d == 64 && !ragged(pr)) {
     rc = launch_k6(*tc, W, kpvp, weight, da, ei, split, pr.BH(), pr.k, pr.p(), (int*)(ws + L.status), st, &cuda_err);
     if (rc) { g_last_cuda_error = cuda_err; return rc; }
     ++*launches;
-  } else if (tcq && P && !few_keys) {
+  } else if (tcq && P) {
     rc = launch_k10(*tc, W, kpvp, weight, da, ei, split, pr.BH(), pr.d, pr.k, pr.p(), (int*)(ws + L.status), st, &cuda_err);
     if (rc) { g_last_cuda_error = cuda_err; return rc; }
     ++*launches;

@@ -1,14 +1,14 @@
-// Backward of the key side on tensor cores for PERFORMER where its weights are kept in 32 bits: d = 128, and ragged lengths
+// Backward of the key side on tensor cores for PERFORMER where its arithmetic keeps 24 bits: d = 128, and ragged lengths
 // (k a multiple of 64 up to 512, p = 64 .. 256).  The formulas are those of k6_bwd_key_side.cuh, which rounds A and dL to bf16.
 //
 // A CTA owns 128 projected keys of a head and walks the features 64 at a time with a key per lane: L = K' W^T and T = V' da^T
-// have a feature per column, so that A and dL go back over them as two bf16 terms each and are the A operands of dV' += A da
-// and dK' += dL W from TMEM, and what belongs to a key (|k'|^2 / 2, the sum of its dL) stays with the two threads that share
-// it.  K' is three bf16 terms (the exponent needs 24 bits); V', da three with d = 64, two with d = 128 (shared memory is full,
-// and the P, c behind that da are bf16).
-// What bounds it is the chain of a block of features: L, exponentials, two products; da is converted under L's products and T
-// formed under the exponentials.  The CUDA-core kernel it stands for -> this, us per call: d = 128, 64 heads, k = 256, m = 128
-// 228 -> 180, 16 heads with their own E, F, k = 512, m = 256 215 -> 144; N = 2003, 64 heads, k = 512, m = 256 330 -> 217.
+// have a feature per column, so that A and dL go back into TMEM as A operands of dV' += A da and dK' += dL W, and what belongs
+// to a key (d = 128: |k'|^2 / 2; the sum of its dL) stays with the two threads that share it.
+// Everything but W (bf16, exact) is three bf16 terms, fp32's 24 bits, and a product of two such is the six pairs of terms down to
+// 2^-24.  With d = 128 shared memory holds two terms of V' and TMEM the third (T's A operand may lie in either).
+// What bounds it is the chain of a block of features: L, exponentials, two products; da is converted under L's products, T formed
+// under the exponentials, dV' under what is done with T.  us per launch, the CUDA-core kernel / two terms of everything but K' / this: 16
+// heads, d = 128, k = 512, m = 256 104 / 31.9 / 36.7; 8 heads, d = 64, k = m = 256 29 / 18.2 / 19.0.
 #pragma once
 
 #include <cuda_bf16.h>
@@ -22,31 +22,19 @@ namespace flurka {
 constexpr int kK10Threads = 256, kK10Feats = 64;
 template <int kD> struct K10Shape {
   static constexpr uint32_t kBlocks = kD / 64;               // blocks of 64 columns
-  static constexpr uint32_t kTerms = kD == 64 ? 3 : 2;       // of V' and da
-  static constexpr uint32_t kVBlock = kTerms * 16384, kABlock = kTerms * 8192;
+  static constexpr uint32_t kVTerms = kD == 64 ? 3 : 2;      // of V' in shared memory
+  static constexpr uint32_t kVBlock = kVTerms * 16384, kABlock = 3 * 8192;
   // shared memory: per block of columns the terms of K' and V' ([128 x 64]), W and the terms of da ([64 x 64])
   static constexpr uint32_t k3 = 0, v = kBlocks * 49152, w = v + kBlocks * kVBlock, da = w + kBlocks * 8192,
-                            be = da + kBlocks * kABlock,     // b_i, e_i of every feature
-                            nrm = be + 2048,                 // |k'_j|^2 / 2
-                            sum = nrm + 512,                 // [2][128] sums of dL
-                            bars = sum + 1024;
+                            be = da + kBlocks * kABlock,     // b_i, e_i of the block's features
+                            nrm = be + 512,                  // |k'_j|^2 / 2: d = 64 as an operand [128 x 16] of L, and [64 x 16] of ones
+                            sum = be,                        // at the end: [2][128] sums of dL
+                            bars = nrm + (kD == 64 ? 6144 : 512);
   static constexpr int bytes = (int)bars + 64 + 1024;
-  // TMEM columns: L, then A; T, then dL (a thread's 32 columns become 16 of high and 16 of low terms); dV'; dK'
-  static constexpr uint32_t kColT = 64, kColDV = 128, kColDK = 128 + kD, kCols = kD == 64 ? 256 : 512;
+  // TMEM columns: L, then A; T, then dL (a thread's 32 columns become 16 of each of two terms); the third terms of A and of dL;
+  // d = 128: that of V'; dV'; dK'
+  static constexpr uint32_t kColT = 64, kColA3 = 128, kColDL3 = 160, kColV3 = 192, kColDV = 256, kColDK = 256 + kD, kCols = 512;
 };
-
-// four fp32 values of a row -> `terms` bf16 terms, tiles of [.. x 64] K-major, 128-byte-swizzled, kStride bytes apart
-template <int kTerms, uint32_t kStride>
-__device__ __forceinline__ void k10_split_store(uint32_t tile0, int r, int c4, float4 x) {
-  const uint32_t off = tile0 + (uint32_t)r * 128u + ((((uint32_t)c4 >> 3) ^ ((uint32_t)r & 7u)) << 4) + (((uint32_t)c4 & 4u) << 1);
-#pragma unroll
-  for (int t = 0; t < kTerms; ++t) {
-    const uint32_t h0 = k6_bf16x2(x.x, x.y), h1 = k6_bf16x2(x.z, x.w);
-    asm volatile("st.shared.v2.b32 [%0], {%1, %2};" ::"r"(off + (uint32_t)t * kStride), "r"(h0), "r"(h1) : "memory");
-    x.x -= __uint_as_float(h0 << 16); x.y -= __uint_as_float(h0 & 0xffff0000u);
-    x.z -= __uint_as_float(h1 << 16); x.w -= __uint_as_float(h1 & 0xffff0000u);
-  }
-}
 
 template <int kD>
 __global__ void __launch_bounds__(kK10Threads, 1)
@@ -87,9 +75,11 @@ k10_bwd_key_performer(const __grid_constant__ CUtensorMap tmW, const K6Params pr
   const int r0 = tid / kLpr, ccol = tid % kLpr * 4;
   const float* __restrict__ dah = prm.da + ((size_t)head * p + r0) * kD + ccol;
   float4 xd[kPerA], y[kPer];
+  float xbe = 0.f;                                           // b_i (threads 0..63) or e_i (64..127)
   auto load_da = [&](int i0) {
 #pragma unroll
     for (int u = 0; u < kPerA; ++u) xd[u] = __ldcg(reinterpret_cast<const float4*>(dah + (size_t)(i0 + u * kStep) * kD));
+    if (tid < 128) xbe = __ldcg((tid < 64 ? prm.weight : prm.ei) + (size_t)head * p + i0 + (tid & 63));
   };
   {
     const float* Kp = prm.kpvp + ((size_t)head * k + j0 + r0) * kD + ccol;
@@ -102,21 +92,31 @@ k10_bwd_key_performer(const __grid_constant__ CUtensorMap tmW, const K6Params pr
       y[u] = r0 + u * kStep < keys ? __ldcg(reinterpret_cast<const float4*>(Vp + (size_t)u * kStep * kD)) : zero;
     }
     load_da(0);
-    float* be = reinterpret_cast<float*>(base_ptr + L::be);
-    if (tid < p) {
-      be[tid] = __ldcg(prm.weight + (size_t)head * p + tid);
-      be[256 + tid] = __ldcg(prm.ei + (size_t)head * p + tid);
-    }
-    float* nrm = reinterpret_cast<float*>(base_ptr + L::nrm);
+    if (kD == 64 && tid < 128)                               // (element (r, c) at (r/8)*256 + (c/8)*128 + (r%8)*16 + (c%8)*2 bytes)
+      reinterpret_cast<uint4*>(base_ptr + L::nrm + 4096)[tid] = (tid & 8) ? make_uint4(0u, 0u, 0u, 0u) : make_uint4(0x3f803f80u, 0x3f80u, 0u, 0u);
 #pragma unroll
     for (int u = 0; u < kPer; ++u) {
       const int r = r0 + u * kStep;
-      k10_split_store<3, 16384>(base + L::k3 + (uint32_t)(ccol >> 6) * 49152u, r, ccol & 63, x[u]);
-      // as the forward's key side adds them up, rounding for rounding: its error then cancels between L_ij and b_i
+      k6_split_store<3>(base + L::k3 + (uint32_t)(ccol >> 6) * 49152u, r, ccol & 63, x[u]);
+      // as the forward's key side adds them up, rounding for rounding: its error then cancels between L_ij and b_i.  d = 64: so does
+      // that of L, which is formed from the same operands in the same order (d = 128 has no room for these, and its P, c, rounded
+      // to bf16, cost more)
       float sq = fmaf(x[u].x, x[u].x, fmaf(x[u].y, x[u].y, fmaf(x[u].z, x[u].z, x[u].w * x[u].w)));
 #pragma unroll
       for (int o = kLpr / 2; o > 0; o >>= 1) sq += __shfl_xor_sync(0xffffffffu, sq, o);
-      if (ccol == 0) nrm[r] = 0.5f * sq;
+      if (ccol == 0) {
+        if constexpr (kD == 64) {
+          const float n0 = -0.5f * sq;
+          const uint32_t t0 = k6_bf16x2(n0, 0.f);
+          const float n1 = n0 - __uint_as_float(t0 << 16);
+          const uint32_t t1 = k6_bf16x2(n1, 0.f);
+          uint4* op = reinterpret_cast<uint4*>(base_ptr + L::nrm + (r >> 3) * 256 + (r & 7) * 16);
+          op[0] = make_uint4(t0 | t1 << 16, k6_bf16x2(n1 - __uint_as_float(t1 << 16), 0.f), 0u, 0u);
+          op[8] = make_uint4(0u, 0u, 0u, 0u);
+        } else {
+          reinterpret_cast<float*>(base_ptr + L::nrm)[r] = 0.5f * sq;
+        }
+      }
     }
   }
   fence_proxy_async_smem();
@@ -134,26 +134,34 @@ k10_bwd_key_performer(const __grid_constant__ CUtensorMap tmW, const K6Params pr
   const int q4 = warp & 3, h = warp >> 2, row = q4 * 32 + lane;
   const uint32_t lane_base = tmem + ((uint32_t)(q4 * 32) << 16) + (uint32_t)h * 32u;
   const bool live = row < keys;
-  const float nj = reinterpret_cast<const float*>(base_ptr + L::nrm)[row];
+  const float nj = kD == 64 ? 0.f : reinterpret_cast<const float*>(base_ptr + L::nrm)[row];
   const float* be = reinterpret_cast<const float*>(base_ptr + L::be) + h * 32;
   float s_j = 0.f;
   bool ok = true;
   uint32_t phase = 0;
   constexpr uint32_t idescT = make_idesc(kFmtBF16, 0, 0, 128, kK10Feats);     // L, T: both operands K-major along d
   constexpr uint32_t idescO = make_idesc(kFmtBF16, 0, 1, 128, kD);            // dV', dK'
-  // T: the pairs of terms (a term's weight is 2^-8 of the one before); what is left out is below 2^-24, with two terms 2^-16
-  constexpr int kPairs = L::kTerms == 3 ? 6 : 3;
+  // the pairs of terms (a term's weight is 2^-8 of the one before); what is left out is below 2^-24
   constexpr uint32_t kTa[6] = {0, 0, 1, 1, 0, 2}, kTb[6] = {0, 1, 0, 1, 2, 0};
-  // 32 values -> their high and low terms over the 32 columns they came from
-  auto put_terms = [&](uint32_t col, const float (&x)[32]) {
-    uint32_t hi[16], lo[16];
+  // 32 values -> two terms over the 32 columns they came from, the third into 16 columns at `col3`
+  auto put_terms = [&](uint32_t col, uint32_t col3, const float (&x)[32]) {
+    uint32_t t0[16], t1[16], t2[16];
 #pragma unroll
     for (int e = 0; e < 16; ++e) {
-      hi[e] = k6_bf16x2(x[2 * e], x[2 * e + 1]);
-      lo[e] = k6_bf16x2(x[2 * e] - __uint_as_float(hi[e] << 16), x[2 * e + 1] - __uint_as_float(hi[e] & 0xffff0000u));
+      float a = x[2 * e], b = x[2 * e + 1];
+      t0[e] = k6_bf16x2(a, b);
+      a -= __uint_as_float(t0[e] << 16); b -= __uint_as_float(t0[e] & 0xffff0000u);
+      t1[e] = k6_bf16x2(a, b);
+      a -= __uint_as_float(t1[e] << 16); b -= __uint_as_float(t1[e] & 0xffff0000u);
+      t2[e] = k6_bf16x2(a, b);
     }
-    tmem_st16(lane_base + col, hi);
-    tmem_st16(lane_base + col + 16, lo);
+    tmem_st16(lane_base + col, t0);
+    tmem_st16(lane_base + col + 16, t1);
+    tmem_st16(lane_base + col3 - (uint32_t)h * 16u, t2);
+  };
+  // the columns of a term of 16 features of A or dL: (column of the values, of their third term) -> step `half` of 2
+  auto term_at = [&](uint32_t col, uint32_t col3, uint32_t t, uint32_t half) {
+    return tmem + (t == 2 ? col3 + half * 16u : col + half * 32u + t * 16u);
   };
 
   for (int i0 = 0; i0 < p; i0 += kK10Feats, phase ^= 1) {
@@ -168,6 +176,8 @@ k10_bwd_key_performer(const __grid_constant__ CUtensorMap tmW, const K6Params pr
           for (uint32_t cb = 0; cb < L::kBlocks; ++cb)
             mma_ss_x4(tmem, make_sdesc(base + L::k3 + cb * 49152u + t * 16384u, 16, 1024, kSwizzle128),
                       make_sdesc(base + L::w + cb * 8192u, 16, 1024, kSwizzle128), 2, 2, idescT, t > 0 || cb > 0 ? 1u : 0u);
+        if (kD == 64)
+          mma_ss(tmem, make_sdesc(base + L::nrm, 128, 256, kSwizzleNone), make_sdesc(base + L::nrm + 4096, 128, 256, kSwizzleNone), idescT, 1u);
         mma_commit(bar_l);
       }
       __syncwarp();
@@ -175,12 +185,32 @@ k10_bwd_key_performer(const __grid_constant__ CUtensorMap tmW, const K6Params pr
     // ---- V' (once) and the block's da -> bf16 terms, under those products
     if (i0 == 0) {
 #pragma unroll
-      for (int u = 0; u < kPer; ++u)
-        k10_split_store<L::kTerms, 16384>(base + L::v + (uint32_t)(ccol >> 6) * L::kVBlock, r0 + u * kStep, ccol & 63, y[u]);
+      for (int u = 0; u < kPer; ++u) {
+        const float4 rest = k6_split_store<L::kVTerms>(base + L::v + (uint32_t)(ccol >> 6) * L::kVBlock, r0 + u * kStep, ccol & 63, y[u]);
+        // d = 128: the third term goes to its rows' threads through the place of da
+        if (L::kVTerms == 2) k6_split_store<1>(base + L::da + (uint32_t)(ccol >> 6) * 16384u, r0 + u * kStep, ccol & 63, rest);
+      }
+      if constexpr (L::kVTerms == 2) {
+        __syncthreads();
+        const uint32_t at = base + L::da + (uint32_t)h * 16384u + (uint32_t)row * 128u;
+#pragma unroll
+        for (uint32_t c = 0; c < 8; c += 2) {
+          uint32_t low[8];
+#pragma unroll
+          for (uint32_t e = 0; e < 2; ++e)
+            asm volatile("ld.shared.v4.b32 {%0, %1, %2, %3}, [%4];" : "=r"(low[4 * e]), "=r"(low[4 * e + 1]), "=r"(low[4 * e + 2]),
+                         "=r"(low[4 * e + 3]) : "r"(at + (((c + e) ^ ((uint32_t)row & 7u)) << 4)) : "memory");
+          tmem_st8(lane_base + L::kColV3 + c * 4, low);
+        }
+        tmem_wait_st();
+        tcgen05_fence_before();
+        __syncthreads();
+      }
     }
 #pragma unroll
     for (int u = 0; u < kPerA; ++u)
-      k10_split_store<L::kTerms, 8192>(base + L::da + (uint32_t)(ccol >> 6) * L::kABlock, r0 + u * kStep, ccol & 63, xd[u]);
+      k6_split_store<3, 8192>(base + L::da + (uint32_t)(ccol >> 6) * L::kABlock, r0 + u * kStep, ccol & 63, xd[u]);
+    if (tid < 128) reinterpret_cast<float*>(base_ptr + L::be)[tid] = xbe;
     if (i0 + kK10Feats < p) load_da(i0 + kK10Feats);
     fence_proxy_async_smem();
     ok = __syncthreads_and(ok) != 0;
@@ -188,11 +218,15 @@ k10_bwd_key_performer(const __grid_constant__ CUtensorMap tmW, const K6Params pr
     if (warp == 0 && elect_one()) {
       tcgen05_fence_after();
 #pragma unroll
-      for (int t = 0; t < kPairs; ++t)
-        for (uint32_t cb = 0; cb < L::kBlocks; ++cb)
-          mma_ss_x4(tmem + L::kColT, make_sdesc(base + L::v + cb * L::kVBlock + kTa[t] * 16384u, 16, 1024, kSwizzle128),
-                    make_sdesc(base + L::da + cb * L::kABlock + kTb[t] * 8192u, 16, 1024, kSwizzle128), 2, 2, idescT,
-                    t > 0 || cb > 0 ? 1u : 0u);
+      for (int t = 0; t < 6; ++t)
+        for (uint32_t cb = 0; cb < L::kBlocks; ++cb) {
+          const uint64_t bd = make_sdesc(base + L::da + cb * L::kABlock + kTb[t] * 8192u, 16, 1024, kSwizzle128);
+          if (kTa[t] >= L::kVTerms)
+            mma_ts_x4(tmem + L::kColT, tmem + L::kColV3 + cb * 32u, bd, 2, idescT, 1u);
+          else
+            mma_ss_x4(tmem + L::kColT, make_sdesc(base + L::v + cb * L::kVBlock + kTa[t] * 16384u, 16, 1024, kSwizzle128), bd, 2, 2,
+                      idescT, t > 0 || cb > 0 ? 1u : 0u);
+        }
       mma_commit(bar_t);
     }
     __syncwarp();
@@ -204,9 +238,26 @@ k10_bwd_key_performer(const __grid_constant__ CUtensorMap tmW, const K6Params pr
       tmem_ld32(lane_base, r);
       tmem_wait_ld(r);
 #pragma unroll
-      for (int e = 0; e < 32; ++e) A[e] = expf(__uint_as_float(r[e]) - nj - be[i0 + e]);      // b_i = log sum_j exp(L_ij): A <= 1
-      put_terms(0, A);
+      for (int e = 0; e < 32; ++e) A[e] = expf((kD == 64 ? __uint_as_float(r[e]) : __uint_as_float(r[e]) - nj) - be[e]);      // b_i = log sum_j exp(L_ij): A <= 1
+      put_terms(0, L::kColA3, A);
     }
+    tmem_wait_st();
+    tcgen05_fence_before();
+    ok = __syncthreads_and(ok) != 0;
+    if (!ok) break;
+    if (warp == 0 && elect_one()) {
+      // dV' comes behind T, under what is done with T.  (The rows of da and of W are the contraction, MN-major: 16 features = 2048 B
+      // per step.)
+      tcgen05_fence_after();
+#pragma unroll
+      for (int t = 0; t < 6; ++t)
+#pragma unroll
+        for (uint32_t half = 0; half < 2; ++half)
+          mma_ts_x2(tmem + L::kColDV, term_at(0, L::kColA3, kTa[t], half),
+                    make_sdesc(base + L::da + kTb[t] * 8192u + half * 4096u, L::kABlock, 1024, kSwizzle128), 128, idescO,
+                    i0 > 0 || t > 0 || half > 0 ? 1u : 0u);
+    }
+    __syncwarp();
     ok = mbar_wait(bar_t, phase, prm.status, &abort_flag) && ok;
     tcgen05_fence_after();
     {
@@ -215,10 +266,10 @@ k10_bwd_key_performer(const __grid_constant__ CUtensorMap tmW, const K6Params pr
       tmem_wait_ld(r);
 #pragma unroll
       for (int e = 0; e < 32; ++e) {
-        A[e] *= __uint_as_float(r[e]) + be[256 + i0 + e];
+        A[e] *= __uint_as_float(r[e]) + be[64 + e];
         s_j += A[e];
       }
-      put_terms(L::kColT, A);
+      put_terms(L::kColT, L::kColDL3, A);
     }
     tmem_wait_st();
     tcgen05_fence_before();
@@ -226,20 +277,11 @@ k10_bwd_key_performer(const __grid_constant__ CUtensorMap tmW, const K6Params pr
     if (!ok) break;
     if (warp == 0 && elect_one()) {
       tcgen05_fence_after();
-      // the rows of da and of W are the contraction (MN-major): 16 features = 2048 B per step.  A is two terms, so that
-      // what it is multiplied with needs no more: hi hi, hi lo, lo hi
 #pragma unroll
       for (uint32_t t = 0; t < 3; ++t)
 #pragma unroll
         for (uint32_t half = 0; half < 2; ++half)
-          mma_ts_x2(tmem + L::kColDV, tmem + half * 32u + (t == 2 ? 16u : 0u),
-                    make_sdesc(base + L::da + (t == 1 ? 8192u : 0u) + half * 4096u, L::kABlock, 1024, kSwizzle128), 128, idescO,
-                    i0 > 0 || t > 0 || half > 0 ? 1u : 0u);
-#pragma unroll
-      for (uint32_t t = 0; t < 2; ++t)
-#pragma unroll
-        for (uint32_t half = 0; half < 2; ++half)
-          mma_ts_x2(tmem + L::kColDK, tmem + L::kColT + half * 32u + t * 16u,
+          mma_ts_x2(tmem + L::kColDK, term_at(L::kColT, L::kColDL3, t, half),
                     make_sdesc(base + L::w + half * 4096u, 8192, 1024, kSwizzle128), 128, idescO,
                     i0 > 0 || t > 0 || half > 0 ? 1u : 0u);
       mma_commit(bar_o);

@@ -56,19 +56,20 @@ __device__ __forceinline__ float k6_ex2(float x) {
   return y;
 }
 
-// four fp32 values of a row -> `terms` bf16 terms, each into its own K-major 128-byte-swizzled [128 x 64] tile
-// (tiles 16384 B apart): row r, columns c4 .. c4 + 3
-template <int kTerms>
-__device__ __forceinline__ void k6_split_store(uint32_t tile0, int r, int c4, float4 x) {
+// four fp32 values of a row -> kTerms bf16 terms, each into its own K-major 128-byte-swizzled [.. x 64] tile
+// (tiles kStride bytes apart): row r, columns c4 .. c4 + 3; returns what they leave
+template <int kTerms, uint32_t kStride = 16384>
+__device__ __forceinline__ float4 k6_split_store(uint32_t tile0, int r, int c4, float4 x) {
   float a = x.x, b = x.y, c = x.z, e = x.w;
   const uint32_t off = tile0 + (uint32_t)r * 128u + ((((uint32_t)c4 >> 3) ^ ((uint32_t)r & 7u)) << 4) + (((uint32_t)c4 & 4u) << 1);
 #pragma unroll
   for (int t = 0; t < kTerms; ++t) {
     const uint32_t h0 = k6_bf16x2(a, b), h1 = k6_bf16x2(c, e);
-    asm volatile("st.shared.v2.b32 [%0], {%1, %2};" ::"r"(off + (uint32_t)t * 16384u), "r"(h0), "r"(h1) : "memory");
+    asm volatile("st.shared.v2.b32 [%0], {%1, %2};" ::"r"(off + (uint32_t)t * kStride), "r"(h0), "r"(h1) : "memory");
     a -= __uint_as_float(h0 << 16); b -= __uint_as_float(h0 & 0xffff0000u);
     c -= __uint_as_float(h1 << 16); e -= __uint_as_float(h1 & 0xffff0000u);
   }
+  return make_float4(a, b, c, e);
 }
 
 __global__ void __launch_bounds__(kK6Threads, 1)
