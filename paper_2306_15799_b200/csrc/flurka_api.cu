@@ -384,7 +384,7 @@ int run_pipeline_with(const Problem& pr, const Layout& L, char* ws, const void* 
   if (tc2) {
     float* part = L.total > L.part ? (float*)(ws + L.part) : nullptr;
     rc = launch_k2(*tc, performer, kpvp, W, weight, abf ? nullptr : aT16, part, status + 4, pr.BH(), pr.d, pr.k, pr.p(), status,
-                   st, &cuda_err, nullptr, abf, abf != nullptr, chained);
+                   st, &cuda_err, nullptr, abf, abf ? 2 : 0, chained);
     if (rc) { g_last_cuda_error = cuda_err; return rc; }
     ++*launches;
   } else {
@@ -1002,7 +1002,8 @@ BackwardLayout make_backward_layout(const Problem& pr) {
   b.efpad = off;
   off = align256(off + efpad_bytes(pr));
   b.abf = off;
-  if (backward_query_tensor_ok(pr)) off = align256(off + (size_t)2 * pr.BH() * pr.p() * pr.d * 2);   // a as two bf16 terms
+  if (backward_query_tensor_ok(pr))                                       // a as two or three bf16 terms
+    off = align256(off + (size_t)bwd_query_a_terms(pr.kernel == FLURKA_PERFORMER, ragged(pr)) * pr.BH() * pr.p() * pr.d * 2);
   b.total = off;
   return b;
 }
@@ -1081,7 +1082,8 @@ int backward_pipeline(const Problem& pr, const BackwardLayout& BL, char* ws, con
                       16 + pairs * 4 <= L.kpvp - L.status;
     rc = launch_k2(*tc, P, kpvp, W, weight, nullptr, room ? (float*)(ws + BL.dkpvp) : nullptr,
                    room ? (int*)(ws + L.status) + 4 : nullptr, pr.BH(), pr.d, pr.k, pr.p(), (int*)(ws + L.status), st,
-                   &cuda_err, tcq ? nullptr : a32, tcq ? (__nv_bfloat16*)(ws + BL.abf) : nullptr, ragged(pr));
+                   &cuda_err, tcq ? nullptr : a32, tcq ? (__nv_bfloat16*)(ws + BL.abf) : nullptr,
+                   ragged(pr) ? bwd_query_a_terms(P, true) : 0);
     if (rc) { g_last_cuda_error = cuda_err; return rc; }
     ++*launches;
   } else {

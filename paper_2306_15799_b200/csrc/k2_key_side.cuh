@@ -17,9 +17,12 @@
 // second product reads the weights from TMEM.  Several blocks: running maximum, accumulator in registers.  RNN: the
 // weights are the fp16 f tile as it lies ([key][feature], the MN-major A operand), and z_i comes from the same tile
 // times a column of ones.
-// kSplit serves sequence lengths whose weights are kept in 32 bits: weights and V' are two bf16 terms each, the low weights
-// where L was read from (RNN: a second f tile), three products instead of two (low x low is 2^-18), and a leaves as the two
-// bf16 terms that the query side reads.  bf16 has fp32's range, so V' may be as large as it may be on CUDA cores.
+// kTerms serves sequence lengths that are no multiple of 8: weights and V' are two bf16 terms each, 16 to 17 bits (the low
+// weights where L was read from; RNN: a second f tile), three products instead of two (low x low is 2^-18), and a leaves as the
+// two bf16 terms that the query side reads.  PERFORMER in the backward pass: three terms and six products, 24 bits, and a as
+// three terms, for with weights near 1 a gradient dL is a difference of nearly equal da.v' and da.a (one head, N = 30001,
+// k = m = 64: dK 2.9e-2 off with two terms, 3.7e-3 with three, 2.8e-3 on CUDA cores; the forward does not notice, and takes 0.8 us more).
+// bf16 has fp32's range, so V' may be as large as it may be on CUDA cores.
 // One block of 256 keys takes about 10 k cycles; the earlier form (eight warps, a staging copy and a block barrier per
 // 128 keys, one thread per row) took 17 us after stage 1's end at B H = 64, k = m = 256, d = 64, this one 9.
 //
@@ -43,7 +46,7 @@ struct K2Params {
   float* weight;            // [BH][p]      b_i (PERFORMER) or z_i (RNN)
   __half* aT16;             // [BH][d][p]   a^T, or NULL
   float* a32;               // [BH][p][d]   a in fp32 as well (the backward pass wants it), or NULL
-  __nv_bfloat16* abf;       // [BH][2][p][d]  a as two bf16 terms (the backward pass), or NULL
+  __nv_bfloat16* abf;       // [BH][abf_terms][p][d]  a as two bf16 terms (the backward pass; kTerms = 3: three), or NULL
   int* status;
   int nsplit;               // CTAs per (head, feature tile) along the keys (1..4; PERFORMER only)
   float* part;              // nsplit > 1: [BH * ftiles][nsplit][d + 2][128]  max, sum, accumulator columns
@@ -52,11 +55,15 @@ struct K2Params {
 
 constexpr int kK2Threads = 512;
 constexpr int kK2BlockElems = 16384;           // keys per block x d
-// shared memory: W tile (<= 32 KB) | ones 4 KB | -|k'|^2/2 tile 8 KB | three 32 KB terms of K' (RNN: f tile, zero slab)
-// | two 32 KB terms of V' | barriers
-constexpr uint32_t kK2Ones = 32768, kK2Nrm = 36864, kK2K3 = 45056, kK2V2 = kK2K3 + 3 * 32768, kK2Bars = kK2V2 + 2 * 32768;
-constexpr int kK2SmemBytes = kK2Bars + 64 + 1024;
-constexpr uint32_t kK2OCol = 256, kK2ZCol = 384;   // TMEM columns of the a accumulator and (RNN) of z
+// shared memory: W tile (<= 32 KB; kTerms = 3: 16) | ones 4 KB | -|k'|^2/2 tile 8 KB | three 32 KB terms of K' (RNN: f tile, zero
+// slab) | two or three 32 KB terms of V' | barriers
+template <int kTerms> struct K2Smem {
+  static constexpr uint32_t ones = kTerms == 3 ? 16384 : 32768, nrm = ones + 4096, k3 = nrm + 8192, v = k3 + 3 * 32768;
+  static constexpr uint32_t bars = v + (kTerms == 3 ? 3 : 2) * 32768;
+  static constexpr int bytes = (int)bars + 64 + 1024;
+};
+// TMEM columns of the a accumulator and of z (RNN) or the third terms of the weights (kTerms = 3)
+constexpr uint32_t kK2OCol = 256, kK2ZCol = 384;
 
 // two floats -> {lo: bf16(a), hi: bf16(b)} with one rounding instruction
 __device__ __forceinline__ uint32_t pack_bf16x2(float a, float b) {
@@ -73,9 +80,9 @@ __device__ __forceinline__ float k2_ex2(float x) {
 __device__ __forceinline__ void st_shared_v2(uint32_t addr, uint32_t a, uint32_t b) {
   asm volatile("st.shared.v2.b32 [%0], {%1, %2};" ::"r"(addr), "r"(a), "r"(b) : "memory");
 }
-// kCols consecutive values of a feature's a, as two bf16 terms `term` elements apart (kInf: an infinite one has no low term)
+// kCols consecutive values of a feature's a, as two bf16 terms `term` elements apart, or three (kInf: an infinite one has no low term)
 template <int kCols, bool kInf = false>
-__device__ __forceinline__ void k2_store_split(__nv_bfloat16* dst, size_t term, const float (&v)[kCols]) {
+__device__ __forceinline__ void k2_store_split(__nv_bfloat16* dst, size_t term, const float (&v)[kCols], bool third = false) {
 #pragma unroll
   for (int c = 0; c < kCols; c += 8) {
     uint32_t hi[4], lo[4];
@@ -92,15 +99,34 @@ __device__ __forceinline__ void k2_store_split(__nv_bfloat16* dst, size_t term, 
     }
     *reinterpret_cast<uint4*>(dst + c) = make_uint4(hi[0], hi[1], hi[2], hi[3]);
     *reinterpret_cast<uint4*>(dst + term + c) = make_uint4(lo[0], lo[1], lo[2], lo[3]);
+    if (third) {
+#pragma unroll
+      for (int e = 0; e < 4; ++e)
+        lo[e] = pack_bf16x2((v[c + 2 * e] - __uint_as_float(hi[e] << 16)) - __uint_as_float(lo[e] << 16),
+                            (v[c + 2 * e + 1] - __uint_as_float(hi[e] & 0xffff0000u)) - __uint_as_float(lo[e] & 0xffff0000u));
+      *reinterpret_cast<uint4*>(dst + 2 * term + c) = make_uint4(lo[0], lo[1], lo[2], lo[3]);
+    }
   }
+}
+// one bf16 term of four values into shared memory, and what it leaves.  Packed conversions: one instruction rounds two values;
+// a bf16 is the top half of an fp32
+__device__ __forceinline__ void k2_put_term(uint32_t addr, float4& v) {
+  const uint32_t h0 = pack_bf16x2(v.x, v.y), h1 = pack_bf16x2(v.z, v.w);
+  st_shared_v2(addr, h0, h1);
+  v.x -= __uint_as_float(h0 << 16); v.y -= __uint_as_float(h0 & 0xffff0000u);
+  v.z -= __uint_as_float(h1 << 16); v.w -= __uint_as_float(h1 & 0xffff0000u);
 }
 __device__ __forceinline__ uint32_t half2_bits(__half2 h) { return *reinterpret_cast<const uint32_t*>(&h); }
 
-// kSplit: weights and V' as two bf16 terms each, without the low x low product (see the header)
-template <bool kPerformer, int kD, bool kSplit = false>
+// kTerms: weights and V' as so many bf16 terms each (see the header); 0: fp16 weights, V' as two fp16 terms
+template <bool kPerformer, int kD, int kTerms = 0>
 __global__ void __launch_bounds__(kK2Threads, 1)
 k2_key_side(const __grid_constant__ CUtensorMap tmW, const K2Params prm) {
   using namespace tc;
+  using L = K2Smem<kTerms>;
+  static_assert(kTerms < 3 || (kPerformer && kD == 64), "room for the third terms");
+  constexpr bool kSplit = kTerms > 0;
+  constexpr int kATerms = kTerms == 3 ? 3 : 2;
   constexpr int KB = kK2BlockElems / kD;                  // keys per block
   constexpr int kq = kD / 64;                             // 64-wide blocks of the head dimension
   constexpr uint32_t kSlab = KB * 128;                    // bytes of one 64-column slab of a term
@@ -112,7 +138,7 @@ k2_key_side(const __grid_constant__ CUtensorMap tmW, const K2Params prm) {
   extern __shared__ uint8_t smem_raw[];
   const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u;
   uint8_t* base_ptr = smem_raw + (base - smem_u32(smem_raw));
-  const uint32_t bar_w = base + kK2Bars, bar_l = bar_w + 8, bar_o = bar_w + 16, tmem_slot = bar_w + 24;
+  const uint32_t bar_w = base + L::bars, bar_l = bar_w + 8, bar_o = bar_w + 16, tmem_slot = bar_w + 24;
   __shared__ int abort_flag;
   __shared__ uint32_t tmem_base_shared;
   __shared__ float red_max[4][128], red_sum[4][128];
@@ -148,18 +174,18 @@ k2_key_side(const __grid_constant__ CUtensorMap tmW, const K2Params prm) {
   if (kPerformer) {
     // A operand of the bias step: [128 x 16] bf16, columns 0..2 = 1, no swizzle
     // (element (r, c) at (r/8)*256 + (c/8)*128 + (r%8)*16 + (c%8)*2 bytes)
-    uint32_t* ones = reinterpret_cast<uint32_t*>(base_ptr + kK2Ones);
+    uint32_t* ones = reinterpret_cast<uint32_t*>(base_ptr + L::ones);
     for (int e = tid; e < 1024; e += kK2Threads) {
       const int c = (e & 3) + ((e >> 5) & 1) * 4;            // which pair of columns
       ones[e] = c == 0 ? 0x3f803f80u : (c == 1 ? 0x00003f80u : 0u);
     }
   } else {
     // B operand of z: [16 x 64 keys] fp16, K-major, no swizzle: row 0 all ones, (c, n) at (c/8)*1024 + (n/8)*128 + (c%8)*16 + (n%8)*2
-    uint32_t* ones = reinterpret_cast<uint32_t*>(base_ptr + kK2Ones);
+    uint32_t* ones = reinterpret_cast<uint32_t*>(base_ptr + L::ones);
     if (tid < 512) ones[tid] = (tid < 256 && (tid & 31) < 4) ? (kSplit ? 0x3f803f80u : 0x3c003c00u) : 0u;
     // d = 64: features 64..127 of the f tile (its second slab) do not exist (kSplit: they are whatever lies there, and not read out)
     if (kD == 64 && !kSplit) {
-      uint4* z4 = reinterpret_cast<uint4*>(base_ptr + kK2K3 + kSlab);
+      uint4* z4 = reinterpret_cast<uint4*>(base_ptr + L::k3 + kSlab);
       for (int e = tid; e < (int)(kSlab / 16); e += kK2Threads) z4[e] = make_uint4(0u, 0u, 0u, 0u);
     }
   }
@@ -218,17 +244,11 @@ k2_key_side(const __grid_constant__ CUtensorMap tmW, const K2Params prm) {
 #pragma unroll
       for (int t = 0; t < kIters; ++t) {
         const int r = crow + t * 16 * kRpi;
-        float x = kx[t].x, y = kx[t].y, z = kx[t].z, w = kx[t].w;
+        const float x = kx[t].x, y = kx[t].y, z = kx[t].z, w = kx[t].w;
         sq[t] = fmaf(x, x, fmaf(y, y, fmaf(z, z, w * w)));
-        const uint32_t off = base + kK2K3 + coff + r * 128 + ((cchunk ^ (r & 7)) << 4);
-        // packed conversions: one instruction rounds two values; a bf16 is the top half of an fp32
+        const uint32_t off = base + L::k3 + coff + r * 128 + ((cchunk ^ (r & 7)) << 4);
 #pragma unroll
-        for (int s3 = 0; s3 < 3; ++s3) {
-          const uint32_t h0 = pack_bf16x2(x, y), h1 = pack_bf16x2(z, w);
-          st_shared_v2(off + s3 * 32768, h0, h1);
-          x -= __uint_as_float(h0 << 16); y -= __uint_as_float(h0 & 0xffff0000u);
-          z -= __uint_as_float(h1 << 16); w -= __uint_as_float(h1 & 0xffff0000u);
-        }
+        for (int s3 = 0; s3 < 3; ++s3) k2_put_term(off + s3 * 32768, kx[t]);
       }
       load_values();
       // |k'_r|^2 of the eight rows over the lanes that share them, halving the number of rows per lane on the way.  The
@@ -254,7 +274,7 @@ k2_key_side(const __grid_constant__ CUtensorMap tmW, const K2Params prm) {
         const __nv_bfloat16 g0 = __float2bfloat16_rn(bb);  bb -= __bfloat162float(g0);
         const __nv_bfloat16 g1 = __float2bfloat16_rn(bb);  bb -= __bfloat162float(g1);
         const __nv_bfloat16 g2 = __float2bfloat16_rn(bb);
-        uint4* na = reinterpret_cast<uint4*>(base_ptr + kK2Nrm + (r >> 3) * 256 + (r & 7) * 16);
+        uint4* na = reinterpret_cast<uint4*>(base_ptr + L::nrm + (r >> 3) * 256 + (r & 7) * 16);
         na[0] = make_uint4((uint32_t)__bfloat16_as_ushort(g0) | ((uint32_t)__bfloat16_as_ushort(g1) << 16),
                            (uint32_t)__bfloat16_as_ushort(g2), 0u, 0u);
         na[8] = make_uint4(0u, 0u, 0u, 0u);
@@ -270,11 +290,11 @@ k2_key_side(const __grid_constant__ CUtensorMap tmW, const K2Params prm) {
         for (int s3 = 0; s3 < 3; ++s3)
           for (int kb = 0; kb < kq; ++kb) {
             const uint64_t ad = make_sdesc(base + kb * 16384, 16, 1024, kSwizzle128);
-            const uint64_t bd = make_sdesc(base + kK2K3 + s3 * 32768 + kb * kSlab, 16, 1024, kSwizzle128);
+            const uint64_t bd = make_sdesc(base + L::k3 + s3 * 32768 + kb * kSlab, 16, 1024, kSwizzle128);
             mma_ss_x4(tmem, ad, bd, 2, 2, idesc1, (s3 > 0 || kb > 0) ? 1u : 0u);
           }
-        const uint64_t ad = make_sdesc(base + kK2Ones, 128, 256, kSwizzleNone);
-        const uint64_t bd = make_sdesc(base + kK2Nrm, 128, 256, kSwizzleNone);
+        const uint64_t ad = make_sdesc(base + L::ones, 128, 256, kSwizzleNone);
+        const uint64_t bd = make_sdesc(base + L::nrm, 128, 256, kSwizzleNone);
         mma_ss(tmem, ad, bd, idesc1, 1u);
         mma_commit(bar_l);
       }
@@ -288,12 +308,11 @@ k2_key_side(const __grid_constant__ CUtensorMap tmW, const K2Params prm) {
         const float x = kx[t].x, y = kx[t].y, z = kx[t].z, w = kx[t].w;
         const float f0 = keep * (fmaxf(x, 0.f) + __expf(fminf(x, 0.f))), f1 = keep * (fmaxf(y, 0.f) + __expf(fminf(y, 0.f)));
         const float f2 = keep * (fmaxf(z, 0.f) + __expf(fminf(z, 0.f))), f3 = keep * (fmaxf(w, 0.f) + __expf(fminf(w, 0.f)));
-        const uint32_t off = base + kK2K3 + coff + r * 128 + ((cchunk ^ (r & 7)) << 4);
+        const uint32_t off = base + L::k3 + coff + r * 128 + ((cchunk ^ (r & 7)) << 4);
         if constexpr (kSplit) {
-          const uint32_t h0 = pack_bf16x2(f0, f1), h1 = pack_bf16x2(f2, f3);
-          st_shared_v2(off, h0, h1);
-          st_shared_v2(off + 32768, pack_bf16x2(f0 - __uint_as_float(h0 << 16), f1 - __uint_as_float(h0 & 0xffff0000u)),
-                       pack_bf16x2(f2 - __uint_as_float(h1 << 16), f3 - __uint_as_float(h1 & 0xffff0000u)));
+          float4 f = make_float4(f0, f1, f2, f3);
+#pragma unroll
+          for (int s2 = 0; s2 < 2; ++s2) k2_put_term(off + s2 * 32768, f);
         } else {
           st_shared_v2(off, half2_bits(__floats2half2_rn(f0, f1)), half2_bits(__floats2half2_rn(f2, f3)));
         }
@@ -303,12 +322,10 @@ k2_key_side(const __grid_constant__ CUtensorMap tmW, const K2Params prm) {
 #pragma unroll
     for (int t = 0; t < kIters; ++t) {
       const int r = crow + t * 16 * kRpi;
-      const uint32_t off = base + kK2V2 + coff + r * 128 + ((cchunk ^ (r & 7)) << 4);
+      const uint32_t off = base + L::v + coff + r * 128 + ((cchunk ^ (r & 7)) << 4);
       if constexpr (kSplit) {
-        const uint32_t h0 = pack_bf16x2(vx[t].x, vx[t].y), h1 = pack_bf16x2(vx[t].z, vx[t].w);
-        st_shared_v2(off, h0, h1);
-        st_shared_v2(off + 32768, pack_bf16x2(vx[t].x - __uint_as_float(h0 << 16), vx[t].y - __uint_as_float(h0 & 0xffff0000u)),
-                     pack_bf16x2(vx[t].z - __uint_as_float(h1 << 16), vx[t].w - __uint_as_float(h1 & 0xffff0000u)));
+#pragma unroll
+        for (int s3 = 0; s3 < kTerms; ++s3) k2_put_term(off + s3 * 32768, vx[t]);
       } else {
         const __half2 hi0 = __floats2half2_rn(vx[t].x, vx[t].y), hi1 = __floats2half2_rn(vx[t].z, vx[t].w);
         const float2 b0 = __half22float2(hi0), b1 = __half22float2(hi1);
@@ -350,21 +367,31 @@ k2_key_side(const __grid_constant__ CUtensorMap tmW, const K2Params prm) {
       float part = 0.f;
       if (have) {
         auto weigh = [&](const uint32_t (&r)[32], uint32_t col) {
-          uint32_t h[16];
           if constexpr (kSplit) {
-            uint32_t lo[16];
 #pragma unroll
-            for (int e = 0; e < 16; ++e) {
-              // (the difference first: the rounding of max * log2 e would go into b_i)
-              const float w0 = k2_ex2((__uint_as_float(r[2 * e]) - new_max) * kLog2e);
-              const float w1 = k2_ex2((__uint_as_float(r[2 * e + 1]) - new_max) * kLog2e);
-              h[e] = pack_bf16x2(w0, w1);
-              const float h0 = __uint_as_float(h[e] << 16), h1 = __uint_as_float(h[e] & 0xffff0000u);
-              lo[e] = pack_bf16x2(w0 - h0, w1 - h1);
-              part += (h0 + __uint_as_float(lo[e] << 16)) + (h1 + __uint_as_float(lo[e] & 0xffff0000u));
+            for (int c = 0; c < 16; c += 8) {
+              uint32_t t0[8], t1[8];
+              [[maybe_unused]] uint32_t t2[8];
+#pragma unroll
+              for (int e = 0; e < 8; ++e) {
+                // (the difference first: the rounding of max * log2 e would go into b_i)
+                float w0 = k2_ex2((__uint_as_float(r[2 * (c + e)]) - new_max) * kLog2e);
+                float w1 = k2_ex2((__uint_as_float(r[2 * (c + e) + 1]) - new_max) * kLog2e);
+                if (kTerms == 3) part += w0 + w1;
+                t0[e] = pack_bf16x2(w0, w1);
+                const float h0 = __uint_as_float(t0[e] << 16), h1 = __uint_as_float(t0[e] & 0xffff0000u);
+                w0 -= h0; w1 -= h1;
+                t1[e] = pack_bf16x2(w0, w1);
+                const float l0 = __uint_as_float(t1[e] << 16), l1 = __uint_as_float(t1[e] & 0xffff0000u);
+                if (kTerms == 2) part += (h0 + l0) + (h1 + l1);
+                else t2[e] = pack_bf16x2(w0 - l0, w1 - l1);
+              }
+              tmem_st8(lane_base + col + c, t0);               // (L has been read by everybody: there is room for two)
+              tmem_st8(lane_base + KB / 2 + col + c, t1);
+              if (kTerms == 3) tmem_st8(lane_base + kK2ZCol + col + c, t2);
             }
-            tmem_st16(lane_base + KB / 2 + col, lo);          // (L has been read by everybody: there is room for both)
           } else {
+            uint32_t h[16];
 #pragma unroll
             for (int e = 0; e < 16; ++e) {
               const __half2 hh = __floats2half2_rn(k2_ex2(fmaf(__uint_as_float(r[2 * e]), kLog2e, -shift)),
@@ -373,8 +400,8 @@ k2_key_side(const __grid_constant__ CUtensorMap tmW, const K2Params prm) {
               part += back.x + back.y;
               h[e] = half2_bits(hh);
             }
+            tmem_st16(lane_base + col, h);
           }
-          tmem_st16(lane_base + col, h);
         };
         weigh(ra, (uint32_t)(qd * kKeysPer / 2));
         if (kKeysPer == 64) weigh(rb, (uint32_t)(qd * kKeysPer / 2 + 16));
@@ -389,32 +416,38 @@ k2_key_side(const __grid_constant__ CUtensorMap tmW, const K2Params prm) {
       tcgen05_fence_after();
       const uint32_t first = (kPerformer || b == b_begin) ? 0u : 1u;
       for (int q4 = 0; q4 < (live >> 6); ++q4) {
-        for (int s2 = 0; s2 < 2; ++s2) {
-          const uint64_t bd = make_sdesc(base + kK2V2 + s2 * 32768 + q4 * 8192, kSlab, 1024, kSwizzle128);
-          const uint32_t add = (q4 > 0 || s2 > 0) ? 1u : first;
-          if constexpr (kSplit && !kPerformer) {
-            constexpr uint32_t idesc = make_idesc(kFmtBF16, 1, 1, 128, kD);
-            mma_ss_x4(tmem + kK2OCol, make_sdesc(base + kK2K3 + q4 * 8192, kSlab, 1024, kSwizzle128), bd, 128, 128, idesc, add);
-            if (s2 == 0)
-              mma_ss_x4(tmem + kK2OCol, make_sdesc(base + kK2K3 + 32768 + q4 * 8192, kSlab, 1024, kSwizzle128), bd, 128, 128, idesc, 1u);
-          } else if constexpr (kSplit) {
-            constexpr uint32_t idesc = make_idesc(kFmtBF16, 0, /*B MN-major*/ 1, 128, kD);
-            mma_ts_x4(tmem + kK2OCol, tmem + q4 * 32, bd, 128, idesc, add);
-            if (s2 == 0) mma_ts_x4(tmem + kK2OCol, tmem + KB / 2 + q4 * 32, bd, 128, idesc, 1u);
-          } else if (kPerformer) {
-            mma_ts_x4(tmem + kK2OCol, tmem + q4 * 32, bd, 128, make_idesc(kFmtF16, 0, /*B MN-major*/ 1, 128, kD), add);
-          } else {
-            const uint64_t ad = make_sdesc(base + kK2K3 + q4 * 8192, kSlab, 1024, kSwizzle128);
-            mma_ss_x4(tmem + kK2OCol, ad, bd, 128, 128, make_idesc(kFmtF16, 1, 1, 128, kD), add);
+        if constexpr (kSplit) {
+          // the pairs of terms (a term's weight is 2^-8 of the one before); what is left out is below 2^-16 or 2^-24
+          constexpr int kTa[6] = {0, 1, 0, 1, 0, 2}, kTb[6] = {0, 0, 1, 1, 2, 0};
+#pragma unroll
+          for (int t = 0; t < (kTerms == 3 ? 6 : 3); ++t) {
+            const uint64_t bd = make_sdesc(base + L::v + kTb[t] * 32768u + q4 * 8192, kSlab, 1024, kSwizzle128);
+            const uint32_t add = (q4 > 0 || t > 0) ? 1u : first;
+            if constexpr (kPerformer) {
+              const uint32_t at = kTa[t] == 2 ? kK2ZCol : kTa[t] * (KB / 2);
+              mma_ts_x4(tmem + kK2OCol, tmem + at + q4 * 32, bd, 128, make_idesc(kFmtBF16, 0, /*B MN-major*/ 1, 128, kD), add);
+            } else {
+              mma_ss_x4(tmem + kK2OCol, make_sdesc(base + L::k3 + kTa[t] * 32768u + q4 * 8192, kSlab, 1024, kSwizzle128), bd, 128, 128,
+                        make_idesc(kFmtBF16, 1, 1, 128, kD), add);
+            }
+          }
+        } else {
+          for (int s2 = 0; s2 < 2; ++s2) {
+            const uint64_t bd = make_sdesc(base + L::v + s2 * 32768u + q4 * 8192, kSlab, 1024, kSwizzle128);
+            const uint32_t add = (q4 > 0 || s2 > 0) ? 1u : first;
+            if (kPerformer) {
+              mma_ts_x4(tmem + kK2OCol, tmem + q4 * 32, bd, 128, make_idesc(kFmtF16, 0, /*B MN-major*/ 1, 128, kD), add);
+            } else {
+              const uint64_t ad = make_sdesc(base + L::k3 + q4 * 8192, kSlab, 1024, kSwizzle128);
+              mma_ss_x4(tmem + kK2OCol, ad, bd, 128, 128, make_idesc(kFmtF16, 1, 1, 128, kD), add);
+            }
           }
         }
         if (!kPerformer) {
-          const uint64_t ad = make_sdesc(base + kK2K3 + q4 * 8192, kSlab, 1024, kSwizzle128);
-          const uint64_t bo = make_sdesc(base + kK2Ones, 128, 1024, kSwizzleNone);
-          mma_ss_x4(tmem + kK2ZCol, ad, bo, 128, 16, make_idesc(kSplit ? kFmtBF16 : kFmtF16, 1, 0, 128, 16), q4 > 0 ? 1u : first);
-          if (kSplit)
-            mma_ss_x4(tmem + kK2ZCol, make_sdesc(base + kK2K3 + 32768 + q4 * 8192, kSlab, 1024, kSwizzle128), bo, 128, 16,
-                      make_idesc(kFmtBF16, 1, 0, 128, 16), 1u);
+          const uint64_t bo = make_sdesc(base + L::ones, 128, 1024, kSwizzleNone);
+          for (int t = 0; t < (kSplit ? 2 : 1); ++t)
+            mma_ss_x4(tmem + kK2ZCol, make_sdesc(base + L::k3 + t * 32768u + q4 * 8192, kSlab, 1024, kSwizzle128), bo, 128, 16,
+                      make_idesc(kSplit ? kFmtBF16 : kFmtF16, 1, 0, 128, 16), q4 > 0 || t > 0 ? 1u : first);
         }
       }
       mma_commit(bar_o);
@@ -474,7 +507,7 @@ k2_key_side(const __grid_constant__ CUtensorMap tmW, const K2Params prm) {
       // (RNN: z_i = 0 where every weight has underflowed; ragged lengths then have a_i = 0, as the CUDA-core kernels do)
       const float inv = 1.f / (kSplit ? fmaxf(zsum, 1.17549435e-38f) : zsum);
       if (qd == 0 && feat < p) prm.weight[(size_t)head * p + feat] = kPerformer ? run_max + (kSplit ? logf(zsum) : __logf(zsum)) : zsum;
-      __half* tile = reinterpret_cast<__half*>(base_ptr + kK2K3) + (size_t)(qd * kColsPer) * 128 + frow;
+      __half* tile = reinterpret_cast<__half*>(base_ptr + L::k3) + (size_t)(qd * kColsPer) * 128 + frow;
 #pragma unroll
       for (int c = 0; c < kColsPer; ++c) {
         acc[c] *= inv;
@@ -486,13 +519,14 @@ k2_key_side(const __grid_constant__ CUtensorMap tmW, const K2Params prm) {
         for (int c = 0; c < kColsPer; c += 4) arow[c >> 2] = make_float4(acc[c], acc[c + 1], acc[c + 2], acc[c + 3]);
       }
       if (prm.abf && feat < p)
-        k2_store_split<kColsPer, kSplit && !kPerformer>(prm.abf + ((size_t)head * 2 * p + feat) * kD + qd * kColsPer, (size_t)p * kD, acc);
+        k2_store_split<kColsPer, kSplit && !kPerformer>(prm.abf + ((size_t)head * kATerms * p + feat) * kD + qd * kColsPer,
+                                                        (size_t)p * kD, acc, kTerms == 3);
     }
     __syncthreads();
     if (ok && prm.aT16) {
       const int cpr = min(128, p - i0) >> 3;                // 16-byte pieces per row
       __half* dst = prm.aT16 + (size_t)head * kD * p + i0;
-      const uint4* tile = reinterpret_cast<const uint4*>(base_ptr + kK2K3);
+      const uint4* tile = reinterpret_cast<const uint4*>(base_ptr + L::k3);
       for (int idx = tid; idx < kD * 16; idx += kK2Threads) {
         const int c = idx >> 4, ch = idx & 15;
         if (ch < cpr) *reinterpret_cast<uint4*>(dst + (size_t)c * p + ch * 8) = tile[idx];
@@ -547,7 +581,9 @@ k2_key_side(const __grid_constant__ CUtensorMap tmW, const K2Params prm) {
           if (prm.aT16) dst[(size_t)c * p] = __float2half_rn(acc[c]);
           if (prm.a32) prm.a32[((size_t)head * p + feat) * kD + qd * kColsPer + c] = acc[c];
         }
-        if (prm.abf) k2_store_split(prm.abf + ((size_t)head * 2 * p + feat) * kD + qd * kColsPer, (size_t)p * kD, acc);
+        if (prm.abf)
+          k2_store_split(prm.abf + ((size_t)head * kATerms * p + feat) * kD + qd * kColsPer, (size_t)p * kD, acc,
+                         kSplit && kPerformer && kATerms == 3);
       }
       if (tid == 0) prm.counters[unit] = 0;
     }

@@ -25,8 +25,9 @@
 //   * What the other CTA adds to this CTA's half of dQ arrives in the P tile, once both CTAs' da have read theirs.
 // Measured at 64 heads x N = 16384, m = 256: all features in one CTA 470 us, one tile in flight 327 us, two 311 us.
 //
-// kSplit (sequence lengths that are no multiple of 8, which keep 32-bit weights): P and C as two bf16 terms each.  The
-// second terms take the P buffer and the G columns of the second group, so one tile is in flight.
+// kSplit (sequence lengths that are no multiple of 8): P and C as two bf16 terms each (16 to 17 bits; da and P^T delta have the
+// same P), a as three, for the key side subtracts what is formed from it (see k2_key_side.cuh).  The second terms take the P
+// buffer and the G columns of the second group, so one tile is in flight.
 #pragma once
 
 #include <cuda_bf16.h>
@@ -47,13 +48,14 @@ template <bool kSplit> struct K8Shape {
 };
 
 // Shared memory: a Q tile is free as soon as S is formed, a dO tile only after da.
-struct K8Smem {
+template <bool kSplit> struct K8Smem {
   static constexpr int kQ = 2, kDO = 3;                                                   // stages of 16 KB
-  static constexpr uint32_t a_hi = 0, a_lo = 16384, w = 32768, p = 49152;                 // P: 32 KB per group (kSplit: per term)
+  static constexpr uint32_t kTerms = kSplit ? 3 : 2, kGroups = kSplit ? 1 : 2;
+  static constexpr uint32_t a = 0, w = kTerms * 16384, p = w + 16384;                     // P: 32 KB per group (kSplit: per term)
   static constexpr uint32_t q = p + 65536, dout = q + kQ * 16384;
   static constexpr uint32_t delta = dout + kDO * 16384;                                   // [16 x 128] bf16 per group
-  static constexpr uint32_t stat = delta + 8192;                                          // [4 parts][128] x (maximum, sum, weighted sum) per group
-  static constexpr uint32_t bias = stat + 16384;                                          // b_i log2 e of two heads
+  static constexpr uint32_t stat = delta + kGroups * 4096;                                // [4 parts][128] x (maximum, sum, weighted sum) per group
+  static constexpr uint32_t bias = stat + kGroups * 8192;                                 // b_i log2 e of two heads
   static constexpr uint32_t bars = bias + 1024;
   static constexpr int bytes = (int)bars + 256 + 1024;
 };
@@ -68,7 +70,7 @@ k8_bwd_query_units(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
                    const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUtensorMap tmA,
                    const K7Params prm) {
   using namespace tc;
-  using L = K8Smem;
+  using L = K8Smem<kSplit>;
   constexpr int kGroups = K8Shape<kSplit>::kGroups, kThreads = K8Shape<kSplit>::kThreads;
   extern __shared__ uint8_t smem_raw[];
   const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u;
@@ -139,7 +141,7 @@ k8_bwd_query_units(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
   {
     // the delta operands [16 x 128] (K-major, no swizzle): rows 0..2 are rewritten per tile, the rest stays zero
     uint32_t* dz = reinterpret_cast<uint32_t*>(base_ptr + L::delta);
-    for (int e = tid; e < 2048; e += kThreads) dz[e] = 0u;
+    for (int e = tid; e < 1024 * kGroups; e += kThreads) dz[e] = 0u;
   }
   fence_proxy_async_smem();
   tcgen05_fence_before();
@@ -219,8 +221,8 @@ k8_bwd_query_units(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
           tcgen05_fence_after();
           const uint64_t ag = make_sdesc(base + L::dout + sd * 16384, 16, 1024, kSwizzle128);
           const uint32_t dst = tmem + kK8ColG + (uint32_t)g * 128u;
-          mma_ss_x4(dst, ag, make_sdesc(base + L::a_hi, 16, 1024, kSwizzle128), 2, 2, idescS, 0u);
-          mma_ss_x4(dst, ag, make_sdesc(base + L::a_lo, 16, 1024, kSwizzle128), 2, 2, idescS, 1u);
+          for (uint32_t t = 0; t < L::kTerms; ++t)
+            mma_ss_x4(dst, ag, make_sdesc(base + L::a + t * 16384u, 16, 1024, kSwizzle128), 2, 2, idescS, t > 0 ? 1u : 0u);
           mma_commit(bar_g + 8 * g);
         };
         if (ok) form_sg(0);
@@ -281,9 +283,9 @@ k8_bwd_query_units(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
           ok = mbar_wait(bar_req, (uint32_t)(head - head0) & 1u, prm.status, &abort_flag);
           if (!ok) break;
           if (lane == 0) {
-            mbar_arrive_expect_tx(bar_head, 32768u);
-            tma_load_3d(base + L::a_hi, &tmA, bar_head, 0, f0, head * 2);
-            tma_load_3d(base + L::a_lo, &tmA, bar_head, 0, f0, head * 2 + 1);
+            mbar_arrive_expect_tx(bar_head, L::kTerms * 16384u);
+            for (uint32_t t = 0; t < L::kTerms; ++t)
+              tma_load_3d(base + L::a + t * 16384u, &tmA, bar_head, 0, f0, head * (int)L::kTerms + (int)t);
           }
           const float* wv = prm.weight + (size_t)head * p;
           float mx = -INFINITY;

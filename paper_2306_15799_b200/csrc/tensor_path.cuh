@@ -411,11 +411,12 @@ inline size_t k2_part_floats(bool performer, int BH, int d, int k, int p) {
 }
 
 // ---- stage 2: per-feature summaries a (fp16, transposed) and weights b / z from K', V' --------
-// split: the weights inside as two bf16 terms (32-bit precision, for ragged lengths)
+// terms: the weights and V' inside as two bf16 terms (for ragged lengths; not PERFORMER with d = 128) or, PERFORMER, as three, and
+// then a as three terms too
 // chained: W is an input of a call whose chain of launches began before this kernel (it is read before the wait)
 inline int launch_k2(TensorContext& tc, bool performer, const float* kpvp, const void* W, float* weight,
                      __half* aT16, float* part, int* counters, int BH, int d, int k, int p, int* status,
-                     cudaStream_t st, int* cuda_err, float* a32 = nullptr, __nv_bfloat16* abf = nullptr, bool split = false,
+                     cudaStream_t st, int* cuda_err, float* a32 = nullptr, __nv_bfloat16* abf = nullptr, int terms = 0,
                      bool chained = true) {
   TensorMaps& tm = tc.maps;
   if (performer) {
@@ -438,14 +439,15 @@ inline int launch_k2(TensorContext& tc, bool performer, const float* kpvp, const
   prm.nsplit = (part && counters) ? k2_nsplit(tc.sm_total(), performer, BH, d, k, p) : 1;
   prm.part = part;
   prm.counters = counters;
-  auto fn = split ? (d == 64 ? (performer ? k2_key_side<true, 64, true> : k2_key_side<false, 64, true>)
-                             : (performer ? k2_key_side<true, 128, true> : k2_key_side<false, 128, true>))
-                  : (d == 64 ? (performer ? k2_key_side<true, 64> : k2_key_side<false, 64>)
-                             : (performer ? k2_key_side<true, 128> : k2_key_side<false, 128>));
-  cudaError_t e = tc.raise_smem((const void*)fn, kK2SmemBytes);
+  auto fn = terms == 3 ? k2_key_side<true, 64, 3>
+            : terms == 2 ? (performer ? k2_key_side<true, 64, 2> : (d == 64 ? k2_key_side<false, 64, 2> : k2_key_side<false, 128, 2>))
+                         : (d == 64 ? (performer ? k2_key_side<true, 64> : k2_key_side<false, 64>)
+                                    : (performer ? k2_key_side<true, 128> : k2_key_side<false, 128>));
+  const int smem = terms == 3 ? K2Smem<3>::bytes : K2Smem<0>::bytes;
+  cudaError_t e = tc.raise_smem((const void*)fn, smem);
   if (e != cudaSuccess) { *cuda_err = (int)e; (void)cudaGetLastError(); return -6; }
   // the RNN kernel ignores tmW; pass any valid map
-  e = launch_chained(chained, fn, BH * prm.ftiles * prm.nsplit, kK2Threads, kK2SmemBytes, st,
+  e = launch_chained(chained, fn, BH * prm.ftiles * prm.nsplit, kK2Threads, smem, st,
                      performer ? tm.W2.map : tm.kpvp.map, prm);
   if (e != cudaSuccess) { *cuda_err = (int)e; (void)cudaGetLastError(); return -6; }
   e = cudaGetLastError();
@@ -515,7 +517,8 @@ inline int launch_k3(TensorContext& tc, bool performer, const void* Q, const voi
 }
 
 // ---- backward of the query side: dQ, and da, e added to -----------------------------------------
-// abf: the two bf16 terms of a, [BH][2][p][d]; split: weights as two bf16 terms (RNN with d = 128: always)
+// abf: a as two bf16 terms, [BH][2][p][d], or (PERFORMER with split) three; split: weights as two (RNN with d = 128: always)
+inline int bwd_query_a_terms(bool performer, bool split) { return performer && split ? 3 : 2; }
 inline int launch_bwd_query(TensorContext& tc, bool performer, bool split, const void* Q, const void* dO, const void* W,
                             const float* weight, const __nv_bfloat16* abf, void* dQ, float* da, float* ei, int BH, int H,
                             int N, int d, int p, int* status, cudaStream_t st, int* cuda_err) {
@@ -525,7 +528,8 @@ inline int launch_bwd_query(TensorContext& tc, bool performer, bool split, const
   const unsigned bQ[3] = {64, 128, 1};
   const unsigned long long dW[2] = {(unsigned long long)d, (unsigned long long)p};
   const unsigned bW[2] = {64, 128};                       // 128 features of a CTA; rows past p read as zero
-  const unsigned long long dA[3] = {(unsigned long long)d, (unsigned long long)p, (unsigned long long)BH * 2};
+  const unsigned long long dA[3] = {(unsigned long long)d, (unsigned long long)p,
+                                    (unsigned long long)(BH * bwd_query_a_terms(performer, split))};
   const unsigned bA[3] = {64, performer ? 128u : (unsigned)d, 1};
   const CUtensorMapDataType bf = CU_TENSOR_MAP_DATA_TYPE_BFLOAT16;
   if (!encode_map(&tm.Q, bf, 2, 3, Q, dQd, bQ) || !encode_map(&tm.dO, bf, 2, 3, dO, dQd, bQ) ||
@@ -554,7 +558,7 @@ inline int launch_bwd_query(TensorContext& tc, bool performer, bool split, const
     auto fn = d == 128 ? (parts == 2 ? k4_bwd_query_wide<2> : k4_bwd_query_wide<1>)
               : split  ? (parts == 2 ? k8_bwd_query_units<2, true> : k8_bwd_query_units<1, true>)
                        : (parts == 2 ? k8_bwd_query_units<2, false> : k8_bwd_query_units<1, false>);
-    const int smem = d == 128 ? K4Smem::bytes : K8Smem::bytes;
+    const int smem = d == 128 ? K4Smem::bytes : (split ? K8Smem<true>::bytes : K8Smem<false>::bytes);
     const int threads = d == 128 ? kK7Threads : (split ? K8Shape<true>::kThreads : K8Shape<false>::kThreads);
     e = tc.raise_smem((const void*)fn, smem);
     if (e == cudaSuccess)
