@@ -89,13 +89,18 @@ k3_query_side(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ C
   extern __shared__ uint8_t smem_raw[];
   const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u;
   uint8_t* base_ptr = smem_raw + (base - smem_u32(smem_raw));
-  constexpr int d = kD;
-  const int p = kPerformer ? prm.p : kD;
+  // RNN with d = 128 takes its sizes from the launch: with constants the compiler opens the loops over d, and a CTA's first tiles wait
+  // for their instructions (us per launch, constants / sizes of the launch: 32 heads x N = 896 12.5 / 11.2, 8 x 1152 7.8 / 7.0, 64 x
+  // 4096 39.3 / 38.0)
+  constexpr bool kRuntime = !kPerformer && kD == 128;
+  const int d = kRuntime ? prm.d : kD;
+  const int p = kPerformer || kRuntime ? prm.p : kD;
   const K3Smem L = k3_smem_plan(d, p, kPerformer, kSplit);
-  constexpr int kGroups = k3_groups(kD), NS = kGroups;
+  constexpr int kGroups = k3_groups(kD);
+  const int NS = kRuntime ? L.q_stages : kGroups;
   // what a tile's row owners arrive with: their warps, or (d = 128, where that was 40.8 us for 40.3 at 64 heads x N = 4096) all of them
   constexpr int kArrivals = kD == 64 ? 4 : 128;
-  constexpr uint32_t q_stage_bytes = 128u * d * 2u;
+  const uint32_t q_stage_bytes = 128u * d * 2u;
 
   // barriers
   const uint32_t bars = base + L.bars;
@@ -103,7 +108,7 @@ k3_query_side(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ C
   const uint32_t bar_qempty = bars + 32;      // [4]   Q tile consumed (MMA commit; RNN: its readers)
   const uint32_t bar_sfull = bars + 64;       // [4]   S ready in TMEM (PERFORMER)
   const uint32_t bar_ofull = bars + 96;       // [4]   O ready in TMEM
-  const uint32_t bar_sfree = bars + 128;      // [4]   TMEM buffer read out, may be overwritten (PERFORMER)
+  const uint32_t bar_sfree = bars + 128;      // [4]   TMEM buffer read out, may be overwritten (PERFORMER waits for it)
   const uint32_t bar_pfull = bars + 160;      // [4][4] a block of 64 features of p written to TMEM by the 128 row owners (kArrivals of them)
   const uint32_t bar_wfull = bars + 288;      //       W resident
   const uint32_t bar_drained = bars + 296;    //       every MMA of the previous head is complete
@@ -169,13 +174,13 @@ k3_query_side(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ C
   __syncthreads();
   const uint32_t tmem = tmem_base_shared;
 
-  constexpr int kq = d >> 6;  // 64-wide K-blocks of the Q / W tiles
+  const int kq = d >> 6;  // 64-wide K-blocks of the Q / W tiles
   const int kp = p >> 6;      // 64-wide K-blocks of a^T
   // TMEM buffers, one per group: tile i uses buffer i % NB, its barriers flip once per NB tiles
-  constexpr int NB = kGroups;
-  constexpr int nb_shift = NB == 4 ? 2 : 1;
-  constexpr uint32_t buf_cols = 512u / NB;
-  constexpr uint32_t o_col = d == 64 ? 64u : 128u;
+  const int NB = d == 64 ? 4 : 2;
+  const int nb_shift = NB == 4 ? 2 : 1;
+  const uint32_t buf_cols = 512u / NB;
+  const uint32_t o_col = d == 64 ? 64u : 128u;
   // O occupies columns [o_col, o_col + d) of the buffer.  Where that range overlaps S (PERFORMER), the
   // second product may start only when pass 2 has consumed those columns: q_first is the first block
   // of 64 features whose completion its issuer waits for (the blocks before it need no signal).
@@ -426,7 +431,7 @@ k3_query_side(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ C
         const uint32_t tb = tmem + buf * buf_cols + lane_off + o_col;
         if (!mbar_wait(bar_ofull + 8 * buf, (j >> nb_shift) & 1, prm.status, &abort_flag)) return false;
         tcgen05_fence_after();
-        if constexpr (d == 64) {
+        if constexpr (kD == 64) {
           // the warp's 32 rows go through a 4 KB slab of shared memory (128-byte rows, 16-byte
           // chunks swizzled like the tensor map expects, so the stores do not collide) and leave as one
           // TMA store of whole lines; rows past the end of the sequence are clipped by the tensor map
@@ -471,7 +476,7 @@ k3_query_side(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ C
           tmem_ld32(tb + c + 32, rb);
           tmem_wait_ld(ra);
           tmem_wait_ld(rb);
-          if (kPerformer && c + 64 >= d) {
+          if (c + 64 >= d) {
             // everything this tile needs from TMEM is in registers: hand the buffer back before storing
             tcgen05_fence_before();
             mbar_arrive(bar_sfree + 8 * buf);
@@ -616,8 +621,6 @@ k3_query_side(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ C
           if (!ok) break;
           const uint32_t qb = base + L.q + st * q_stage_bytes;
           const float* sc = reinterpret_cast<const float*>(base_ptr + L.scale);
-          // (d = 128 unrolled: 40.4 -> 39.2 us at 64 heads x N = 4096; d = 64 has no registers for it)
-#pragma unroll (kD == 64 ? 1 : 4)
           for (int c = 0; c < d; c += 32) {
             uint32_t h[16];
             [[maybe_unused]] uint32_t lo[16];
