@@ -1110,6 +1110,11 @@ int backward_pipeline(const Problem& pr, const BackwardLayout& BL, char* ws, con
     ++*launches;
   }
   __nv_bfloat16* split = tc ? (__nv_bfloat16*)(ws + BL.split) : nullptr;
+  // RNN with d = 64 and few keys: the CUDA-core kernel's CTAs of 32 keys are one wave, and its chain is shorter.  us per launch, CUDA
+  // cores / k9: 8 heads, k = 512 7.1 / 9.9, 64 heads, k = 64 7.3 / 8.7; two waves, 16 heads, k = 512 10.3 / 9.8, 96 heads, k = 64
+  // 10.2 / 7.9.  (d = 128: 16.6 / 17.7 at 8 heads, k = 256, but 16.4 / 14.1 with k = 64.)  PERFORMER's key side on tensor cores wants its
+  // other half there too: b_i has the rounding of L as the tensor cores form it.
+  const bool few_keys = !P && pr.d == 64 && pr.BH() * (pr.k / 32) <= device_sms();
   if (tcq && P && pr.d == 64 && !ragged(pr)) {
     rc = launch_k6(*tc, W, kpvp, weight, da, ei, split, pr.BH(), pr.k, pr.p(), (int*)(ws + L.status), st, &cuda_err);
     if (rc) { g_last_cuda_error = cuda_err; return rc; }
@@ -1118,7 +1123,7 @@ int backward_pipeline(const Problem& pr, const BackwardLayout& BL, char* ws, con
     rc = launch_k10(*tc, W, kpvp, weight, da, ei, split, pr.BH(), pr.d, pr.k, pr.p(), (int*)(ws + L.status), st, &cuda_err);
     if (rc) { g_last_cuda_error = cuda_err; return rc; }
     ++*launches;
-  } else if (tcq && !P) {
+  } else if (tcq && !P && !few_keys) {
     rc = launch_k9(*tc, kpvp, weight, da, ei, split, pr.BH(), pr.d, pr.k, (int*)(ws + L.status), st, &cuda_err);
     if (rc) { g_last_cuda_error = cuda_err; return rc; }
     ++*launches;
