@@ -227,7 +227,7 @@ k5_bwd_projections(const __grid_constant__ CUtensorMap tmP0, const __grid_consta
       const uint32_t piece = base + (uint32_t)(q * 32 + lane) * 16u;
       if constexpr (kParts == 2) {
         if (part == 1) {
-          ok = mbar_wait(bar_ring, 0, p.status, &abort_flag);
+          ok = mbar_wait_cluster(bar_ring, 0, p.status, &abort_flag);
           if (!ok) break;
           const uint32_t to = map_to_cta(piece, rank), bar = map_to_cta(bar_sums, rank);
 #pragma unroll 1
@@ -244,7 +244,7 @@ k5_bwd_projections(const __grid_constant__ CUtensorMap tmP0, const __grid_consta
         }
         // every load of this CTA's ring has landed and has been read: the accumulators are complete
         if (lane == 0) {
-          mbar_arrive_remote(map_to_cta(bar_ring, 2u + rank));
+          mbar_arrive_cluster(map_to_cta(bar_ring, 2u + rank));     // (with it the ring is the other pair's to write)
           if (warp == 2) mbar_arrive_expect_tx(bar_sums, 512u * kN);
         }
         ok = mbar_wait(bar_sums, 0, p.status, &abort_flag);
