@@ -2,15 +2,18 @@
 flurka_forward and flurka_backward take their way through csrc/marshal.cpp, which does the same on the tensors themselves.
 
 Every step of the forward pass runs inside the CUDA library.  If the library has not been built
-(``python -m paper_2306_15799_b200.build``) loading raises; there is no fallback.
+(``python -m paper_2306_15799_b200.build``) loading raises; there is no fallback.  (Without the marshalling module, or with
+one that was built for another torch or Python, loading warns, and the plain calls are marshalled here too.)
 """
 from __future__ import annotations
 
 import ctypes
 import os
+import warnings
 
 import torch
 
+from . import build
 from .configs import PERFORMER, RNN
 
 IO_BF16 = 0x000
@@ -105,9 +108,7 @@ def load() -> ctypes.CDLL:
     lib.flurka_set_stage1_pairs.argtypes = [ci]
     lib.flurka_measure_ex2_rate.restype = ci
     lib.flurka_measure_ex2_rate.argtypes = [ctypes.POINTER(ctypes.c_double)]
-    from . import _marshal as marshal
-    marshal.init(ctypes.cast(lib.flurka_forward, vp).value, ctypes.cast(lib.flurka_backward, vp).value)
-    _marshal = marshal
+    _marshal = _load_marshal(lib)
     _lib = lib
     return lib
 
@@ -123,7 +124,30 @@ def version() -> int:
 _LAYOUTS = ("bhnd", "bnhd")
 
 
-def _load_marshal():
+class _NoMarshal:
+    """In place of the module: every call takes the way through this file."""
+
+    @staticmethod
+    def forward(*args):
+        return None
+
+    backward = forward
+
+
+def _load_marshal(lib):
+    try:
+        if not build.marshal_fits():
+            raise ImportError("it was built for another torch or Python, or not at all")
+        from . import _marshal as marshal
+    except ImportError as e:
+        warnings.warn("flurka: calls are marshalled in Python, _marshal.so was not loaded (%s); "
+                      "`python -m paper_2306_15799_b200.build` builds it" % e, RuntimeWarning, stacklevel=3)
+        return _NoMarshal
+    marshal.init(*[ctypes.cast(f, ctypes.c_void_p).value for f in (lib.flurka_forward, lib.flurka_backward)])
+    return marshal
+
+
+def _marshal_of_loaded_library():
     load()
     return _marshal
 
@@ -200,7 +224,7 @@ def flurka_forward(Q, K, V, E, F, W, variant, out=None, stream=None, layout="bhn
     layout: 'bhnd' for [B,H,N,d] tensors, 'bnhd' for [B,N,H,d]."""
     if out is None:
         if stream is None and layout in _LAYOUTS:
-            done = (_marshal or _load_marshal()).forward(Q, K, V, E, F, W, variant, layout == "bnhd")
+            done = (_marshal or _marshal_of_loaded_library()).forward(Q, K, V, E, F, W, variant, layout == "bnhd")
             if done is not None:
                 if done[0]:
                     raise FlurkaError(done[0], "flurka_forward")
@@ -326,7 +350,7 @@ def flurka_backward(Q, K, V, E, F, W, dO, variant, stream=None, layout="bhnd", o
     """Gradients of the forward's output with respect to Q, K, V, E, F, given dO (device tensors).
     Returns (dQ, dK, dV, dE, dF), shaped and typed like the inputs (`out`: five such tensors to write into)."""
     if out is None and stream is None and layout in _LAYOUTS:
-        done = (_marshal or _load_marshal()).backward(Q, K, V, E, F, W, variant, layout == "bnhd", dO)
+        done = (_marshal or _marshal_of_loaded_library()).backward(Q, K, V, E, F, W, variant, layout == "bnhd", dO)
         if done is not None:
             if done[0]:
                 raise FlurkaError(done[0], "flurka_backward")

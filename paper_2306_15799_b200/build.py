@@ -31,13 +31,27 @@ def is_stale() -> bool:
     return any(os.path.getmtime(p) > t for p in _deps())
 
 
+def marshal_tag() -> bytes:
+    """What the module is built for: it holds this text."""
+    import torch
+    return ("marshalling for torch %s, %s" % (torch.__version__, sys.implementation.cache_tag)).encode()
+
+
+def marshal_fits() -> bool:
+    """Whether _marshal.so is there and was built for the torch and the Python that run now."""
+    if not os.path.exists(MARSHAL):
+        return False
+    with open(MARSHAL, "rb") as f:
+        return marshal_tag() in f.read()
+
+
 def compile_marshal(source: str, target: str) -> None:
     """g++ against torch's headers: marshal.cpp -> a Python module"""
     import sysconfig
     import torch
     root = os.path.join(os.path.dirname(os.path.abspath(torch.__file__)))
     tmp = target + ".tmp.%d" % os.getpid()
-    cmd = [os.environ.get("CXX", "g++"), "-O2", "-std=c++17", "-shared", "-fPIC",
+    cmd = [os.environ.get("CXX", "g++"), "-O2", "-std=c++17", "-shared", "-fPIC", "-DFLURKA_MARSHAL_TAG=\"%s\"" % marshal_tag().decode(),
            "-D_GLIBCXX_USE_CXX11_ABI=%d" % int(torch._C._GLIBCXX_USE_CXX11_ABI),
            "-isystem", os.path.join(root, "include"), "-isystem", os.path.join(root, "include", "torch", "csrc", "api", "include"),
            "-isystem", os.path.join(os.environ.get("CUDA_HOME", "/usr/local/cuda"), "include"),
@@ -52,7 +66,7 @@ def compile_marshal(source: str, target: str) -> None:
 
 def build_marshal(force: bool = False) -> str:
     """paper_2306_15799_b200/_marshal.so"""
-    if force or not os.path.exists(MARSHAL) or os.path.getmtime(MARSHAL) < os.path.getmtime(MARSHAL_SOURCE):
+    if force or not marshal_fits() or os.path.getmtime(MARSHAL) < os.path.getmtime(MARSHAL_SOURCE):
         compile_marshal(MARSHAL_SOURCE, MARSHAL)
     return MARSHAL
 

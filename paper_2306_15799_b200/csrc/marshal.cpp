@@ -154,7 +154,7 @@ PyMethodDef kMethods[] = {
     {"forward", (PyCFunction)(void*)forward, METH_FASTCALL, "forward(Q, K, V, E, F, W, variant, bnhd)"},
     {"backward", (PyCFunction)(void*)backward, METH_FASTCALL, "backward(Q, K, V, E, F, W, variant, bnhd, dO)"},
     {nullptr, nullptr, 0, nullptr}};
-PyModuleDef kModule = {PyModuleDef_HEAD_INIT, "_marshal", nullptr, -1, kMethods, nullptr, nullptr, nullptr, nullptr};
+PyModuleDef kModule = {PyModuleDef_HEAD_INIT, "_marshal", FLURKA_MARSHAL_TAG, -1, kMethods, nullptr, nullptr, nullptr, nullptr};
 
 }  // namespace
 

@@ -4,6 +4,7 @@ import ctypes
 import importlib.util
 import os
 import re
+import sys
 
 import pytest
 import torch
@@ -154,6 +155,28 @@ def test_tensors_without_memory_are_left_to_the_python_path(cpu_marshal, transfo
     else:
         torch.func.grad(others)(Q.clone())
     assert seen and all(s is None for s in seen)
+
+
+@pytest.mark.parametrize("fault", ["built for another torch", "does not load"])
+def test_library_works_without_the_marshalling_module(monkeypatch, fault):
+    """No entry point depends on _marshal.so: the library loads with a warning, calls are checked and refused in Python."""
+    build.build()
+    if fault == "does not load":
+        monkeypatch.setitem(sys.modules, "paper_2306_15799_b200._marshal", None)
+        monkeypatch.delattr("paper_2306_15799_b200._marshal", raising=False)
+    else:
+        monkeypatch.setattr(build, "marshal_tag", lambda: b"marshalling for torch 0.0")
+        assert not build.marshal_fits()
+    monkeypatch.setattr(binding, "_lib", None)
+    monkeypatch.setattr(binding, "_marshal", None)
+    with pytest.warns(RuntimeWarning, match="_marshal.so"):
+        binding.load()
+    assert binding.version() == 100 and not binding._marshal.__name__.endswith("._marshal")
+    _, args, dO = _small_call()
+    with pytest.raises(ValueError):
+        binding.flurka_forward(*args, PERFORMER)
+    with pytest.raises(ValueError):
+        binding.flurka_backward(*args, dO, PERFORMER)
 
 
 @pytest.mark.gpu
