@@ -73,7 +73,7 @@ typedef enum {
   FLURKA_PATH_SIMT = 1,   /* fp32 CUDA-core kernels: any shape within the limits, both element types */
   FLURKA_PATH_TENSOR = 2, /* tcgen05 / TMEM / TMA kernels: bf16 only, shape rules below; else error  */
   FLURKA_PATH_TENSOR_STAGE1 = 3, /* for bisecting: tensor-core down-projection, the rest on CUDA cores (as a name that
-                                    flurka_last_path() gives: tensor-core down-projection, weights of 32 bits) */
+                                    flurka_last_path() gives: tensor-core down-projection, weights of more than 16 bits) */
   FLURKA_PATH_TENSOR_STAGE3 = 4, /* for bisecting: tensor-core query side, the rest on CUDA cores      */
   FLURKA_PATH_TENSOR_STAGE23 = 5 /* for bisecting: tensor-core key and query side, CUDA-core stage 1   */
 } flurka_path_t;
@@ -90,8 +90,8 @@ typedef enum {
  * Pointers 16-byte aligned.  The tensor-core path additionally needs bf16, d in {64, 128},
  * N % 8 == 0, k % 64 == 0 with k <= 512, and (PERFORMER) m in {64, 128, 192, 256}; other shapes run on the
  * SIMT path.  Under FLURKA_PATH_AUTO it also takes other N >= 256, with E, F copied once into rows on 16-byte
- * boundaries (in the workspace) and with weights of 32-bit precision: all three stages for PERFORMER with
- * d = 64, and (named FLURKA_PATH_TENSOR_STAGE1) for RNN, else stage 1 alone.  The call enqueues work and returns; it never
+ * boundaries (in the workspace): all three stages, with weights, V' and the key-side summaries as two bf16 terms each (16 to 17
+ * bits and fp32's range), for PERFORMER with d = 64 and (named FLURKA_PATH_TENSOR_STAGE1) for RNN; else stage 1 alone.  The call enqueues work and returns; it never
  * synchronises.  Scratch comes from the workspace set by flurka_set_workspace(), or from one the library obtains on first need and re-uses:
  * when a later problem needs more, the old block is released and a larger one obtained in stream order
  * on `stream` (cudaFreeAsync / cudaMallocAsync), so calls that share the library-owned workspace must
@@ -180,12 +180,14 @@ int flurka_forward_finish(const void* Q, const void* W, int variant, int B, int 
  * forward pass.  No output may overlap an input or another output.
  * Kernels: where flurka_forward's tensor-core path takes the shape (bf16, the rules below) the two
  * down-projections, the key-side summaries and the gradients dK, dV, dE, dF
- * (products with E, F, K, V: dK', dV' enter as two bf16 terms) run on tcgen05 kernels; so does the query side
- * (dQ and the gradients of the key-side summaries), and the key side's backward half (dK', dV' from those gradients)
- * for RNN and for PERFORMER with d = 64.  N no multiple of 8: weights keep 32 bits, as two bf16 terms on tensor cores
- * or, the key side's backward half of PERFORMER and its query side with d = 128, in fp32 on CUDA cores; the products
- * with E, F, K, V follow where they are short.  flurka_last_path() then reports FLURKA_PATH_TENSOR, or
- * FLURKA_PATH_TENSOR_STAGE1 where weights have 32 bits (ragged N, RNN with d = 128).
+ * (products with E, F, K, V: dK', dV' enter as two bf16 terms) run on tcgen05 kernels; so do the query side
+ * (dQ and the gradients of the key-side summaries) and the key side's backward half (dK', dV' from those gradients; RNN with
+ * d = 64 and few keys: on CUDA cores).  N no multiple of 8: the same where the products are long enough, but for PERFORMER with
+ * d = 128, whose key and query side run in fp32 on CUDA cores.
+ * What is held in how many bits: the query side's weights 8 (bf16), or 16 to 17 as two bf16 terms (N no multiple of 8, RNN with
+ * d = 128); the forward's key-side summaries 16 to 17, or 24 as three terms (PERFORMER, N no multiple of 8); the key side's backward
+ * half 24, or (PERFORMER with d = 64, N a multiple of 8) its weights 8.  flurka_last_path() then reports FLURKA_PATH_TENSOR, or
+ * FLURKA_PATH_TENSOR_STAGE1 where the query side's weights have more than 8 bits.
  * Everything else, and every shape under FLURKA_PATH_SIMT, runs on CUDA cores with fp32 arithmetic;
  * FLURKA_PATH_TENSOR forced on a shape without a tensor-core query side returns FLURKA_ERR_SHAPE.
  */

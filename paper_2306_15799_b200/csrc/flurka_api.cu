@@ -61,9 +61,9 @@ bool tensor_path_ok(const Problem& pr) {
   return true;
 }
 
-// Ragged lengths keep 32-bit weights: they came to the tensor cores from the CUDA-core kernels, whose weights, a and V' are
+// Ragged lengths: they came to the tensor cores from the CUDA-core kernels, whose weights, a and V' are
 // fp32, while the kernels of the other lengths round weights and a to fp16 (the backward: P, c to bf16).  Stage 1 gives
-// fp32 sums of exact products either way.  Stages 2 and 3 have a form with two bf16 terms of everything (fp32's range; error of
+// fp32 sums of exact products either way.  Stages 2 and 3 have a form with two bf16 terms of everything (16 to 17 bits, fp32's range; error of
 // the output against 64 bits as with fp32 weights, 1.649e-3 at B H = 8, N = 3001, k = m = 256, all of it the output's own
 // rounding, where fp16 weights give 1.667e-3); PERFORMER with d = 128, where those terms do not fit beside W, runs on CUDA cores.
 bool ragged(const Problem& pr) { return pr.N % 8 != 0; }
@@ -976,7 +976,7 @@ bool backward_tensor_ok(const Problem& pr) {
   return tensor_path_ok(pr) && !ragged(pr) && (pr.d == 64 || pr.kernel == FLURKA_PERFORMER);
 }
 // Shapes whose query side has a tensor-core kernel.  Beyond those above: RNN with d = 128 and ragged lengths, whose weights
-// keep 32 bits (P, c as two bf16 terms); those terms do not fit beside d = 128 and W.
+// are held in 16 to 17 bits (P, c as two bf16 terms); those terms do not fit beside d = 128 and W.
 bool backward_query_tensor_ok(const Problem& pr) {
   return tensor_path_ok(pr) && !(ragged(pr) && pr.d == 128 && pr.kernel == FLURKA_PERFORMER);
 }
@@ -1045,7 +1045,7 @@ int backward_pipeline(const Problem& pr, const BackwardLayout& BL, char* ws, con
                       void* dV, void* dE, void* dF, cudaStream_t st, int* launches, TensorContext* tc, bool tcq) {
   // tc != NULL: stage 1 and the gradients that are products with E, F, K, V run on the tensor-core kernels (exact
   // products of bf16 inputs, fp32 sums; dK', dV' as two bf16 terms), and but for ragged lengths the key side's forward
-  // half does; tcq: so do the query side and both halves of the key side at any length (but for a few
+  // half does; tcq: so do the query side and both halves of the key side at any length (but for the RNN's few
   // keys, below)
   const Layout& L = BL.L;
   float* kpvp = (float*)(ws + L.kpvp);
@@ -1230,7 +1230,7 @@ int flurka_backward(const void* Q, const void* K, const void* V, const void* E, 
   if (rc) return rc;
   ds.partial_pending = false;
   ds.timer.have = false;
-  // (TENSOR_STAGE1 wherever weights keep 32 bits, whichever kernels the key and the query side run on)
+  // (TENSOR_STAGE1 wherever weights have more than 8 bits, whichever kernels the key and the query side run on)
   ds.last_path = tc && tensor_ok ? FLURKA_PATH_TENSOR : (tc ? FLURKA_PATH_TENSOR_STAGE1 : FLURKA_PATH_SIMT);
   ds.last_launches = launches;
   ds.have_last = true;

@@ -17,7 +17,7 @@
 // RNN is bound by what its row owners issue and wait for (HBM at 96 heads x N = 4096, d = 64: 15 us).  Four groups of one tile
 // and an arrival per warp, against two groups of two tiles and one per thread: 24.3 us for 27.2 there, the call 65.3 for 68.4; twice
 // as many Q tiles in flight 24.1.
-// kSplit (RNN): lengths whose weights are kept in 32 bits (ragged N).  p as two bf16 terms, the second in the columns between
+// kSplit (RNN): ragged N.  p as two bf16 terms (16 to 17 bits), the second in the columns between
 // the first and O, times a as two bf16 terms ([feature][column], as stage 2 leaves them for the backward as well): three
 // products instead of one (low x low is 2^-18).
 // PERFORMER with d = 64 has a kernel of its own (k3_query_units.cuh), which keeps four tiles at work at a time;

@@ -19,7 +19,7 @@
 // special-function; what is left is latency: a block's round trip through two chains of products is 1000 cycles.  Three groups
 // with S of the next block formed under the exponentials of this one came out the same (108 us).
 //
-// kSplit: lengths whose weights are kept in 32 bits (ragged N).  p as two bf16 terms, which fill S's 64 columns, times a as two
+// kSplit: ragged N.  p as two bf16 terms (16 to 17 bits), which fill S's 64 columns, times a as two
 // bf16 terms ([feature][column], as stage 2 leaves them for the backward as well): three products instead of one (low x low
 // is 2^-18).  a's second term takes the room of the output slabs, so every thread stores its own row.  2 x 8 heads x N = 6001,
 // k = m = 256: the call 60.3 us, 51.9 with fp16 weights, 281 with stages 2 and 3 on CUDA cores.

@@ -9,7 +9,7 @@
 //
 // d = 64 moves 48 KB and takes 1150 cycles of MMA per tile, but a tile's chain from its loads to da is four times that: two
 // groups of eight warps (two threads per row) have a tile each.
-// kSplit (sequence lengths that are no multiple of 8, and d = 128: weights there have 32 bits): P as two bf16 terms.  With
+// kSplit (sequence lengths that are no multiple of 8, and d = 128): P as two bf16 terms, 16 to 17 bits.  With
 // d = 64 the second term takes rows 64..127 of the A operand, which has 128 rows either way: da's lanes 64..127 are its share
 // of the sums, and the flush adds both.  With d = 128 it is a second product; one group (the operands fill shared memory).
 #pragma once

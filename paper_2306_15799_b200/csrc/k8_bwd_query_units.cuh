@@ -23,7 +23,7 @@
 //     (32 cycles a step instead of 48); dQ goes over the other half.  So that every thread overwrites only columns of its
 //     own, a thread takes features 32 h .. 32 h + 31 of each half of the 128.
 //   * What the other CTA adds to this CTA's half of dQ arrives in the P tile, once both CTAs' da have read theirs.
-// Measured at 64 heads x N = 16384, m = 256: all features in one CTA 470 us, one tile in flight 327 us, two 311 us.
+// Measured at 64 heads x N = 16384, m = 256: all features in one CTA 470 us, one tile in flight 327 us, two 322 us.
 //
 // kSplit (sequence lengths that are no multiple of 8): P and C as two bf16 terms each (16 to 17 bits; da and P^T delta have the
 // same P), a as three, for the key side subtracts what is formed from it (see k2_key_side.cuh).  The second terms take the P

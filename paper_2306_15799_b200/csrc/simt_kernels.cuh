@@ -1,6 +1,6 @@
 // CUDA-core (fp32 FFMA) kernels for the three stages of the FLuRKA forward pass
 // (arxiv 2306.15799, Eq. (2)).  They serve the float32 I/O configuration, every shape the
-// tensor-core kernels do not cover, and stages 2 and 3 where those have no form with 32-bit weights.
+// tensor-core kernels do not cover, and stages 2 and 3 where those have no form with more than 16-bit weights.
 //
 // Stage 1  down-projection   K' = E K, V' = F V          (Section 2.1; sequence contraction)
 // Stage 2  key side          per feature i:  b_i = log sum_j exp(L_ji),  a_i = softmax_j(L_.i)^T V'

@@ -603,8 +603,9 @@ inline int launch_k5(TensorContext& tc, const void* E, const void* F, const void
   const bool narrow0 = 2 * groups * ((N + 255) / 256) * ((p.slabs + 3) / 4) < few;
   const int row_tiles1 = 2 * groups * ((k + 255) / 256);
   // mode 1 with so few tiles that two pairs of CTAs can share each: clusters of four, of which an SM count of 148 holds 32 at
-  // once, and enough column blocks that half of them are worth the exchange (us per launch, one pair per tile / two: 128 columns, 96 blocks,
-  // N = 1024 44 / 30; 256 columns, 96 blocks, N = 4096 52 / 47, 32 blocks, N = 3001 21 / 24)
+  // once, and enough column blocks that half of them are worth the exchange.  us per launch, one pair per tile / two, k = 256: 128 columns,
+  // N = 1024: 16 blocks 11.3 / 12.0, 20 12.1 / 12.2, 24 13.5 / 12.9, 48 22.0 / 17.7, 96 44.2 / 29.9 (N = 2048: 16 12.5 / 13.7, 24 15.0 / 14.8, 96
+  // 47 / 33); 256 columns, N = 3000: 32 21.0 / 24.0, 48 28.4 / 29.6, 64 35.4 / 34.4, 96 50 / 45 (N = 4096: 48 29.9 / 30.6, 64 37.2 / 36.1)
   const int at_once = tc.sm_count() * 32 / 148;
   const bool shared128 = row_tiles1 * ((N + 127) / 128) <= at_once && p.slabs >= 24;
   const bool shared256 = !shared128 && row_tiles1 * ((N + 255) / 256) <= at_once && p.slabs >= 64;
@@ -658,7 +659,7 @@ inline int launch_k6(TensorContext& tc, const void* W, const float* kpvp, const 
   return 0;
 }
 
-// ---- the same with weights of 32 bits
+// ---- the same with 24 bits
 inline int launch_k10(TensorContext& tc, const void* W, const float* kpvp, const float* weight, const float* da,
                       const float* ei, __nv_bfloat16* split, int BH, int d, int k, int p, int* status, cudaStream_t st,
                       int* cuda_err) {

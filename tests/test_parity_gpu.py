@@ -495,7 +495,7 @@ def _ragged_path(w):
 ], ids=lambda v: v.name if hasattr(v, "name") else str(v))
 def test_ragged_lengths_on_the_tensor_path(w, layout, per_head):
     """N no multiple of 8: E, F are read from copies whose rows start on 16-byte boundaries.  (The key and query side of
-    d = 128 and RNN, which have no tensor-core form with 32-bit weights, run on CUDA cores.)"""
+    PERFORMER with d = 128 and of short RNN calls run on CUDA cores.)"""
     x = synth.make_inputs(w)
     if per_head:
         gen = torch.Generator().manual_seed(w.seed)
