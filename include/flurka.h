@@ -182,8 +182,8 @@ int flurka_forward_finish(const void* Q, const void* W, int variant, int B, int 
  * down-projections, the key-side summaries and the gradients dK, dV, dE, dF
  * (products with E, F, K, V: dK', dV' enter as two bf16 terms) run on tcgen05 kernels; so do the query side
  * (dQ and the gradients of the key-side summaries) and the key side's backward half (dK', dV' from those gradients; RNN with
- * d = 64 and few keys: on CUDA cores).  N no multiple of 8: the same where the products are long enough, but for PERFORMER with
- * d = 128, whose key and query side run in fp32 on CUDA cores.
+ * d = 64 and PERFORMER with d = 128, m = 64, both with few keys: on CUDA cores).  N no multiple of 8: the same where the products
+ * are long enough, but for PERFORMER with d = 128, whose key and query side run in fp32 on CUDA cores.
  * What is held in how many bits: the query side's weights 8 (bf16), or 16 to 17 as two bf16 terms (N no multiple of 8, RNN with
  * d = 128); the forward's key-side summaries 16 to 17, or 24 as three terms (PERFORMER, N no multiple of 8); the key side's backward
  * half 24, or (PERFORMER with d = 64, N a multiple of 8) its weights 8.  flurka_last_path() then reports FLURKA_PATH_TENSOR, or

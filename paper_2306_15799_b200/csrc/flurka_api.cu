@@ -1045,7 +1045,7 @@ int backward_pipeline(const Problem& pr, const BackwardLayout& BL, char* ws, con
                       void* dV, void* dE, void* dF, cudaStream_t st, int* launches, TensorContext* tc, bool tcq) {
   // tc != NULL: stage 1 and the gradients that are products with E, F, K, V run on the tensor-core kernels (exact
   // products of bf16 inputs, fp32 sums; dK', dV' as two bf16 terms), and but for ragged lengths the key side's forward
-  // half does; tcq: so do the query side and both halves of the key side at any length (but for the RNN's few
+  // half does; tcq: so do the query side and both halves of the key side at any length (but for few
   // keys, below)
   const Layout& L = BL.L;
   float* kpvp = (float*)(ws + L.kpvp);
@@ -1110,16 +1110,18 @@ int backward_pipeline(const Problem& pr, const BackwardLayout& BL, char* ws, con
     ++*launches;
   }
   __nv_bfloat16* split = tc ? (__nv_bfloat16*)(ws + BL.split) : nullptr;
-  // RNN with d = 64 and few keys: the CUDA-core kernel's CTAs of 32 keys are one wave, and its chain is shorter.  us per launch, CUDA
-  // cores / k9: 8 heads, k = 512 7.1 / 9.9, 64 heads, k = 64 7.3 / 8.7; two waves, 16 heads, k = 512 10.3 / 9.8, 96 heads, k = 64
-  // 10.2 / 7.9.  (d = 128: 16.6 / 17.7 at 8 heads, k = 256, but 16.4 / 14.1 with k = 64.)  PERFORMER's key side on tensor cores wants its
-  // other half there too: b_i has the rounding of L as the tensor cores form it.
-  const bool few_keys = !P && pr.d == 64 && pr.BH() * (pr.k / 32) <= device_sms();
+  // One block of features (RNN with d = 64, PERFORMER with d = 128 and m = 64) and few keys: the CUDA-core kernel's CTAs of 32 keys are one
+  // wave, and its chain is shorter.  us per launch, CUDA cores / k9: 8 heads, k = 512 7.1 / 9.9, 64 heads, k = 64 7.3 / 8.7; two waves, 16
+  // heads, k = 512 10.3 / 9.8, 96 heads, k = 64 10.2 / 7.9.  CUDA cores / k10, d = 128: 8 heads, k = 128 15.6 / 22.5, k = 64 15.5 / 16.4; two
+  // waves, 16 heads, k = 512 30.6 / 22.6; two blocks, m = 128, 8 heads, k = 64 27.7 / 21.0, k = 256 28.0 / 27.6.  (The RNN with d = 128 has
+  // two blocks: 16.6 / 17.7 at 8 heads, k = 256, but 16.4 / 14.1 with k = 64.)  PERFORMER with d = 64 and a ragged length wants its other half
+  // on tensor cores too: b_i has the rounding of L as they form it.
+  const bool few_keys = pr.d == (P ? 128 : 64) && pr.p() <= 64 && pr.BH() * (pr.k / 32) <= device_sms();
   if (tcq && P && pr.d == 64 && !ragged(pr)) {
     rc = launch_k6(*tc, W, kpvp, weight, da, ei, split, pr.BH(), pr.k, pr.p(), (int*)(ws + L.status), st, &cuda_err);
     if (rc) { g_last_cuda_error = cuda_err; return rc; }
     ++*launches;
-  } else if (tcq && P) {
+  } else if (tcq && P && !few_keys) {
     rc = launch_k10(*tc, W, kpvp, weight, da, ei, split, pr.BH(), pr.d, pr.k, pr.p(), (int*)(ws + L.status), st, &cuda_err);
     if (rc) { g_last_cuda_error = cuda_err; return rc; }
     ++*launches;
