@@ -132,6 +132,8 @@ k3_query_side(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ C
   if (threadIdx.x == 0) {
     abort_flag = 0;
     scale_epoch = 0;
+    if (kSplit)
+      for (int i = 0; i < 2 * kGroups; ++i) reinterpret_cast<uint32_t*>(base_ptr + L.scale)[128 + i * (kD / 8)] = 0u;
     for (int i = 0; i < NS; ++i) {
       mbar_init(bar_qfull + 8 * i, 1);
       mbar_init(bar_qempty + 8 * i, kPerformer ? 1 : kArrivals);
@@ -365,8 +367,13 @@ k3_query_side(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ C
           float* sc = reinterpret_cast<float*>(base_ptr + L.scale);
           const float inv = 1.f / mx;
           for (int f = lane; f < p; f += 32) sc[f] = wv[f] * inv;
+          __syncwarp();
+          if (lane == 0) {
+            __threadfence_block();
+            scale_epoch = events + 1;
+          }
           if constexpr (kSplit) {
-            uint32_t* odd = reinterpret_cast<uint32_t*>(sc) + 128 + events % (2 * kGroups) * (d / 8);
+            volatile uint32_t* odd = reinterpret_cast<volatile uint32_t*>(sc) + 128 + events % (2 * kGroups) * (d / 8);
             uint32_t any = 0u;
 #pragma unroll
             for (int q = 0; q < kD / 32; ++q) {
@@ -384,12 +391,10 @@ k3_query_side(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ C
               }
               any |= plus | minus;
             }
-            if (lane == 0) odd[0] = any;
-          }
-          __syncwarp();
-          if (lane == 0) {
-            __threadfence_block();
-            scale_epoch = events + 1;
+            if (lane == 0) {
+              __threadfence_block();
+              odd[0] = (uint32_t)(events + 1) << 1 | (any ? 1u : 0u);
+            }
           }
         }
         mbar_arrive(bar_biasready);
@@ -405,17 +410,35 @@ k3_query_side(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ C
       const float kLog2e = 1.4426950408889634f;
       int events = 0;
       bool ok = true;
+      // a count in shared memory that another warp raises (bounded)
+      auto await_count = [&](auto reached) -> bool {
+        if (reached()) return true;
+        const uint64_t t0 = global_timer_ns();
+        uint32_t spins = 0;
+        while (!reached()) {
+          if ((++spins & 63u) == 0) {
+            if (abort_flag) return false;
+            if (global_timer_ns() - t0 > kWaitLimitNs) {
+              atomicOr(prm.status, 1);
+              abort_flag = 1;
+              return false;
+            }
+          }
+        }
+        return true;
+      };
       // read-out of tile j: O / sum -> bf16 -> the output rows
       // (head and first row of the tile are tracked by the caller: no divisions on this path)
       const uint32_t slab = base + L.ostage + (uint32_t)(warp - 4) * 4096u;
       // kSplit: columns in which a is infinite, for an infinite V' has (all features with one sign: every weight is > 0).  The low
       // terms' products make them NaN, here they become infinite again, but for rows whose sum of weights is no number.
-      // Words of the head, behind the scales: any; 4 + 2 q, 5 + 2 q: +, - of column block q.  As many heads as the tiles
-      // in flight can belong to, twice.
+      // Words of the head, behind the scales: 2 x the number of heads met + any; 4 + 2 q, 5 + 2 q: +, - of column block q.  As many
+      // heads as the tiles in flight can belong to, twice.  They are there well before a tile of the head is read out.
+      const uint32_t* odd = nullptr;
+      uint32_t odd_word = 0u;
       auto infinite_columns = [&](uint32_t (&ra)[32], uint32_t (&rb)[32], int c, float sum) {
         if constexpr (kSplit) {
-          const uint32_t* odd = reinterpret_cast<const uint32_t*>(base_ptr + L.scale) + 128 + (events - 1) % (2 * kGroups) * (d / 8);
-          if (odd[0] != 0u && sum < INFINITY) {
+          if ((odd_word & 1u) != 0u && sum < INFINITY) {
             const uint4 w = *reinterpret_cast<const uint4*>(odd + 4 + (c >> 4));
 #pragma unroll
             for (int e = 0; e < 32; ++e) {
@@ -430,6 +453,11 @@ k3_query_side(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ C
         const int buf = j & (NB - 1);
         const uint32_t tb = tmem + buf * buf_cols + lane_off + o_col;
         if (!mbar_wait(bar_ofull + 8 * buf, (j >> nb_shift) & 1, prm.status, &abort_flag)) return false;
+        if constexpr (kSplit) {
+          odd = reinterpret_cast<const uint32_t*>(base_ptr + L.scale) + 128 + (events - 1) % (2 * kGroups) * (d / 8);
+          if (!await_count([&] { return (odd_word = *(volatile const uint32_t*)odd) >> 1 == (uint32_t)events; })) return false;
+          __threadfence_block();
+        }
         tcgen05_fence_after();
         if constexpr (kD == 64) {
           // the warp's 32 rows go through a 4 KB slab of shared memory (128-byte rows, 16-byte
@@ -601,21 +629,7 @@ k3_query_side(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ C
           // the second product starts only when all 128 owners have said so)
           // this head's scale vector is in place (it is replaced only after every product of this head, hence
           // every row owner's use of it, is complete)
-          if (scale_epoch < events) {
-            const uint64_t t0 = global_timer_ns();
-            uint32_t spins = 0;
-            while (scale_epoch < events) {
-              if ((++spins & 63u) == 0) {
-                if (abort_flag) { ok = false; break; }
-                if (global_timer_ns() - t0 > kWaitLimitNs) {
-                  atomicOr(prm.status, 1);
-                  abort_flag = 1;
-                  ok = false;
-                  break;
-                }
-              }
-            }
-          }
+          ok = await_count([&] { return scale_epoch >= events; });
           __threadfence_block();
           if (ok) ok = mbar_wait(bar_qfull + 8 * st, (i >> nb_shift) & 1, prm.status, &abort_flag);
           if (!ok) break;
