@@ -1111,12 +1111,13 @@ int backward_pipeline(const Problem& pr, const BackwardLayout& BL, char* ws, con
   }
   __nv_bfloat16* split = tc ? (__nv_bfloat16*)(ws + BL.split) : nullptr;
   // One block of features (RNN with d = 64, PERFORMER with d = 128 and m = 64) and few keys: the CUDA-core kernel's CTAs of 32 keys are one
-  // wave, and its chain is shorter.  us per launch, CUDA cores / k9: 8 heads, k = 512 7.1 / 9.9, 64 heads, k = 64 7.3 / 8.7; two waves, 16
-  // heads, k = 512 10.3 / 9.8, 96 heads, k = 64 10.2 / 7.9.  CUDA cores / k10, d = 128: 8 heads, k = 128 15.6 / 22.5, k = 64 15.5 / 16.4; two
+  // wave, and its chain is shorter.  (Four of them stand for one of k9's or k10's: with k = 64, half a block of keys, that is half a wave.)
+  // us per launch, CUDA cores / k9: 8 heads, k = 512 7.1 / 9.9; two waves, 16 heads, k = 512 10.3 / 9.8; the call with k = 64, N = 376: 32
+  // heads 41.5 / 42.7, 64 heads 53.6 / 51.0.  CUDA cores / k10, d = 128: 8 heads, k = 128 15.6 / 22.5, k = 64 15.5 / 16.4; two
   // waves, 16 heads, k = 512 30.6 / 22.6; two blocks, m = 128, 8 heads, k = 64 27.7 / 21.0, k = 256 28.0 / 27.6.  (The RNN with d = 128 has
   // two blocks: 16.6 / 17.7 at 8 heads, k = 256, but 16.4 / 14.1 with k = 64.)  PERFORMER with d = 64 and a ragged length wants its other half
   // on tensor cores too: b_i has the rounding of L as they form it.
-  const bool few_keys = pr.d == (P ? 128 : 64) && pr.p() <= 64 && pr.BH() * (pr.k / 32) <= device_sms();
+  const bool few_keys = pr.d == (P ? 128 : 64) && pr.p() <= 64 && pr.BH() * ((pr.k + 127) / 128) * 4 <= device_sms();
   if (tcq && P && pr.d == 64 && !ragged(pr)) {
     rc = launch_k6(*tc, W, kpvp, weight, da, ei, split, pr.BH(), pr.k, pr.p(), (int*)(ws + L.status), st, &cuda_err);
     if (rc) { g_last_cuda_error = cuda_err; return rc; }
